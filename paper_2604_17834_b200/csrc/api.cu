@@ -11,6 +11,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "device_memory.h"
 #include "format.h"
 #include "kernels.h"
 #include "spmm_b200.h"
@@ -74,8 +75,7 @@ int encode_2d(CUtensorMap* map, int dtype, const void* base, uint64_t rows, uint
 template <class T>
 int upload(T** dptr, const void* src, size_t bytes) {
     *dptr = nullptr;
-    const size_t alloc = bytes ? bytes : 16;
-    if (cudaMalloc(reinterpret_cast<void**>(dptr), alloc) != cudaSuccess) return SPMM_ERR_ALLOC;
+    if (!dev_alloc_ok(dptr, bytes, nullptr)) return SPMM_ERR_ALLOC;
     if (bytes && cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return SPMM_ERR_CUDA;
     return SPMM_OK;
 }
@@ -126,16 +126,19 @@ struct spmm_handle_s {
     int32_t* d_tiles = nullptr;      // {block-row, token tile} pairs (the exported schedule)
     int32_t* d_tile_recs = nullptr;  // the kernel's records: {block-row, token tile, first block, end block}
     int32_t* d_cta_ptr = nullptr;
-    WcsrDevTask* d_tasks = nullptr;
-    int32_t* d_bin_ptr = nullptr;
-    int32_t* d_bin_tasks = nullptr;
-    int32_t* d_items = nullptr;
-    int32_t* d_fills = nullptr;
-    int32_t* d_bin_fill = nullptr;
-    int32_t* d_fills_narrow = nullptr;    // WCSR narrow-operand variant (2-byte types, height 16)
-    int32_t* d_bin_fill_narrow = nullptr;
-    uint8_t* d_grp_class = nullptr;  // WCSR: reuse class per group of four padded columns (gather hints)
-    int32_t* d_merge = nullptr;      // window | first | nparts, each [n_merge]
+    // WCSR schedule: sections of d_plan (d_grp_class: or an array of its own, d_class, from the GPU builder)
+    int32_t* d_plan = nullptr;
+    const WcsrDevTask* d_tasks = nullptr;
+    const int32_t* d_bin_ptr = nullptr;
+    const int32_t* d_bin_tasks = nullptr;
+    const int32_t* d_items = nullptr;
+    const int32_t* d_fills = nullptr;
+    const int32_t* d_bin_fill = nullptr;
+    const int32_t* d_fills_narrow = nullptr;    // WCSR narrow-operand variant (2-byte types, height 16)
+    const int32_t* d_bin_fill_narrow = nullptr;
+    uint8_t* d_class = nullptr;
+    const uint8_t* d_grp_class = nullptr;  // WCSR: reuse class per group of four padded columns (gather hints)
+    const int32_t* d_merge = nullptr;      // window | first | nparts, each [n_merge]
     int n_merge = 0;
     int* d_status = nullptr;
 
@@ -171,31 +174,16 @@ namespace {
 void free_handle(spmm_handle_s* h) {
     if (!h) return;
     if (!h->host_only) {
-        cudaFree(h->d_ptr);
-        cudaFree(h->d_idx);
-        cudaFree(h->d_vals);
-        cudaFree(h->d_order);
-        cudaFree(h->d_tiles);
-        cudaFree(h->d_tile_recs);
-        cudaFree(h->d_cta_ptr);
-        cudaFree(h->d_kmerge);
-        cudaFree(h->d_sidx);
-        cudaFree(h->d_srows);
-        cudaFree(h->d_svals);
-        cudaFree(h->d_stile_recs);
-        cudaFree(h->d_scta_ptr);
-        cudaFree(h->d_tasks);
-        cudaFree(h->d_bin_ptr);
-        cudaFree(h->d_bin_tasks);
-        cudaFree(h->d_items);
-        cudaFree(h->d_fills);
-        cudaFree(h->d_bin_fill);
-        cudaFree(h->d_fills_narrow);
-        cudaFree(h->d_bin_fill_narrow);
-        cudaFree(h->d_grp_class);
-        cudaFree(h->d_merge);
-        cudaFree(h->d_status);
-        cudaFree(h->d_partial);
+        // the handle's last run may still be on the GPU; its memory goes back to the pool of its own device
+        int dev = -1;
+        const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != h->device && cudaSetDevice(h->device) == cudaSuccess;
+        cudaDeviceSynchronize();
+        void* const arrays[] = {
+            h->d_ptr, h->d_idx, h->d_vals, h->d_order, h->d_tiles, h->d_tile_recs, h->d_cta_ptr, h->d_kmerge,
+            h->d_sidx, h->d_srows, h->d_svals, h->d_stile_recs, h->d_scta_ptr, h->d_status, h->d_partial,
+            h->d_plan, h->d_class};
+        for (void* ptr : arrays) dev_free(ptr, nullptr);
+        if (other) cudaSetDevice(dev);
         cudaFree(h->d_Bstage);
         cudaFree(h->d_Cstage);
         if (h->s_in) cudaStreamDestroy(h->s_in);
@@ -217,13 +205,15 @@ int device_setup(spmm_handle_s* h, const spmm_opts_t* opts) {
     }
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
-    cudaDeviceProp prop;
-    if (cudaGetDeviceProperties(&prop, dev) != cudaSuccess) return SPMM_ERR_CUDA;
-    if (prop.major != 10) return SPMM_ERR_UNSUPPORTED;   // sm_100a code only
+    int major = 0, sms = 0;
+    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return SPMM_ERR_CUDA;
+    if (major != 10) return SPMM_ERR_UNSUPPORTED;   // sm_100a code only
     h->device = dev;
-    h->sms = prop.multiProcessorCount;
+    h->sms = sms;
     h->n_ctas = (opts && opts->n_ctas > 0) ? opts->n_ctas : h->sms;
-    if (cudaMalloc(reinterpret_cast<void**>(&h->d_status), 4 * sizeof(int)) != cudaSuccess) return SPMM_ERR_ALLOC;
+    if (!dev_alloc_ok(&h->d_status, 4 * sizeof(int), nullptr)) return SPMM_ERR_ALLOC;
     if (cudaMemset(h->d_status, 0, 4 * sizeof(int)) != cudaSuccess) return SPMM_ERR_CUDA;
     return SPMM_OK;
 }
@@ -377,48 +367,67 @@ int create_bcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     return SPMM_OK;
 }
 
-// Uploads the schedule arrays of a WCSR handle (everything but the three format arrays).
+// Uploads the schedule arrays of a WCSR handle (everything but the three format arrays): one allocation, one copy.
 int upload_wcsr_plan(spmm_handle_s* h) {
     const WcsrHost& f = h->wcsr;
-    std::vector<WcsrDevTask> dt(f.tasks.size());
-    for (size_t i = 0; i < f.tasks.size(); ++i) {
-        dt[i].col_begin = f.window_row_ptr[f.tasks[i].window] + f.tasks[i].q0;
-        dt[i].count = f.tasks[i].count;
-        dt[i].window = f.tasks[i].window;
-        dt[i].slot = f.tasks[i].slot;
+    const size_t nt = f.tasks.size(), nm = f.merge_window.size(), ni = f.bin_tasks.size();
+    const bool narrow = !f.bin_fill_narrow.empty();
+    // sections in 4-byte words, each on a 16-byte boundary
+    size_t words = 0;
+    auto section = [&](size_t n) {
+        const size_t at = words;
+        words += (n + 3) / 4 * 4;
+        return at;
+    };
+    const size_t o_tasks = section(4 * nt), o_bin_ptr = section(f.bin_ptr.size()), o_bin_tasks = section(ni), o_items = section(4 * ni);
+    const size_t o_fills = section(f.fills.size()), o_bin_fill = section(f.bin_fill.size());
+    const size_t o_fills_n = section(f.fills_narrow.size()), o_bin_fill_n = section(f.bin_fill_narrow.size());
+    const size_t o_merge = section(3 * nm), o_class = section((f.grp_class.size() + 3) / 4);
+    std::vector<int32_t> w(words, 0);
+    static_assert(sizeof(WcsrDevTask) == 16, "four words per task");
+    for (size_t i = 0; i < nt; ++i) {
+        const WcsrTask& t = f.tasks[i];
+        const WcsrDevTask d = {f.window_row_ptr[t.window] + t.q0, t.count, t.window, t.slot};
+        std::memcpy(&w[o_tasks + 4 * i], &d, 16);
     }
-    const size_t nm = f.merge_window.size();
-    std::vector<int32_t> mg(3 * nm);
-    for (size_t i = 0; i < nm; ++i) {
-        mg[i] = f.merge_window[i];
-        mg[nm + i] = f.merge_first[i];
-        mg[2 * nm + i] = f.merge_nparts[i];
+    for (size_t i = 0; i < ni; ++i) {
+        const WcsrTask& t = f.tasks[f.bin_tasks[i]];
+        w[o_items + 4 * i] = t.window;
+        w[o_items + 4 * i + 1] = t.slot;
+        w[o_items + 4 * i + 2] = t.count;
     }
+    auto put = [&](size_t at, const void* src, size_t bytes) {
+        if (bytes) std::memcpy(&w[at], src, bytes);
+    };
+    put(o_bin_ptr, f.bin_ptr.data(), f.bin_ptr.size() * 4);
+    put(o_bin_tasks, f.bin_tasks.data(), ni * 4);
+    put(o_fills, f.fills.data(), f.fills.size() * 4);
+    put(o_bin_fill, f.bin_fill.data(), f.bin_fill.size() * 4);
+    put(o_fills_n, f.fills_narrow.data(), f.fills_narrow.size() * 4);
+    put(o_bin_fill_n, f.bin_fill_narrow.data(), f.bin_fill_narrow.size() * 4);
+    put(o_merge, f.merge_window.data(), nm * 4);
+    put(o_merge + nm, f.merge_first.data(), nm * 4);
+    put(o_merge + 2 * nm, f.merge_nparts.data(), nm * 4);
+    put(o_class, f.grp_class.data(), f.grp_class.size());
+    int rc = upload(&h->d_plan, w.data(), words * 4);
+    if (rc) return rc;
     h->n_merge = static_cast<int>(nm);
-    int rc = upload(&h->d_tasks, dt.data(), dt.size() * sizeof(WcsrDevTask));
-    if (!rc) rc = upload(&h->d_bin_ptr, f.bin_ptr.data(), f.bin_ptr.size() * 4);
-    if (!rc) rc = upload(&h->d_bin_tasks, f.bin_tasks.data(), f.bin_tasks.size() * 4);
-    if (!rc) {
-        std::vector<int32_t> items(4 * f.bin_tasks.size(), 0);
-        for (size_t i = 0; i < f.bin_tasks.size(); ++i) {
-            items[4 * i] = f.tasks[f.bin_tasks[i]].window;
-            items[4 * i + 1] = f.tasks[f.bin_tasks[i]].slot;
-            items[4 * i + 2] = f.tasks[f.bin_tasks[i]].count;
-        }
-        rc = upload(&h->d_items, items.data(), items.size() * 4);
+    h->d_tasks = reinterpret_cast<WcsrDevTask*>(h->d_plan + o_tasks);
+    h->d_bin_ptr = h->d_plan + o_bin_ptr;
+    h->d_bin_tasks = h->d_plan + o_bin_tasks;
+    h->d_items = h->d_plan + o_items;
+    h->d_fills = h->d_plan + o_fills;
+    h->d_bin_fill = h->d_plan + o_bin_fill;
+    if (narrow) {
+        h->d_fills_narrow = h->d_plan + o_fills_n;
+        h->d_bin_fill_narrow = h->d_plan + o_bin_fill_n;
     }
-    if (!rc) rc = upload(&h->d_fills, f.fills.data(), f.fills.size() * 4);
-    if (!rc) rc = upload(&h->d_bin_fill, f.bin_fill.data(), f.bin_fill.size() * 4);
-    if (!rc && !f.bin_fill_narrow.empty()) {
-        rc = upload(&h->d_fills_narrow, f.fills_narrow.data(), f.fills_narrow.size() * 4);
-        if (!rc) rc = upload(&h->d_bin_fill_narrow, f.bin_fill_narrow.data(), f.bin_fill_narrow.size() * 4);
+    h->d_merge = h->d_plan + o_merge;
+    if (!f.grp_class.empty()) {
+        h->d_grp_class = reinterpret_cast<const uint8_t*>(h->d_plan + o_class);
+        std::vector<uint8_t>().swap(h->wcsr.grp_class);
     }
-    if (!rc) rc = upload(&h->d_merge, mg.data(), mg.size() * 4);
-    if (!rc && !f.grp_class.empty()) {
-        rc = upload(&h->d_grp_class, f.grp_class.data(), f.grp_class.size());
-        if (!rc) std::vector<uint8_t>().swap(h->wcsr.grp_class);
-    }
-    return rc;
+    return SPMM_OK;
 }
 
 // Option and size checks shared by the host and the device builder; on success *hp is a fresh handle.
@@ -497,7 +506,8 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     try {
         rc = build_wcsr_device(m, k, d_row_ptr, d_col_idx, static_cast<const uint8_t*>(d_vals), h->es, wh, b_col, T,
                                h->n_ctas * wcsr_bins_per_sm(h->es, wh), stream, &h->wcsr, &h->nnz, &h->d_ptr, &h->d_idx,
-                               &h->d_vals, &h->d_grp_class);
+                               &h->d_vals, &h->d_class);
+        h->d_grp_class = h->d_class;
         if (!rc) rc = upload_wcsr_plan(h);
     } catch (const std::bad_alloc&) {
         rc = SPMM_ERR_ALLOC;
@@ -729,12 +739,12 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     if (!h->host_only) {
         if (h->d_tiles) {   // a previous schedule may still be in use by a running kernel
             if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
-            cudaFree(h->d_tiles);
-            cudaFree(h->d_tile_recs);
-            cudaFree(h->d_cta_ptr);
-            cudaFree(h->d_stile_recs);
-            cudaFree(h->d_scta_ptr);
-            cudaFree(h->d_kmerge);
+            dev_free(h->d_tiles, nullptr);
+            dev_free(h->d_tile_recs, nullptr);
+            dev_free(h->d_cta_ptr, nullptr);
+            dev_free(h->d_stile_recs, nullptr);
+            dev_free(h->d_scta_ptr, nullptr);
+            dev_free(h->d_kmerge, nullptr);
             h->d_tiles = h->d_tile_recs = h->d_cta_ptr = h->d_stile_recs = h->d_scta_ptr = h->d_kmerge = nullptr;
             h->n_kmerge = 0;
             h->tmP_ok = false;
@@ -781,10 +791,11 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             rc = upload(&h->d_kmerge, mg.data(), mg.size() * 4);
             const size_t need = static_cast<size_t>(sc.n_slots) * f.b * static_cast<size_t>(N) * 4;
             if (!rc && need > h->partial_bytes) {
-                cudaFree(h->d_partial);
+                if (h->d_partial && cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
+                dev_free(h->d_partial, nullptr);
                 h->d_partial = nullptr;
                 h->partial_bytes = 0;
-                if (cudaMalloc(reinterpret_cast<void**>(&h->d_partial), need) != cudaSuccess) rc = SPMM_ERR_ALLOC;
+                if (!dev_alloc_ok(&h->d_partial, need, nullptr)) rc = SPMM_ERR_ALLOC;
                 else h->partial_bytes = need;
             }
             if (!rc) {
@@ -947,23 +958,23 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
 }
 
 // The handle's workspace for the partial tiles of split windows at dense width N (grown, never shrunk).
-int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N) {
+int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, cudaStream_t stream) {
     const size_t need = static_cast<size_t>(wcsr_workspace_bytes(h, N));
     if (need > h->partial_bytes) {
         if (h->d_partial) {
             if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
-            cudaFree(h->d_partial);
+            dev_free(h->d_partial, nullptr);
             h->d_partial = nullptr;
             h->partial_bytes = 0;
         }
-        if (cudaMalloc(reinterpret_cast<void**>(&h->d_partial), need) != cudaSuccess) return SPMM_ERR_ALLOC;
+        if (!dev_alloc_ok(&h->d_partial, need, stream)) return SPMM_ERR_ALLOC;
         h->partial_bytes = need;
     }
     return SPMM_OK;
 }
 
 int run_wcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t stream) {
-    if (int rc = ensure_wcsr_workspace(h, N)) return rc;
+    if (int rc = ensure_wcsr_workspace(h, N, stream)) return rc;
     return launch_wcsr_all(h, B, C, h->d_partial, N, stream);
 }
 
@@ -1095,7 +1106,9 @@ int spmm_prepare(spmm_handle_t h, int64_t N) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
     if (dev != h->device) return SPMM_ERR_INVALID_ARG;
-    return ensure_wcsr_workspace(h, N);
+    if (int rc = ensure_wcsr_workspace(h, N, nullptr)) return rc;
+    // (the run may use any stream: the allocation has to be complete, not only ordered on this one)
+    return cudaStreamSynchronize(nullptr) == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
 }
 
 int spmm_wcsr_run_static(spmm_handle_t h, const void* B_dev, void* C_dev, int64_t N, void* stream) {

@@ -401,6 +401,39 @@ void wcsr_reuse_classes(const int32_t* window_col_idx, int64_t P, int64_t k, std
         }
 }
 
+namespace {
+
+// The bins of the longest-processing-time rule: the lightest one (ties: the lowest index) on top.  A binary heap of
+// {load, bin} in one 64-bit key; taking the top and giving it back heavier is one sift down.
+class LightestBin {
+public:
+    static constexpr int kBinBits = 29;
+    explicit LightestBin(int n) : key_(static_cast<size_t>(n)) {
+        for (int i = 0; i < n; ++i) key_[i] = static_cast<uint64_t>(i);
+    }
+    int32_t bin() const { return static_cast<int32_t>(key_[0] & ((uint64_t{1} << kBinBits) - 1)); }
+    int64_t load() const { return static_cast<int64_t>(key_[0] >> kBinBits); }
+    void add(int64_t cost) {
+        const uint64_t k = key_[0] + (static_cast<uint64_t>(cost) << kBinBits);
+        const size_t n = key_.size();
+        size_t i = 0;
+        for (;;) {
+            size_t c = 2 * i + 1;
+            if (c >= n) break;
+            c += c + 1 < n && key_[c + 1] < key_[c];
+            if (key_[c] >= k) break;
+            key_[i] = key_[c];
+            i = c;
+        }
+        key_[i] = k;
+    }
+
+private:
+    std::vector<uint64_t> key_;     // load << kBinBits | bin; loads stay below 2^35 (columns are int32, a task has 8 or more)
+};
+
+}  // namespace
+
 // Largest bin load of the longest-processing-time assignment when windows are cut into chunks of T.
 static int64_t lpt_max_load(const std::vector<int32_t>& window_row_ptr, int64_t nwin, int T, int n_bins) {
     std::vector<int32_t> counts;
@@ -410,14 +443,11 @@ static int64_t lpt_max_load(const std::vector<int32_t>& window_row_ptr, int64_t 
         if (len > 0) counts.push_back(len);
     }
     std::sort(counts.begin(), counts.end(), std::greater<int32_t>());
-    std::priority_queue<int64_t, std::vector<int64_t>, std::greater<int64_t>> heap;
-    for (int j = 0; j < n_bins; ++j) heap.push(0);
+    LightestBin bins(n_bins);
     int64_t mx = 0;
     for (int32_t c : counts) {
-        const int64_t l = heap.top() + c + kTaskFixedCost;
-        heap.pop();
-        heap.push(l);
-        mx = std::max(mx, l);
+        mx = std::max(mx, bins.load() + c + kTaskFixedCost);
+        bins.add(c + kTaskFixedCost);
     }
     return mx;
 }
@@ -439,6 +469,7 @@ int default_split_cols(const std::vector<int32_t>& window_row_ptr, int64_t nwin,
 
 int plan_wcsr(WcsrHost* out, int T, int n_bins, int es) {
     const int64_t nwin = out->nwin, P = out->P;
+    if (n_bins >= 1 << LightestBin::kBinBits) return SPMM_ERR_TOO_LARGE;
     if (T == 0) T = default_split_cols(out->window_row_ptr, nwin, P, n_bins);
     out->T = T;
 
@@ -484,18 +515,13 @@ int plan_wcsr(WcsrHost* out, int T, int n_bins, int es) {
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(),
                      [&](int32_t x, int32_t y) { return out->tasks[x].count > out->tasks[y].count; });
-    using Load = std::pair<int64_t, int32_t>;   // (load, bin): smallest load, then lowest bin, on top
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-    for (int32_t bsel = 0; bsel < n_bins; ++bsel) heap.push(Load(0, bsel));
+    LightestBin bins(n_bins);
     std::vector<int32_t> bin_of(static_cast<size_t>(ntasks));
     std::vector<int32_t> bin_count(static_cast<size_t>(n_bins), 0);
     for (int32_t t : order) {
-        Load top = heap.top();
-        heap.pop();
-        bin_of[t] = top.second;
-        bin_count[top.second]++;
-        top.first += out->tasks[t].count + kTaskFixedCost;
-        heap.push(top);
+        bin_of[t] = bins.bin();
+        bin_count[bins.bin()]++;
+        bins.add(out->tasks[t].count + kTaskFixedCost);
     }
     out->bin_ptr.assign(static_cast<size_t>(n_bins) + 1, 0);
     for (int j = 0; j < n_bins; ++j) out->bin_ptr[j + 1] = out->bin_ptr[j] + bin_count[j];

@@ -25,7 +25,9 @@
 #include <cstring>
 #include <numeric>
 #include <algorithm>
+#include <new>
 
+#include "device_memory.h"
 #include "format.h"
 #include "kernels.h"
 #include "spmm_b200.h"
@@ -56,6 +58,41 @@ __global__ void csr_check_cols_kernel(int64_t m, int64_t k, const int64_t* row_p
             prev = c;
         }
     }
+}
+
+// The same rules entry by entry, whatever the row lengths (a row of 5000 entries kept one thread of the kernel
+// above busy for 140 us): *bad is set when any entry breaks one; the row-wise kernel then finds the error code.
+// A column that does not ascend must be the first of its row: its position is looked up in row_ptr.
+__global__ void csr_check_entries_kernel(int64_t m, int64_t k, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, int* bad) {
+    const int64_t nnz = row_ptr[m];
+    for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < nnz;
+         p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t c = col_idx[p];
+        bool ok = c >= 0 && c < k;
+        if (ok && p > 0 && c <= col_idx[p - 1]) {
+            int64_t lo = 0, hi = m;                      // first row that starts at or behind p
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (row_ptr[mid] < p) lo = mid + 1; else hi = mid;
+            }
+            ok = row_ptr[lo] == p;
+        }
+        if (!ok) *bad = 1;
+    }
+}
+
+// Checks the columns of a CSR matrix whose row pointers are known to be sound; synchronises `st`.
+int check_csr_cols(int64_t m, int64_t k, int64_t nnz, const int64_t* d_row_ptr, const int32_t* d_col_idx, int* d_bad, int* d_err, cudaStream_t st) {
+    const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 8192));
+    csr_check_entries_kernel<<<entry_grid, 256, 0, st>>>(m, k, d_row_ptr, d_col_idx, d_bad);
+    int bad = 0, err = 0;
+    if (cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+        return SPMM_ERR_CUDA;
+    if (!bad) return SPMM_OK;
+    csr_check_cols_kernel<<<static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048)), 256, 0, st>>>(m, k, d_row_ptr, d_col_idx, d_err);
+    if (cudaMemcpyAsync(&err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+        return SPMM_ERR_CUDA;
+    return err;
 }
 
 // Shared-memory bitmap of the block columns of block-row I.
@@ -231,9 +268,9 @@ int stack_bcsr_device(const uint8_t* d_blocks, const BcsrStack& st, int b, int e
     const int pieces = b * b * es / 16;
     const int64_t n_pieces = st.ns * st.R * pieces;
     int32_t* d_src = nullptr;
-    if (cudaMalloc(reinterpret_cast<void**>(&d_src), st.src.size() * 4) != cudaSuccess) return SPMM_ERR_ALLOC;
-    if (cudaMalloc(reinterpret_cast<void**>(d_stacked), static_cast<size_t>(n_pieces) * 16) != cudaSuccess) {
-        cudaFree(d_src);
+    if (!dev_alloc_ok(&d_src, st.src.size() * 4, nullptr)) return SPMM_ERR_ALLOC;
+    if (!dev_alloc_ok(d_stacked, static_cast<size_t>(n_pieces) * 16, nullptr)) {
+        dev_free(d_src, nullptr);
         return SPMM_ERR_ALLOC;
     }
     int rc = SPMM_OK;
@@ -245,8 +282,8 @@ int stack_bcsr_device(const uint8_t* d_blocks, const BcsrStack& st, int b, int e
                                                                    reinterpret_cast<uint4*>(*d_stacked), st.R, pieces, n_pieces);
         if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) rc = SPMM_ERR_CUDA;
     }
-    cudaFree(d_src);
-    if (rc) { cudaFree(*d_stacked); *d_stacked = nullptr; }
+    dev_free(d_src, nullptr);
+    if (rc) { dev_free(*d_stacked, nullptr); *d_stacked = nullptr; }
     return rc;
 }
 
@@ -267,23 +304,23 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     out->nbr = nbr;
     out->nbc = nbc;
 
-    int* d_flags = nullptr;                     // [0] CSR error code (min), [1] scan overflow
+    int* d_flags = nullptr;                     // [0] CSR error code (min), [1] scan overflow, [2] a bad entry
     int32_t* d_counts = nullptr;
     auto fail = [&](int code) {
-        cudaFree(d_flags);
-        cudaFree(d_counts);
-        cudaFree(*d_block_row_ptr);
-        cudaFree(*d_block_col_idx);
-        cudaFree(*d_blocks);
+        dev_free(d_flags, st);
+        dev_free(d_counts, st);
+        dev_free(*d_block_row_ptr, st);
+        dev_free(*d_block_col_idx, st);
+        dev_free(*d_blocks, st);
         *d_block_row_ptr = nullptr;
         *d_block_col_idx = nullptr;
         *d_blocks = nullptr;
         return code;
     };
-    if (cudaMalloc(reinterpret_cast<void**>(&d_flags), 2 * sizeof(int)) != cudaSuccess) return fail(SPMM_ERR_ALLOC);
-    if (cudaMemsetAsync(d_flags, 0, 2 * sizeof(int), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    if (cudaMalloc(reinterpret_cast<void**>(&d_counts), static_cast<size_t>(nbr + 1) * 4) != cudaSuccess) return fail(SPMM_ERR_ALLOC);
-    if (cudaMalloc(reinterpret_cast<void**>(d_block_row_ptr), static_cast<size_t>(nbr + 1) * 4) != cudaSuccess) return fail(SPMM_ERR_ALLOC);
+    if (!dev_alloc_ok(&d_flags, 4 * sizeof(int), st)) return fail(SPMM_ERR_ALLOC);
+    if (cudaMemsetAsync(d_flags, 0, 4 * sizeof(int), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
+    if (!dev_alloc_ok(&d_counts, static_cast<size_t>(nbr + 1) * 4, st)) return fail(SPMM_ERR_ALLOC);
+    if (!dev_alloc_ok(d_block_row_ptr, static_cast<size_t>(nbr + 1) * 4, st)) return fail(SPMM_ERR_ALLOC);
 
     // 1. the CSR must be canonical (the count and fill passes rely on in-range columns)
     int64_t nnz = 0;
@@ -298,10 +335,7 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     if (flags[0] != 0) return fail(flags[0]);
     if (nnz < 0 || (nnz > 0 && (!d_col_idx || !d_vals))) return fail(SPMM_ERR_INVALID_ARG);
     if (nnz > 0) {
-        csr_check_cols_kernel<<<check_grid, 256, 0, st>>>(m, k, d_row_ptr, d_col_idx, d_flags);
-        if (cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        if (cudaStreamSynchronize(st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        if (flags[0] != 0) return fail(flags[0]);
+        if (int rc = check_csr_cols(m, k, nnz, d_row_ptr, d_col_idx, d_flags + 2, d_flags, st)) return fail(rc);
     }
     *nnz_out = nnz;
 
@@ -325,8 +359,8 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     // 4. block columns and values
     const size_t tile_bytes = static_cast<size_t>(b) * b * es;
     const size_t idx_bytes = static_cast<size_t>(nnzb) * 4, val_bytes = static_cast<size_t>(nnzb) * tile_bytes;
-    if (cudaMalloc(reinterpret_cast<void**>(d_block_col_idx), idx_bytes ? idx_bytes : 16) != cudaSuccess) return fail(SPMM_ERR_ALLOC);
-    if (cudaMalloc(reinterpret_cast<void**>(d_blocks), val_bytes ? val_bytes : 16) != cudaSuccess) return fail(SPMM_ERR_ALLOC);
+    if (!dev_alloc_ok(d_block_col_idx, idx_bytes ? idx_bytes : 16, st)) return fail(SPMM_ERR_ALLOC);
+    if (!dev_alloc_ok(d_blocks, val_bytes ? val_bytes : 16, st)) return fail(SPMM_ERR_ALLOC);
     if (val_bytes && cudaMemsetAsync(*d_blocks, 0, val_bytes, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
     if (nbr > 0 && nnzb > 0) {
         if (es == 1)
@@ -340,32 +374,34 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     if (nnzb && cudaMemcpyAsync(out->block_col_idx.data(), *d_block_col_idx, idx_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return fail(SPMM_ERR_CUDA);
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    cudaFree(d_flags);
-    cudaFree(d_counts);
+    dev_free(d_flags, st);
+    dev_free(d_counts, st);
     finish_bcsr_host(out);       // row order, empty block-rows, distinct block columns: host, from the index arrays
     return SPMM_OK;
 }
 
 namespace {
 
-__global__ void wcsr_keys_kernel(int64_t m, int wh, const int64_t* row_ptr, const int32_t* col_idx, uint64_t* keys) {
+// key = window << cb | column, cb = bits of a column: no empty bits for the radix sort to pass over
+__global__ void wcsr_keys_kernel(int64_t m, int wh, int cb, const int64_t* row_ptr, const int32_t* col_idx, uint64_t* keys) {
     const int lane = threadIdx.x & 31;
     const int64_t warp0 = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
     for (int64_t i = warp0; i < m; i += nwarps) {
-        const uint64_t hi = static_cast<uint64_t>(i / wh) << 32;
+        const uint64_t hi = static_cast<uint64_t>(i / wh) << cb;
         for (int64_t p = row_ptr[i] + lane; p < row_ptr[i + 1]; p += 32) keys[p] = hi | static_cast<uint32_t>(col_idx[p]);
     }
 }
 
 // per window: how many distinct columns; per column: is it referenced at all
-__global__ void wcsr_count_kernel(const uint64_t* ukeys, const int* n_unique, int32_t* cnt, uint8_t* used) {
+__global__ void wcsr_count_kernel(const uint64_t* ukeys, const int* n_unique, int cb, int32_t* cnt, uint8_t* used) {
     const int64_t n = *n_unique;
+    const uint64_t col_mask = (uint64_t{1} << cb) - 1;
     for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < n;
          j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const uint64_t key = ukeys[j];
-        atomicAdd(&cnt[key >> 32], 1);
-        used[static_cast<uint32_t>(key)] = 1;
+        atomicAdd(&cnt[key >> cb], 1);
+        used[key & col_mask] = 1;
     }
 }
 
@@ -384,14 +420,15 @@ __global__ void wcsr_sum_used_kernel(const uint8_t* used, int64_t k, unsigned lo
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(total, n);
 }
 
-__global__ void wcsr_cols_kernel(const uint64_t* ukeys, const int* n_unique, const int32_t* ustart,
+__global__ void wcsr_cols_kernel(const uint64_t* ukeys, const int* n_unique, int cb, const int32_t* ustart,
                                  const int32_t* window_row_ptr, int32_t* window_col_idx) {
     const int64_t n = *n_unique;
+    const uint64_t col_mask = (uint64_t{1} << cb) - 1;
     for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < n;
          j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const uint64_t key = ukeys[j];
-        const int64_t w = static_cast<int64_t>(key >> 32);
-        window_col_idx[window_row_ptr[w] + (j - ustart[w])] = static_cast<int32_t>(static_cast<uint32_t>(key));
+        const int64_t w = static_cast<int64_t>(key >> cb);
+        window_col_idx[window_row_ptr[w] + (j - ustart[w])] = static_cast<int32_t>(key & col_mask);
     }
 }
 
@@ -464,39 +501,41 @@ __global__ void wcsr_group_class_kernel(const int32_t* __restrict__ col_idx, int
     }
 }
 
-// Allocates and fills *d_grp_class [P / 4] from the device copy of window_col_idx.
-int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, int64_t k, cudaStream_t st, uint8_t** d_grp_class) {
+// Allocates and fills *d_grp_class [P / 4] from the device copy of window_col_idx, in the order of `st`.
+int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, int64_t k, int64_t nwin, cudaStream_t st, uint8_t** d_grp_class) {
     *d_grp_class = nullptr;
     if (P <= 0 || k <= 0) return SPMM_OK;
     int32_t *refs = nullptr, *refs_sorted = nullptr, *ids = nullptr, *order = nullptr;
     uint8_t* cls = nullptr;
     void* temp = nullptr;
-    auto release = [&]() { cudaFree(refs); cudaFree(refs_sorted); cudaFree(ids); cudaFree(order); cudaFree(cls); cudaFree(temp); };
+    auto release = [&]() { dev_free(refs, st); dev_free(refs_sorted, st); dev_free(ids, st); dev_free(order, st); dev_free(cls, st); dev_free(temp, st); };
     const size_t kb = static_cast<size_t>(k) * 4;
-    if (cudaMalloc(reinterpret_cast<void**>(&refs), kb) != cudaSuccess || cudaMalloc(reinterpret_cast<void**>(&refs_sorted), kb) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&ids), kb) != cudaSuccess || cudaMalloc(reinterpret_cast<void**>(&order), kb) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&cls), static_cast<size_t>(k)) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(d_grp_class), static_cast<size_t>(P / 4)) != cudaSuccess) {
+    if (!dev_alloc_ok(&refs, kb, st) || !dev_alloc_ok(&refs_sorted, kb, st) ||
+        !dev_alloc_ok(&ids, kb, st) || !dev_alloc_ok(&order, kb, st) ||
+        !dev_alloc_ok(&cls, static_cast<size_t>(k), st) ||
+        !dev_alloc_ok(d_grp_class, static_cast<size_t>(P / 4), st)) {
         release();
-        cudaFree(*d_grp_class);
+        dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
         return SPMM_ERR_ALLOC;
     }
     cudaMemsetAsync(refs, 0, kb, st);
     wcsr_refs_kernel<<<2048, 256, 0, st>>>(d_window_col_idx, P, refs);
     iota_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 2048)), 256, 0, st>>>(ids, k);
+    int count_bits = 1;                       // a row of B is gathered by nwin windows at most
+    while (count_bits < 31 && (int64_t{1} << count_bits) <= nwin) ++count_bits;
     size_t tb = 0;
-    cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, 32, st);
-    bool ok = cudaMalloc(&temp, tb ? tb : 16) == cudaSuccess &&
-              cub::DeviceRadixSort::SortPairsDescending(temp, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, 32, st) == cudaSuccess;
+    cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st);
+    bool ok = dev_alloc_ok(&temp, tb, st) &&
+              cub::DeviceRadixSort::SortPairsDescending(temp, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st) == cudaSuccess;
     if (ok) {
         wcsr_class_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 2048)), 256, 0, st>>>(refs_sorted, order, k, cls);
         wcsr_group_class_kernel<<<2048, 256, 0, st>>>(d_window_col_idx, P / 4, cls, *d_grp_class);
-        ok = cudaStreamSynchronize(st) == cudaSuccess && cudaGetLastError() == cudaSuccess;
+        ok = cudaGetLastError() == cudaSuccess;
     }
     release();
     if (!ok) {
-        cudaFree(*d_grp_class);
+        dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
         return SPMM_ERR_CUDA;
     }
@@ -528,16 +567,16 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     unsigned long long* d_total = nullptr;
     void* d_temp = nullptr;
     auto release = [&]() {
-        cudaFree(d_flags); cudaFree(d_keys); cudaFree(d_keys2); cudaFree(d_cnt); cudaFree(d_len);
-        cudaFree(d_ustart); cudaFree(d_used); cudaFree(d_total); cudaFree(d_temp);
+        dev_free(d_flags, st); dev_free(d_keys, st); dev_free(d_keys2, st); dev_free(d_cnt, st); dev_free(d_len, st);
+        dev_free(d_ustart, st); dev_free(d_used, st); dev_free(d_total, st); dev_free(d_temp, st);
     };
     auto fail = [&](int code) {
         release();
-        cudaFree(*d_window_row_ptr); cudaFree(*d_window_col_idx); cudaFree(*d_packed);
+        dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st);
         *d_window_row_ptr = nullptr; *d_window_col_idx = nullptr; *d_packed = nullptr;
         return code;
     };
-    auto alloc = [&](void** ptr, size_t bytes) { return cudaMalloc(ptr, bytes ? bytes : 16) == cudaSuccess; };
+    auto alloc = [&](void** ptr, size_t bytes) { return dev_alloc(ptr, bytes, st) == cudaSuccess; };
 
     if (!alloc(reinterpret_cast<void**>(&d_flags), 4 * sizeof(int))) return fail(SPMM_ERR_ALLOC);
     if (cudaMemsetAsync(d_flags, 0, 4 * sizeof(int), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
@@ -554,10 +593,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     if (nnz < 0 || (nnz > 0 && (!d_col_idx || !d_vals))) return fail(SPMM_ERR_INVALID_ARG);
     if (nnz >= (int64_t{1} << 31)) return fail(SPMM_ERR_TOO_LARGE);
     if (nnz > 0) {
-        csr_check_cols_kernel<<<check_grid, 256, 0, st>>>(m, k, d_row_ptr, d_col_idx, d_flags);
-        if (cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        if (cudaStreamSynchronize(st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        if (flags[0] != 0) return fail(flags[0]);
+        if (int rc = check_csr_cols(m, k, nnz, d_row_ptr, d_col_idx, d_flags + 2, d_flags, st)) return fail(rc);
     }
     *nnz_out = nnz;
 
@@ -575,10 +611,12 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     cudaMemsetAsync(d_used, 0, static_cast<size_t>(k ? k : 1), st);
     cudaMemsetAsync(d_total, 0, 8, st);
     const int n = static_cast<int>(nnz);
-    int end_bit = 32;
-    while (end_bit < 64 && (int64_t{1} << (end_bit - 32)) < nwin) ++end_bit;
+    int cb = 1;
+    while ((int64_t{1} << cb) < k) ++cb;
+    int end_bit = cb + 1;
+    while ((int64_t{1} << (end_bit - cb)) < nwin) ++end_bit;
     if (n > 0) {
-        wcsr_keys_kernel<<<static_cast<unsigned>(std::min<int64_t>((m + 7) / 8, 4096)), 256, 0, st>>>(m, wh, d_row_ptr, d_col_idx, d_keys);
+        wcsr_keys_kernel<<<static_cast<unsigned>(std::min<int64_t>((m + 7) / 8, 4096)), 256, 0, st>>>(m, wh, cb, d_row_ptr, d_col_idx, d_keys);
         size_t t1 = 0, t2 = 0;
         cub::DeviceRadixSort::SortKeys(nullptr, t1, d_keys, d_keys2, n, 0, end_bit, st);
         cub::DeviceSelect::Unique(nullptr, t2, d_keys2, d_keys, d_flags + 2, n, st);
@@ -588,7 +626,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         tb = std::max(t1, t2);
         if (cub::DeviceSelect::Unique(d_temp, tb, d_keys2, d_keys, d_flags + 2, n, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
         // d_keys now holds the unique keys, d_flags[2] their number
-        wcsr_count_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, d_cnt, d_used);
+        wcsr_count_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, cb, d_cnt, d_used);
     }
     wcsr_pad_kernel<<<static_cast<unsigned>(std::min<int64_t>((nwin + 255) / 256 + 1, 2048)), 256, 0, st>>>(d_cnt, nwin, b_col, d_len);
     exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_len, nwin, *d_window_row_ptr, d_flags + 1);
@@ -616,7 +654,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         cudaMemsetAsync(*d_packed, 0, packed_bytes, st);
     }
     if (n > 0) {
-        wcsr_cols_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, d_ustart, *d_window_row_ptr, *d_window_col_idx);
+        wcsr_cols_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, cb, d_ustart, *d_window_row_ptr, *d_window_col_idx);
         const unsigned vgrid = static_cast<unsigned>(std::min<int64_t>((m + 7) / 8, 8192));
         if (es == 1)
             wcsr_values_kernel<1><<<vgrid, 256, 0, st>>>(m, wh, b_col, d_row_ptr, d_col_idx, d_vals, d_cnt, *d_window_row_ptr, *d_window_col_idx, *d_packed);
@@ -625,12 +663,19 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         else
             wcsr_values_kernel<4><<<vgrid, 256, 0, st>>>(m, wh, b_col, d_row_ptr, d_col_idx, d_vals, d_cnt, *d_window_row_ptr, *d_window_col_idx, *d_packed);
     }
-    if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    release();
-    int rc = wcsr_reuse_classes_device(*d_window_col_idx, P, k, st, d_grp_class);
-    if (!rc) rc = plan_wcsr(out, T, n_bins, es);
+    release();                                // (ordered behind the kernels that use them)
+    int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
+    // the split plan needs the window lengths only: the host makes it while the kernels above run
+    if (!rc) {
+        try {
+            rc = plan_wcsr(out, T, n_bins, es);
+        } catch (const std::bad_alloc&) {
+            rc = SPMM_ERR_ALLOC;
+        }
+    }
+    if (cudaStreamSynchronize(st) != cudaSuccess && !rc) rc = SPMM_ERR_CUDA;
     if (rc) {
-        cudaFree(*d_window_row_ptr); cudaFree(*d_window_col_idx); cudaFree(*d_packed); cudaFree(*d_grp_class);
+        dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st); dev_free(*d_grp_class, st);
         *d_window_row_ptr = nullptr; *d_window_col_idx = nullptr; *d_packed = nullptr; *d_grp_class = nullptr;
     }
     return rc;
