@@ -368,7 +368,8 @@ int create_bcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
 }
 
 // Uploads the schedule arrays of a WCSR handle (everything but the three format arrays): one allocation, one copy.
-int upload_wcsr_plan(spmm_handle_s* h) {
+// Synchronises `stream`.
+int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
     const WcsrHost& f = h->wcsr;
     const size_t nt = f.tasks.size(), nm = f.merge_window.size(), ni = f.bin_tasks.size();
     const bool narrow = !f.bin_fill_narrow.empty();
@@ -380,10 +381,13 @@ int upload_wcsr_plan(spmm_handle_s* h) {
         return at;
     };
     const size_t o_tasks = section(4 * nt), o_bin_ptr = section(f.bin_ptr.size()), o_bin_tasks = section(ni), o_items = section(4 * ni);
-    const size_t o_fills = section(f.fills.size()), o_bin_fill = section(f.bin_fill.size());
-    const size_t o_fills_n = section(f.fills_narrow.size()), o_bin_fill_n = section(f.bin_fill_narrow.size());
+    const size_t o_item_fill = section(f.item_fill.size()), o_bin_fill = section(f.bin_fill.size());
+    const size_t o_item_fill_n = section(f.item_fill_narrow.size()), o_bin_fill_n = section(f.bin_fill_narrow.size());
     const size_t o_merge = section(3 * nm), o_class = section((f.grp_class.size() + 3) / 4);
     std::vector<int32_t> w(words, 0);
+    // the fills themselves are written on the GPU, behind what is copied
+    const size_t o_fills = section(2 * static_cast<size_t>(f.item_fill.empty() ? 0 : f.item_fill.back()));
+    const size_t o_fills_n = section(2 * static_cast<size_t>(narrow ? f.item_fill_narrow.back() : 0));
     static_assert(sizeof(WcsrDevTask) == 16, "four words per task");
     for (size_t i = 0; i < nt; ++i) {
         const WcsrTask& t = f.tasks[i];
@@ -401,25 +405,32 @@ int upload_wcsr_plan(spmm_handle_s* h) {
     };
     put(o_bin_ptr, f.bin_ptr.data(), f.bin_ptr.size() * 4);
     put(o_bin_tasks, f.bin_tasks.data(), ni * 4);
-    put(o_fills, f.fills.data(), f.fills.size() * 4);
+    put(o_item_fill, f.item_fill.data(), f.item_fill.size() * 4);
     put(o_bin_fill, f.bin_fill.data(), f.bin_fill.size() * 4);
-    put(o_fills_n, f.fills_narrow.data(), f.fills_narrow.size() * 4);
+    put(o_item_fill_n, f.item_fill_narrow.data(), f.item_fill_narrow.size() * 4);
     put(o_bin_fill_n, f.bin_fill_narrow.data(), f.bin_fill_narrow.size() * 4);
     put(o_merge, f.merge_window.data(), nm * 4);
     put(o_merge + nm, f.merge_first.data(), nm * 4);
     put(o_merge + 2 * nm, f.merge_nparts.data(), nm * 4);
     put(o_class, f.grp_class.data(), f.grp_class.size());
-    int rc = upload(&h->d_plan, w.data(), words * 4);
-    if (rc) return rc;
+    if (!dev_alloc_ok(&h->d_plan, words * 4, stream)) return SPMM_ERR_ALLOC;
+    if (cudaMemcpyAsync(h->d_plan, w.data(), w.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SPMM_ERR_CUDA;
+    int32_t* fills = h->d_plan + o_fills;
+    int32_t* fills_n = h->d_plan + o_fills_n;
+    if (expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill, f.kt, fills, stream) != cudaSuccess ||
+        (narrow && expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill_n,
+                                     kWcsrNarrowCols, fills_n, stream) != cudaSuccess) ||
+        cudaStreamSynchronize(stream) != cudaSuccess)
+        return SPMM_ERR_CUDA;
     h->n_merge = static_cast<int>(nm);
     h->d_tasks = reinterpret_cast<WcsrDevTask*>(h->d_plan + o_tasks);
     h->d_bin_ptr = h->d_plan + o_bin_ptr;
     h->d_bin_tasks = h->d_plan + o_bin_tasks;
     h->d_items = h->d_plan + o_items;
-    h->d_fills = h->d_plan + o_fills;
+    h->d_fills = fills;
     h->d_bin_fill = h->d_plan + o_bin_fill;
     if (narrow) {
-        h->d_fills_narrow = h->d_plan + o_fills_n;
+        h->d_fills_narrow = fills_n;
         h->d_bin_fill_narrow = h->d_plan + o_bin_fill_n;
     }
     h->d_merge = h->d_plan + o_merge;
@@ -484,7 +495,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
         rc = upload(&h->d_ptr, f.window_row_ptr.data(), f.window_row_ptr.size() * 4);
         if (!rc) rc = upload(&h->d_idx, f.window_col_idx.data(), f.window_col_idx.size() * 4);
         if (!rc) rc = upload(&h->d_vals, f.packed.data(), f.packed.size());
-        if (!rc) rc = upload_wcsr_plan(h);
+        if (!rc) rc = upload_wcsr_plan(h, nullptr);
         if (rc) { free_handle(h); return rc; }
         std::vector<uint8_t>().swap(h->wcsr.packed);
     }
@@ -508,7 +519,7 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
                                h->n_ctas * wcsr_bins_per_sm(h->es, wh), stream, &h->wcsr, &h->nnz, &h->d_ptr, &h->d_idx,
                                &h->d_vals, &h->d_class);
         h->d_grp_class = h->d_class;
-        if (!rc) rc = upload_wcsr_plan(h);
+        if (!rc) rc = upload_wcsr_plan(h, stream);
     } catch (const std::bad_alloc&) {
         rc = SPMM_ERR_ALLOC;
     }

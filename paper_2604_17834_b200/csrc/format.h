@@ -113,15 +113,16 @@ struct WcsrHost {
     std::vector<int32_t> bin_ptr;         // [n_bins+1]
     std::vector<int32_t> bin_tasks;       // [n_tasks] task indices, bin-major
     // Device-private pipeline schedule: every task cut into "fills" of at most kt columns (one
-    // shared-memory stage each), stored bin-major in the bins' task order.
-    // fills[i] = {first padded column, count | first<<16 | last<<17} where first / last mark
-    // the first / last fill of a task; bin_fill[j] = index of the first fill of bin j.
+    // shared-memory stage each), stored bin-major in the bins' task order: fill i =
+    // {first padded column, count | first<<16 | last<<17} where first / last mark the first / last fill
+    // of a task.  The list itself is written on the GPU (expand_wcsr_fills); here only its cuts:
+    // item_fill[i] = index of the first fill of bin_tasks[i], bin_fill[j] = of the first fill of bin j.
     int kt = 0;
-    std::vector<int32_t> fills;           // 2 * n_fills
+    std::vector<int32_t> item_fill;       // [n_tasks+1]
     std::vector<int32_t> bin_fill;        // [n_bins+1]
     // the same for the narrow-operand kernel variant (stages of kWcsrNarrowCols columns); empty
     // unless the value type is 2 bytes wide and the window height 16
-    std::vector<int32_t> fills_narrow, bin_fill_narrow;
+    std::vector<int32_t> item_fill_narrow, bin_fill_narrow;
     // Device-private gather hint (no effect on results): reuse class of every group of four
     // consecutive padded columns, one byte each.  A column's class says how high its B row ranks
     // by the number of windows that gather it: 7 = among the 16 Ki most gathered rows, 6 = 32 Ki,
@@ -177,6 +178,9 @@ constexpr int kWcsrTopClassRows = 16384;   // rows in class 7; every class below
 void wcsr_reuse_classes(const int32_t* window_col_idx, int64_t P, int64_t k, std::vector<uint8_t>* grp_class);
 // Second half of build_wcsr: split plan, bins, fills and merge lists from out->window_row_ptr / out->P.
 int plan_wcsr(WcsrHost* out, int T, int n_bins, int es);
+// Writes the fills of n_items items ({first column, count, ..} descriptors tasks[bin_tasks[i]]) in the order of `stream`.
+cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_t* d_bin_tasks, const int32_t* d_item_fill, int kt,
+                              int32_t* d_fills, cudaStream_t stream);
 // The WCSR format arrays built on the GPU from a CSR matrix in device memory (format_gpu.cu):
 // validates the CSR, allocates and fills window_row_ptr, window_col_idx and the packed values on
 // the device (owned by the caller afterwards) together with the column groups' reuse classes

@@ -461,6 +461,20 @@ __global__ void wcsr_values_kernel(int64_t m, int wh, int b_col, const int64_t* 
     }
 }
 
+// eight lanes per item
+__global__ void wcsr_fills_kernel(int64_t n_items, const WcsrDevTask* __restrict__ tasks, const int32_t* __restrict__ bin_tasks,
+                                  const int32_t* __restrict__ item_fill, int kt, int2* __restrict__ fills) {
+    for (int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 3; i < n_items;
+         i += (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 3) {
+        const WcsrDevTask t = tasks[bin_tasks[i]];
+        const int f0 = item_fill[i], n = item_fill[i + 1] - f0;
+        for (int j = threadIdx.x & 7; j < n; j += 8) {
+            const int done = j * kt;
+            fills[f0 + j] = make_int2(t.col_begin + done, min(kt, t.count - done) | (j == 0) << 16 | (j == n - 1) << 17);
+        }
+    }
+}
+
 // ---- reuse classes of the column groups (gather hints; the host rule of wcsr_reuse_classes)
 
 __global__ void wcsr_refs_kernel(const int32_t* __restrict__ col_idx, int64_t P, int32_t* __restrict__ refs) {
@@ -543,6 +557,14 @@ int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, int64_
 }
 
 }  // namespace
+
+cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_t* d_bin_tasks, const int32_t* d_item_fill, int kt,
+                              int32_t* d_fills, cudaStream_t stream) {
+    if (n_items <= 0) return cudaSuccess;
+    wcsr_fills_kernel<<<static_cast<unsigned>(std::min<int64_t>((n_items + 31) / 32, 4096)), 256, 0, stream>>>(
+        n_items, static_cast<const WcsrDevTask*>(d_tasks), d_bin_tasks, d_item_fill, kt, reinterpret_cast<int2*>(d_fills));
+    return cudaGetLastError();
+}
 
 int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
                       int es, int wh, int b_col, int T, int n_bins, cudaStream_t st, WcsrHost* out, int64_t* nnz_out,
