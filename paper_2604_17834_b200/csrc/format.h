@@ -136,6 +136,45 @@ struct WcsrHost {
     std::vector<int32_t> merge_nparts;    // number of slots (split) or 0 (empty)
 };
 
+// The row stream: a device-private copy of the nonzeros of a WCSR handle whose windows condense
+// almost nothing (about one stored value per padded column), in the order the row kernel
+// (wcsr_rows_kernel.cu) consumes them.  No counterpart in the paper; the exported format arrays and
+// the tensor-core plan are unaffected.
+//   order      rows sorted (stably) into length classes: long rows (more than task_max nonzeros), then
+//              rows above task_max / 2, / 4, ... down to pack, then all rows of at most `pack`
+//              nonzeros, each class in row order.
+//   tasks      a row above `pack` is a task of its own; the packed rows are cut into runs: a row
+//              belongs to run (entries of the packed rows before it) / pack.  A row without nonzeros
+//              counts as one entry (no gather; it still writes its zeros).
+//   entries    {column | sign bit on a row's last entry, value}; task t starts at the first multiple of
+//              four from (entries of the tasks before it) + 3 t on; padding and empty rows have column
+//              0x7fffffff.
+//   long rows  after the tasks' entries, each starting on a multiple of eight, no sign bits, cut into
+//              parts of part_len entries (one CTA each).
+struct WcsrRowStream {
+    int pack = 0, task_max = 0, part_len = 0;
+    int32_t n_tasks = 0, n_parts = 0, n_long = 0, n_slots = 0;
+    int32_t* d_order = nullptr;      // [m + 1]
+    int32_t* d_tasks = nullptr;      // int4 [n_tasks]
+    int32_t* d_parts = nullptr;      // int4 [n_parts]
+    int32_t* d_longs = nullptr;      // int4 [n_long]
+    int32_t* d_col = nullptr;
+    uint8_t* d_val = nullptr;
+    unsigned* d_counters = nullptr;  // 32 zero bytes (what the kernel gathers for an entry without column), then the counters
+    int32_t* d_total = nullptr;      // {tasks, parts, long rows, slots}, read by finish_wcsr_rows
+};
+// Whether the row kernel serves a handle: 2- or 4-byte values, and at most kRowsMaxPerCol stored
+// values per padded column.
+constexpr double kRowsMaxPerCol = 2.0;
+constexpr int kRowsMaxSlots = 65536;    // partial rows of long rows cut into parts
+// Builds the stream on the GPU from a (validated) CSR matrix in device memory, in the order of `stream`; leaves
+// *out empty when the matrix has no rows or is too large for 32-bit entry positions.
+int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
+                           int es, int sms, cudaStream_t stream, WcsrRowStream* out);
+// Reads the counts the launches need; synchronises `stream`.  Until then n_tasks = n_parts = 0.
+int finish_wcsr_rows(WcsrRowStream* s, cudaStream_t stream);
+void free_wcsr_rows(WcsrRowStream* s, cudaStream_t stream);
+
 // All return 0 or a negative spmm_status_t value.
 int validate_csr(const CsrView& a);
 int coo_to_csr(int64_t m, int64_t k, int64_t nnz, const int32_t* rows, const int32_t* cols,
@@ -187,9 +226,14 @@ cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_
 // (*d_grp_class, the rule of wcsr_reuse_classes), leaves window_row_ptr, P and distinct_cols in *out
 // (out->window_col_idx, out->packed and out->grp_class stay empty) and runs plan_wcsr.
 // Synchronises `stream`.
+// Where the row kernel is to serve the handle (wcsr_wants_rows), *rows is built as well.
 int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
-                      int es, int wh, int b_col, int T, int n_bins, cudaStream_t stream, WcsrHost* out, int64_t* nnz_out,
-                      int32_t** d_window_row_ptr, int32_t** d_window_col_idx, uint8_t** d_packed, uint8_t** d_grp_class);
+                      int es, int wh, int b_col, int T, int n_bins, int sms, cudaStream_t stream, WcsrHost* out, int64_t* nnz_out,
+                      int32_t** d_window_row_ptr, int32_t** d_window_col_idx, uint8_t** d_packed, uint8_t** d_grp_class,
+                      WcsrRowStream* rows);
+inline bool wcsr_wants_rows(int es, int64_t m, int64_t nnz, int64_t P) {
+    return es != 1 && m > 0 && static_cast<double>(nnz) <= kRowsMaxPerCol * static_cast<double>(P);
+}
 
 // Byte offset of element (row r, padded column q) inside the packed WCSR value array.
 #ifdef __CUDACC__

@@ -148,6 +148,32 @@ struct MergeParams {
 };
 cudaError_t launch_wcsr_merge(const MergeParams& p, int wh, int ctype, cudaStream_t stream);   // ctype: 0 fp32, 1 fp16, 2 bf16
 
+// WCSR product from the row stream (wcsr_rows_kernel.cu; the stream: WcsrRowStream in format.h).
+struct WcsrRowsParams {
+    const int4* tasks;           // [n_tasks] {first entry, entries, position in order of the first row, 0}
+    const int4* parts;           // [n_parts] {first entry, entries, long row, part}: one CTA per column tile, first in the grid
+    const int4* longs;           // [long rows] {row, first partial slot, parts, 0}
+    const int32_t* order;        // rows in task order
+    const int32_t* col;          // entries: column, sign bit = last of its row, 0x7fffffff = no gather
+    const uint8_t* val;
+    unsigned* counters;          // [long rows][kRowsMaxTiles], zero between launches
+    float* partial;              // [slots][tiles of the launch][tile columns]
+    const uint8_t* zeros;        // 32 zero bytes
+    const void* B;
+    void* C;
+    int64_t N;
+    int32_t n_tasks, n_parts;
+    int32_t lanes, groups, tile0;    // set by launch_wcsr_rows
+};
+constexpr int kRowsThreads = 128;
+constexpr int kRowsMaxTiles = 8;     // column tiles one launch covers at most
+// How a dense width is cut: a column tile is lanes vectors of vec bytes (a group of lanes).
+struct RowsShape { int vec, lanes, tiles, tile_cols; };
+// aligned32: every row of B and of C starts on a 32-byte boundary.
+RowsShape wcsr_rows_shape(int64_t N, int es, bool aligned32);
+// bf16, fp16, tf32.  Column tiles [tile0, tile0 + tiles), at most kRowsMaxTiles of them.
+cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, cudaStream_t stream);
+
 // Device address and size in bytes of the library's built-in partial-tile scratch on the
 // current device (resolved on the first call per device).
 cudaError_t wcsr_static_scratch(float** ptr, size_t* bytes);

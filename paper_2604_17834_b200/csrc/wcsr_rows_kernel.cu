@@ -138,3 +138,171 @@ __device__ __forceinline__ void store_c(uint8_t* dst, const float (&acc)[VE]) {
         st_vec<VE * 2>(dst, w);
     }
 }
+
+// Resident CTAs per SM: registers cap the bytes in flight.  Wide vectors: 7 (72 registers) measured 805 us
+// on R-MAT 2^21 fp16 N = 128, 5 CTAs 858, 8 CTAs 893; 16-byte vectors: 8.
+template <int FMT, int CT, int VB>
+__global__ void __launch_bounds__(kRowsThreads, VB == 32 ? 7 : 8)
+wcsr_rows_kernel(const WcsrRowsParams p) {
+    constexpr int ES = FMT == 2 ? 4 : 2;
+    constexpr int VE = VB / ES;                           // dense columns per lane
+    using CElem = typename CType<FMT, CT>::type;
+    extern __shared__ float red[];                        // long rows: [kStrands][VE][lanes]
+    __shared__ unsigned arrived;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = lane / p.lanes, l = lane - g * p.lanes;
+    const int tile = p.tile0 + blockIdx.y;
+    const int64_t n = (static_cast<int64_t>(tile) * p.lanes + l) * VE;         // first dense column of this lane
+    const bool on = g < p.groups && n < p.N;
+    const uint8_t* B = static_cast<const uint8_t*>(p.B) + n * ES;
+    const uint32_t pitch = static_cast<uint32_t>(p.N) * ES;
+    const int64_t c_pitch = p.N * static_cast<int64_t>(sizeof(CElem));
+
+    float acc[VE];
+#pragma unroll
+    for (int i = 0; i < VE; ++i) acc[i] = 0.f;
+
+    // an entry without a gather reads zeros of the library's own
+    auto gather = [&](int c) -> Vec<VB> {
+        const uint32_t j = static_cast<uint32_t>(c) & 0x7fffffffu;
+        const uint8_t* src = B + static_cast<uint64_t>(j) * pitch;
+        return ld_row<VB>(j != static_cast<uint32_t>(kNoCol) ? src : p.zeros);
+    };
+
+    if (static_cast<int>(blockIdx.x) >= p.n_parts) {
+        // ------------------------------------------------------------------ whole rows, one task per group
+        const int id = ((static_cast<int>(blockIdx.x) - p.n_parts) * kWarps + warp) * p.groups + g;
+        if (!on || id >= p.n_tasks) return;
+        const int4 d = __ldg(p.tasks + id);               // first entry, entries, position in order
+        const int32_t* order = p.order + d.z;
+        uint8_t* C = static_cast<uint8_t*>(p.C) + n * sizeof(CElem);
+        Ent4<ES> cur = ld_ent4<ES>(p.col, p.val, d.x, d.y > 0);
+        int row = __ldg(order);
+        for (int e = 0; e < d.y; e += 4) {
+            Vec<VB> b[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) b[u] = gather(cur.c[u]);
+            const Ent4<ES> nxt = ld_ent4<ES>(p.col, p.val, d.x + e + 4, e + 4 < d.y);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                fma_vec<FMT, VB, VE>(acc, cur.val(u), b[u]);
+                if (cur.c[u] < 0) {                       // the row's last entry
+                    store_c<FMT, CT, VB, VE>(C + row * c_pitch, acc);
+#pragma unroll
+                    for (int i = 0; i < VE; ++i) acc[i] = 0.f;
+                    row = __ldg(++order);                 // (order has one element more than there are rows)
+                }
+            }
+            cur = nxt;
+        }
+        return;
+    }
+
+    // ---------------------------------------------------------------------- one part of a long row
+    const int4 d = __ldg(p.parts + blockIdx.x);           // first entry, entries, long row, part
+    const int4 lr = __ldg(p.longs + d.z);                 // row, first slot, parts
+    const int n_groups = kWarps * p.groups;
+    const int tile_cols = p.lanes * VE;
+    if (g < p.groups) {
+        for (int strand = warp * p.groups + g; strand < kStrands; strand += n_groups) {
+#pragma unroll
+            for (int i = 0; i < VE; ++i) acc[i] = 0.f;
+            if (on) {
+                Ent4<ES> cur = ld_ent4<ES>(p.col, p.val, d.x + strand * 8, strand * 8 < d.y);
+                for (int e = strand * 8; e < d.y;) {
+                    Vec<VB> b[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) b[u] = gather(cur.c[u]);
+                    const int en = (e & 4) ? e + kStrands * 8 - 4 : e + 4;      // the strand's next four entries
+                    const Ent4<ES> nxt = ld_ent4<ES>(p.col, p.val, d.x + en, en < d.y);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) fma_vec<FMT, VB, VE>(acc, cur.val(u), b[u]);
+                    cur = nxt;
+                    e = en;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < VE; ++i) red[strand * tile_cols + i * p.lanes + l] = acc[i];
+        }
+    }
+    __syncthreads();
+    const int64_t n_tile = static_cast<int64_t>(tile) * tile_cols;
+    CElem* Crow = static_cast<CElem*>(p.C) + lr.x * p.N + n_tile;
+    const int64_t slot_pitch = static_cast<int64_t>(gridDim.y) * tile_cols;
+    float* part0 = p.partial + static_cast<int64_t>(lr.y) * slot_pitch + static_cast<int64_t>(blockIdx.y) * tile_cols;
+    for (int t = threadIdx.x; t < tile_cols; t += kRowsThreads) {
+        float s = 0.f;
+#pragma unroll
+        for (int i = 0; i < kStrands; ++i) s += red[i * tile_cols + (t % VE) * p.lanes + t / VE];
+        if (lr.z == 1) {
+            if (n_tile + t < p.N) Crow[t] = from_f32<CElem>(s);
+        } else {
+            part0[d.w * slot_pitch + t] = s;
+        }
+    }
+    if (lr.z == 1) return;
+    // several parts: the CTA that arrives last adds them in part order.  The counter wraps to zero, so
+    // it is ready for the next launch.
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) arrived = atomicInc(p.counters + d.z * kRowsMaxTiles + blockIdx.y, static_cast<unsigned>(lr.z) - 1u);
+    __syncthreads();
+    if (arrived != static_cast<unsigned>(lr.z) - 1u) return;
+    __threadfence();
+    for (int t = threadIdx.x; t < tile_cols; t += kRowsThreads) {
+        if (n_tile + t >= p.N) break;
+        float s = 0.f;
+        int i = 0;
+        for (; i + 8 <= lr.z; i += 8) {
+            float x[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = __ldcg(part0 + (i + j) * slot_pitch + t);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s += x[j];
+        }
+        for (; i < lr.z; ++i) s += __ldcg(part0 + i * slot_pitch + t);
+        Crow[t] = from_f32<CElem>(s);
+    }
+}
+
+template <int VB>
+cudaError_t launch_vb(int dtype, int c16, const WcsrRowsParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
+    if (dtype == 2) wcsr_rows_kernel<2, 0, VB><<<grid, kRowsThreads, smem, stream>>>(p);
+    else if (dtype == 1 && c16) wcsr_rows_kernel<0, 1, VB><<<grid, kRowsThreads, smem, stream>>>(p);
+    else if (dtype == 1) wcsr_rows_kernel<0, 0, VB><<<grid, kRowsThreads, smem, stream>>>(p);
+    else if (dtype == 0 && c16) wcsr_rows_kernel<1, 1, VB><<<grid, kRowsThreads, smem, stream>>>(p);
+    else if (dtype == 0) wcsr_rows_kernel<1, 0, VB><<<grid, kRowsThreads, smem, stream>>>(p);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+// 32-byte vectors from 128-byte rows on (R-MAT 2^21 fp16 N = 128: 805 against 864 us with 16 bytes;
+// TF32 N = 128, 100,000 rows: 36.6 against 38.6); below, 16-byte vectors keep more lanes busy (the same
+// graph at N = 32: 339 against 454 us).
+RowsShape wcsr_rows_shape(int64_t N, int es, bool aligned32) {
+    RowsShape s;
+    s.vec = aligned32 && N * es >= 128 ? 32 : 16;
+    const int64_t vecs = (N * es + s.vec - 1) / s.vec;
+    const int64_t tiles = (vecs + 31) / 32;               // a group is part of one warp
+    s.lanes = static_cast<int>((vecs + tiles - 1) / tiles);
+    s.tiles = static_cast<int>((vecs + s.lanes - 1) / s.lanes);
+    s.tile_cols = s.lanes * (s.vec / es);
+    return s;
+}
+
+cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, cudaStream_t stream) {
+    p.lanes = s.lanes;
+    p.groups = 32 / s.lanes;
+    p.tile0 = tile0;
+    const int per_cta = kWarps * p.groups;
+    const int64_t ctas = p.n_parts + (static_cast<int64_t>(p.n_tasks) + per_cta - 1) / per_cta;
+    if (ctas <= 0 || tiles <= 0) return cudaSuccess;
+    const dim3 grid(static_cast<unsigned>(ctas), static_cast<unsigned>(tiles));
+    const size_t smem = p.n_parts > 0 ? static_cast<size_t>(kStrands) * s.tile_cols * 4 : 0;     // at most 32 KB
+    return s.vec == 32 ? launch_vb<32>(dtype, c16, p, grid, smem, stream) : launch_vb<16>(dtype, c16, p, grid, smem, stream);
+}
+
+}  // namespace spmm
