@@ -703,4 +703,190 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     return rc;
 }
 
+// ----------------------------------------------------------------------------- row stream
+
+namespace {
+
+constexpr int kRowClasses = 8;
+
+// length class of a row: 0 = longer than task_max, then one class per factor of two down to `pack`, last = packed
+__device__ __forceinline__ int row_class(int64_t len, int pack, int task_max) {
+    if (len > task_max) return 0;
+    int c = 1;
+    for (int lim = task_max / 2; lim >= pack; lim /= 2, ++c)
+        if (len > lim) return c;
+    return c;
+}
+
+__global__ void rows_class_kernel(int64_t m, const int64_t* __restrict__ row_ptr, int pack, int task_max, uint8_t* __restrict__ cls,
+                                  int32_t* __restrict__ ids, int32_t* __restrict__ counts) {
+    __shared__ int n[kRowClasses];
+    if (threadIdx.x < kRowClasses) n[threadIdx.x] = 0;
+    __syncthreads();
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int c = row_class(row_ptr[i + 1] - row_ptr[i], pack, task_max);
+        cls[i] = static_cast<uint8_t>(c);
+        ids[i] = static_cast<int32_t>(i);
+        atomicAdd(&n[c], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < kRowClasses && n[threadIdx.x]) atomicAdd(&counts[threadIdx.x], n[threadIdx.x]);
+}
+
+struct Int4Sum {
+    __host__ __device__ int4 operator()(const int4& a, const int4& b) const { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+};
+
+// Per position of `order`: {entries (an empty row counts one; a long row none here), padded entries of a long row,
+// its parts, its partial slots}; position m closes the scan.
+__global__ void rows_size_kernel(int64_t m, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr, int task_max, int part_len,
+                                 int4* __restrict__ size) {
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i <= m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        int4 s = make_int4(0, 0, 0, 0);
+        if (i < m) {
+            const int32_t r = order[i];
+            const int n = static_cast<int>(row_ptr[r + 1] - row_ptr[r]);
+            if (n <= task_max) {
+                s.x = n > 0 ? n : 1;
+            } else {
+                s.y = (n + 7) / 8 * 8;
+                s.z = (n + part_len - 1) / part_len;
+                s.w = s.z > 1 ? s.z : 0;
+            }
+        }
+        size[i] = s;
+    }
+}
+
+// What the later passes need of a plan: positions below n_long are long rows, then n_single tasks of one row, then
+// packed rows.
+struct RowsPlan {
+    int64_t m;
+    int pack, part_len, long_base;       // long_base: the long rows' first entry
+    const int32_t* counts;
+    const int4* start;                   // exclusive sums of rows_size_kernel's fields
+    int n_classes;
+    __device__ __forceinline__ int n_long() const { return counts[0]; }
+    __device__ __forceinline__ int n_single() const {
+        int s = 0;
+        for (int c = 1; c + 1 < n_classes; ++c) s += counts[c];
+        return s;
+    }
+    // task of position i (not a long row)
+    __device__ __forceinline__ int task(int64_t i, int nl, int ns) const {
+        const int64_t p0 = static_cast<int64_t>(nl) + ns;
+        return i < p0 ? static_cast<int>(i) - nl : ns + (start[i].x - start[p0].x) / pack;
+    }
+    __device__ __forceinline__ int begin(int task, int first_entry) const { return (first_entry + 3 * task + 3) / 4 * 4; }
+};
+
+// task heads; descriptors of the long rows and their parts; totals {tasks, parts, long rows, slots}
+__global__ void rows_plan_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr, int32_t* __restrict__ head,
+                                 int4* __restrict__ parts, int4* __restrict__ longs, int4* __restrict__ total) {
+    const int nl = p.n_long(), ns = p.n_single();
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i <= p.m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        if (i == p.m) {
+            const int tasks = nl < p.m ? p.task(p.m - 1, nl, ns) + 1 : 0;
+            head[tasks] = static_cast<int32_t>(p.m);
+            *total = make_int4(tasks, p.start[p.m].z, nl, p.start[p.m].w);
+        } else if (i < nl) {
+            const int4 s = p.start[i];
+            const int np = p.start[i + 1].z - s.z;
+            const int32_t r = order[i];
+            const int n = static_cast<int>(row_ptr[r + 1] - row_ptr[r]);
+            longs[i] = make_int4(r, s.w, np, 0);
+            for (int j = 0; j < np; ++j)
+                parts[s.z + j] = make_int4(p.long_base + s.y + j * p.part_len, min(p.part_len, n - j * p.part_len), static_cast<int>(i), j);
+        } else {
+            const int t = p.task(i, nl, ns);
+            if (i == nl || t != p.task(i - 1, nl, ns)) head[t] = static_cast<int32_t>(i);
+        }
+    }
+}
+
+template <int ES> struct RowsValue { using type = uint16_t; };
+template <> struct RowsValue<4> { using type = uint32_t; };
+
+// eight lanes per position: a row's nonzeros to their place in its task, the task's descriptor and padding
+template <int ES>
+__global__ void rows_fill_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int32_t* __restrict__ head,
+                                 const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ vals,
+                                 int4* __restrict__ tasks, int32_t* __restrict__ col, uint8_t* __restrict__ val) {
+    using T = typename RowsValue<ES>::type;
+    const T* src = reinterpret_cast<const T*>(vals);
+    T* dst = reinterpret_cast<T*>(val);
+    const int nl = p.n_long(), ns = p.n_single();
+    const int sub = threadIdx.x & 7;
+    for (int64_t i = nl + ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 3); i < p.m;
+         i += (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 3) {
+        const int t = p.task(i, nl, ns);
+        const int h = head[t], h1 = head[t + 1];
+        const int first = p.start[h].x;
+        const int64_t base = p.begin(t, first);
+        const int64_t at = base + (p.start[i].x - first);
+        const int32_t r = order[i];
+        const int64_t s = row_ptr[r];
+        const int n = static_cast<int>(row_ptr[r + 1] - s);
+        if (n == 0 && sub == 0) {
+            col[at] = -1;                                  // the sign bit and no gather
+            dst[at] = 0;
+        }
+        for (int j = sub; j < n; j += 8) {
+            col[at + j] = col_idx[s + j] | (j == n - 1 ? static_cast<int32_t>(0x80000000u) : 0);
+            dst[at + j] = src[s + j];
+        }
+        if (i == h) {
+            const int len = p.start[h1].x - first;
+            if (sub == 0) tasks[t] = make_int4(static_cast<int>(base), len, h, 0);
+            if (sub < 4 && len + sub < (len + 3) / 4 * 4) {
+                col[base + len + sub] = 0x7fffffff;
+                dst[base + len + sub] = 0;
+            }
+        }
+    }
+}
+
+// one CTA per long row
+template <int ES>
+__global__ void rows_fill_long_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr,
+                                      const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ vals, int32_t* __restrict__ col,
+                                      uint8_t* __restrict__ val) {
+    using T = typename RowsValue<ES>::type;
+    const T* src = reinterpret_cast<const T*>(vals);
+    T* dst = reinterpret_cast<T*>(val);
+    const int nl = p.n_long();
+    for (int i = blockIdx.x; i < nl; i += gridDim.x) {
+        const int32_t r = order[i];
+        const int64_t s = row_ptr[r], n = row_ptr[r + 1] - s, at = p.long_base + p.start[i].y;
+        for (int64_t j = threadIdx.x; j < (n + 7) / 8 * 8; j += blockDim.x) {
+            col[at + j] = j < n ? col_idx[s + j] : 0x7fffffff;
+            dst[at + j] = j < n ? src[s + j] : T(0);
+        }
+    }
+}
+
+unsigned grid_for(int64_t n, int per) { return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>((n + per - 1) / per, 4096))); }
+
+}  // namespace
+
+void free_wcsr_rows(WcsrRowStream* s, cudaStream_t st) {
+    void* const arrays[] = {s->d_order, s->d_tasks, s->d_parts, s->d_longs, s->d_col, s->d_val, s->d_counters, s->d_total};
+    for (void* ptr : arrays) dev_free(ptr, st);
+    *s = WcsrRowStream();
+}
+
+int finish_wcsr_rows(WcsrRowStream* s, cudaStream_t st) {
+    if (!s->d_total) return SPMM_OK;
+    int32_t total[4] = {0, 0, 0, 0};
+    if (cudaMemcpyAsync(total, s->d_total, sizeof(total), cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+        return SPMM_ERR_CUDA;
+    dev_free(s->d_total, st);
+    s->d_total = nullptr;
+    s->n_tasks = total[0];
+    s->n_parts = total[1];
+    s->n_long = total[2];
+    s->n_slots = total[3];
+    return SPMM_OK;
+}
+
 }  // namespace spmm
