@@ -141,6 +141,7 @@ struct spmm_handle_s {
     const int32_t* d_merge = nullptr;      // window | first | nparts, each [n_merge]
     int n_merge = 0;
     int* d_status = nullptr;
+    WcsrRowStream rows;              // WCSR: the nonzeros for the row kernel (empty: the window kernel serves the handle)
 
     float* d_partial = nullptr;      // WCSR workspace
     size_t partial_bytes = 0;
@@ -183,6 +184,7 @@ void free_handle(spmm_handle_s* h) {
             h->d_sidx, h->d_srows, h->d_svals, h->d_stile_recs, h->d_scta_ptr, h->d_status, h->d_partial,
             h->d_plan, h->d_class};
         for (void* ptr : arrays) dev_free(ptr, nullptr);
+        free_wcsr_rows(&h->rows, nullptr);
         if (other) cudaSetDevice(dev);
         cudaFree(h->d_Bstage);
         cudaFree(h->d_Cstage);
@@ -496,6 +498,19 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
         if (!rc) rc = upload(&h->d_idx, f.window_col_idx.data(), f.window_col_idx.size() * 4);
         if (!rc) rc = upload(&h->d_vals, f.packed.data(), f.packed.size());
         if (!rc) rc = upload_wcsr_plan(h, nullptr);
+        if (!rc && wcsr_wants_rows(a.es, a.m, a.nnz, f.P)) {
+            int64_t* d_rp = nullptr;
+            int32_t* d_ci = nullptr;
+            uint8_t* d_va = nullptr;
+            rc = upload(&d_rp, a.row_ptr, static_cast<size_t>(a.m + 1) * 8);
+            if (!rc) rc = upload(&d_ci, a.col_idx, static_cast<size_t>(a.nnz) * 4);
+            if (!rc) rc = upload(&d_va, a.vals, static_cast<size_t>(a.nnz) * a.es);
+            if (!rc) rc = build_wcsr_rows_device(a.m, a.nnz, d_rp, d_ci, d_va, a.es, h->sms, nullptr, &h->rows);
+            if (!rc) rc = finish_wcsr_rows(&h->rows, nullptr);
+            dev_free(d_rp, nullptr);
+            dev_free(d_ci, nullptr);
+            dev_free(d_va, nullptr);
+        }
         if (rc) { free_handle(h); return rc; }
         std::vector<uint8_t>().swap(h->wcsr.packed);
     }
@@ -516,8 +531,8 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     if (rc) { free_handle(h); return rc; }
     try {
         rc = build_wcsr_device(m, k, d_row_ptr, d_col_idx, static_cast<const uint8_t*>(d_vals), h->es, wh, b_col, T,
-                               h->n_ctas * wcsr_bins_per_sm(h->es, wh), stream, &h->wcsr, &h->nnz, &h->d_ptr, &h->d_idx,
-                               &h->d_vals, &h->d_class);
+                               h->n_ctas * wcsr_bins_per_sm(h->es, wh), h->sms, stream, &h->wcsr, &h->nnz, &h->d_ptr, &h->d_idx,
+                               &h->d_vals, &h->d_class, &h->rows);
         h->d_grp_class = h->d_class;
         if (!rc) rc = upload_wcsr_plan(h, stream);
     } catch (const std::bad_alloc&) {
@@ -917,6 +932,62 @@ int64_t wcsr_workspace_bytes(const spmm_handle_s* h, int64_t N) {
     return h->wcsr.n_slots * int64_t{h->wcsr.wh} * N * 4;
 }
 
+// Whether a run takes the row kernel: the handle has a row stream, and the wait limit is not zero, the documented
+// hook for the path where a wait runs out, which the window kernel serves (the row kernel waits for nothing).
+bool use_rows(const spmm_handle_s* h, int64_t N) {
+    return (h->rows.n_tasks > 0 || h->rows.n_parts > 0) && g_wait_limit_ns.load() != 0 && N * h->es < (int64_t{1} << 32);
+}
+
+// Bytes of partial rows one launch of the row kernel wants for `tiles` column tiles.
+size_t rows_partial_bytes(const spmm_handle_s* h, const RowsShape& s, int tiles) {
+    return static_cast<size_t>(h->rows.n_slots) * s.tile_cols * 4 * tiles;
+}
+
+RowsShape rows_shape(const spmm_handle_s* h, const void* B, const void* C, int64_t N) {
+    // (N * es % 32 == 0 makes C's rows multiples of 32 bytes as well: its elements are at least as wide)
+    const bool aligned32 = (N * h->es) % 32 == 0 && ((reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 31) == 0;
+    return wcsr_rows_shape(N, h->es, aligned32);
+}
+
+// partial: room for cap bytes of partial rows, one column tile's at least; the column tiles go in as few
+// launches as that and the counters allow.
+int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partial, size_t cap, int64_t N, cudaStream_t stream) {
+    const WcsrRowStream& r = h->rows;
+    const RowsShape s = rows_shape(h, B, C, N);
+    WcsrRowsParams p;
+    p.tasks = reinterpret_cast<const int4*>(r.d_tasks);
+    p.parts = reinterpret_cast<const int4*>(r.d_parts);
+    p.longs = reinterpret_cast<const int4*>(r.d_longs);
+    p.order = r.d_order;
+    p.col = r.d_col;
+    p.val = r.d_val;
+    p.zeros = reinterpret_cast<const uint8_t*>(r.d_counters);
+    p.counters = r.d_counters + 8;
+    p.partial = partial;
+    p.B = B;
+    p.C = C;
+    p.N = N;
+    p.n_tasks = r.n_tasks;
+    p.n_parts = r.n_parts;
+    int step = std::min(s.tiles, kRowsMaxTiles);
+    while (step > 1 && rows_partial_bytes(h, s, step) > cap) --step;
+    if (rows_partial_bytes(h, s, step) > cap) return SPMM_ERR_TOO_LARGE;
+    for (int t = 0; t < s.tiles; t += step)
+        if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), stream) != cudaSuccess)
+            return SPMM_ERR_CUDA;
+    return SPMM_OK;
+}
+
+// What spmm_run wants at a dense width, whatever the alignment of its operands.
+size_t rows_workspace_bytes(const spmm_handle_s* h, int64_t N) {
+    size_t most = 0;
+    for (int wide = 0; wide < 2; ++wide) {
+        const RowsShape s = wcsr_rows_shape(N, h->es, wide != 0);
+        most = std::max(most, rows_partial_bytes(h, s, std::min(s.tiles, kRowsMaxTiles)));
+    }
+    return most;
+}
+
 int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, int64_t N, cudaStream_t stream) {
     const WcsrHost& f = h->wcsr;
     const int bnt = 128;                    // tokens per tile; wider B takes one pass per tile
@@ -970,7 +1041,7 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
 
 // The handle's workspace for the partial tiles of split windows at dense width N (grown, never shrunk).
 int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, cudaStream_t stream) {
-    const size_t need = static_cast<size_t>(wcsr_workspace_bytes(h, N));
+    const size_t need = use_rows(h, N) ? rows_workspace_bytes(h, N) : static_cast<size_t>(wcsr_workspace_bytes(h, N));
     if (need > h->partial_bytes) {
         if (h->d_partial) {
             if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
@@ -986,6 +1057,7 @@ int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, cudaStream_t stream) {
 
 int run_wcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t stream) {
     if (int rc = ensure_wcsr_workspace(h, N, stream)) return rc;
+    if (use_rows(h, N)) return launch_wcsr_rows_all(h, B, C, h->d_partial, h->partial_bytes, N, stream);
     return launch_wcsr_all(h, B, C, h->d_partial, N, stream);
 }
 
@@ -1131,6 +1203,8 @@ int spmm_wcsr_run_static(spmm_handle_t h, const void* B_dev, void* C_dev, int64_
     size_t cap = 0;
     if (wcsr_static_scratch(&scratch, &cap) != cudaSuccess) return SPMM_ERR_CUDA;
     if (static_cast<size_t>(wcsr_workspace_bytes(h, N)) > cap) return SPMM_ERR_TOO_LARGE;
+    if (use_rows(h, N) && rows_partial_bytes(h, rows_shape(h, B_dev, C_dev, N), 1) <= cap)
+        return launch_wcsr_rows_all(h, B_dev, C_dev, scratch, cap, N, static_cast<cudaStream_t>(stream));
     return launch_wcsr_all(h, B_dev, C_dev, scratch, N, static_cast<cudaStream_t>(stream));
 }
 

@@ -567,8 +567,9 @@ cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_
 }
 
 int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
-                      int es, int wh, int b_col, int T, int n_bins, cudaStream_t st, WcsrHost* out, int64_t* nnz_out,
-                      int32_t** d_window_row_ptr, int32_t** d_window_col_idx, uint8_t** d_packed, uint8_t** d_grp_class) {
+                      int es, int wh, int b_col, int T, int n_bins, int sms, cudaStream_t st, WcsrHost* out, int64_t* nnz_out,
+                      int32_t** d_window_row_ptr, int32_t** d_window_col_idx, uint8_t** d_packed, uint8_t** d_grp_class,
+                      WcsrRowStream* rows) {
     *d_grp_class = nullptr;
     if (wh != 16 && wh != 64) return SPMM_ERR_UNSUPPORTED;
     if ((es != 1 && es != 2 && es != 4) || b_col * es != 32) return SPMM_ERR_UNSUPPORTED;
@@ -687,6 +688,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     }
     release();                                // (ordered behind the kernels that use them)
     int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
+    if (!rc && wcsr_wants_rows(es, m, nnz, P)) rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, st, rows);
     // the split plan needs the window lengths only: the host makes it while the kernels above run
     if (!rc) {
         try {
@@ -695,8 +697,10 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
             rc = SPMM_ERR_ALLOC;
         }
     }
+    if (!rc) rc = finish_wcsr_rows(rows, st);
     if (cudaStreamSynchronize(st) != cudaSuccess && !rc) rc = SPMM_ERR_CUDA;
     if (rc) {
+        free_wcsr_rows(rows, st);
         dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st); dev_free(*d_grp_class, st);
         *d_window_row_ptr = nullptr; *d_window_col_idx = nullptr; *d_packed = nullptr; *d_grp_class = nullptr;
     }
@@ -887,6 +891,84 @@ int finish_wcsr_rows(WcsrRowStream* s, cudaStream_t st) {
     s->n_long = total[2];
     s->n_slots = total[3];
     return SPMM_OK;
+}
+
+int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
+                           int es, int sms, cudaStream_t st, WcsrRowStream* out) {
+    *out = WcsrRowStream();
+    if (m <= 0 || (es != 2 && es != 4)) return SPMM_OK;
+    // Task sizes by the entries there are per SM and 128 groups: small matrices need short tasks to fill the
+    // GPU, large ones long tasks so that fewer warps start up.  Measured (us), {pack, task_max, part_len} =
+    // {8, 64, 512} / {16, 32, 256} / {16, 64, 512} / {32, 128, 512}: 4000 rows TF32 N = 36 (2 entries):
+    // 13.7 / 8.7 / 13.7 / 23.2; 100,000 rows TF32 N = 128 (34): 34.9 / 37.8 / 36.0 / 43.1; R-MAT 2^17 bf16
+    // N = 40 (157): 49.1 / 53.5 / 49.2 / 43.5; R-MAT 2^21 fp16 N = 128 (1820): 872 / 992 / 869 / 821.
+    const int64_t per = (nnz + m) / (int64_t{sms} * 128);
+    if (per >= 100) { out->pack = 32; out->task_max = 128; out->part_len = 512; }
+    else if (per >= 16) { out->pack = 16; out->task_max = 64; out->part_len = 512; }
+    else { out->pack = 16; out->task_max = 32; out->part_len = 256; }
+    // rows of more than one part have more than part_len nonzeros: at most kRowsMaxSlots parts
+    out->part_len = static_cast<int>(std::max<int64_t>(out->part_len, (2 * nnz / kRowsMaxSlots + 127) / 128 * 128));
+    // upper bounds for the arrays, so that nothing has to be read back before the end
+    const int64_t max_tasks = 2 * ((nnz + m) / out->pack) + 2;
+    const int64_t max_long = nnz / out->task_max + 1;
+    const int64_t max_parts = max_long + nnz / out->part_len + 1;
+    const int64_t long_base = (nnz + m + 3 * max_tasks + 15) / 8 * 8;
+    const int64_t entries = long_base + nnz + 8 * max_long;
+    if (entries >= (int64_t{1} << 31) || m >= (int64_t{1} << 31) - 1) return SPMM_OK;
+
+    uint8_t *d_cls = nullptr, *d_cls2 = nullptr;
+    int32_t *d_ids = nullptr, *d_counts = nullptr, *d_head = nullptr;
+    int4 *d_size = nullptr, *d_start = nullptr;
+    void* d_temp = nullptr;
+    auto done = [&](int code) {
+        void* const arrays[] = {d_cls, d_cls2, d_ids, d_counts, d_head, d_size, d_start, d_temp};
+        for (void* ptr : arrays) dev_free(ptr, st);
+        if (code) free_wcsr_rows(out, st);
+        return code;
+    };
+    auto alloc = [&](auto** ptr, int64_t bytes) { return dev_alloc_ok(ptr, static_cast<size_t>(bytes), st); };
+    size_t t1 = 0, t2 = 0;
+    const int4 zero = make_int4(0, 0, 0, 0);
+    cub::DeviceRadixSort::SortPairs(nullptr, t1, d_cls, d_cls2, d_ids, out->d_order, static_cast<int>(m), 0, 3, st);
+    cub::DeviceScan::ExclusiveScan(nullptr, t2, d_size, d_start, Int4Sum(), zero, static_cast<int>(m + 1), st);
+    size_t tb = std::max(t1, t2);
+    const int64_t counter_bytes = 32 + max_long * kRowsMaxTiles * 4;
+    if (!alloc(&d_cls, m) || !alloc(&d_cls2, m) || !alloc(&d_ids, m * 4) || !alloc(&d_counts, kRowClasses * 4) || !alloc(&d_head, (max_tasks + 1) * 4) ||
+        !alloc(&d_size, (m + 1) * 16) || !alloc(&d_start, (m + 1) * 16) || !alloc(&d_temp, static_cast<int64_t>(tb)) ||
+        !alloc(&out->d_order, (m + 1) * 4) || !alloc(&out->d_tasks, max_tasks * 16) || !alloc(&out->d_parts, max_parts * 16) ||
+        !alloc(&out->d_longs, max_long * 16) || !alloc(&out->d_col, entries * 4) || !alloc(&out->d_val, entries * es) ||
+        !alloc(&out->d_counters, counter_bytes) || !alloc(&out->d_total, 16))
+        return done(SPMM_ERR_ALLOC);
+    cudaMemsetAsync(d_counts, 0, kRowClasses * 4, st);
+    cudaMemsetAsync(out->d_order + m, 0, 4, st);
+    cudaMemsetAsync(out->d_counters, 0, static_cast<size_t>(counter_bytes), st);
+    rows_class_kernel<<<grid_for(m, 256), 256, 0, st>>>(m, d_row_ptr, out->pack, out->task_max, d_cls, d_ids, d_counts);
+    if (cub::DeviceRadixSort::SortPairs(d_temp, tb, d_cls, d_cls2, d_ids, out->d_order, static_cast<int>(m), 0, 3, st) != cudaSuccess)
+        return done(SPMM_ERR_CUDA);
+    rows_size_kernel<<<grid_for(m + 1, 256), 256, 0, st>>>(m, out->d_order, d_row_ptr, out->task_max, out->part_len, d_size);
+    if (cub::DeviceScan::ExclusiveScan(d_temp, tb, d_size, d_start, Int4Sum(), zero, static_cast<int>(m + 1), st) != cudaSuccess)
+        return done(SPMM_ERR_CUDA);
+    RowsPlan p;
+    p.m = m;
+    p.pack = out->pack;
+    p.part_len = out->part_len;
+    p.long_base = static_cast<int>(long_base);
+    p.counts = d_counts;
+    p.start = d_start;
+    p.n_classes = 2;                                         // long, packed, and the classes between
+    for (int lim = out->task_max / 2; lim >= out->pack; lim /= 2) ++p.n_classes;
+    int4* tasks = reinterpret_cast<int4*>(out->d_tasks);
+    rows_plan_kernel<<<grid_for(m + 1, 256), 256, 0, st>>>(p, out->d_order, d_row_ptr, d_head, reinterpret_cast<int4*>(out->d_parts),
+                                                          reinterpret_cast<int4*>(out->d_longs), reinterpret_cast<int4*>(out->d_total));
+    const unsigned lg = static_cast<unsigned>(std::min<int64_t>(max_long, 1024));
+    if (es == 2) {
+        rows_fill_kernel<2><<<grid_for(m * 8, 256), 256, 0, st>>>(p, out->d_order, d_head, d_row_ptr, d_col_idx, d_vals, tasks, out->d_col, out->d_val);
+        rows_fill_long_kernel<2><<<lg, 256, 0, st>>>(p, out->d_order, d_row_ptr, d_col_idx, d_vals, out->d_col, out->d_val);
+    } else {
+        rows_fill_kernel<4><<<grid_for(m * 8, 256), 256, 0, st>>>(p, out->d_order, d_head, d_row_ptr, d_col_idx, d_vals, tasks, out->d_col, out->d_val);
+        rows_fill_long_kernel<4><<<lg, 256, 0, st>>>(p, out->d_order, d_row_ptr, d_col_idx, d_vals, out->d_col, out->d_val);
+    }
+    return done(cudaGetLastError() == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA);
 }
 
 }  // namespace spmm
