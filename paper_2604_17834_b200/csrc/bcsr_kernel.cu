@@ -8,11 +8,12 @@
 // block, K-major).  One shape therefore serves b = 16, 32, 64 and 128, and an epilogue thread
 // holds one token: a warp's registers are a [C row][32 tokens] tile, row-major like C.
 //
-// Roles (192 threads, one CTA per SM, persistent):
-//   warp 0      TMA producer: per pipeline stage (1, 2 or 4 stored blocks) one request for
-//               the A blocks and one 3-D request per block for its B tile (2*GROUPS boxes of
-//               b x 64 tokens), issued by different lanes of one warp-instruction, into a
-//               STAGES-deep shared-memory ring; full/empty mbarriers with phase bits.
+// Roles (192 to 288 threads, one CTA per SM, persistent):
+//   warps 0, 6 ..   TMA producers (one to four, BcsrProducers), taking the stages in turn: per pipeline
+//               stage (1, 2 or 4 stored blocks) one request for the A blocks and one 3-D request per
+//               block for its B tile (2*GROUPS boxes of b x 64 tokens), issued by different lanes of
+//               one warp-instruction, into a STAGES-deep shared-memory ring; full/empty mbarriers
+//               with phase bits.
 //   warp 1      MMA issuer: one thread issues tcgen05.mma into one of two TMEM accumulator
 //               buffers; tcgen05.commit frees the ring slot / publishes the accumulator.
 //   warps 2-5   epilogue: tcgen05.ld -> registers -> one of the warp's staging tiles in shared
@@ -100,7 +101,7 @@ struct BcsrCfg {
     static_assert(kEpiCols <= B && H % kEpiCols == 0, "a staging tile never straddles two block-rows");
     static_assert(2 * kAccCols <= 512, "accumulators exceed TMEM");
     static_assert(kSmemBytes <= 227 * 1024, "stage ring exceeds shared memory");
-    static_assert((2 * STAGES + 7 + 8) * 8 + 64 <= kBarrierBytes, "barrier area");
+    static_assert((2 * STAGES + 7 + 8) * 8 + 64 + 32 <= kBarrierBytes, "barrier area");
     static_assert(kBps == 1 || (B <= 32 && kKS == 1), "multi-block stages are for the small block sizes");
     static_assert(kKS == 1 || kBB <= 128, "a column slice is at most one 128-byte row piece");
     static_assert(kBB % 32 == 0, "a block row must hold whole K steps");
@@ -118,8 +119,26 @@ constexpr int bcsr_fit_stages() {
 
 constexpr int kSchedDepth = 4;      // tile indices fetched ahead by the dynamic scheduler
 
+// TMA producer warps.  One warp takes ~470 cycles per stage to see it free and to issue its two to five requests,
+// whatever their size (one CTA alone, 64 x 64 blocks at 128 tokens, 24 KB a stage: 471 cycles a block without the
+// MMAs, 311 with the MMAs and without the loads, 517 with both), so up to four warps take the stages in turn.
+// Measured with one -> four warps (us): down-projection 3584 x 18944, N = 128, bf16 21.1 -> 14.3; N = 2048, E4M3
+// 68.1 -> 36.9; TF32, 64 x 64, N = 3000 115.5 -> 91.1; b = 32, N = 1000 229 -> 161; the prefill shapes within 1 %.
+// 512-token stages of 64-row blocks (or of 1-byte values) stay with one: a request is 32 KB there and the loads
+// are not short of issue; with four, E4M3 with fp32 C was slower, the loads crowding out the stores (N = 9001
+// 185 -> 234).
+// At most one warp per stage: a warp's parity wait on a stage's empty barrier is exact only while that barrier is
+// at most one phase behind the use the warp is about to fill, that is, while unit it - 2 STAGES has been consumed;
+// the warp's own previous unit it - NP tells it that unit it - NP - STAGES has.
+template <int B, int GROUPS, int STAGES, int ES, int DYN>
+struct BcsrProducers {
+    static constexpr int kMost = STAGES < 4 ? STAGES : 4;
+    static constexpr int n = (DYN || (GROUPS == 4 && (B >= 64 || ES == 1))) ? 1 : kMost;
+    static constexpr int kThreads = DYN ? 224 : 160 + 32 * n;
+};
+
 template <int B, int H, int GROUPS, int STAGES, int FMT, int CT, int CM, int DYN>
-__global__ void __launch_bounds__(DYN ? 224 : 192, 1)
+__global__ void __launch_bounds__((BcsrProducers<B, GROUPS, STAGES, FMT == 3 ? 1 : (FMT == 2 ? 4 : 2), DYN>::kThreads), 1)
 bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmB3, const __grid_constant__ CUtensorMap tmC,
                  const __grid_constant__ CUtensorMap tmP, const BcsrParams p) {
@@ -221,13 +240,18 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
     };
 
-    if (warp == 0) {
-        // ------------------------------------------------------------------ TMA producer
+    constexpr int NP = BcsrProducers<B, GROUPS, STAGES, ES, DYN>::n;
+    static_assert(NP <= STAGES && NP <= 4, "parity waits; slots of `issued`");
+    // units issued by every producer warp (its own among those below this count): for the abort path
+    volatile uint32_t* issued = reinterpret_cast<volatile uint32_t*>(reinterpret_cast<uint8_t*>(bars) + Cfg::kBarrierBytes - 16);
+    if (warp == 0 || (!DYN && warp >= 6)) {
+        // ------------------------------------------------------------------ TMA producers
         // A warp serialises the TMA requests of its lanes (~60 cycles each) but needs far
         // longer for requests issued one after the other by a single thread, so the loads of
         // a stage are spread over the lanes: lane x < nbox fetches B box x, lanes 8 / 9 the
         // A block (two halves when b = 128).  Lane 0 posts the stage's byte count first.
         {
+            const uint32_t pw = warp == 0 ? 0 : warp - 5;   // this warp takes the stage units pw, pw + NP, ...
             uint32_t it = 0;
             bool ok = true;
             // A blocks and the B slab are re-read by other CTAs while the slab lasts: ask L2 to
@@ -255,6 +279,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     for (int jq = 0; jq < nq && ok; jq += Cfg::kBps)
 #pragma unroll 1
                     for (int kp = 0; kp < Cfg::kKS; ++kp, ++it) {       // column slices of the block (1 unless TF32, b >= 64)
+                        if (NP > 1 && it % NP != pw) continue;
                         const int q = q0 + jq;
                         const int kx = kp * Cfg::kKB;                    // first column of A / first row of B of this unit
                         const int nb = min(Cfg::kBps, nq - jq);          // stored blocks in this stage
@@ -313,12 +338,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 }
             }
-            if (!ok && lane == 0) {
-                // leave no bulk copy in flight: wait (bounded) for the fills already issued
-                const uint32_t first = it > STAGES ? it - STAGES : 0;
-                for (uint32_t j = first; j < it; ++j)
-                    if (!mbar_drain_wait(full_bar(j % STAGES), (j / STAGES) & 1u, ctl, 21)) break;
-            }
+            if (lane == 0) issued[pw] = it;
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
@@ -517,6 +537,19 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
     tc_fence_before_sync();
     __syncthreads();
+    if (threadIdx.x == 0 && *abort_flag) {
+        // leave no bulk copy in flight: wait (bounded) for the last fill issued into every stage
+        uint32_t most = 0;
+        for (int w = 0; w < NP; ++w) most = issued[w] > most ? issued[w] : most;
+        bool ok = true;
+        for (uint32_t s = 0; s < STAGES && ok; ++s) {
+            for (uint32_t j = most; j-- > 0;) {              // a stage's last fill is among the last few units
+                if (j % STAGES != s || j >= issued[j % NP]) continue;
+                ok = mbar_drain_wait(full_bar(s), (j / STAGES) & 1u, ctl, 21);
+                break;
+            }
+        }
+    }
     // launched while the previous grid of the stream was still running: do not finish before it
     if (p.overlap == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (warp == 1) {
@@ -544,6 +577,7 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
     constexpr int CS = static_cast<int>(sizeof(typename CType<FMT, CT>::type));
     constexpr int STAGES = bcsr_fit_stages<B, H, GROUPS, CAP, ES, CS, CM>();
     using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, CS, CM>;
+    constexpr int kThreads = BcsrProducers<B, GROUPS, STAGES, ES, DYN>::kThreads;
     auto kfn = bcsr_spmm_kernel<B, H, GROUPS, STAGES, FMT, CT, CM, DYN>;
     // the attribute belongs to the (function, device) pair: set it once per device
     static std::mutex mu;
@@ -563,7 +597,7 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
     if (p.overlap == 2) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(static_cast<unsigned>(grid));
-        cfg.blockDim = dim3(DYN ? 224 : 192);
+        cfg.blockDim = dim3(kThreads);
         cfg.dynamicSmemBytes = Cfg::kSmemBytes;
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];
@@ -573,7 +607,7 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
         cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kfn, tmA, tmB, tmB3, tmC, tmP, p);
     }
-    kfn<<<grid, DYN ? 224 : 192, Cfg::kSmemBytes, stream>>>(tmA, tmB, tmB3, tmC, tmP, p);
+    kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmB, tmB3, tmC, tmP, p);
     return cudaGetLastError();
 }
 
