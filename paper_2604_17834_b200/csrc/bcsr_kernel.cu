@@ -192,18 +192,21 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
-    // the row groups' launch: the launch of the remaining block-rows may begin on the SMs this
-    // grid leaves idle (the two write disjoint rows of C)
-    if (p.overlap == 1) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
     const int64_t N = p.N;
     // Static schedule: this CTA's range of the tile list.  Dynamic: tile blockIdx.x, then the
     // indices the scheduler warp obtains; every working warp walks the same sequence.
     int tile_begin = 0, tile_end = 0;
+    int4 rec0 = make_int4(0, 0, 0, 0);               // record of this CTA's first tile
     if constexpr (!DYN) {
         tile_begin = __ldg(p.cta_ptr + blockIdx.x);
         tile_end = __ldg(p.cta_ptr + blockIdx.x + 1);
+        if (tile_begin < tile_end) rec0 = __ldg(p.tiles + tile_begin);
     }
+    // The row groups' launch (overlap = 1): the launch of the remaining block-rows runs beside this one (the two
+    // write disjoint rows of C), so it is let go only when the operands are ready.
+    if (p.overlap != 1) grid_trigger();
+    if (p.overlap != 2) grid_wait();
+    if (p.overlap == 1) grid_trigger();
     // Next tile of this warp's walk; nth = number of tiles it has taken so far.  A tile's record
     // {block-row, token tile, first stored block, end block} is all a role needs to know about
     // it; with the static schedule the following tile's record is requested one tile ahead
@@ -212,7 +215,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         if constexpr (!DYN) {
             const int ti = tile_begin + static_cast<int>(nth);
             if (ti >= tile_end) return false;
-            *rec = nth == 0 ? __ldg(p.tiles + ti) : *rec_next;
+            *rec = nth == 0 ? rec0 : *rec_next;
             if (ti + 1 < tile_end) *rec_next = __ldg(p.tiles + ti + 1);
             return true;
         } else {
@@ -551,7 +554,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
     }
     // launched while the previous grid of the stream was still running: do not finish before it
-    if (p.overlap == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (p.overlap == 2) grid_wait();
     if (warp == 1) {
         if (*abort_flag) {
             // abort path: let the MMAs this warp's elected lane already issued finish before
@@ -594,21 +597,12 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
             attr_done[dev] = true;
         }
     }
-    if (p.overlap == 2) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(grid));
-        cfg.blockDim = dim3(kThreads);
-        cfg.dynamicSmemBytes = Cfg::kSmemBytes;
-        cfg.stream = stream;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        return cudaLaunchKernelEx(&cfg, kfn, tmA, tmB, tmB3, tmC, tmP, p);
+    if constexpr (DYN) {        // (its grid is a queue of CTAs that running ones cancel: launched when the stream gets there)
+        kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmB, tmB3, tmC, tmP, p);
+        return cudaGetLastError();
+    } else {
+        return launch_dependent(kfn, dim3(static_cast<unsigned>(grid)), kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmB3, tmC, tmP, p);
     }
-    kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmB, tmB3, tmC, tmP, p);
-    return cudaGetLastError();
 }
 
 template <int FMT, int CT, int CM, int DYN>
@@ -753,7 +747,8 @@ __global__ void __launch_bounds__(256) bcsr_merge_kernel(const BcsrMergeParams p
     const int i = blockIdx.x;
     const int I = p.row[i], first = p.first[i], nparts = p.nparts[i];
     // the partial tiles belong to the SpMM kernel launched just before on the same stream
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    grid_trigger();
+    grid_wait();
     const int64_t N = p.N, n4 = N >> 2;                 // N is a multiple of 4 (16-byte rows)
     const int64_t row0 = static_cast<int64_t>(I) * p.b;
     const int64_t rows = min_i64(p.b, p.m - row0);
@@ -786,18 +781,9 @@ __global__ void __launch_bounds__(256) bcsr_merge_kernel(const BcsrMergeParams p
 
 cudaError_t launch_bcsr_merge(const BcsrMergeParams& p, cudaStream_t stream) {
     if (p.n <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
     const int64_t pieces = static_cast<int64_t>(p.b) * (p.N >> 2);
-    cfg.gridDim = dim3(static_cast<unsigned>(p.n), static_cast<unsigned>((pieces + 256 * kMergePieces - 1) / (256 * kMergePieces)));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, bcsr_merge_kernel, p);
+    const dim3 grid(static_cast<unsigned>(p.n), static_cast<unsigned>((pieces + 256 * kMergePieces - 1) / (256 * kMergePieces)));
+    return launch_dependent(bcsr_merge_kernel, grid, 256, 0, stream, p);
 }
 
 }  // namespace spmm

@@ -7,6 +7,24 @@
 
 namespace spmm {
 
+// Launch with programmatic stream serialisation (see grid_wait in ptx.cuh).  Measured back to back: BCSR
+// 512 x 512, N = 256 6.15 -> 4.25 us, 3584 x 18944 N = 128
+// 14.3 -> 11.4; WCSR 4000 rows, N = 36 8.2 -> 6.5, 100,000 rows, N = 128 38.0 -> 35.1; long launches unchanged.
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(static_cast<unsigned>(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // per-device caches (kernel attributes, the built-in scratch address) are arrays of this length
 constexpr int kMaxDevices = 64;
 
@@ -24,9 +42,9 @@ struct BcsrParams {
     // tile records then name {group, token tile, first stacked block, end stacked block} and
     // block_col_idx is the stacked blocks' column index
     const int32_t* stack_rows;
-    // 1: this grid lets the next launch of the stream start while it runs (its first
-    // instruction after set-up is griddepcontrol.launch_dependents); 2: this grid was launched
-    // that way behind another one and waits for it (griddepcontrol.wait) before its CTAs exit
+    // 0: waits for the launch before it in the stream before it touches an operand (grid_wait).
+    // 1: the same, and the next launch may run beside it: it is let go (grid_trigger) after that wait.
+    // 2: such a next launch: it may start at once, and waits for the one before it before its CTAs exit
     int32_t overlap;
 };
 

@@ -38,6 +38,16 @@ __device__ __forceinline__ bool elect_one() {
     return pred != 0;
 }
 
+// ----------------------------------------------------------------------------- dependent launches
+
+// Every kernel of a run is launched with programmatic stream serialisation: its CTAs may start, and set
+// themselves up from creation-time data, while the kernel before it in the stream is still running.
+// grid_wait returns once that kernel has completed and its writes are visible; nothing that it may
+// write (the dense operand) or still read or write (C, workspaces) is touched before.  grid_trigger lets
+// the next launch of the stream start in the same way.  (No effect in launches without the attribute.)
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ----------------------------------------------------------------------------- mbarrier
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {

@@ -129,10 +129,9 @@ wcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmB, const WcsrParams p) {
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    // The merge kernel is launched as a programmatic dependent: let its CTAs be scheduled (and
-    // fetch their lists) while this grid runs; they block in griddepcontrol.wait until this
-    // grid has completed and its writes are visible.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the merge kernel's CTAs may be scheduled (and fetch their lists) while this grid runs
+    grid_trigger();
+    grid_wait();
     const uint32_t tmem_base = *tmem_slot;
     const int64_t N = p.N;
     const int2 kNoDesc = make_int2(0, 0);
@@ -525,7 +524,8 @@ wcsr_merge_kernel(const MergeParams p) {
     const int nparts = p.nparts[i];
     // everything above is creation-time data; the partial tiles and C belong to the SpMM
     // kernel launched just before on the same stream: wait until it has completed
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    grid_trigger();
+    grid_wait();
     const int64_t N = p.N;
     const int64_t row0 = static_cast<int64_t>(w) * kWH;
     const int rows = static_cast<int>(min_i64(kWH, p.m - row0));
@@ -577,8 +577,7 @@ cudaError_t launch_one(const CUtensorMap& tmB, const WcsrParams& p, int sms, cud
     int grid = sms * Cfg::kCtasPerSm;
     if (grid > p.n_bins) grid = p.n_bins;
     if (grid < 1) return cudaSuccess;
-    kfn<<<grid, (PW + 5) * 32, Cfg::kSmemBytes, stream>>>(tmB, p);
-    return cudaGetLastError();
+    return launch_dependent(kfn, dim3(static_cast<unsigned>(grid)), (PW + 5) * 32, Cfg::kSmemBytes, stream, tmB, p);
 }
 
 template <int WH>
@@ -642,24 +641,10 @@ cudaError_t wcsr_static_scratch(float** ptr, size_t* bytes) {
 // ctype: 0 = fp32 C, 1 = fp16, 2 = bf16
 cudaError_t launch_wcsr_merge(const MergeParams& p, int wh, int ctype, cudaStream_t stream) {
     if (p.n <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(p.n));
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (wh == 64) {
-        if (ctype == 1) return cudaLaunchKernelEx(&cfg, wcsr_merge_kernel<__half, 64>, p);
-        if (ctype == 2) return cudaLaunchKernelEx(&cfg, wcsr_merge_kernel<__nv_bfloat16, 64>, p);
-        return cudaLaunchKernelEx(&cfg, wcsr_merge_kernel<float, 64>, p);
-    }
-    if (ctype == 1) return cudaLaunchKernelEx(&cfg, wcsr_merge_kernel<__half, 16>, p);
-    if (ctype == 2) return cudaLaunchKernelEx(&cfg, wcsr_merge_kernel<__nv_bfloat16, 16>, p);
-    return cudaLaunchKernelEx(&cfg, wcsr_merge_kernel<float, 16>, p);
+    const dim3 grid(static_cast<unsigned>(p.n));
+    auto go = [&](auto kfn) { return launch_dependent(kfn, grid, 256, 0, stream, p); };
+    if (wh == 64) return ctype == 1 ? go(wcsr_merge_kernel<__half, 64>) : (ctype == 2 ? go(wcsr_merge_kernel<__nv_bfloat16, 64>) : go(wcsr_merge_kernel<float, 64>));
+    return ctype == 1 ? go(wcsr_merge_kernel<__half, 16>) : (ctype == 2 ? go(wcsr_merge_kernel<__nv_bfloat16, 16>) : go(wcsr_merge_kernel<float, 16>));
 }
 
 }  // namespace spmm

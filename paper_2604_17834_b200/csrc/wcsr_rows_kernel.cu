@@ -150,6 +150,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     extern __shared__ float red[];                        // long rows: [kStrands][VE][lanes]
     __shared__ unsigned arrived;
 
+    grid_trigger();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane / p.lanes, l = lane - g * p.lanes;
     const int tile = p.tile0 + blockIdx.y;
@@ -173,12 +174,16 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     if (static_cast<int>(blockIdx.x) >= p.n_parts) {
         // ------------------------------------------------------------------ whole rows, one task per group
         const int id = ((static_cast<int>(blockIdx.x) - p.n_parts) * kWarps + warp) * p.groups + g;
-        if (!on || id >= p.n_tasks) return;
+        if (!on || id >= p.n_tasks) {
+            grid_wait();                                  // (a CTA of this grid has always waited: the next launch relies on it)
+            return;
+        }
         const int4 d = __ldg(p.tasks + id);               // first entry, entries, position in order
         const int32_t* order = p.order + d.z;
         uint8_t* C = static_cast<uint8_t*>(p.C) + n * sizeof(CElem);
         Ent4<ES> cur = ld_ent4<ES>(p.col, p.val, d.x, d.y > 0);
         int row = __ldg(order);
+        grid_wait();
         for (int e = 0; e < d.y; e += 4) {
             Vec<VB> b[4];
 #pragma unroll
@@ -202,6 +207,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     // ---------------------------------------------------------------------- one part of a long row
     const int4 d = __ldg(p.parts + blockIdx.x);           // first entry, entries, long row, part
     const int4 lr = __ldg(p.longs + d.z);                 // row, first slot, parts
+    grid_wait();
     const int n_groups = kWarps * p.groups;
     const int tile_cols = p.lanes * VE;
     if (g < p.groups) {
@@ -268,13 +274,11 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
 
 template <int VB>
 cudaError_t launch_vb(int dtype, int c16, const WcsrRowsParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
-    if (dtype == 2) wcsr_rows_kernel<2, 0, VB><<<grid, kRowsThreads, smem, stream>>>(p);
-    else if (dtype == 1 && c16) wcsr_rows_kernel<0, 1, VB><<<grid, kRowsThreads, smem, stream>>>(p);
-    else if (dtype == 1) wcsr_rows_kernel<0, 0, VB><<<grid, kRowsThreads, smem, stream>>>(p);
-    else if (dtype == 0 && c16) wcsr_rows_kernel<1, 1, VB><<<grid, kRowsThreads, smem, stream>>>(p);
-    else if (dtype == 0) wcsr_rows_kernel<1, 0, VB><<<grid, kRowsThreads, smem, stream>>>(p);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    auto go = [&](auto kfn) { return launch_dependent(kfn, grid, kRowsThreads, smem, stream, p); };
+    if (dtype == 2) return go(wcsr_rows_kernel<2, 0, VB>);
+    if (dtype == 1) return c16 ? go(wcsr_rows_kernel<0, 1, VB>) : go(wcsr_rows_kernel<0, 0, VB>);
+    if (dtype == 0) return c16 ? go(wcsr_rows_kernel<1, 1, VB>) : go(wcsr_rows_kernel<1, 0, VB>);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace

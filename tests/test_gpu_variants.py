@@ -581,3 +581,38 @@ def test_bcsr_fp8_e4m3_rowmajor(lib, b, N):
     finally:
         lib.spmm_destroy(h0)
         lib.spmm_destroy(h1)
+
+
+@pytest.mark.parametrize("kind,opt", [("bcsr", {}), ("bcsr", dict(stack_min_fill=-1)), ("wcsr", {}), ("wcsr", dict(split_cols=64))])
+def test_runs_that_feed_one_another_on_a_stream(lib, kind, opt):
+    """Launches overlap (each sets itself up while the one before it is running): a run whose dense operand
+    is the previous run's result, and whose result overwrites what that run read, sees every value in place.
+    A chain of eight unsynchronised products equals the same chain with a synchronise after every run."""
+    import torch
+    n, N, dtype = 1536, 192, "fp16"
+    if kind == "bcsr":                     # 10 % full block-rows: row groups unless switched off
+        a = wl.bcsr_sweep(611, m=n, k=n, b=16, density=0.1, dtype=dtype)
+        mk, size = lib.spmm_bcsr_create_csr, 16
+    else:                                  # one nonzero per window column, or (dense windows) the window kernel
+        a = wl.wcsr_irregular(seed=612, m=n, dtype=dtype, max_len=400) if opt == {} else wl.random_csr(613, n, n, 0.3, dtype)
+        mk, size = lib.spmm_wcsr_create_csr, 16
+    vals = wl.to_storage(wl.widen(a["vals"], dtype) * (1.0 / 16), dtype)
+    h = mk(n, n, a["row_ptr"], a["col_idx"], vals, dtype, size, c_type=lib.C_SAME_AS_INPUT, **opt)
+    st = torch.cuda.current_stream().cuda_stream
+    try:
+        x0 = to_device(wl.dense(614, n, N, ("normal", 0.0, 1.0), dtype))
+        outs = []
+        for sync in (True, False, False):
+            x, y = x0.clone(), torch.empty_like(x0)
+            for _ in range(8):
+                lib.spmm_run(h, x.data_ptr(), y.data_ptr(), N, st)
+                if sync:
+                    torch.cuda.synchronize()
+                x, y = y, x
+            torch.cuda.synchronize()
+            lib.spmm_check(h)
+            outs.append(x.clone())
+        assert bool(torch.isfinite(outs[0]).all())
+        assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
+    finally:
+        lib.spmm_destroy(h)
