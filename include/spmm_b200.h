@@ -68,7 +68,7 @@ typedef enum {
                                     k8 instruction shape of Sec. 3.1; Sec. 4.1 evaluates both
                                     formats in it).  WCSR, and BCSR with every block size and
                                     both layouts; C is fp32, the BCSR schedule static, and
-                                    BCSR row groups are not formed.                           */
+                                    BCSR row groups are formed for block 16 and 32.           */
     SPMM_FP8_E4M3 = 3            /* 1-byte E4M3 storage (Sec. 5 names 8-bit inputs as the next
                                     step); fp32 C.  BCSR: static schedule, block 32, 64 or
                                     128; row-major operands need N >= 128 and N % 16 == 0,
@@ -111,6 +111,11 @@ typedef enum {
     SPMM_GATHER_TMA = 0,         /* TMA row gather (four rows x 128 bytes per request), the
                                     default: the indirect load Sec. 3.2 says TMA cannot do is
                                     available on this architecture                            */
+                                 /* (a WCSR handle whose windows condense almost nothing -- at most
+                                    two nonzeros per padded column; 2- and 4-byte values -- sums C
+                                    row by row from a private copy of the nonzeros instead of
+                                    gathering for window tiles; this option is then without effect,
+                                    and SPMM_TF32 operands are multiplied as full fp32 values)   */
     SPMM_GATHER_LSU = 1          /* the paper's own scheme (Sec. 3.2): the producer warps copy
                                     the rows with 128-bit loads through the load/store units
                                     (16-byte cp.async) to the swizzled positions the MMA reads.

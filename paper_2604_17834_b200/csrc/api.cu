@@ -116,7 +116,9 @@ struct spmm_handle_s {
     int32_t* d_stile_recs = nullptr; // {group, token tile, first stacked block, end}
     int32_t* d_scta_ptr = nullptr;
     CUtensorMap tmAs;                // map of d_svals
-    CUtensorMap tmB3s;               // whole-tile map of B for the stacked launch's 256-token tile
+    int stack_groups = 0;            // token groups of the stacked launch's tile (2, or 1: see ensure_schedule)
+    int32_t* d_rec_ptr = nullptr;    // ranges of d_tile_recs per CTA
+    CUtensorMap tmB3s;               // whole-tile map of B for the stacked launch's token tile
     bool tmB3s_ok = false;
     int k_split = 0;                 // opts.k_split (1: cut outlier block-rows into parts)
     int32_t* d_kmerge = nullptr;     // K-split merge lists: row | first slot | parts, each [n_kmerge]
@@ -182,7 +184,7 @@ void free_handle(spmm_handle_s* h) {
         void* const arrays[] = {
             h->d_ptr, h->d_idx, h->d_vals, h->d_order, h->d_tiles, h->d_tile_recs, h->d_cta_ptr, h->d_kmerge,
             h->d_sidx, h->d_srows, h->d_svals, h->d_stile_recs, h->d_scta_ptr, h->d_status, h->d_partial,
-            h->d_plan, h->d_class};
+            h->d_plan, h->d_class, h->d_rec_ptr};
         for (void* ptr : arrays) dev_free(ptr, nullptr);
         free_wcsr_rows(&h->rows, nullptr);
         if (other) cudaSetDevice(dev);
@@ -287,8 +289,8 @@ int encode_tmA(spmm_handle_s* h) {
 int setup_stack(spmm_handle_s* h) {
     const BcsrHost& f = h->bcsr;
     // static schedule only; b = 128 blocks already are 128 rows high
-    // (row groups exist for the 16-bit types, and for E4M3 with column-major operands)
-    const bool eligible = !h->dynamic && f.b < 128 && h->stack_min_fill >= 0 && h->dtype != SPMM_TF32 &&
+    // (row groups exist for the 16-bit types, for TF32 with block rows of up to 128 bytes, and for E4M3 with column-major operands)
+    const bool eligible = !h->dynamic && f.b < 128 && h->stack_min_fill >= 0 && !(h->dtype == SPMM_TF32 && f.b > 32) &&
                           !(h->dtype == SPMM_FP8_E4M3 && !h->col_major);
     int rc = build_bcsr_stack(f, eligible ? h->stack_min_fill : -1, &h->stack);
     if (rc || h->host_only || h->stack.ng == 0) return rc;
@@ -607,7 +609,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
             if (!*ok) *out = h->tmB;
         };
         whole_tile_map(groups, &h->tmB3, &h->tmB3_ok);
-        if (h->stack.ng > 0) whole_tile_map(kStackGroups, &h->tmB3s, &h->tmB3s_ok);
+        if (h->stack.ng > 0 && h->stack_groups > 0) whole_tile_map(h->stack_groups, &h->tmB3s, &h->tmB3s_ok);
     } else {
         // B as [k][N]: box = kb rows (the block's k extent, or one column slice of A's block:
         // bcsr_k_split) x 128 bytes of tokens; 4-byte elements take the 128-byte swizzle with
@@ -634,7 +636,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
             if (!*ok) *out = h->tmB;
         };
         whole_tile_map(groups, &h->tmB3, &h->tmB3_ok);
-        if (h->stack.ng > 0) whole_tile_map(kStackGroups, &h->tmB3s, &h->tmB3s_ok);
+        if (h->stack.ng > 0 && h->stack_groups > 0) whole_tile_map(h->stack_groups, &h->tmB3s, &h->tmB3s_ok);
     }
     if (rc) return rc;
     h->tmB_ptr = B;
@@ -695,6 +697,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     if (sw < 1) sw = 1;
     if (sw > n_tt) sw = n_tt;
     BcsrSchedule sc, ss;
+    BcsrSchedule kc, ks;             // what the kernels run where it is not the exported plan: narrower tiles of the row groups
+    bool narrow = false;
     const BcsrStack& st = h->stack;
     int rc;
     try {
@@ -739,7 +743,7 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             }
             std::vector<int64_t> loads;
             rc = build_tile_schedule(units, lens, kStackTileFixedCost, n_tt_s, static_cast<int>(sws), h->n_ctas, &ss,
-                                     bcsr_stack_block_cost(), nullptr, &loads);
+                                     bcsr_stack_block_cost(kStackGroups), nullptr, &loads);
             ss.groups = kStackGroups;
             ss.N = N;
             if (!rc) {
@@ -752,8 +756,35 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                     units.push_back(I);
                     lens.push_back(f.block_row_ptr[I + 1] - f.block_row_ptr[I]);
                 }
+                std::vector<int64_t> totals;
                 rc = build_tile_schedule(units, lens, kTileFixedCost, n_tt, static_cast<int>(sw), h->n_ctas, &sc,
-                                         bcsr_block_cost(f.b, groups), &loads);
+                                         bcsr_block_cost(f.b, groups), &loads, &totals);
+                // Where the longest tile of a row group alone exceeds a CTA's share of the whole work by half (few groups,
+                // a narrow dense operand), its launch is a handful of CTAs working while the others are done: the
+                // groups then run with 128-token tiles, twice as many and less than half as long.  Results are the
+                // same bits (a token's sums do not depend on its tile).  10 % full block-rows, us: 6000 x 5000 TF32,
+                // b = 32, N = 1500 (24 tiles of 157 stacked blocks, an 80 us launch whose CTAs were busy for 18 us on
+                // average) 79.6 -> 50.4; 8192 x 8192 fp16, b = 32, N = 504 78.7 -> 53.0; with the share exceeded by
+                // 15 % only (b = 16, N = 1000) 99.7 -> 103.6, the stacked blocks being fetched twice as often.
+                int64_t work = 0, longest = 0;
+                for (int64_t x : totals) work += x;
+                for (int64_t g = 0; g < st.ng; ++g) longest = std::max<int64_t>(longest, st.ptr[g + 1] - st.ptr[g]);
+                longest = (longest + kStackTileFixedCost) * bcsr_stack_block_cost(kStackGroups);
+                if (!rc && N > 128 && 2 * longest * h->n_ctas > 3 * work) {
+                    narrow = true;
+                    std::vector<int32_t> gu, gl;
+                    for (int64_t g = 0; g < st.ng; ++g) {
+                        gu.push_back(static_cast<int32_t>(g));
+                        gl.push_back(st.ptr[g + 1] - st.ptr[g]);
+                    }
+                    rc = build_tile_schedule(gu, gl, kStackTileFixedCost, static_cast<int>((N + 127) / 128), static_cast<int>(2 * sws), h->n_ctas, &ks,
+                                             bcsr_stack_block_cost(1), nullptr, &loads);
+                    if (!rc) {
+                        std::sort(loads.begin(), loads.end());
+                        rc = build_tile_schedule(units, lens, kTileFixedCost, n_tt, static_cast<int>(sw), h->n_ctas, &kc,
+                                                 bcsr_block_cost(f.b, groups), &loads);
+                    }
+                }
             }
         }
     } catch (const std::bad_alloc&) {
@@ -767,23 +798,25 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
             dev_free(h->d_tiles, nullptr);
             dev_free(h->d_tile_recs, nullptr);
+            dev_free(h->d_rec_ptr, nullptr);
             dev_free(h->d_cta_ptr, nullptr);
             dev_free(h->d_stile_recs, nullptr);
             dev_free(h->d_scta_ptr, nullptr);
             dev_free(h->d_kmerge, nullptr);
-            h->d_tiles = h->d_tile_recs = h->d_cta_ptr = h->d_stile_recs = h->d_scta_ptr = h->d_kmerge = nullptr;
+            h->d_tiles = h->d_tile_recs = h->d_rec_ptr = h->d_cta_ptr = h->d_stile_recs = h->d_scta_ptr = h->d_kmerge = nullptr;
             h->n_kmerge = 0;
             h->tmP_ok = false;
         }
         rc = upload(&h->d_tiles, sc.tiles.data(), sc.tiles.size() * 4);
         if (!rc) {
             // self-contained records, so that a role needs one load per tile (and can fetch it a tile ahead)
-            const size_t nt = sc.tiles.size() / 2;
+            const BcsrSchedule& run = narrow ? kc : sc;
+            const size_t nt = run.tiles.size() / 2;
             std::vector<int32_t> recs(4 * nt);
             for (size_t i = 0; i < nt; ++i) {
-                recs[4 * i + 1] = sc.tiles[2 * i + 1];
-                if (sc.units.empty()) {
-                    const int32_t I = sc.tiles[2 * i];
+                recs[4 * i + 1] = run.tiles[2 * i + 1];
+                if (run.units.empty()) {
+                    const int32_t I = run.tiles[2 * i];
                     recs[4 * i] = I;
                     recs[4 * i + 2] = f.block_row_ptr[I];
                     recs[4 * i + 3] = f.block_row_ptr[I + 1];
@@ -797,6 +830,7 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                 }
             }
             rc = upload(&h->d_tile_recs, recs.data(), recs.size() * 4);
+            if (!rc) rc = upload(&h->d_rec_ptr, run.cta_ptr.data(), run.cta_ptr.size() * 4);
         }
         if (!rc && sc.n_slots > 0) {
             // merge lists (split block-rows in ascending order: their slots are consecutive), the
@@ -840,20 +874,23 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
         }
         if (!rc) rc = upload(&h->d_cta_ptr, sc.cta_ptr.data(), sc.cta_ptr.size() * 4);
         if (!rc && !ss.tiles.empty()) {
-            const size_t nt = ss.tiles.size() / 2;
+            const BcsrSchedule& run = narrow ? ks : ss;
+            const size_t nt = run.tiles.size() / 2;
             std::vector<int32_t> recs(4 * nt);
             for (size_t i = 0; i < nt; ++i) {
-                const int32_t g = ss.tiles[2 * i];
+                const int32_t g = run.tiles[2 * i];
                 recs[4 * i] = g;
-                recs[4 * i + 1] = ss.tiles[2 * i + 1];
+                recs[4 * i + 1] = run.tiles[2 * i + 1];
                 recs[4 * i + 2] = st.ptr[g];
                 recs[4 * i + 3] = st.ptr[g + 1];
             }
             rc = upload(&h->d_stile_recs, recs.data(), recs.size() * 4);
-            if (!rc) rc = upload(&h->d_scta_ptr, ss.cta_ptr.data(), ss.cta_ptr.size() * 4);
+            if (!rc) rc = upload(&h->d_scta_ptr, run.cta_ptr.data(), run.cta_ptr.size() * 4);
         }
         if (rc) return rc;
     }
+    h->stack_groups = ss.tiles.empty() ? 0 : (narrow ? 1 : kStackGroups);
+    h->tmB_N = -1;                   // (the stacked launch's map of B depends on its tile)
     h->sched_stack = std::move(ss);
     h->sched = std::move(sc);
     return SPMM_OK;
@@ -870,7 +907,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.block_row_ptr = h->d_ptr;
     p.block_col_idx = h->d_idx;
     p.tiles = reinterpret_cast<const int4*>(h->d_tile_recs);
-    p.cta_ptr = h->d_cta_ptr;
+    p.cta_ptr = h->d_rec_ptr;
     p.C = C;
     p.m = h->m;
     p.N = N;
@@ -899,7 +936,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         ps.use_3d = h->tmB3s_ok ? 1 : 0;
         ps.overlap = 1;
         p.overlap = 2;
-        cudaError_t es = launch_bcsr_stacked(h->dtype, f.b, h->c16, h->col_major, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
+        cudaError_t es = launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
                                              h->n_ctas, stream);
         if (es != cudaSuccess) return SPMM_ERR_CUDA;
         if (h->sched.tiles.empty()) return SPMM_OK;

@@ -75,7 +75,7 @@ struct BcsrCfg {
     // Small blocks carry too little work for the fixed cost of a pipeline stage (barrier
     // round trip, request issue, MMA hand-off): a stage holds several consecutive stored
     // blocks of the block-row, their B tiles first, then their A blocks (one request).
-    static constexpr int kBps = bcsr_blocks_per_stage(B);
+    static constexpr int kBps = H == B ? bcsr_blocks_per_stage(B) : bcsr_stacked_per_stage(B, ES);
     static constexpr int kStageBytes = ((kBps * (kDenseBytes + kABytes) + 1023) / 1024) * 1024;
     static constexpr int kAOff = kBps * kDenseBytes;         // A blocks inside the stage
     static constexpr int kARowBytes = kBB < 128 ? kBB : 128;
@@ -143,7 +143,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                  const __grid_constant__ CUtensorMap tmB3, const __grid_constant__ CUtensorMap tmC,
                  const __grid_constant__ CUtensorMap tmP, const BcsrParams p) {
     constexpr int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2);
-    static_assert(FMT != 2 || (!CT && !DYN && H == B), "TF32: fp32 C, static schedule, no row groups");
+    static_assert(FMT != 2 || (!CT && !DYN && (H == B || B <= 32)), "TF32: fp32 C, static schedule, row groups of rows up to 128 bytes");
     static_assert(H == B || !DYN, "stacked blocks: static schedule only");
     using CElem = typename CType<FMT, CT>::type;
     using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, static_cast<int>(sizeof(CElem)), CM>;
@@ -357,7 +357,13 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             constexpr int kStepBytes = (32 / ES) * 128;     // k-rows of one MMA x 128 bytes (row-major token tile)
             const uint64_t bdesc0 = make_smem_desc(0, 16, 8 * Cfg::kARowBytes, Cfg::kASwizzle);
             const bool leader = elect_one();
+            // Whether the next stage's full barrier was already seen complete: with one token group the next stage is
+            // tested before this stage's MMAs are issued, so that its answer is there when they have
+            // been (a stage cost the issuer 172 cycles beside its four MMAs of 48, during which the tensor pipe ran
+            // dry; down-projection 3584 x 18944, N = 128: 11.3 -> 10.6 us, b = 32, N = 1000: 87.7 -> 80.3).  Wider
+            // tiles have MMAs enough to cover it and measured up to 3 % slower with the extra test.
             uint32_t it = 0, tile_i = 0;
+            bool ready = false;
             bool ok = true;
             int4 tcd, tcd_next;
             for (; ok && next_tile(tile_i, &tcd, &tcd_next, &ok); ++tile_i) {
@@ -377,9 +383,11 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     const int nb = min(Cfg::kBps, min(pe - q, 32 - ((q - pb) & 31)));
                     const int s = it % STAGES;
                     const uint32_t ph = (it / STAGES) & 1u;
-                    if (!__all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, ctl, 3))) { ok = false; break; }
+                    if (!ready && !__all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, ctl, 3))) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t sb = smem_base + s * Cfg::kStageBytes;
+                    if constexpr (GROUPS == 1)
+                        ready = __all_sync(0xffffffffu, mbar_test_wait(full_bar((it + 1) % STAGES), ((it + 1) / STAGES) & 1u));
 #pragma unroll
                     for (int i = 0; i < Cfg::kBps; ++i) {
                         if (i < nb) {
@@ -624,25 +632,34 @@ cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtens
     }
 }
 
-// Stacked blocks (row groups): 128 rows x b, token tile 256, four stages of 48 KB.
+// Stacked blocks (row groups): 128 rows x b; token tile 256 and four stages of 48 KB, or 128 and six of 32 KB.
 template <int FMT, int CT, int CM>
-cudaError_t launch_stack_shape(int b, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_stack_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                                const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
-    switch (b) {
-        case 16: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 32: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 64: return launch_one<64, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        default: return cudaErrorInvalidValue;
+    switch (b * 10 + groups) {
+        case 161: return launch_one<16, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        default: break;
     }
+    if constexpr (FMT != 2) {
+        if (b == 64 && groups == 1) return launch_one<64, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        if (b == 64 && groups == 2) return launch_one<64, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int FMT>
-cudaError_t launch_stack_fmt(int b, int c16, int cm, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_stack_fmt(int b, int groups, int c16, int cm, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                              const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
-    if (cm) return c16 ? launch_stack_shape<FMT, 1, 1>(b, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-                       : launch_stack_shape<FMT, 0, 1>(b, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-    return c16 ? launch_stack_shape<FMT, 1, 0>(b, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-               : launch_stack_shape<FMT, 0, 0>(b, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+    if constexpr (FMT != 2) {
+        if (c16) return cm ? launch_stack_shape<FMT, 1, 1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
+                           : launch_stack_shape<FMT, 1, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+    }
+    if (c16) return cudaErrorInvalidValue;
+    return cm ? launch_stack_shape<FMT, 0, 1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
+              : launch_stack_shape<FMT, 0, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
 }
 
 // E4M3 inputs: fp32 C, static schedule; b = 32, 64 or 128 (a block row must hold at least one
@@ -724,15 +741,21 @@ cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, in
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_bcsr_stacked(int dtype, int b, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,
+cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,
                                 const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid,
                                 cudaStream_t stream) {
-    if (dtype == 1) return launch_stack_fmt<0>(b, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
-    if (dtype == 0) return launch_stack_fmt<1>(b, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
+    if (dtype == 1) return launch_stack_fmt<0>(b, groups, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
+    if (dtype == 0) return launch_stack_fmt<1>(b, groups, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
+    if (dtype == 2) return launch_stack_fmt<2>(b, groups, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // TF32: b = 16, 32
     if (dtype == 3 && !c16 && col_major) {
-        // E4M3: half the bytes per stage, twice the ring depth
-        if (b == 32) return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        if (b == 64) return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        // E4M3: half the bytes per stage, deeper rings
+        switch (b * 10 + groups) {
+            case 321: return launch_one<32, 128, 1, 10, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            default: break;
+        }
     }
     return cudaErrorInvalidValue;
 }

@@ -200,9 +200,9 @@ int build_tile_schedule(const std::vector<int32_t>& units, const std::vector<int
                         int slab_w, int n_ctas, BcsrSchedule* out, int64_t unit_cost = 1,
                         const std::vector<int64_t>* initial = nullptr, std::vector<int64_t>* final_loads = nullptr);
 // Relative cost of one stored block in the two launches of a handle with row groups, in bytes
-// staged per block divided by b: a stacked block brings 256 tokens x b and 128 x b of A, a b x b
+// staged per block divided by b: a stacked block brings 128 * groups tokens x b and 128 x b of A, a b x b
 // block 128 * groups tokens x b and b x b of A (both launches are bound by that traffic).
-constexpr int64_t bcsr_stack_block_cost() { return 2 * (256 + 128); }
+constexpr int64_t bcsr_stack_block_cost(int groups) { return 2 * (128 * groups + 128); }
 constexpr int64_t bcsr_block_cost(int b, int groups) { return 2 * (128 * groups + b); }
 // a row group's tile writes 128 rows of C whatever its length
 constexpr int kStackTileFixedCost = 8;

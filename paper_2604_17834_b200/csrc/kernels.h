@@ -64,11 +64,12 @@ struct BcsrParams {
 cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA,
                         const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP,
                         const BcsrParams& p, int grid, cudaStream_t stream);
-// Row groups: the same kernel with 128 x b stacked blocks (MMA N = 128) and a 256-token tile.
-// tmA: the stacked values as [blocks * 128][b], box 128 x b; tmB3 built for groups = 2; b = 16, 32, 64.
+// Row groups: the same kernel with 128 x b stacked blocks (MMA N = 128) and a 256-token tile (groups = 2), or a
+// 128-token one (groups = 1; see ensure_schedule).
+// tmA: the stacked values as [blocks * 128][b], box 128 x b; tmB3 built for `groups`; b = 16, 32, 64 (tf32: 16, 32).
 constexpr int kStackRows = 128;
 constexpr int kStackGroups = 2;
-cudaError_t launch_bcsr_stacked(int dtype, int b, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,
+cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,
                                 const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
                                 int grid, cudaStream_t stream);
 // K-split: tmP = the partial tiles as [slots * b][N] fp32, box as tmC's (the tile record of a
@@ -92,6 +93,8 @@ int bcsr_token_groups_max(int dtype, int b, int c16, int col_major);
 constexpr int bcsr_epi_cols(int b, bool c16, bool col_major) { return (b < 32 || !c16) ? 16 : 32; }
 // stored blocks that share one pipeline stage (and one A request): 4 / 2 for b = 16 / 32
 constexpr int bcsr_blocks_per_stage(int b) { return b == 16 ? 4 : (b == 32 ? 2 : 1); }
+// stacked blocks (row groups) per stage: 4 / 2 / 1 blocks; 4-byte values are twice as wide
+constexpr int bcsr_stacked_per_stage(int b, int es) { return es == 4 ? bcsr_blocks_per_stage(b) / 2 : bcsr_blocks_per_stage(b); }
 // Column slices a stored block is cut into, one pipeline stage each: blocks of 4-byte elements
 // with rows longer than 128 bytes (TF32, b = 64 / 128) go through the ring 32 columns at a time;
 // every other block is one unit.

@@ -616,3 +616,26 @@ def test_runs_that_feed_one_another_on_a_stream(lib, kind, opt):
         assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
     finally:
         lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("b,col_major", [(16, False), (32, False), (32, True)])
+@pytest.mark.parametrize("N", [256, 392, 2048])
+def test_bcsr_tf32_row_groups_and_narrow_tiles(lib, b, col_major, N):
+    """Row groups of TF32 blocks (rows of up to 128 bytes), and of any type with 128-token tiles: few groups and a
+    narrow dense operand take those (N = 256, 392), many tokens the 256-token ones.  Same MMAs in the same
+    order as without groups: equal to the last bit, and to the oracle within the bound."""
+    for dtype in ("tf32", "fp16"):
+        a = wl.bcsr_sweep(700 + b, m=2048, k=1536, b=b, density=0.05, dtype=dtype)
+        Bs = wl.dense(701, 1536, N, ("uniform", -1.0, 1.0), dtype)
+        outs = []
+        for fill in (0, -1):
+            h = lib.spmm_bcsr_create_csr(2048, 1536, a["row_ptr"], a["col_idx"], a["vals"], dtype, b, stack_min_fill=fill,
+                                         layout=lib.COLMAJOR if col_major else lib.ROWMAJOR)
+            try:
+                assert (lib.spmm_get_info(h, N)["n_stacked_rows"] > 0) == (fill == 0)
+                outs.append(run_gpu_variant(lib, h, Bs, 2048, N, dtype, col_major=col_major))
+            finally:
+                lib.spmm_destroy(h)
+        assert np.array_equal(outs[0], outs[1])
+        Cr, S = reference(a, Bs, dtype)
+        assert_close(outs[0], Cr, S, dtype, "%s row groups b=%d N=%d" % (dtype, b, N))
