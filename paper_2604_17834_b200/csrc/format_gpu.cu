@@ -16,8 +16,8 @@
 //
 // WCSR (window condensation of Sec. 2.3): every stored entry becomes the 64-bit key
 // (window << 32 | column); a radix sort and a unique pass (CUB primitives) leave, window after
-// window, the ascending union of each window's columns; counting keys per window and two prefix
-// sums give window_row_ptr (lengths padded to b_col) and each window's place in the key list;
+// window, the ascending union of each window's columns; where the window changes gives each window's
+// place in the key list, a prefix sum window_row_ptr (lengths padded to b_col);
 // window_col_idx is those columns over a -1 fill, and every value finds its condensed column by
 // binary search in its window's list and goes straight into the packed tile layout.
 #include <cub/cub.cuh>
@@ -382,33 +382,41 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
 
 namespace {
 
-// key = window << cb | column, cb = bits of a column: no empty bits for the radix sort to pass over
-__global__ void wcsr_keys_kernel(int64_t m, int wh, int cb, const int64_t* row_ptr, const int32_t* col_idx, uint64_t* keys) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    for (int64_t i = warp0; i < m; i += nwarps) {
-        const uint64_t hi = static_cast<uint64_t>(i / wh) << cb;
-        for (int64_t p = row_ptr[i] + lane; p < row_ptr[i + 1]; p += 32) keys[p] = hi | static_cast<uint32_t>(col_idx[p]);
+// Entry by entry (a warp per row took four times as long: a row of 5000 entries was one warp's work): the row of
+// every entry, looked up in row_ptr, and its key = window << cb | column, cb = bits of a column: no empty bits for
+// the radix sort to pass over.
+__global__ void wcsr_keys_kernel(int64_t m, int wh, int cb, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+                                 uint64_t* __restrict__ keys, int32_t* __restrict__ row_of) {
+    const int64_t nnz = row_ptr[m];
+    for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        int64_t lo = 0, hi = m - 1;                       // last row that starts at or before p
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (row_ptr[mid] <= p) lo = mid; else hi = mid - 1;
+        }
+        row_of[p] = static_cast<int32_t>(lo);
+        keys[p] = static_cast<uint64_t>(lo / wh) << cb | static_cast<uint32_t>(col_idx[p]);
     }
 }
 
-// per window: how many distinct columns; per column: is it referenced at all
-__global__ void wcsr_count_kernel(const uint64_t* ukeys, const int* n_unique, int cb, int32_t* cnt, uint8_t* used) {
+// The unique keys ascend, so a window's keys are a run: where each run starts (ustart[nwin] = their number);
+// per column: is it referenced at all
+__global__ void wcsr_starts_kernel(const uint64_t* __restrict__ ukeys, const int* __restrict__ n_unique, int64_t nwin, int cb,
+                                   int32_t* __restrict__ ustart, uint8_t* __restrict__ used) {
     const int64_t n = *n_unique;
     const uint64_t col_mask = (uint64_t{1} << cb) - 1;
-    for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < n;
-         j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const uint64_t key = ukeys[j];
-        atomicAdd(&cnt[key >> cb], 1);
-        used[key & col_mask] = 1;
+    for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j <= n; j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int64_t w = j < n ? static_cast<int64_t>(ukeys[j] >> cb) : nwin;
+        const int64_t before = j > 0 ? static_cast<int64_t>(ukeys[j - 1] >> cb) : -1;
+        for (int64_t x = before + 1; x <= w; ++x) ustart[x] = static_cast<int32_t>(j);
+        if (j < n) used[ukeys[j] & col_mask] = 1;
     }
 }
 
-__global__ void wcsr_pad_kernel(const int32_t* cnt, int64_t nwin, int b_col, int32_t* len) {
+__global__ void wcsr_pad_kernel(const int32_t* __restrict__ ustart, int64_t nwin, int b_col, int32_t* __restrict__ len) {
     for (int64_t w = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; w < nwin;
          w += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        len[w] = (cnt[w] + b_col - 1) / b_col * b_col;
+        len[w] = (ustart[w + 1] - ustart[w] + b_col - 1) / b_col * b_col;
 }
 
 __global__ void wcsr_sum_used_kernel(const uint8_t* used, int64_t k, unsigned long long* total) {
@@ -432,32 +440,27 @@ __global__ void wcsr_cols_kernel(const uint64_t* ukeys, const int* n_unique, int
     }
 }
 
+// One thread per entry: its column's place in its window's list, by binary search.
 template <int ES>
-__global__ void wcsr_values_kernel(int64_t m, int wh, int b_col, const int64_t* row_ptr, const int32_t* col_idx,
-                                   const uint8_t* vals, const int32_t* cnt, const int32_t* window_row_ptr,
-                                   const int32_t* window_col_idx, uint8_t* packed) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp0 = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    for (int64_t i = warp0; i < m; i += nwarps) {
-        const int64_t w = i / wh;
-        const int r = static_cast<int>(i - w * wh);
+__global__ void wcsr_values_kernel(int64_t nnz, int wh, int b_col, const int32_t* __restrict__ row_of, const int32_t* __restrict__ col_idx,
+                                   const uint8_t* __restrict__ vals, const int32_t* __restrict__ ustart, const int32_t* __restrict__ window_row_ptr,
+                                   const int32_t* __restrict__ window_col_idx, uint8_t* __restrict__ packed) {
+    for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int i = row_of[p];
+        const int w = i / wh, r = i - w * wh;
         const int64_t base = window_row_ptr[w];
         const int32_t* seg = window_col_idx + base;
-        const int n = cnt[w];
-        for (int64_t p = row_ptr[i] + lane; p < row_ptr[i + 1]; p += 32) {
-            const int32_t c = col_idx[p];
-            int lo = 0, hi = n;                      // first position with seg[pos] >= c; c is in the list
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (seg[mid] < c) lo = mid + 1; else hi = mid;
-            }
-            uint8_t* dst = packed + wcsr_packed_offset(wh, b_col, ES, r, base + lo);
-            const uint8_t* src = vals + static_cast<size_t>(p) * ES;
-            if constexpr (ES == 1) *dst = *src;
-            else if constexpr (ES == 2) *reinterpret_cast<uint16_t*>(dst) = *reinterpret_cast<const uint16_t*>(src);
-            else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(src);
+        const int32_t c = col_idx[p];
+        int lo = 0, hi = ustart[w + 1] - ustart[w];      // first position with seg[pos] >= c; c is in the list
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (seg[mid] < c) lo = mid + 1; else hi = mid;
         }
+        uint8_t* dst = packed + wcsr_packed_offset(wh, b_col, ES, r, base + lo);
+        const uint8_t* src = vals + static_cast<size_t>(p) * ES;
+        if constexpr (ES == 1) *dst = *src;
+        else if constexpr (ES == 2) *reinterpret_cast<uint16_t*>(dst) = *reinterpret_cast<const uint16_t*>(src);
+        else *reinterpret_cast<uint32_t*>(dst) = *reinterpret_cast<const uint32_t*>(src);
     }
 }
 
@@ -583,14 +586,14 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     *d_window_col_idx = nullptr;
     *d_packed = nullptr;
 
-    int* d_flags = nullptr;                   // [0] CSR error code, [1] scan overflow, [2] number of unique keys
+    int* d_flags = nullptr;                   // [0] CSR error code, [1] scan overflow, [2] a bad entry, then the number of unique keys
     uint64_t *d_keys = nullptr, *d_keys2 = nullptr;
-    int32_t *d_cnt = nullptr, *d_len = nullptr, *d_ustart = nullptr;
+    int32_t *d_row_of = nullptr, *d_len = nullptr, *d_ustart = nullptr;
     uint8_t* d_used = nullptr;
     unsigned long long* d_total = nullptr;
     void* d_temp = nullptr;
     auto release = [&]() {
-        dev_free(d_flags, st); dev_free(d_keys, st); dev_free(d_keys2, st); dev_free(d_cnt, st); dev_free(d_len, st);
+        dev_free(d_flags, st); dev_free(d_keys, st); dev_free(d_keys2, st); dev_free(d_row_of, st); dev_free(d_len, st);
         dev_free(d_ustart, st); dev_free(d_used, st); dev_free(d_total, st); dev_free(d_temp, st);
     };
     auto fail = [&](int code) {
@@ -623,23 +626,24 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     // keys -> sorted -> unique
     if (!alloc(reinterpret_cast<void**>(&d_keys), static_cast<size_t>(nnz) * 8) ||
         !alloc(reinterpret_cast<void**>(&d_keys2), static_cast<size_t>(nnz) * 8) ||
-        !alloc(reinterpret_cast<void**>(&d_cnt), static_cast<size_t>(nwin + 1) * 4) ||
+        !alloc(reinterpret_cast<void**>(&d_row_of), static_cast<size_t>(nnz) * 4) ||
         !alloc(reinterpret_cast<void**>(&d_len), static_cast<size_t>(nwin + 1) * 4) ||
         !alloc(reinterpret_cast<void**>(&d_ustart), static_cast<size_t>(nwin + 1) * 4) ||
         !alloc(reinterpret_cast<void**>(&d_used), static_cast<size_t>(k)) ||
         !alloc(reinterpret_cast<void**>(&d_total), 8) ||
         !alloc(reinterpret_cast<void**>(d_window_row_ptr), static_cast<size_t>(nwin + 1) * 4))
         return fail(SPMM_ERR_ALLOC);
-    cudaMemsetAsync(d_cnt, 0, static_cast<size_t>(nwin + 1) * 4, st);
+    cudaMemsetAsync(d_ustart, 0, static_cast<size_t>(nwin + 1) * 4, st);
     cudaMemsetAsync(d_used, 0, static_cast<size_t>(k ? k : 1), st);
     cudaMemsetAsync(d_total, 0, 8, st);
     const int n = static_cast<int>(nnz);
+    const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 16384));
     int cb = 1;
     while ((int64_t{1} << cb) < k) ++cb;
     int end_bit = cb + 1;
     while ((int64_t{1} << (end_bit - cb)) < nwin) ++end_bit;
     if (n > 0) {
-        wcsr_keys_kernel<<<static_cast<unsigned>(std::min<int64_t>((m + 7) / 8, 4096)), 256, 0, st>>>(m, wh, cb, d_row_ptr, d_col_idx, d_keys);
+        wcsr_keys_kernel<<<entry_grid, 256, 0, st>>>(m, wh, cb, d_row_ptr, d_col_idx, d_keys, d_row_of);
         size_t t1 = 0, t2 = 0;
         cub::DeviceRadixSort::SortKeys(nullptr, t1, d_keys, d_keys2, n, 0, end_bit, st);
         cub::DeviceSelect::Unique(nullptr, t2, d_keys2, d_keys, d_flags + 2, n, st);
@@ -649,11 +653,10 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         tb = std::max(t1, t2);
         if (cub::DeviceSelect::Unique(d_temp, tb, d_keys2, d_keys, d_flags + 2, n, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
         // d_keys now holds the unique keys, d_flags[2] their number
-        wcsr_count_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, cb, d_cnt, d_used);
+        wcsr_starts_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, nwin, cb, d_ustart, d_used);
     }
-    wcsr_pad_kernel<<<static_cast<unsigned>(std::min<int64_t>((nwin + 255) / 256 + 1, 2048)), 256, 0, st>>>(d_cnt, nwin, b_col, d_len);
+    wcsr_pad_kernel<<<static_cast<unsigned>(std::min<int64_t>((nwin + 255) / 256 + 1, 2048)), 256, 0, st>>>(d_ustart, nwin, b_col, d_len);
     exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_len, nwin, *d_window_row_ptr, d_flags + 1);
-    exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_cnt, nwin, d_ustart, d_flags + 3);
     if (k > 0) wcsr_sum_used_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 1024)), 256, 0, st>>>(d_used, k, d_total);
     out->window_row_ptr.assign(static_cast<size_t>(nwin) + 1, 0);
     unsigned long long distinct = 0;
@@ -678,13 +681,12 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     }
     if (n > 0) {
         wcsr_cols_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, cb, d_ustart, *d_window_row_ptr, *d_window_col_idx);
-        const unsigned vgrid = static_cast<unsigned>(std::min<int64_t>((m + 7) / 8, 8192));
         if (es == 1)
-            wcsr_values_kernel<1><<<vgrid, 256, 0, st>>>(m, wh, b_col, d_row_ptr, d_col_idx, d_vals, d_cnt, *d_window_row_ptr, *d_window_col_idx, *d_packed);
+            wcsr_values_kernel<1><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
         else if (es == 2)
-            wcsr_values_kernel<2><<<vgrid, 256, 0, st>>>(m, wh, b_col, d_row_ptr, d_col_idx, d_vals, d_cnt, *d_window_row_ptr, *d_window_col_idx, *d_packed);
+            wcsr_values_kernel<2><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
         else
-            wcsr_values_kernel<4><<<vgrid, 256, 0, st>>>(m, wh, b_col, d_row_ptr, d_col_idx, d_vals, d_cnt, *d_window_row_ptr, *d_window_col_idx, *d_packed);
+            wcsr_values_kernel<4><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
     }
     release();                                // (ordered behind the kernels that use them)
     int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
@@ -960,7 +962,7 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     int4* tasks = reinterpret_cast<int4*>(out->d_tasks);
     rows_plan_kernel<<<grid_for(m + 1, 256), 256, 0, st>>>(p, out->d_order, d_row_ptr, d_head, reinterpret_cast<int4*>(out->d_parts),
                                                           reinterpret_cast<int4*>(out->d_longs), reinterpret_cast<int4*>(out->d_total));
-    const unsigned lg = static_cast<unsigned>(std::min<int64_t>(max_long, 1024));
+    const unsigned lg = static_cast<unsigned>(std::min<int64_t>(max_long, 8192));
     if (es == 2) {
         rows_fill_kernel<2><<<grid_for(m * 8, 256), 256, 0, st>>>(p, out->d_order, d_head, d_row_ptr, d_col_idx, d_vals, tasks, out->d_col, out->d_val);
         rows_fill_long_kernel<2><<<lg, 256, 0, st>>>(p, out->d_order, d_row_ptr, d_col_idx, d_vals, out->d_col, out->d_val);
