@@ -372,7 +372,7 @@ int create_bcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
 }
 
 // Uploads the schedule arrays of a WCSR handle (everything but the three format arrays): one allocation, one copy.
-// Synchronises `stream`.
+// In the order of `stream` (the host arrays have been read when it returns).
 int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
     const WcsrHost& f = h->wcsr;
     const size_t nt = f.tasks.size(), nm = f.merge_window.size(), ni = f.bin_tasks.size();
@@ -423,8 +423,7 @@ int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
     int32_t* fills_n = h->d_plan + o_fills_n;
     if (expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill, f.kt, fills, stream) != cudaSuccess ||
         (narrow && expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill_n,
-                                     kWcsrNarrowCols, fills_n, stream) != cudaSuccess) ||
-        cudaStreamSynchronize(stream) != cudaSuccess)
+                                     kWcsrNarrowCols, fills_n, stream) != cudaSuccess))
         return SPMM_ERR_CUDA;
     h->n_merge = static_cast<int>(nm);
     h->d_tasks = reinterpret_cast<WcsrDevTask*>(h->d_plan + o_tasks);
@@ -513,6 +512,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
             dev_free(d_ci, nullptr);
             dev_free(d_va, nullptr);
         }
+        if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = SPMM_ERR_CUDA;
         if (rc) { free_handle(h); return rc; }
         std::vector<uint8_t>().swap(h->wcsr.packed);
     }
@@ -537,9 +537,11 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
                                &h->d_vals, &h->d_class, &h->rows);
         h->d_grp_class = h->d_class;
         if (!rc) rc = upload_wcsr_plan(h, stream);
+        if (!rc) rc = finish_wcsr_rows(&h->rows, stream);
     } catch (const std::bad_alloc&) {
         rc = SPMM_ERR_ALLOC;
     }
+    if (!rc && cudaStreamSynchronize(stream) != cudaSuccess) rc = SPMM_ERR_CUDA;
     if (rc) { free_handle(h); return rc; }
     *out = h;
     return SPMM_OK;

@@ -40,8 +40,12 @@ constexpr int kThreads = 256;
 
 // Validation in two passes, so that the second one never reads past the arrays: once row_ptr is
 // known to start at 0 and to be monotone, every position below row_ptr[m] lies inside col_idx.
-__global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* err) {
-    if (blockIdx.x == 0 && threadIdx.x == 0 && row_ptr[0] != 0) atomicMin(err, SPMM_ERR_INVALID_ARG);
+// (nnz: receives row_ptr[m] where the caller reads it together with *err; may be null)
+__global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* err, int64_t* nnz) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (row_ptr[0] != 0) atomicMin(err, SPMM_ERR_INVALID_ARG);
+        if (nnz) *nnz = row_ptr[m];
+    }
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < m;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x)
         if (row_ptr[i + 1] < row_ptr[i]) atomicMin(err, SPMM_ERR_INVALID_ARG);
@@ -327,7 +331,7 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     int flags[2] = {0, 0};
     const unsigned check_grid = static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048));
     if (m > 0) {
-        csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, d_flags);
+        csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, d_flags, nullptr);
         if (cudaMemcpyAsync(&nnz, d_row_ptr + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
     }
     if (cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
@@ -385,8 +389,9 @@ namespace {
 // Entry by entry (a warp per row took four times as long: a row of 5000 entries was one warp's work): the row of
 // every entry, looked up in row_ptr, and its key = window << cb | column, cb = bits of a column: no empty bits for
 // the radix sort to pass over.
-__global__ void wcsr_keys_kernel(int64_t m, int wh, int cb, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                                 uint64_t* __restrict__ keys, int32_t* __restrict__ row_of) {
+// An entry out of range or not ascending in its row sets *bad and counts as column 0.
+__global__ void wcsr_keys_kernel(int64_t m, int64_t k, int wh, int cb, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+                                 uint64_t* __restrict__ keys, int32_t* __restrict__ row_of, int* bad) {
     const int64_t nnz = row_ptr[m];
     for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         int64_t lo = 0, hi = m - 1;                       // last row that starts at or before p
@@ -394,8 +399,13 @@ __global__ void wcsr_keys_kernel(int64_t m, int wh, int cb, const int64_t* __res
             const int64_t mid = (lo + hi + 1) >> 1;
             if (row_ptr[mid] <= p) lo = mid; else hi = mid - 1;
         }
+        int64_t c = col_idx[p];
+        if (c < 0 || c >= k || (p > row_ptr[lo] && col_idx[p - 1] >= c)) {
+            *bad = 1;
+            c = 0;
+        }
         row_of[p] = static_cast<int32_t>(lo);
-        keys[p] = static_cast<uint64_t>(lo / wh) << cb | static_cast<uint32_t>(col_idx[p]);
+        keys[p] = static_cast<uint64_t>(lo / wh) << cb | static_cast<uint64_t>(c);
     }
 }
 
@@ -522,35 +532,35 @@ __global__ void wcsr_group_class_kernel(const int32_t* __restrict__ col_idx, int
 int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, int64_t k, int64_t nwin, cudaStream_t st, uint8_t** d_grp_class) {
     *d_grp_class = nullptr;
     if (P <= 0 || k <= 0) return SPMM_OK;
+    int count_bits = 1;                       // a row of B is gathered by nwin windows at most
+    while (count_bits < 31 && (int64_t{1} << count_bits) <= nwin) ++count_bits;
     int32_t *refs = nullptr, *refs_sorted = nullptr, *ids = nullptr, *order = nullptr;
-    uint8_t* cls = nullptr;
-    void* temp = nullptr;
-    auto release = [&]() { dev_free(refs, st); dev_free(refs_sorted, st); dev_free(ids, st); dev_free(order, st); dev_free(cls, st); dev_free(temp, st); };
-    const size_t kb = static_cast<size_t>(k) * 4;
-    if (!dev_alloc_ok(&refs, kb, st) || !dev_alloc_ok(&refs_sorted, kb, st) ||
-        !dev_alloc_ok(&ids, kb, st) || !dev_alloc_ok(&order, kb, st) ||
-        !dev_alloc_ok(&cls, static_cast<size_t>(k), st) ||
-        !dev_alloc_ok(d_grp_class, static_cast<size_t>(P / 4), st)) {
-        release();
+    size_t tb = 0;
+    cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st);
+    const size_t kb = static_cast<size_t>(k) * 4, step = (kb + 255) / 256 * 256;
+    uint8_t* block = nullptr;                 // refs | sorted refs | ids | order | classes | CUB's
+    if (!dev_alloc_ok(&block, 5 * step + tb, st) || !dev_alloc_ok(d_grp_class, static_cast<size_t>(P / 4), st)) {
+        dev_free(block, st);
         dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
         return SPMM_ERR_ALLOC;
     }
+    refs = reinterpret_cast<int32_t*>(block);
+    refs_sorted = reinterpret_cast<int32_t*>(block + step);
+    ids = reinterpret_cast<int32_t*>(block + 2 * step);
+    order = reinterpret_cast<int32_t*>(block + 3 * step);
+    uint8_t* cls = block + 4 * step;
+    void* temp = block + 5 * step;
     cudaMemsetAsync(refs, 0, kb, st);
     wcsr_refs_kernel<<<2048, 256, 0, st>>>(d_window_col_idx, P, refs);
     iota_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 2048)), 256, 0, st>>>(ids, k);
-    int count_bits = 1;                       // a row of B is gathered by nwin windows at most
-    while (count_bits < 31 && (int64_t{1} << count_bits) <= nwin) ++count_bits;
-    size_t tb = 0;
-    cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st);
-    bool ok = dev_alloc_ok(&temp, tb, st) &&
-              cub::DeviceRadixSort::SortPairsDescending(temp, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st) == cudaSuccess;
+    bool ok = cub::DeviceRadixSort::SortPairsDescending(temp, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st) == cudaSuccess;
     if (ok) {
         wcsr_class_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 2048)), 256, 0, st>>>(refs_sorted, order, k, cls);
         wcsr_group_class_kernel<<<2048, 256, 0, st>>>(d_window_col_idx, P / 4, cls, *d_grp_class);
         ok = cudaGetLastError() == cudaSuccess;
     }
-    release();
+    dev_free(block, st);
     if (!ok) {
         dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
@@ -586,16 +596,18 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     *d_window_col_idx = nullptr;
     *d_packed = nullptr;
 
-    int* d_flags = nullptr;                   // [0] CSR error code, [1] scan overflow, [2] a bad entry, then the number of unique keys
-    uint64_t *d_keys = nullptr, *d_keys2 = nullptr;
-    int32_t *d_row_of = nullptr, *d_len = nullptr, *d_ustart = nullptr;
-    uint8_t* d_used = nullptr;
-    unsigned long long* d_total = nullptr;
-    void* d_temp = nullptr;
-    auto release = [&]() {
-        dev_free(d_flags, st); dev_free(d_keys, st); dev_free(d_keys2, st); dev_free(d_row_of, st); dev_free(d_len, st);
-        dev_free(d_ustart, st); dev_free(d_used, st); dev_free(d_total, st); dev_free(d_temp, st);
-    };
+    // what the GPU tells the host, read with one copy at a time
+    struct Flags {
+        int err;                              // CSR error code
+        int overflow;                         // of the scan
+        int n_unique;                         // unique keys
+        int bad;                              // an entry out of range or not ascending
+        int64_t nnz;
+        unsigned long long distinct;          // columns that are referenced
+    } flags = {};
+    Flags* d_flags = nullptr;
+    uint8_t* d_work = nullptr;                // keys, sorted keys, rows of the entries, window lengths and starts, column marks, CUB's
+    auto release = [&]() { dev_free(d_flags, st); dev_free(d_work, st); };
     auto fail = [&](int code) {
         release();
         dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st);
@@ -604,71 +616,77 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     };
     auto alloc = [&](void** ptr, size_t bytes) { return dev_alloc(ptr, bytes, st) == cudaSuccess; };
 
-    if (!alloc(reinterpret_cast<void**>(&d_flags), 4 * sizeof(int))) return fail(SPMM_ERR_ALLOC);
-    if (cudaMemsetAsync(d_flags, 0, 4 * sizeof(int), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    int64_t nnz = 0;
-    int flags[4] = {0, 0, 0, 0};
+    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags))) return fail(SPMM_ERR_ALLOC);
+    if (cudaMemsetAsync(d_flags, 0, sizeof(Flags), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
+    auto read_flags = [&]() {
+        return cudaMemcpyAsync(&flags, d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    };
     const unsigned check_grid = static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048));
-    if (m > 0) {
-        csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, d_flags);
-        if (cudaMemcpyAsync(&nnz, d_row_ptr + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    }
-    if (cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    if (cudaStreamSynchronize(st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    if (flags[0] != 0) return fail(flags[0]);
+    if (m > 0) csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, &d_flags->err, &d_flags->nnz);
+    if (!read_flags()) return fail(SPMM_ERR_CUDA);
+    if (flags.err != 0) return fail(flags.err);
+    const int64_t nnz = flags.nnz;
     if (nnz < 0 || (nnz > 0 && (!d_col_idx || !d_vals))) return fail(SPMM_ERR_INVALID_ARG);
     if (nnz >= (int64_t{1} << 31)) return fail(SPMM_ERR_TOO_LARGE);
-    if (nnz > 0) {
-        if (int rc = check_csr_cols(m, k, nnz, d_row_ptr, d_col_idx, d_flags + 2, d_flags, st)) return fail(rc);
-    }
     *nnz_out = nnz;
 
     // keys -> sorted -> unique
-    if (!alloc(reinterpret_cast<void**>(&d_keys), static_cast<size_t>(nnz) * 8) ||
-        !alloc(reinterpret_cast<void**>(&d_keys2), static_cast<size_t>(nnz) * 8) ||
-        !alloc(reinterpret_cast<void**>(&d_row_of), static_cast<size_t>(nnz) * 4) ||
-        !alloc(reinterpret_cast<void**>(&d_len), static_cast<size_t>(nwin + 1) * 4) ||
-        !alloc(reinterpret_cast<void**>(&d_ustart), static_cast<size_t>(nwin + 1) * 4) ||
-        !alloc(reinterpret_cast<void**>(&d_used), static_cast<size_t>(k)) ||
-        !alloc(reinterpret_cast<void**>(&d_total), 8) ||
-        !alloc(reinterpret_cast<void**>(d_window_row_ptr), static_cast<size_t>(nwin + 1) * 4))
-        return fail(SPMM_ERR_ALLOC);
-    cudaMemsetAsync(d_ustart, 0, static_cast<size_t>(nwin + 1) * 4, st);
-    cudaMemsetAsync(d_used, 0, static_cast<size_t>(k ? k : 1), st);
-    cudaMemsetAsync(d_total, 0, 8, st);
     const int n = static_cast<int>(nnz);
     const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 16384));
     int cb = 1;
     while ((int64_t{1} << cb) < k) ++cb;
     int end_bit = cb + 1;
     while ((int64_t{1} << (end_bit - cb)) < nwin) ++end_bit;
+    uint64_t *d_keys = nullptr, *d_keys2 = nullptr;
+    size_t t1 = 0, t2 = 0;
     if (n > 0) {
-        wcsr_keys_kernel<<<entry_grid, 256, 0, st>>>(m, wh, cb, d_row_ptr, d_col_idx, d_keys, d_row_of);
-        size_t t1 = 0, t2 = 0;
         cub::DeviceRadixSort::SortKeys(nullptr, t1, d_keys, d_keys2, n, 0, end_bit, st);
-        cub::DeviceSelect::Unique(nullptr, t2, d_keys2, d_keys, d_flags + 2, n, st);
-        if (!alloc(&d_temp, std::max(t1, t2))) return fail(SPMM_ERR_ALLOC);
-        size_t tb = std::max(t1, t2);
+        cub::DeviceSelect::Unique(nullptr, t2, d_keys2, d_keys, &d_flags->n_unique, n, st);
+    }
+    size_t work_bytes = 0, tb = std::max(t1, t2);
+    auto section = [&](size_t bytes) {
+        const size_t at = work_bytes;
+        work_bytes += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t o_keys = section(static_cast<size_t>(nnz) * 8), o_keys2 = section(static_cast<size_t>(nnz) * 8);
+    const size_t o_row_of = section(static_cast<size_t>(nnz) * 4), o_len = section(static_cast<size_t>(nwin + 1) * 4);
+    const size_t o_ustart = section(static_cast<size_t>(nwin + 1) * 4), o_used = section(static_cast<size_t>(k)), o_temp = section(tb);
+    if (!alloc(reinterpret_cast<void**>(&d_work), work_bytes) ||
+        !alloc(reinterpret_cast<void**>(d_window_row_ptr), static_cast<size_t>(nwin + 1) * 4))
+        return fail(SPMM_ERR_ALLOC);
+    d_keys = reinterpret_cast<uint64_t*>(d_work + o_keys);
+    d_keys2 = reinterpret_cast<uint64_t*>(d_work + o_keys2);
+    int32_t* d_row_of = reinterpret_cast<int32_t*>(d_work + o_row_of);
+    int32_t* d_len = reinterpret_cast<int32_t*>(d_work + o_len);
+    int32_t* d_ustart = reinterpret_cast<int32_t*>(d_work + o_ustart);
+    uint8_t* d_used = d_work + o_used;
+    void* d_temp = d_work + o_temp;
+    cudaMemsetAsync(d_ustart, 0, o_temp - o_ustart, st);       // the starts and the marks behind them
+    if (n > 0) {
+        wcsr_keys_kernel<<<entry_grid, 256, 0, st>>>(m, k, wh, cb, d_row_ptr, d_col_idx, d_keys, d_row_of, &d_flags->bad);
         if (cub::DeviceRadixSort::SortKeys(d_temp, tb, d_keys, d_keys2, n, 0, end_bit, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        tb = std::max(t1, t2);
-        if (cub::DeviceSelect::Unique(d_temp, tb, d_keys2, d_keys, d_flags + 2, n, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        // d_keys now holds the unique keys, d_flags[2] their number
-        wcsr_starts_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, nwin, cb, d_ustart, d_used);
+        if (cub::DeviceSelect::Unique(d_temp, tb, d_keys2, d_keys, &d_flags->n_unique, n, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
+        // d_keys now holds the unique keys
+        wcsr_starts_kernel<<<2048, 256, 0, st>>>(d_keys, &d_flags->n_unique, nwin, cb, d_ustart, d_used);
     }
     wcsr_pad_kernel<<<static_cast<unsigned>(std::min<int64_t>((nwin + 255) / 256 + 1, 2048)), 256, 0, st>>>(d_ustart, nwin, b_col, d_len);
-    exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_len, nwin, *d_window_row_ptr, d_flags + 1);
-    if (k > 0) wcsr_sum_used_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 1024)), 256, 0, st>>>(d_used, k, d_total);
+    exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_len, nwin, *d_window_row_ptr, &d_flags->overflow);
+    if (k > 0) wcsr_sum_used_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 1024)), 256, 0, st>>>(d_used, k, &d_flags->distinct);
     out->window_row_ptr.assign(static_cast<size_t>(nwin) + 1, 0);
-    unsigned long long distinct = 0;
     if (cudaMemcpyAsync(out->window_row_ptr.data(), *d_window_row_ptr, static_cast<size_t>(nwin + 1) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&distinct, d_total, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+        !read_flags())
         return fail(SPMM_ERR_CUDA);
-    if (cudaStreamSynchronize(st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-    if (flags[1]) return fail(SPMM_ERR_TOO_LARGE);
+    if (flags.bad) {
+        // (an entry that broke a rule was taken as column 0, so nothing above left its arrays)
+        csr_check_cols_kernel<<<check_grid, 256, 0, st>>>(m, k, d_row_ptr, d_col_idx, &d_flags->err);
+        if (!read_flags()) return fail(SPMM_ERR_CUDA);
+        return fail(flags.err != 0 ? flags.err : SPMM_ERR_INVALID_ARG);
+    }
+    if (flags.overflow) return fail(SPMM_ERR_TOO_LARGE);
     const int64_t P = out->window_row_ptr[static_cast<size_t>(nwin)];
     out->P = P;
-    out->distinct_cols = static_cast<int64_t>(distinct);
+    out->distinct_cols = static_cast<int64_t>(flags.distinct);
 
     // window_col_idx over a -1 fill, values into the zero-filled packed tiles
     const size_t packed_bytes = static_cast<size_t>(P) * wh * es;
@@ -680,7 +698,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         cudaMemsetAsync(*d_packed, 0, packed_bytes, st);
     }
     if (n > 0) {
-        wcsr_cols_kernel<<<2048, 256, 0, st>>>(d_keys, d_flags + 2, cb, d_ustart, *d_window_row_ptr, *d_window_col_idx);
+        wcsr_cols_kernel<<<2048, 256, 0, st>>>(d_keys, &d_flags->n_unique, cb, d_ustart, *d_window_row_ptr, *d_window_col_idx);
         if (es == 1)
             wcsr_values_kernel<1><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
         else if (es == 2)
@@ -699,8 +717,6 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
             rc = SPMM_ERR_ALLOC;
         }
     }
-    if (!rc) rc = finish_wcsr_rows(rows, st);
-    if (cudaStreamSynchronize(st) != cudaSuccess && !rc) rc = SPMM_ERR_CUDA;
     if (rc) {
         free_wcsr_rows(rows, st);
         dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st); dev_free(*d_grp_class, st);
