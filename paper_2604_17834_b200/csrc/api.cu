@@ -971,10 +971,34 @@ int64_t wcsr_workspace_bytes(const spmm_handle_s* h, int64_t N) {
     return h->wcsr.n_slots * int64_t{h->wcsr.wh} * N * 4;
 }
 
-// Whether a run takes the row kernel: the handle has a row stream, and the wait limit is not zero, the documented
-// hook for the path where a wait runs out, which the window kernel serves (the row kernel waits for nothing).
+// Stored values per padded column up to which the row kernel is the faster one at dense width N.  The window kernel
+// takes 128-token tiles whose row of B is 256 (2-byte types; from 64 tokens on it has a variant for half of that) or
+// 512 bytes, so it is at its best from N = 64 / 128 on; a launch the row kernel's short tasks alone can spread over
+// the GPU (load < 16) is latency, which condensing does not help.  Row / window kernel, us, 16 entries a row in a
+// band, at 1.2 / 1.4 / 1.9 values per column:
+//   100,000 rows  fp16 N = 32   0.62 / 0.81 / 0.97 of the window kernel's time    TF32 N = 64    0.64 / 0.79 / 1.10
+//                 fp16 N = 128  1.05 / 1.29 / 1.70                                TF32 N = 128   0.95 / 1.13 / 1.56
+//   8000 rows     fp16 N = 128  0.60 / 0.84 / 1.43                                TF32 N = 128   0.72 / 0.85 / 1.03
+// Where a row of B leaves more than a quarter of a warp's lanes idle, the large launches of the 2-byte types (load
+// >= 100) are the window kernel's as well: N = 320 on R-MAT 2^20, 24 a row, 1450 us against 1600, on 200,000 rows of
+// power-law length 285 against 344; with the lanes full, N = 256, 1046 against 998 and 209 against 214.
+double wcsr_rows_limit(const spmm_handle_s* h, int64_t N) {
+    const int64_t load = wcsr_rows_load(h->m, h->nnz, h->sms);
+    const int es = h->es;
+    if (load < 16 || N < (es == 4 ? 128 : 64)) return kRowsMaxPerCol;
+    if (es == 4) return 1.4;
+    if (load < 100) return 1.22;
+    const RowsShape s = wcsr_rows_shape(N, es, (N * es) % 32 == 0);
+    const int64_t busy = int64_t{32 / s.lanes} * s.lanes * (N * es), all = int64_t{32} * s.lanes * s.tiles * s.vec;
+    return busy * 4 < all * 3 ? 0.0 : 1.22;
+}
+
+// Whether a run takes the row kernel: the handle has a row stream, it is the faster one, and the wait limit is not
+// zero, the documented hook for the path where a wait runs out, which the window kernel serves (the row kernel waits
+// for nothing).
 bool use_rows(const spmm_handle_s* h, int64_t N) {
-    return (h->rows.n_tasks > 0 || h->rows.n_parts > 0) && g_wait_limit_ns.load() != 0 && N * h->es < (int64_t{1} << 32);
+    return (h->rows.n_tasks > 0 || h->rows.n_parts > 0) && g_wait_limit_ns.load() != 0 && N * h->es < (int64_t{1} << 32) &&
+           static_cast<double>(h->nnz) <= wcsr_rows_limit(h, N) * static_cast<double>(h->wcsr.P);
 }
 
 // Bytes of partial rows one launch of the row kernel wants for `tiles` column tiles.
@@ -1079,8 +1103,8 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
 }
 
 // The handle's workspace for the partial tiles of split windows at dense width N (grown, never shrunk).
-int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, cudaStream_t stream) {
-    const size_t need = use_rows(h, N) ? rows_workspace_bytes(h, N) : static_cast<size_t>(wcsr_workspace_bytes(h, N));
+int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, bool rows, cudaStream_t stream) {
+    const size_t need = rows ? rows_workspace_bytes(h, N) : static_cast<size_t>(wcsr_workspace_bytes(h, N));
     if (need > h->partial_bytes) {
         if (h->d_partial) {
             if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
@@ -1094,9 +1118,10 @@ int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, cudaStream_t stream) {
     return SPMM_OK;
 }
 
-int run_wcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t stream) {
-    if (int rc = ensure_wcsr_workspace(h, N, stream)) return rc;
-    if (use_rows(h, N)) return launch_wcsr_rows_all(h, B, C, h->d_partial, h->partial_bytes, N, stream);
+// rows: use_rows for the whole operand of which these are N columns (the kernels add in different orders)
+int run_wcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, bool rows, cudaStream_t stream) {
+    if (int rc = ensure_wcsr_workspace(h, N, rows, stream)) return rc;
+    if (rows) return launch_wcsr_rows_all(h, B, C, h->d_partial, h->partial_bytes, N, stream);
     return launch_wcsr_all(h, B, C, h->d_partial, N, stream);
 }
 
@@ -1207,7 +1232,7 @@ int spmm_run(spmm_handle_t h, const void* B_dev, void* C_dev, int64_t N, void* s
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (h->format == 0) return run_bcsr(h, B_dev, C_dev, N, st);
-    return run_wcsr(h, B_dev, C_dev, N, st);
+    return run_wcsr(h, B_dev, C_dev, N, use_rows(h, N), st);
 }
 
 int spmm_bcsr_plan(spmm_handle_t h, int64_t N) {
@@ -1228,7 +1253,7 @@ int spmm_prepare(spmm_handle_t h, int64_t N) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
     if (dev != h->device) return SPMM_ERR_INVALID_ARG;
-    if (int rc = ensure_wcsr_workspace(h, N, nullptr)) return rc;
+    if (int rc = ensure_wcsr_workspace(h, N, use_rows(h, N), nullptr)) return rc;
     // (the run may use any stream: the allocation has to be complete, not only ordered on this one)
     return cudaStreamSynchronize(nullptr) == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
 }
@@ -1309,6 +1334,7 @@ int spmm_run_host(spmm_handle_t h, const void* B_host, void* C_host, int64_t N, 
                 return SPMM_ERR_CUDA;
     }
     const int64_t nc = N / nchunks;
+    const bool rows = h->format == 1 && use_rows(h, N);
     const size_t bchunk = bbytes / nchunks, cchunk = cbytes / nchunks;
     const uint8_t* Bh = static_cast<const uint8_t*>(B_host);
     uint8_t* Chost = static_cast<uint8_t*>(C_host);
@@ -1330,7 +1356,8 @@ int spmm_run_host(spmm_handle_t h, const void* B_host, void* C_host, int64_t N, 
     for (int c = 0; c < nchunks && !bad && !rc; ++c) {
         bad |= cudaStreamWaitEvent(st, h->ev_in[c], 0) != cudaSuccess;
         if (bad) break;
-        rc = spmm_run(h, dB + c * bchunk, dC + c * cchunk, nc, stream);
+        rc = check_run_args(h, dB + c * bchunk, dC + c * cchunk, nc);
+        if (!rc) rc = h->format == 0 ? run_bcsr(h, dB + c * bchunk, dC + c * cchunk, nc, st) : run_wcsr(h, dB + c * bchunk, dC + c * cchunk, nc, rows, st);
         if (rc) break;
         bad |= cudaEventRecord(h->ev_run[c], st) != cudaSuccess;
         bad |= cudaStreamWaitEvent(h->s_out, h->ev_run[c], 0) != cudaSuccess;

@@ -163,9 +163,11 @@ struct WcsrRowStream {
     unsigned* d_counters = nullptr;  // 32 zero bytes (what the kernel gathers for an entry without column), then the counters
     int32_t* d_total = nullptr;      // {tasks, parts, long rows, slots}, read by finish_wcsr_rows
 };
-// Whether the row kernel serves a handle: 2- or 4-byte values, and at most kRowsMaxPerCol stored
-// values per padded column.
-constexpr double kRowsMaxPerCol = 2.0;
+// A handle has a row stream where the row kernel is the faster one at some dense width: 2- or 4-byte values, at
+// most kRowsMaxPerCol stored values per padded column (wcsr_wants_rows; by width: wcsr_rows_limit in api.cu).
+constexpr double kRowsMaxPerCol = 1.75;
+// Entries per SM and 128 groups of the row kernel: what its task sizes and its limits go by.
+inline int64_t wcsr_rows_load(int64_t m, int64_t nnz, int sms) { return (nnz + m) / (int64_t{sms} * 128); }
 constexpr int kRowsMaxSlots = 65536;    // partial rows of long rows cut into parts
 // Builds the stream on the GPU from a (validated) CSR matrix in device memory, in the order of `stream`; leaves
 // *out empty when the matrix has no rows or is too large for 32-bit entry positions.

@@ -915,13 +915,21 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
                            int es, int sms, cudaStream_t st, WcsrRowStream* out) {
     *out = WcsrRowStream();
     if (m <= 0 || (es != 2 && es != 4)) return SPMM_OK;
-    // Task sizes by the entries there are per SM and 128 groups: small matrices need short tasks to fill the
-    // GPU, large ones long tasks so that fewer warps start up.  Measured (us), {pack, task_max, part_len} =
-    // {8, 64, 512} / {16, 32, 256} / {16, 64, 512} / {32, 128, 512}: 4000 rows TF32 N = 36 (2 entries):
-    // 13.7 / 8.7 / 13.7 / 23.2; 100,000 rows TF32 N = 128 (34): 34.9 / 37.8 / 36.0 / 43.1; R-MAT 2^17 bf16
-    // N = 40 (157): 49.1 / 53.5 / 49.2 / 43.5; R-MAT 2^21 fp16 N = 128 (1820): 872 / 992 / 869 / 821.
-    const int64_t per = (nnz + m) / (int64_t{sms} * 128);
-    if (per >= 100) { out->pack = 32; out->task_max = 128; out->part_len = 512; }
+    // Task sizes by the entries there are per SM and 128 groups: small matrices need short tasks and parts to fill
+    // the GPU; in large ones a CTA's start and the reduction at its end weigh more (a part of 512 entries is eight
+    // steps of a group).  task_max is pack times a power of two, so that the last length class holds the rows of
+    // at most `pack` entries and no others.  Measured (us), {pack, task_max, part_len}, fp16 N = 128 / 320:
+    //                                        {16,32,256}  {16,64,512}  {16,64,1024}  {16,128,1024}  {32,128,512}  {32,128,2048}
+    //   4000 rows TF32 N = 36 (2 entries)        8.7          13.7                                      23.2
+    //   R-MAT 2^15, 16 a row (28)                              21.2 / 39    20.8 / 47     23.7 / 43      24.5 / 40     23.7 / 68
+    //   60,000 rows (66)                                      37.8 / 93    34.3 / 98     40.8 / 89      45.7 / 94     39.4 / 118
+    //   200,000 rows (137)                                    83.4 / 242   78.4 / 237    75.6 / 237     84.7 / 241    76.4 / 235
+    //   R-MAT 2^17 (160)                                      82.0 / 193   77.3 / 187    67.3 / 182     76.1 / 190    71.3 / 183
+    //   R-MAT 2^20 (1320)                                     623 / 1694   593 / 1652    527 / 1615     560 / 1648    518 / 1590
+    const int64_t per = wcsr_rows_load(m, nnz, sms);
+    if (per >= 500) { out->pack = 32; out->task_max = 128; out->part_len = 2048; }
+    else if (per >= 100) { out->pack = 16; out->task_max = 128; out->part_len = 1024; }
+    else if (per >= 50) { out->pack = 16; out->task_max = 64; out->part_len = 1024; }
     else if (per >= 16) { out->pack = 16; out->task_max = 64; out->part_len = 512; }
     else { out->pack = 16; out->task_max = 32; out->part_len = 256; }
     // rows of more than one part have more than part_len nonzeros: at most kRowsMaxSlots parts

@@ -283,14 +283,19 @@ cudaError_t launch_vb(int dtype, int c16, const WcsrRowsParams& p, dim3 grid, si
 
 }  // namespace
 
-// 32-byte vectors from 128-byte rows on (R-MAT 2^21 fp16 N = 128: 805 against 864 us with 16 bytes;
-// TF32 N = 128, 100,000 rows: 36.6 against 38.6); below, 16-byte vectors keep more lanes busy (the same
-// graph at N = 32: 339 against 454 us).
+// 32-byte vectors for rows of more than 128 bytes (R-MAT 2^21 fp16 N = 128: 805 against 864 us with 16 bytes;
+// 192-byte rows, R-MAT 2^20, fp16 / TF32: 518 / 454 against 592 / 537); up to there 16-byte vectors: fewer rows
+// share a warp, and its store at a row's end stops the others less often (128 bytes, 200,000 rows, fp16 / TF32:
+// 52 / 45 against 75 / 58).  Rows that are cut anyhow get one column tile more where that fills the lanes (1280
+// bytes, three tiles of 14 lanes instead of two of 20, R-MAT 2^20 TF32 N = 320: 2577 against 2819; two tiles for
+// one of 20 lanes read the entries twice: 1655 against 1661 there, 41 against 39 on R-MAT 2^15).
 RowsShape wcsr_rows_shape(int64_t N, int es, bool aligned32) {
     RowsShape s;
-    s.vec = aligned32 && N * es >= 128 ? 32 : 16;
+    s.vec = aligned32 && N * es > 128 ? 32 : 16;
     const int64_t vecs = (N * es + s.vec - 1) / s.vec;
-    const int64_t tiles = (vecs + 31) / 32;               // a group is part of one warp
+    int64_t tiles = (vecs + 31) / 32;               // a group is part of one warp
+    auto used = [&](int64_t t) { const int64_t l = (vecs + t - 1) / t; return 32 / l * l * vecs * 100 / (l * t); };
+    if (tiles > 1 && used(tiles + 1) > used(tiles) * 5 / 4) ++tiles;
     s.lanes = static_cast<int>((vecs + tiles - 1) / tiles);
     s.tiles = static_cast<int>((vecs + s.lanes - 1) / s.lanes);
     s.tile_cols = s.lanes * (s.vec / es);
