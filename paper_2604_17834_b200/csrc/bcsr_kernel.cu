@@ -357,11 +357,12 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             constexpr int kStepBytes = (32 / ES) * 128;     // k-rows of one MMA x 128 bytes (row-major token tile)
             const uint64_t bdesc0 = make_smem_desc(0, 16, 8 * Cfg::kARowBytes, Cfg::kASwizzle);
             const bool leader = elect_one();
-            // Whether the next stage's full barrier was already seen complete: with one token group the next stage is
-            // tested before this stage's MMAs are issued, so that its answer is there when they have
+            // Whether the next stage's full barrier was already seen complete: with one token group and b < 128 the
+            // next stage is tested before this stage's MMAs are issued, so that its answer is there when they have
             // been (a stage cost the issuer 172 cycles beside its four MMAs of 48, during which the tensor pipe ran
             // dry; down-projection 3584 x 18944, N = 128: 11.3 -> 10.6 us, b = 32, N = 1000: 87.7 -> 80.3).  Wider
-            // tiles have MMAs enough to cover it and measured up to 3 % slower with the extra test.
+            // tiles have MMAs enough to cover it and measured up to 3 % slower with the extra test; so have blocks of 128
+            // (8192 x 8192, b = 128, density 0.2: 156.1 us with it, 154.2 without).
             uint32_t it = 0, tile_i = 0;
             bool ready = false;
             bool ok = true;
@@ -386,7 +387,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     if (!ready && !__all_sync(0xffffffffu, mbar_wait(full_bar(s), ph, ctl, 3))) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint32_t sb = smem_base + s * Cfg::kStageBytes;
-                    if constexpr (GROUPS == 1)
+                    if constexpr (GROUPS == 1 && B < 128)
                         ready = __all_sync(0xffffffffu, mbar_test_wait(full_bar((it + 1) % STAGES), ((it + 1) / STAGES) & 1u));
 #pragma unroll
                     for (int i = 0; i < Cfg::kBps; ++i) {
