@@ -926,12 +926,15 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     //   200,000 rows (137)                                    83.4 / 242   78.4 / 237    75.6 / 237     84.7 / 241    76.4 / 235
     //   R-MAT 2^17 (160)                                      82.0 / 193   77.3 / 187    67.3 / 182     76.1 / 190    71.3 / 183
     //   R-MAT 2^20 (1320)                                     623 / 1694   593 / 1652    527 / 1615     560 / 1648    518 / 1590
+    // Below 16, {8, 32, 256} / {16, 32, 256} / {8, 32, 128} / {16, 64, 512}, fp16 N = 64 / 320: 45,000 rows (6)
+    // 8.2 / 26.0, 12.5 / 26.5, 8.2 / 23.1, 12.6 / 34.3; R-MAT 2^13, 24 a row (10) 7.1 / 18.6, 7.7 / 18.5, 8.1 / 18.4,
+    // 8.0 / 21.3; TF32 N = 64: 7.9, 9.6, 7.8, 11.8 and 8.6, 9.1, 9.4, 14.1.
     const int64_t per = wcsr_rows_load(m, nnz, sms);
     if (per >= 500) { out->pack = 32; out->task_max = 128; out->part_len = 2048; }
     else if (per >= 100) { out->pack = 16; out->task_max = 128; out->part_len = 1024; }
     else if (per >= 50) { out->pack = 16; out->task_max = 64; out->part_len = 1024; }
     else if (per >= 16) { out->pack = 16; out->task_max = 64; out->part_len = 512; }
-    else { out->pack = 16; out->task_max = 32; out->part_len = 256; }
+    else { out->pack = 8; out->task_max = 32; out->part_len = 256; }
     // rows of more than one part have more than part_len nonzeros: at most kRowsMaxSlots parts
     out->part_len = static_cast<int>(std::max<int64_t>(out->part_len, (2 * nnz / kRowsMaxSlots + 127) / 128 * 128));
     // upper bounds for the arrays, so that nothing has to be read back before the end
