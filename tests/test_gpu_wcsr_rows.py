@@ -1,0 +1,113 @@
+"""WCSR row kernel (windows that condense almost nothing): row lengths at the edges of its tasks, parts and
+length classes, every task size, both vector widths, several column tiles, ragged tails, against the fp64 oracle.
+Bound: that of the other WCSR tests; products are exact or rounded once, sums are fp32, a 16-bit C adds 2^-9.
+"""
+import numpy as np
+import pytest
+
+from paper_2604_17834_b200 import workloads as wl
+
+from helpers import CANARY, GUARD, assert_close, check_guards, reference, run_gpu_variant, to_device
+
+pytestmark = pytest.mark.gpu
+
+EDGES = [0, 1, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1025, 2048, 2049, 5000]
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2604_17834_b200 import binding
+    return binding
+
+
+def _matrix(m, k, mean, dtype, seed=61):
+    """EDGES, 16 rows apart and in both orders, among rows of 0 .. 2 * mean entries; a row's columns are k / length
+    apart from a random start, so neighbouring rows share almost none."""
+    rng = np.random.default_rng(seed)
+    lens = rng.integers(0, 2 * mean + 1, m)
+    lens[np.arange(len(EDGES)) * 16] = EDGES
+    lens[m - 1 - np.arange(len(EDGES)) * 16] = EDGES
+    rp = np.zeros(m + 1, np.int64)
+    rp[1:] = np.cumsum(lens)
+    step = k // np.maximum(lens, 1)
+    start = (rng.random(m) * step).astype(np.int64)
+    j = np.arange(rp[-1]) - np.repeat(rp[:-1], lens)
+    col = (np.repeat(start, lens) + j * np.repeat(step, lens)).astype(np.int32)
+    vals = wl.dense(seed + 1, 1, int(rp[-1]), ("normal", 0.0, 1.0), dtype).ravel()
+    return {"m": m, "k": k, "row_ptr": rp, "col_idx": col, "vals": vals}
+
+
+# rows, mean length: 4, 20, 54, 122 and 539 entries per SM and 128 groups, one for every choice of task sizes;
+# N: a row of B that is one vector, 16-byte vectors (to 128 bytes, or 144 and 8400 bytes: no multiple of 32),
+# 32-byte vectors with a ragged last tile, and more column tiles than one launch covers (8400 bytes)
+@pytest.mark.parametrize("dtype,c16,m,mean,N", [
+    ("fp16", False, 3001, 16, 8), ("tf32", False, 3001, 16, 36), ("bf16", True, 3001, 16, 64), ("fp16", False, 3001, 16, 4200),
+    ("tf32", False, 3001, 16, 328), ("bf16", True, 3001, 16, 1040), ("fp16", True, 40007, 8, 80), ("tf32", False, 100003, 9, 32),
+    ("bf16", False, 100003, 22, 32), ("tf32", False, 600011, 16, 8)])
+def test_wcsr_row_kernel(lib, dtype, c16, m, mean, N):
+    import torch
+    k = max(m, 20000)
+    a = _matrix(m, k, mean, dtype)
+    Bs = wl.dense(63, k, N, ("uniform", -1.0, 1.0), dtype)
+    Cr, S = reference(a, Bs, dtype)
+    out = []
+    dev = [to_device(x) for x in (a["row_ptr"], a["col_idx"], a["vals"])]
+    opts = dict(c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
+    for built_on_gpu in (True, False):
+        if built_on_gpu:
+            h = lib.spmm_wcsr_create_csr_device(m, k, *[d.data_ptr() for d in dev], dtype, 16, **opts)
+        else:
+            h = lib.spmm_wcsr_create_csr(m, k, a["row_ptr"], a["col_idx"], a["vals"], dtype, 16, **opts)
+        try:
+            info = lib.spmm_get_info(h, N)
+            assert info["nnz"] * 16 <= 1.2 * info["stored_values"]          # the row kernel's at every width
+            out.append(run_gpu_variant(lib, h, Bs, m, N, dtype, c16=c16))
+            if built_on_gpu:
+                # operands on a 16-byte boundary only: the 16-byte vectors, whatever the width; same sums
+                es, cs = a["vals"].itemsize, 2 if c16 else 4
+                raw = torch.empty(k * N * es + 16, dtype=torch.uint8, device="cuda")
+                raw[16:] = to_device(Bs).view(torch.uint8).reshape(-1)
+                cdt = {4: torch.float32, 2: torch.bfloat16 if dtype == "bf16" else torch.float16}[cs]
+                buf = torch.full((2 * GUARD + m * N + 16 // cs,), CANARY, dtype=cdt, device="cuda")
+                C = buf[GUARD + 16 // cs:GUARD + 16 // cs + m * N].view(m, N)
+                lib.spmm_run(h, raw.data_ptr() + 16, C.data_ptr(), N, torch.cuda.current_stream().cuda_stream)
+                torch.cuda.synchronize()
+                check_guards(buf, "spmm_run")
+                out.append(C.float().cpu().numpy())
+        finally:
+            lib.spmm_destroy(h)
+    assert_close(out[0], Cr, S, dtype, "row kernel %s N=%d" % (dtype, N))
+    assert np.array_equal(out[0], out[1]) and np.array_equal(out[0], out[2])
+
+
+@pytest.mark.parametrize("dtype,N,expect", [("fp16", 32, True), ("fp16", 64, False), ("tf32", 64, True), ("tf32", 128, False)])
+def test_wcsr_kernel_by_width(lib, dtype, N, expect):
+    """A band that condenses 1.5 values per column: the row kernel below 64 (TF32: 128) tokens, the window kernel
+    from there on (their sums differ in the last bits); a run over column chunks goes by the whole width."""
+    m = 50000
+    rng = np.random.default_rng(3)
+    col = np.sort((np.arange(m)[:, None] + rng.permuted(np.tile(np.arange(240), (m, 1)), axis=1)[:, :16]), axis=1)
+    a = {"m": m, "k": m + 240, "row_ptr": np.arange(m + 1, dtype=np.int64) * 16, "col_idx": col.astype(np.int32).ravel(),
+         "vals": wl.dense(5, 1, m * 16, ("normal", 0.0, 1.0), dtype).ravel()}
+    h = lib.spmm_wcsr_create_csr(m, m + 240, a["row_ptr"], a["col_idx"], a["vals"], dtype, 16)
+    try:
+        info = lib.spmm_get_info(h, N)
+        assert 1.25 < info["nnz"] * 16 / info["stored_values"] < 1.7
+        Bs = wl.dense(6, m + 240, N, ("uniform", -1.0, 1.0), dtype)
+        C = run_gpu_variant(lib, h, Bs, m, N, dtype)
+        Cr, S = reference(a, Bs, dtype)
+        assert_close(C, Cr, S, dtype, "band N=%d" % N)
+        # the row kernel adds a row of up to 32 values in their order, one rounding each
+        B64 = wl.widen(Bs, dtype)
+        v = wl.widen(a["vals"], dtype).reshape(m, 16)
+        acc = np.zeros((64, N), np.float32)
+        for j in range(16):
+            acc = (acc.astype(np.float64) + v[:64, j, None] * B64[col[:64, j]]).astype(np.float32)
+        assert np.array_equal(C[:64], acc) == expect
+        if N == 128:
+            import torch
+            host = np.empty((m, N), np.float32)                            # chunks of 64 columns
+            lib.spmm_run_host(h, np.ascontiguousarray(Bs), host, N, torch.cuda.current_stream().cuda_stream)
+            assert np.array_equal(host, C)
+    finally:
+        lib.spmm_destroy(h)
