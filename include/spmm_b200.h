@@ -337,6 +337,9 @@ int spmm_prepare(spmm_handle_t h, int64_t N);
  * WCSR keeps the partial tiles of split windows in a device workspace owned by the handle;
  * it is (re)allocated here the first time a given N needs more than it holds, so two runs
  * of one handle must not overlap on the GPU, and the first run at a new N may synchronise.
+ * Under stream capture a run that would have to allocate returns an error and launches
+ * nothing (in cudaStreamCaptureModeRelaxed it allocates, outside the graph): call
+ * spmm_prepare before the capture.  A captured run keeps the addresses of capture time.
  * Split windows are merged by a fixed-order sum, so results are run-to-run identical.
  * A BCSR handle with row groups launches its kernel twice (groups, then the other block-rows;
  * the second launch starts on the SMs the first leaves idle and does not finish before it).

@@ -147,6 +147,7 @@ struct spmm_handle_s {
 
     float* d_partial = nullptr;      // WCSR workspace
     size_t partial_bytes = 0;
+    bool partial_pooled = true;      // false: from cudaMalloc (see ensure_wcsr_workspace)
 
     // BCSR tensor maps
     CUtensorMap tmA;
@@ -174,6 +175,14 @@ struct spmm_handle_s {
 
 namespace {
 
+void free_partial(spmm_handle_s* h) {
+    if (h->partial_pooled) dev_free(h->d_partial, nullptr);
+    else cudaFree(h->d_partial);
+    h->d_partial = nullptr;
+    h->partial_bytes = 0;
+    h->partial_pooled = true;
+}
+
 void free_handle(spmm_handle_s* h) {
     if (!h) return;
     if (!h->host_only) {
@@ -183,9 +192,10 @@ void free_handle(spmm_handle_s* h) {
         cudaDeviceSynchronize();
         void* const arrays[] = {
             h->d_ptr, h->d_idx, h->d_vals, h->d_order, h->d_tiles, h->d_tile_recs, h->d_cta_ptr, h->d_kmerge,
-            h->d_sidx, h->d_srows, h->d_svals, h->d_stile_recs, h->d_scta_ptr, h->d_status, h->d_partial,
+            h->d_sidx, h->d_srows, h->d_svals, h->d_stile_recs, h->d_scta_ptr, h->d_status,
             h->d_plan, h->d_class, h->d_rec_ptr};
         for (void* ptr : arrays) dev_free(ptr, nullptr);
+        free_partial(h);
         free_wcsr_rows(&h->rows, nullptr);
         if (other) cudaSetDevice(dev);
         cudaFree(h->d_Bstage);
@@ -854,10 +864,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             const size_t need = static_cast<size_t>(sc.n_slots) * f.b * static_cast<size_t>(N) * 4;
             if (!rc && need > h->partial_bytes) {
                 if (h->d_partial && cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
-                dev_free(h->d_partial, nullptr);
-                h->d_partial = nullptr;
-                h->partial_bytes = 0;
-                if (!dev_alloc_ok(&h->d_partial, need, nullptr)) rc = SPMM_ERR_ALLOC;
+                free_partial(h);
+                if (!dev_alloc_ready_ok(&h->d_partial, need)) rc = SPMM_ERR_ALLOC;
                 else h->partial_bytes = need;
             }
             if (!rc) {
@@ -1102,19 +1110,34 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
     return e == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
 }
 
-// The handle's workspace for the partial tiles of split windows at dense width N (grown, never shrunk).
+// The handle's workspace for the partial tiles of split windows at dense width N (grown, never shrunk).  It outlives
+// the run and serves runs on any stream, so it is never a stream-ordered allocation of the run's own stream -- under
+// stream capture that would be a node of the graph, whose memory exists while the graph runs only.  A run that needs
+// to grow it under capture asks for memory outside the pool instead: refused (SPMM_ERR_ALLOC, nothing launched) in
+// the capture modes that forbid an allocation, lasting in the relaxed one.
 int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, bool rows, cudaStream_t stream) {
     const size_t need = rows ? rows_workspace_bytes(h, N) : static_cast<size_t>(wcsr_workspace_bytes(h, N));
-    if (need > h->partial_bytes) {
-        if (h->d_partial) {
-            if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
-            dev_free(h->d_partial, nullptr);
-            h->d_partial = nullptr;
-            h->partial_bytes = 0;
-        }
-        if (!dev_alloc_ok(&h->d_partial, need, stream)) return SPMM_ERR_ALLOC;
-        h->partial_bytes = need;
+    if (need <= h->partial_bytes) return SPMM_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {    // (the legacy stream while a blocking one is captured)
+        cudaGetLastError();
+        capture = cudaStreamCaptureStatusActive;
     }
+    if (h->d_partial) {
+        if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
+        free_partial(h);
+    }
+    if (capture == cudaStreamCaptureStatusNone) {
+        if (!dev_alloc_ready_ok(&h->d_partial, need)) return SPMM_ERR_ALLOC;
+    } else {
+        if (cudaMalloc(reinterpret_cast<void**>(&h->d_partial), need) != cudaSuccess) {
+            cudaGetLastError();
+            h->d_partial = nullptr;
+            return SPMM_ERR_ALLOC;
+        }
+        h->partial_pooled = false;
+    }
+    h->partial_bytes = need;
     return SPMM_OK;
 }
 
@@ -1253,9 +1276,7 @@ int spmm_prepare(spmm_handle_t h, int64_t N) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
     if (dev != h->device) return SPMM_ERR_INVALID_ARG;
-    if (int rc = ensure_wcsr_workspace(h, N, use_rows(h, N), nullptr)) return rc;
-    // (the run may use any stream: the allocation has to be complete, not only ordered on this one)
-    return cudaStreamSynchronize(nullptr) == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
+    return ensure_wcsr_workspace(h, N, use_rows(h, N), nullptr);
 }
 
 int spmm_wcsr_run_static(spmm_handle_t h, const void* B_dev, void* C_dev, int64_t N, void* stream) {

@@ -8,27 +8,33 @@ namespace spmm {
 
 namespace {
 
-cudaError_t device_pool(cudaMemPool_t* pool) {
+struct Pool {
+    cudaMemPool_t pool = nullptr;
+    cudaStream_t service = nullptr;      // carries allocations only (dev_alloc_ready): never waits for a user's work
+};
+
+cudaError_t device_pool(Pool* pool) {
     static std::mutex mu;
-    static cudaMemPool_t pools[kMaxDevices] = {};
+    static Pool pools[kMaxDevices];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
-    if (!pools[dev]) {
+    if (!pools[dev].pool) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.handleTypes = cudaMemHandleTypeNone;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
-        cudaMemPool_t p = nullptr;
-        e = cudaMemPoolCreate(&p, &props);
+        Pool p;
+        e = cudaMemPoolCreate(&p.pool, &props);
         if (e != cudaSuccess) return e;
         unsigned long long keep = kPoolKeepBytes;
-        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        e = cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p.service, cudaStreamNonBlocking);
         if (e != cudaSuccess) {
-            cudaMemPoolDestroy(p);
+            cudaMemPoolDestroy(p.pool);
             return e;
         }
         pools[dev] = p;
@@ -37,19 +43,23 @@ cudaError_t device_pool(cudaMemPool_t* pool) {
     return cudaSuccess;
 }
 
-}  // namespace
-
-cudaError_t dev_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
+// `stream` null with `ready`: the service stream, waited for.
+cudaError_t alloc_from_pool(void** ptr, size_t bytes, cudaStream_t stream, bool ready) {
     *ptr = nullptr;
-    cudaMemPool_t pool = nullptr;
+    Pool pool;
     cudaError_t e = device_pool(&pool);
     if (e != cudaSuccess) return e;
+    if (ready) stream = pool.service;
     if (bytes == 0) bytes = 16;
-    e = cudaMallocFromPoolAsync(ptr, bytes, pool, stream);
+    e = cudaMallocFromPoolAsync(ptr, bytes, pool.pool, stream);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        cudaMemPoolTrimTo(pool, 0);
-        e = cudaMallocFromPoolAsync(ptr, bytes, pool, stream);
+        cudaMemPoolTrimTo(pool.pool, 0);
+        e = cudaMallocFromPoolAsync(ptr, bytes, pool.pool, stream);
+    }
+    if (e == cudaSuccess && ready) {
+        e = cudaStreamSynchronize(stream);
+        if (e != cudaSuccess) cudaFreeAsync(*ptr, stream);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -57,6 +67,12 @@ cudaError_t dev_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
     }
     return e;
 }
+
+}  // namespace
+
+cudaError_t dev_alloc(void** ptr, size_t bytes, cudaStream_t stream) { return alloc_from_pool(ptr, bytes, stream, false); }
+
+cudaError_t dev_alloc_ready(void** ptr, size_t bytes) { return alloc_from_pool(ptr, bytes, nullptr, true); }
 
 void dev_free(void* ptr, cudaStream_t stream) {
     if (ptr) cudaFreeAsync(ptr, stream);

@@ -94,3 +94,35 @@ def assert_close(C_gpu, C_ref, S, dtype, what=""):
         raise AssertionError("%s: %d of %d outside the bound; worst at (%d,%d): gpu %.6g ref %.6g err %.3g bound %.3g"
                              % (what, int(bad.sum()), err.size, i, j, C_gpu[i, j], C_ref[i, j], err[i, j], bound[i, j]))
     return float(np.max(err / bound))
+
+
+def captured_run(lib, h, B, C, N, relaxed=False, replay=False):
+    """One spmm_run inside a stream capture of its own stream.  -> (status code of the run, kinds of the captured
+    nodes, or None where the capture gave no graph).  replay: launch the graph once, unless the run was refused."""
+    import torch
+    from cuda.bindings import runtime as rt
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    mode = rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed if relaxed else rt.cudaStreamCaptureMode.cudaStreamCaptureModeGlobal
+    assert rt.cudaStreamBeginCapture(stream.cuda_stream, mode)[0] == rt.cudaError_t.cudaSuccess
+    code = lib.SPMM_OK
+    try:
+        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, stream.cuda_stream)
+    except lib.SpmmError as e:
+        code = e.code
+    err, graph = rt.cudaStreamEndCapture(stream.cuda_stream)
+    rt.cudaGetLastError()
+    if err != rt.cudaError_t.cudaSuccess or int(graph) == 0:
+        return code, None
+    n = rt.cudaGraphGetNodes(graph, 0)[-1]
+    nodes = rt.cudaGraphGetNodes(graph, n)[1] if n else []
+    kinds = [str(rt.cudaGraphNodeGetType(x)[1]).split(".")[-1].split("NodeType")[-1].split(":")[0].strip().lower() for x in nodes]
+    if replay and code == lib.SPMM_OK:
+        err, ex = rt.cudaGraphInstantiate(graph, 0)
+        assert err == rt.cudaError_t.cudaSuccess
+        assert rt.cudaGraphLaunch(ex, stream.cuda_stream)[0] == rt.cudaError_t.cudaSuccess
+        stream.synchronize()
+        lib.spmm_check(h)
+        rt.cudaGraphExecDestroy(ex)
+    rt.cudaGraphDestroy(graph)
+    return code, kinds

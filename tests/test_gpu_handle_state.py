@@ -1,0 +1,77 @@
+"""What a handle keeps between calls: the run's workspace, the memory behind it, what stream capture may see of it.
+
+A run inside a stream capture is also the test for "makes no allocating or synchronising call": in the global capture
+mode such a call is refused by CUDA, so a run that is captured into kernel nodes only has made none.
+"""
+import numpy as np
+import pytest
+
+from paper_2604_17834_b200 import workloads as wl
+
+from helpers import assert_close, captured_run, reference, run_gpu, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lib():
+    from paper_2604_17834_b200 import binding
+    return binding
+
+
+def _long_rows(dtype, m=512, k=60000, n=900, seed=3):
+    """Rows of n entries whose columns neighbouring rows share almost never: the row kernel's, several parts a row."""
+    rng = np.random.default_rng(seed)
+    step = k // n
+    col = (np.arange(n, dtype=np.int64)[None, :] * step + rng.integers(0, step, (m, 1))).astype(np.int32)
+    return {"m": m, "k": k, "row_ptr": np.arange(m + 1, dtype=np.int64) * n, "col_idx": col.ravel(),
+            "vals": wl.dense(seed, 1, m * n, ("normal", 0.0, 1.0), dtype).ravel()}
+
+
+@pytest.mark.parametrize("kind", ["rows", "window"])
+def test_a_run_under_capture_never_takes_its_workspace_from_the_graph(lib, kind):
+    """Without spmm_prepare a captured run has no workspace: it is refused and launches nothing, and the handle then
+    works as if it had not been tried.  After spmm_prepare the same run is captured, and its replay and ordinary
+    runs agree.  (The workspace must never be an allocation node: its memory would be the graph's.)"""
+    import torch
+    dtype, N = "fp16", 128
+    a = _long_rows(dtype) if kind == "rows" else wl.random_csr(51, 1000, 900, 0.3, dtype)
+    h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16,
+                                 **({} if kind == "rows" else dict(split_cols=64)))
+    try:
+        Bs = wl.dense(8, a["k"], N, ("normal", 0.0, 1.0), dtype)
+        B = to_device(Bs)
+        C = torch.zeros((a["m"], N), dtype=torch.float32, device="cuda")
+        code, nodes = captured_run(lib, h, B, C, N)
+        assert code == lib.SPMM_ERR_ALLOC and nodes is None
+        want = run_gpu(lib, h, Bs, a["m"], N)
+        Cr, S = reference(a, Bs, dtype)
+        assert_close(want, Cr, S, dtype, "after a refused capture")
+        code, nodes = captured_run(lib, h, B, C, N, replay=True)
+        assert code == lib.SPMM_OK and nodes and set(nodes) == {"kernel"}
+        assert np.array_equal(C.cpu().numpy(), want)
+        assert np.array_equal(run_gpu(lib, h, Bs, a["m"], N), want)
+    finally:
+        lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["rows", "window"])
+def test_a_relaxed_capture_allocates_outside_the_graph(lib, kind):
+    """cudaStreamCaptureModeRelaxed allows allocations: the workspace is then ordinary memory that outlives the graph."""
+    import torch
+    dtype, N = "fp16", 96
+    a = _long_rows(dtype, seed=4) if kind == "rows" else wl.random_csr(52, 1000, 900, 0.3, dtype)
+    h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16,
+                                 **({} if kind == "rows" else dict(split_cols=64)))
+    try:
+        Bs = wl.dense(9, a["k"], N, ("normal", 0.0, 1.0), dtype)
+        B = to_device(Bs)
+        C = torch.zeros((a["m"], N), dtype=torch.float32, device="cuda")
+        code, nodes = captured_run(lib, h, B, C, N, relaxed=True, replay=True)
+        assert code == lib.SPMM_OK and set(nodes) == {"kernel"}
+        first = C.cpu().numpy().copy()
+        assert np.array_equal(run_gpu(lib, h, Bs, a["m"], N), first)
+        Cr, S = reference(a, Bs, dtype)
+        assert_close(first, Cr, S, dtype, "relaxed capture")
+    finally:
+        lib.spmm_destroy(h)
