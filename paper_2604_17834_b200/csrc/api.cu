@@ -72,11 +72,13 @@ int encode_2d(CUtensorMap* map, int dtype, const void* base, uint64_t rows, uint
     return r == CUDA_SUCCESS ? SPMM_OK : SPMM_ERR_CUDA;
 }
 
+// Ready for every stream when it returns (a copy from pageable memory may still be on its way when cudaMemcpy does).
 template <class T>
 int upload(T** dptr, const void* src, size_t bytes) {
     *dptr = nullptr;
-    if (!dev_alloc_ok(dptr, bytes, nullptr)) return SPMM_ERR_ALLOC;
-    if (bytes && cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (!dev_alloc_ready_ok(dptr, bytes)) return SPMM_ERR_ALLOC;
+    if (bytes && (cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess))
+        return SPMM_ERR_CUDA;
     return SPMM_OK;
 }
 
@@ -211,7 +213,8 @@ void free_handle(spmm_handle_s* h) {
     delete h;
 }
 
-int device_setup(spmm_handle_s* h, const spmm_opts_t* opts) {
+// `stream`: the creation's own, which it synchronises before it returns the handle.
+int device_setup(spmm_handle_s* h, const spmm_opts_t* opts, cudaStream_t stream) {
     if (h->host_only) {
         h->sms = 148;
         h->n_ctas = (opts && opts->n_ctas > 0) ? opts->n_ctas : 148;
@@ -227,8 +230,8 @@ int device_setup(spmm_handle_s* h, const spmm_opts_t* opts) {
     h->device = dev;
     h->sms = sms;
     h->n_ctas = (opts && opts->n_ctas > 0) ? opts->n_ctas : h->sms;
-    if (!dev_alloc_ok(&h->d_status, 4 * sizeof(int), nullptr)) return SPMM_ERR_ALLOC;
-    if (cudaMemset(h->d_status, 0, 4 * sizeof(int)) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (!dev_alloc_ok(&h->d_status, 4 * sizeof(int), stream)) return SPMM_ERR_ALLOC;
+    if (cudaMemsetAsync(h->d_status, 0, 4 * sizeof(int), stream) != cudaSuccess) return SPMM_ERR_CUDA;
     return SPMM_OK;
 }
 
@@ -323,7 +326,7 @@ int create_bcsr(spmm_handle_t* out, const CsrView& a, int dtype, int block, cons
     rc = validate_csr(a);
     if (rc) { delete h; return rc; }
     h->nnz = a.nnz;
-    rc = device_setup(h, opts);
+    rc = device_setup(h, opts, nullptr);
     if (rc) { free_handle(h); return rc; }
     try {
         rc = build_bcsr(a, block, &h->bcsr);
@@ -359,7 +362,7 @@ int create_bcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     spmm_handle_s* h = nullptr;
     int rc = new_bcsr_handle(&h, m, k, dtype, block, opts);
     if (rc) return rc;
-    rc = device_setup(h, opts);
+    rc = device_setup(h, opts, stream);
     if (rc) { free_handle(h); return rc; }
     try {
         rc = build_bcsr_device(m, k, d_row_ptr, d_col_idx, static_cast<const uint8_t*>(d_vals), h->es, block, stream,
@@ -495,7 +498,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
     rc = validate_csr(a);
     if (rc) { delete h; return rc; }
     h->nnz = a.nnz;
-    rc = device_setup(h, opts);
+    rc = device_setup(h, opts, nullptr);
     if (rc) { free_handle(h); return rc; }
     try {
         rc = build_wcsr(a, wh, b_col, T, h->n_ctas * wcsr_bins_per_sm(h->es, wh), &h->wcsr);
@@ -539,7 +542,7 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     int rc = new_wcsr_handle(&h, m, k, dtype, opts, &b_col, &T);
     if (rc) return rc;
     if (h->lsu_gather && wh != 16) { delete h; return SPMM_ERR_UNSUPPORTED; }
-    rc = device_setup(h, opts);
+    rc = device_setup(h, opts, stream);
     if (rc) { free_handle(h); return rc; }
     try {
         rc = build_wcsr_device(m, k, d_row_ptr, d_col_idx, static_cast<const uint8_t*>(d_vals), h->es, wh, b_col, T,
@@ -1403,6 +1406,7 @@ int spmm_check(spmm_handle_t h) {
     if (cudaMemcpy(st, h->d_status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return SPMM_ERR_CUDA;
     if (st[0] != 0) {
         cudaMemset(h->d_status, 0, sizeof(st));
+        cudaStreamSynchronize(nullptr);          // (the next run may come on a stream that does not wait for this one)
         if (st[0] == 2) return SPMM_ERR_DEV_BOUNDS;
         return st[3] != 0 ? SPMM_ERR_DEV_UNDRAINED : SPMM_ERR_DEV_TIMEOUT;
     }

@@ -75,3 +75,32 @@ def test_a_relaxed_capture_allocates_outside_the_graph(lib, kind):
         assert_close(first, Cr, S, dtype, "relaxed capture")
     finally:
         lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["bcsr", "wcsr"])
+def test_a_handle_is_complete_when_its_creation_returns(lib, kind):
+    """Built and run on a stream of its own while the default stream is busy: nothing of the handle may still wait
+    behind that work.  A status word cleared late would wipe what the run reported (here a wait that runs out)."""
+    import torch
+    a = wl.bcsr_sweep(404, m=2048, k=2048, b=64, density=0.3, dtype="fp16") if kind == "bcsr" else wl.wcsr_irregular(seed=405, m=20000, dtype="tf32")
+    dtype, size, N = ("fp16", 64, 1024) if kind == "bcsr" else ("tf32", 16, 128)
+    mk = lib.spmm_bcsr_create_csr_device if kind == "bcsr" else lib.spmm_wcsr_create_csr_device
+    dev = [to_device(a[x]) for x in ("row_ptr", "col_idx", "vals")]
+    B = to_device(wl.dense(6, a["k"], N, ("normal", 0.0, 1.0), dtype))
+    C = torch.empty((a["m"], N), dtype=torch.float32, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(500_000_000)                         # a quarter of a second on the default stream
+    h = mk(a["m"], a["k"], *[d.data_ptr() for d in dev], dtype, size, side.cuda_stream)
+    try:
+        lib.spmm_set_wait_limit_ns(0)
+        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, side.cuda_stream)
+        side.synchronize()
+        torch.cuda.synchronize()
+        with pytest.raises(lib.SpmmError) as e:
+            lib.spmm_check(h)
+        assert e.value.code == lib.SPMM_ERR_DEV_TIMEOUT
+        lib.spmm_check(h)
+    finally:
+        lib.spmm_set_wait_limit_ns(2_000_000_000)
+        lib.spmm_destroy(h)
