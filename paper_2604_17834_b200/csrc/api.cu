@@ -199,6 +199,7 @@ void free_handle(spmm_handle_s* h) {
         for (void* ptr : arrays) dev_free(ptr, nullptr);
         free_partial(h);
         free_wcsr_rows(&h->rows, nullptr);
+        dev_give_back();
         if (other) cudaSetDevice(dev);
         cudaFree(h->d_Bstage);
         cudaFree(h->d_Cstage);
@@ -1312,14 +1313,14 @@ int spmm_run_host(spmm_handle_t h, const void* B_host, void* C_host, int64_t N, 
         cudaFree(h->d_Bstage);
         h->d_Bstage = nullptr;
         h->Bstage_bytes = 0;
-        if (cudaMalloc(&h->d_Bstage, bbytes ? bbytes : 16) != cudaSuccess) return SPMM_ERR_ALLOC;
+        if (dev_malloc(&h->d_Bstage, bbytes) != cudaSuccess) return SPMM_ERR_ALLOC;
         h->Bstage_bytes = bbytes;
     }
     if (cbytes > h->Cstage_bytes) {
         cudaFree(h->d_Cstage);
         h->d_Cstage = nullptr;
         h->Cstage_bytes = 0;
-        if (cudaMalloc(reinterpret_cast<void**>(&h->d_Cstage), cbytes ? cbytes : 16) != cudaSuccess) return SPMM_ERR_ALLOC;
+        if (dev_malloc(reinterpret_cast<void**>(&h->d_Cstage), cbytes) != cudaSuccess) return SPMM_ERR_ALLOC;
         h->Cstage_bytes = cbytes;
     }
     // Large operands go in column chunks (token chunks), so that the copy of one chunk's result to

@@ -78,4 +78,29 @@ void dev_free(void* ptr, cudaStream_t stream) {
     if (ptr) cudaFreeAsync(ptr, stream);
 }
 
+void dev_give_back(size_t keep) {
+    Pool pool;
+    unsigned long long reserved = 0;
+    if (device_pool(&pool) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool.pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess || reserved <= keep)
+        return;
+    cudaStreamSynchronize(nullptr);              // the frees count once they are known to have happened
+    cudaMemPoolTrimTo(pool.pool, keep);
+}
+
+cudaError_t dev_malloc(void** ptr, size_t bytes) {
+    if (bytes == 0) bytes = 16;
+    cudaError_t e = cudaMalloc(ptr, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        dev_give_back(0);
+        e = cudaMalloc(ptr, bytes);
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *ptr = nullptr;
+    }
+    return e;
+}
+
 }  // namespace spmm

@@ -104,3 +104,20 @@ def test_a_handle_is_complete_when_its_creation_returns(lib, kind):
     finally:
         lib.spmm_set_wait_limit_ns(2_000_000_000)
         lib.spmm_destroy(h)
+
+
+def test_destroying_a_handle_gives_its_memory_back(lib):
+    """What a large handle held is the device's again when spmm_destroy returns, but for the pool's 256 MB."""
+    import torch
+    m, n = 32768, 1024                                     # 2 M blocks of 16 x 16: 1 GB
+    rp = torch.arange(m + 1, device="cuda", dtype=torch.int64) * n
+    ci = (torch.arange(n, device="cuda", dtype=torch.int32) * 32).repeat(m)
+    va = torch.ones(m * n, dtype=torch.float16, device="cuda")
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    h = lib.spmm_bcsr_create_csr_device(m, m, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), "fp16", 16, stack_min_fill=-1)
+    held = free0 - torch.cuda.mem_get_info()[0]
+    lib.spmm_destroy(h)
+    left = free0 - torch.cuda.mem_get_info()[0]
+    assert held > 700 << 20
+    assert left <= (256 << 20) + (64 << 20), "%.0f MB still held" % (left / 2 ** 20)       # (64: the pool grows in steps)
