@@ -156,7 +156,10 @@ typedef struct {
                             for b = 16 / 32 / 64), -1 = off, 1..100 = threshold.  A private
                             second copy of the grouped rows' values is kept on the device; the
                             exported format arrays and nnz_stored are unaffected.  Ignored for
-                            b = 128 and the dynamic schedule.                                 */
+                            b = 128 and the dynamic schedule.  A non-finite entry of B makes
+                            NaN of its column's outputs in the block-rows that store a block
+                            there, as without groups; with 16-bit and E4M3 values also in the
+                            other block-rows of a group whose union holds that block column.  */
     int32_t gather;      /* spmm_gather_t; WCSR only (a BCSR handle ignores it)              */
     int32_t k_split;     /* BCSR: 1 = a block-row whose stored blocks exceed a quarter of one
                             CTA's mean load for the dense width at hand is cut into contiguous

@@ -928,6 +928,10 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.status = h->d_status;
     p.wait_limit_ns = g_wait_limit_ns.load();
     p.stack_rows = nullptr;
+    p.plain_col_idx = nullptr;
+    p.plain_vals = nullptr;
+    p.B = nullptr;
+    p.k = h->k;
     p.overlap = 0;
     CUtensorMap tmA = h->tmA;
     if (!h->tmA_ok) {
@@ -947,6 +951,11 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         ps.tiles = reinterpret_cast<const int4*>(h->d_stile_recs);
         ps.cta_ptr = h->d_scta_ptr;
         ps.stack_rows = h->d_srows;
+        if (h->dtype == SPMM_TF32) {
+            ps.plain_col_idx = h->d_idx;
+            ps.plain_vals = reinterpret_cast<const float*>(h->d_vals);
+            ps.B = static_cast<const float*>(B);
+        }
         ps.use_3d = h->tmB3s_ok ? 1 : 0;
         ps.overlap = 1;
         p.overlap = 2;

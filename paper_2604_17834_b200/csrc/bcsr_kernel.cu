@@ -137,6 +137,28 @@ struct BcsrProducers {
     static constexpr int kThreads = DYN ? 224 : 160 + 32 * n;
 };
 
+// What the tensor core takes of a 4-byte operand.
+__device__ __forceinline__ float tf32_operand(float x) { return x != x ? x : __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
+
+// C[row][n] of a TF32 matrix from the blocks its block-row stores.  A stacked block multiplies the absent sub-blocks
+// of its other block-rows as zeros, and a zero times Inf or NaN is NaN: where a row group's accumulator is NaN, this
+// says whether the row's own blocks make it one.  Never reached with finite operands and sums.
+template <int B, int CM>
+__device__ __noinline__ float plain_product(const int32_t* block_row_ptr, const int32_t* block_col_idx, const float* vals,
+                                            const float* dense, int64_t k, int64_t N, int64_t row, int64_t n) {
+    const int64_t I = row / B;
+    const int q1 = block_row_ptr[I + 1];
+    float s = 0.f;
+    for (int q = block_row_ptr[I]; q < q1; ++q) {
+        const int64_t k0 = static_cast<int64_t>(block_col_idx[q]) * B;
+        const float* a = vals + (static_cast<int64_t>(q) * B + (row - I * B)) * B;
+        const int width = static_cast<int>(min_i64(B, k - k0));
+        for (int j = 0; j < width; ++j)
+            s = fmaf(tf32_operand(a[j]), tf32_operand(CM ? dense[n * k + k0 + j] : dense[(k0 + j) * N + n]), s);
+    }
+    return s;
+}
+
 template <int B, int H, int GROUPS, int STAGES, int FMT, int CT, int CM, int DYN>
 __global__ void __launch_bounds__((BcsrProducers<B, GROUPS, STAGES, FMT == 3 ? 1 : (FMT == 2 ? 4 : 2), DYN>::kThreads), 1)
 bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -461,6 +483,21 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                         for (int j = 0; j < W; ++j) v[j] = 0u;
                     }
+                    int32_t crow = static_cast<int32_t>(row0) + c0;
+                    if constexpr (H != B) crow = __shfl_sync(0xffffffffu, member, c0 / B) * B + (c0 % B);
+                    if constexpr (H != B && FMT == 2) {
+                        bool nan = false;
+#pragma unroll
+                        for (int j = 0; j < W; ++j) nan |= __uint_as_float(v[j]) != __uint_as_float(v[j]);
+                        if (__any_sync(0xffffffffu, nan)) {
+#pragma unroll
+                            for (int j = 0; j < W; ++j)
+                                if (__uint_as_float(v[j]) != __uint_as_float(v[j]) && crow + j < p.m && nw + lane < N)
+                                    v[j] = __float_as_uint(plain_product<B, CM>(p.block_row_ptr, p.plain_col_idx, p.plain_vals, p.B, p.k, N,
+                                                                               crow + j, nw + lane));
+                            __syncwarp();
+                        }
+                    }
                     // registers -> the next tile of this warp's staging ring -> one TMA store.  The
                     // store that used this tile kEpiBufs chunks ago must have read it first.
                     const uint32_t stg = stg0 + (chunk % Cfg::kEpiBufs) * Cfg::kEpiTileBytes;
@@ -506,8 +543,6 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
-                    int32_t crow = static_cast<int32_t>(row0) + c0;
-                    if constexpr (H != B) crow = __shfl_sync(0xffffffffu, member, c0 / B) * B + (c0 % B);
                     if (lane == 0) {
                         // row-major: box = 32 tokens x W rows at (token, row); column-major: box =
                         // W columns x 32 tokens at (column, token).  Out-of-range parts are clipped.

@@ -42,6 +42,11 @@ struct BcsrParams {
     // tile records then name {group, token tile, first stacked block, end stacked block} and
     // block_col_idx is the stacked blocks' column index
     const int32_t* stack_rows;
+    // TF32 row groups: the format's own blocks and the dense operand (see plain_product in bcsr_kernel.cu)
+    const int32_t* plain_col_idx;
+    const float* plain_vals;
+    const float* B;
+    int64_t k;
     // 0: waits for the launch before it in the stream before it touches an operand (grid_wait).
     // 1: the same, and the next launch may run beside it: it is let go (grid_trigger) after that wait.
     // 2: such a next launch: it may start at once, and waits for the one before it before its CTAs exit

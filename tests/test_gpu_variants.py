@@ -639,3 +639,42 @@ def test_bcsr_tf32_row_groups_and_narrow_tiles(lib, b, col_major, N):
         assert np.array_equal(outs[0], outs[1])
         Cr, S = reference(a, Bs, dtype)
         assert_close(outs[0], Cr, S, dtype, "%s row groups b=%d N=%d" % (dtype, b, N))
+
+
+@pytest.mark.parametrize("b,col_major,N", [(16, False, 256), (16, True, 712), (32, False, 2048), (32, True, 132)])
+def test_bcsr_tf32_row_groups_keep_non_finite_operands_to_their_rows(lib, b, col_major, N):
+    """Row groups multiply absent sub-blocks as zeros, and 0 x Inf is NaN: with TF32 values an Inf or NaN in B
+    must reach the block-rows that store a block in its block column, and no others, as without groups.  Outputs whose
+    own blocks meet only finite operands are compared with the oracle on B with the others set to zero."""
+    m, k = 1992, 1528
+    a = _grouped_matrix(70 + b, m, k, b, "tf32")
+    Bs = wl.dense(702, k, N, ("uniform", -1.0, 1.0), "tf32")
+    rng = np.random.default_rng(703)
+    for value in (np.inf, -np.inf, np.nan):                # scattered entries, one whole row, one whole token
+        Bs[rng.integers(0, k, 40), rng.integers(0, N, 40)] = value
+    Bs[k - 1] = np.inf
+    Bs[:, 5] = np.nan
+    outs = []
+    for fill in (0, -1):
+        h = lib.spmm_bcsr_create_csr(m, k, a["row_ptr"], a["col_idx"], a["vals"], "tf32", b, stack_min_fill=fill,
+                                     layout=lib.COLMAJOR if col_major else lib.ROWMAJOR)
+        try:
+            assert (lib.spmm_get_info(h, N)["n_stacked_rows"] > 0) == (fill == 0)
+            outs.append(run_gpu_variant(lib, h, Bs, m, N, "tf32", col_major=col_major))
+        finally:
+            lib.spmm_destroy(h)
+    finite = np.isfinite(Bs)
+    nbr, nbc = -(-m // b), -(-k // b)
+    stored = np.zeros((nbr, nbc), bool)
+    stored[np.repeat(np.arange(m), np.diff(a["row_ptr"])) // b, a["col_idx"] // b] = True
+    bad = np.zeros((nbc * b, N), bool)
+    bad[:k] = ~finite
+    hit = (stored.astype(np.int32) @ bad.reshape(nbc, b, N).any(1).astype(np.int32)) > 0
+    hit = np.repeat(hit, b, axis=0)[:m]
+    assert hit.any() and not hit.all()
+    for C in outs:
+        assert np.isfinite(C[~hit]).all()
+        assert not np.isfinite(C[hit]).any()               # (a stored block holds a zero times Inf or an Inf of its own)
+    Cr, S = reference(a, np.where(finite, Bs, 0.0).astype(np.float32), "tf32")
+    for C in outs:
+        assert_close(np.where(hit, 0.0, C).astype(np.float32), np.where(hit, 0.0, Cr), S, "tf32", "non-finite B b=%d" % b)
