@@ -106,21 +106,32 @@ typedef enum {
                                     block scheduler; this is the hardware queue itself.       */
 } spmm_sched_t;
 
-/* How the WCSR kernel brings the gathered rows of B into shared memory (opts.gather). */
+/* How a WCSR handle computes C (opts.gather). */
 typedef enum {
-    SPMM_GATHER_TMA = 0,         /* TMA row gather (four rows x 128 bytes per request), the
-                                    default: the indirect load Sec. 3.2 says TMA cannot do is
-                                    available on this architecture                            */
-                                 /* (a WCSR handle whose windows condense almost nothing -- at most
-                                    two nonzeros per padded column; 2- and 4-byte values -- sums C
-                                    row by row from a private copy of the nonzeros instead of
-                                    gathering for window tiles; this option is then without effect,
-                                    and SPMM_TF32 operands are multiplied as full fp32 values)   */
-    SPMM_GATHER_LSU = 1          /* the paper's own scheme (Sec. 3.2): the producer warps copy
+    SPMM_GATHER_AUTO = 0,        /* default.  The window kernel with the TMA gather; or, for handles
+                                    whose windows condense almost nothing, the row kernel, which
+                                    sums C row by row on the CUDA cores from a private copy of the
+                                    nonzeros.  A handle can take the row kernel when its values are
+                                    2 or 4 bytes wide, it holds at most 1.75 nonzeros per padded
+                                    column (nnz / n_units of spmm_get_info) and split_cols and
+                                    n_ctas are left at 0 (both describe the window kernel's plan);
+                                    whether it does depends on N as well (at narrow N up to
+                                    1.75; from N = 64, TF32 128, only up to 1.4 for TF32 and 1.22 for
+                                    2-byte values unless the matrix is small, and not at all for
+                                    large 2-byte matrices at widths that leave lanes idle).
+                                    The two kernels add in different orders (last bits), and the
+                                    row kernel multiplies SPMM_TF32 operands as full fp32 values
+                                    where the tensor core drops their low 13 bits: never less
+                                    exact, but not the same bits at every N.  Ask for
+                                    SPMM_GATHER_TMA to have one kernel, and TF32, at every N.      */
+    SPMM_GATHER_LSU = 1,         /* the paper's own scheme (Sec. 3.2): the producer warps copy
                                     the rows with 128-bit loads through the load/store units
                                     (16-byte cp.async) to the swizzled positions the MMA reads.
                                     Kept for the side-by-side measurement; window height 16,
                                     fp32 C.                                                   */
+    SPMM_GATHER_TMA = 2          /* the window kernel with the TMA row gather (four rows x 128
+                                    bytes per request): the indirect load Sec. 3.2 says TMA cannot
+                                    do is available on this architecture                       */
 } spmm_gather_t;
 
 /* Optional creation parameters; pass NULL for all defaults.  Zero = default. */

@@ -122,11 +122,11 @@ ROWMAJOR, COLMAJOR = 0, 1
 
 
 SCHED_STATIC, SCHED_DYNAMIC = 0, 1
-GATHER_TMA, GATHER_LSU = 0, 1
+GATHER_AUTO, GATHER_LSU, GATHER_TMA = 0, 1, 2
 
 
 def _opts(b_col=0, split_cols=0, host_only=False, n_ctas=0, c_type=C_FP32, layout=ROWMAJOR, schedule=SCHED_STATIC,
-          stack_min_fill=0, gather=GATHER_TMA, k_split=0):
+          stack_min_fill=0, gather=GATHER_AUTO, k_split=0):
     """Keyword options of the create functions -> spmm_opts_t (zero = the library's default; the
     header documents every field).  stack_min_fill: BCSR row groups, 0 = default threshold,
     -1 = off, 1..100 = minimum percentage of stored sub-blocks for a group to be formed."""

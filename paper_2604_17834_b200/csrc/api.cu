@@ -93,6 +93,7 @@ struct spmm_handle_s {
     bool c16 = false;        // C in the input's 16-bit type (never with TF32, whose input type is fp32)
     bool col_major = false;  // BCSR: B given as X[N][k], C as Y[N][m]
     bool dynamic = false;    // BCSR: tiles handed out at run time through Cluster Launch Control
+    bool want_rows = false;  // WCSR: no option asks for the window kernel or describes its plan
     bool lsu_gather = false; // WCSR: B rows gathered by the load/store units (comparison variant) instead of TMA
     int cs = 4;              // bytes per C element
     int n_ctas = 148;
@@ -241,7 +242,7 @@ int check_opts(const spmm_opts_t* opts) {
     if (opts->c_type != SPMM_C_FP32 && opts->c_type != SPMM_C_SAME_AS_INPUT) return SPMM_ERR_INVALID_ARG;
     if (opts->layout != SPMM_ROWMAJOR && opts->layout != SPMM_COLMAJOR) return SPMM_ERR_INVALID_ARG;
     if (opts->schedule != SPMM_SCHED_STATIC && opts->schedule != SPMM_SCHED_DYNAMIC) return SPMM_ERR_INVALID_ARG;
-    if (opts->gather != SPMM_GATHER_TMA && opts->gather != SPMM_GATHER_LSU) return SPMM_ERR_INVALID_ARG;
+    if (opts->gather < SPMM_GATHER_AUTO || opts->gather > SPMM_GATHER_TMA) return SPMM_ERR_INVALID_ARG;
     return SPMM_OK;
 }
 
@@ -464,7 +465,7 @@ int new_wcsr_handle(spmm_handle_s** hp, int64_t m, int64_t k, int dtype, const s
     if (int orc = check_opts(opts)) return orc;
     if (opts && opts->layout == SPMM_COLMAJOR) return SPMM_ERR_UNSUPPORTED;   // BCSR only
     // 8-bit inputs: fp32 C, the TMA gather
-    if (dtype == SPMM_FP8_E4M3 && opts && (opts->c_type != SPMM_C_FP32 || opts->gather != SPMM_GATHER_TMA)) return SPMM_ERR_UNSUPPORTED;
+    if (dtype == SPMM_FP8_E4M3 && opts && (opts->c_type != SPMM_C_FP32 || opts->gather == SPMM_GATHER_LSU)) return SPMM_ERR_UNSUPPORTED;
     if (opts && opts->schedule == SPMM_SCHED_DYNAMIC) return SPMM_ERR_UNSUPPORTED;
     const int es = elem_size(dtype);
     const int b_col_default = 32 / es;
@@ -483,6 +484,7 @@ int new_wcsr_handle(spmm_handle_s** hp, int64_t m, int64_t k, int dtype, const s
     h->c16 = opts && opts->c_type == SPMM_C_SAME_AS_INPUT && dtype != SPMM_TF32;
     h->cs = h->c16 ? 2 : 4;
     h->lsu_gather = opts && opts->gather == SPMM_GATHER_LSU;
+    h->want_rows = !opts || (opts->gather == SPMM_GATHER_AUTO && opts->split_cols <= 0 && opts->n_ctas <= 0);
     if (h->lsu_gather && h->c16) { delete h; return SPMM_ERR_UNSUPPORTED; }   // the comparison variant writes fp32 C
     *hp = h;
     *b_col_out = b_col;
@@ -513,7 +515,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
         if (!rc) rc = upload(&h->d_idx, f.window_col_idx.data(), f.window_col_idx.size() * 4);
         if (!rc) rc = upload(&h->d_vals, f.packed.data(), f.packed.size());
         if (!rc) rc = upload_wcsr_plan(h, nullptr);
-        if (!rc && wcsr_wants_rows(a.es, a.m, a.nnz, f.P)) {
+        if (!rc && h->want_rows && wcsr_wants_rows(a.es, a.m, a.nnz, f.P)) {
             int64_t* d_rp = nullptr;
             int32_t* d_ci = nullptr;
             uint8_t* d_va = nullptr;
@@ -548,7 +550,7 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     try {
         rc = build_wcsr_device(m, k, d_row_ptr, d_col_idx, static_cast<const uint8_t*>(d_vals), h->es, wh, b_col, T,
                                h->n_ctas * wcsr_bins_per_sm(h->es, wh), h->sms, stream, &h->wcsr, &h->nnz, &h->d_ptr, &h->d_idx,
-                               &h->d_vals, &h->d_class, &h->rows);
+                               &h->d_vals, &h->d_class, h->want_rows ? &h->rows : nullptr);
         h->d_grp_class = h->d_class;
         if (!rc) rc = upload_wcsr_plan(h, stream);
         if (!rc) rc = finish_wcsr_rows(&h->rows, stream);

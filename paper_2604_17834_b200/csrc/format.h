@@ -228,7 +228,7 @@ cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_
 // (*d_grp_class, the rule of wcsr_reuse_classes), leaves window_row_ptr, P and distinct_cols in *out
 // (out->window_col_idx, out->packed and out->grp_class stay empty) and runs plan_wcsr.
 // Synchronises `stream` on the way; the last kernels may still be running when it returns.
-// Where the row kernel is to serve the handle (wcsr_wants_rows), *rows is built as well.
+// Where the row kernel is to serve the handle (rows not null and wcsr_wants_rows), *rows is built as well.
 int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
                       int es, int wh, int b_col, int T, int n_bins, int sms, cudaStream_t stream, WcsrHost* out, int64_t* nnz_out,
                       int32_t** d_window_row_ptr, int32_t** d_window_col_idx, uint8_t** d_packed, uint8_t** d_grp_class,

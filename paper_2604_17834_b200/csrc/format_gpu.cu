@@ -708,7 +708,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     }
     release();                                // (ordered behind the kernels that use them)
     int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
-    if (!rc && wcsr_wants_rows(es, m, nnz, P)) rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, st, rows);
+    if (!rc && rows && wcsr_wants_rows(es, m, nnz, P)) rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, st, rows);
     // the split plan needs the window lengths only: the host makes it while the kernels above run
     if (!rc) {
         try {
@@ -718,7 +718,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         }
     }
     if (rc) {
-        free_wcsr_rows(rows, st);
+        if (rows) free_wcsr_rows(rows, st);
         dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st); dev_free(*d_grp_class, st);
         *d_window_row_ptr = nullptr; *d_window_col_idx = nullptr; *d_packed = nullptr; *d_grp_class = nullptr;
     }

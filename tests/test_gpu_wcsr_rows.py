@@ -111,3 +111,45 @@ def test_wcsr_kernel_by_width(lib, dtype, N, expect):
             assert np.array_equal(host, C)
     finally:
         lib.spmm_destroy(h)
+
+
+def _rows_kernel_ran(a, Bs, C):
+    """TF32 handles: the window kernel multiplies what the tensor core keeps of an operand (its low 13 bits dropped),
+    the row kernel the whole value; a row of one entry shows which it was."""
+    one = np.flatnonzero(np.diff(a["row_ptr"]) == 1)[:200]
+    p = a["row_ptr"][one]
+    v, b = a["vals"][p][:, None], Bs[a["col_idx"][p]]
+    cut = [(x.view(np.uint32) & np.uint32(0xffffe000)).view(np.float32) for x in (np.ascontiguousarray(v), np.ascontiguousarray(b))]
+    full, tf32 = np.array_equal(C[one], v * b), np.array_equal(C[one], cut[0] * cut[1])
+    assert one.size > 20 and full != tf32
+    return full
+
+
+@pytest.mark.parametrize("on_gpu", [False, True])
+def test_options_of_the_window_kernel_are_honoured(lib, on_gpu):
+    """A matrix the row kernel takes by default: asking for a gather, a sub-task size or a grid size gets the window
+    kernel, which they describe; the two gathers then agree to the last bit, and so does an explicit default T."""
+    a = wl.wcsr_irregular(seed=31, m=5000, dtype="tf32")
+    N = 128
+    Bs = wl.dense(32, a["k"], N, ("normal", 0.0, 1.0), "tf32")
+    Cr, S = reference(a, Bs, "tf32")
+    dev = [to_device(a[x]) for x in ("row_ptr", "col_idx", "vals")]
+
+    def run(**opt):
+        if on_gpu:
+            h = lib.spmm_wcsr_create_csr_device(a["m"], a["k"], *[d.data_ptr() for d in dev], "tf32", 16, **opt)
+        else:
+            h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], "tf32", 16, **opt)
+        try:
+            C = run_gpu_variant(lib, h, Bs, a["m"], N, "tf32")
+            assert_close(C, Cr, S, "tf32", str(opt))
+            return C, lib.spmm_get_info(h, N)
+        finally:
+            lib.spmm_destroy(h)
+
+    C0, info = run()
+    assert _rows_kernel_ran(a, Bs, C0)
+    outs = [run(**opt)[0] for opt in (dict(gather=lib.GATHER_TMA), dict(gather=lib.GATHER_LSU), dict(split_cols=info["split_cols"]),
+                                      dict(split_cols=64), dict(n_ctas=info["n_ctas"]))]
+    assert not any(_rows_kernel_ran(a, Bs, C) for C in outs)
+    assert all(np.array_equal(outs[0], outs[i]) for i in (1, 2, 4))
