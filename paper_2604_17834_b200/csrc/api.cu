@@ -1016,11 +1016,10 @@ double wcsr_rows_limit(const spmm_handle_s* h, int64_t N) {
     return busy * 4 < all * 3 ? 0.0 : 1.22;
 }
 
-// Whether a run takes the row kernel: the handle has a row stream, it is the faster one, and the wait limit is not
-// zero, the documented hook for the path where a wait runs out, which the window kernel serves (the row kernel waits
-// for nothing).
+// Whether a run takes the row kernel: the handle has a row stream and it is the faster one.  A function of the handle
+// and the dense width alone.
 bool use_rows(const spmm_handle_s* h, int64_t N) {
-    return (h->rows.n_tasks > 0 || h->rows.n_parts > 0) && g_wait_limit_ns.load() != 0 && N * h->es < (int64_t{1} << 32) &&
+    return (h->rows.n_tasks > 0 || h->rows.n_parts > 0) && N * h->es < (int64_t{1} << 32) &&
            static_cast<double>(h->nnz) <= wcsr_rows_limit(h, N) * static_cast<double>(h->wcsr.P);
 }
 
@@ -1053,6 +1052,8 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     p.B = B;
     p.C = C;
     p.N = N;
+    p.status = h->d_status;
+    p.give_up = g_wait_limit_ns.load() == 0 ? 1 : 0;
     p.n_tasks = r.n_tasks;
     p.n_parts = r.n_parts;
     int step = std::min(s.tiles, kRowsMaxTiles);

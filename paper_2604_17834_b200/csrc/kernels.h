@@ -188,6 +188,8 @@ struct WcsrRowsParams {
     const void* B;
     void* C;
     int64_t N;
+    int* status;
+    int32_t give_up;             // the wait limit is zero: leave at once and report a wait that ran out (below)
     int32_t n_tasks, n_parts;
     int32_t lanes, groups, tile0;    // set by launch_wcsr_rows
 };

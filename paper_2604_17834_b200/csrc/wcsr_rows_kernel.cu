@@ -34,6 +34,7 @@ namespace {
 
 constexpr int kWarps = kRowsThreads / 32;
 constexpr int kStrands = 16;            // partial sums of a part: strand = (entry / 8) % kStrands, whatever the dense width
+constexpr int kGiveUpSite = 31;         // in the status word, where other kernels name the wait that ran out
 constexpr int kNoCol = 0x7fffffff;      // an entry without a gather: row without nonzeros, or padding
 
 template <int VB> struct Vec { uint32_t w[VB / 4]; };
@@ -151,6 +152,16 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     __shared__ unsigned arrived;
 
     grid_trigger();
+    // This kernel waits for nothing of its own.  With a wait limit of zero, which makes the kernels that do wait give
+    // up at their first wait, it does what they do: it leaves early and says so.
+    if (p.give_up) {
+        grid_wait();
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && atomicCAS(p.status, 0, 1) == 0) {
+            p.status[1] = kGiveUpSite;
+            p.status[2] = 0;
+        }
+        return;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane / p.lanes, l = lane - g * p.lanes;
     const int tile = p.tile0 + blockIdx.y;

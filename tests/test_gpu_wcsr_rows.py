@@ -7,7 +7,7 @@ import pytest
 
 from paper_2604_17834_b200 import workloads as wl
 
-from helpers import CANARY, GUARD, assert_close, check_guards, reference, run_gpu_variant, to_device
+from helpers import CANARY, GUARD, assert_close, captured_run, check_guards, reference, run_gpu_variant, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -153,3 +153,30 @@ def test_options_of_the_window_kernel_are_honoured(lib, on_gpu):
                                       dict(split_cols=64), dict(n_ctas=info["n_ctas"]))]
     assert not any(_rows_kernel_ran(a, Bs, C) for C in outs)
     assert all(np.array_equal(outs[0], outs[i]) for i in (1, 2, 4))
+
+
+def test_a_wait_limit_of_zero_does_not_change_the_kernel(lib):
+    """The limit is process wide: set between the preparation of a handle and its run it makes the run give up, and
+    must not send it to another kernel with another workspace (a captured run shows that nothing was allocated)."""
+    import torch
+    a = _matrix(3001, 20000, 16, "tf32")
+    N = 128
+    Bs = wl.dense(33, a["k"], N, ("normal", 0.0, 1.0), "tf32")
+    B, C = to_device(Bs), torch.empty((a["m"], N), dtype=torch.float32, device="cuda")
+    h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], "tf32", 16)
+    try:
+        want = run_gpu_variant(lib, h, Bs, a["m"], N, "tf32")
+        assert _rows_kernel_ran(a, Bs, want)
+        lib.spmm_set_wait_limit_ns(0)
+        code, nodes = captured_run(lib, h, B, C, N)
+        assert code == lib.SPMM_OK and nodes == ["kernel"]                   # (the window kernel would be two)
+        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        with pytest.raises(lib.SpmmError) as e:
+            lib.spmm_check(h)
+        assert e.value.code == lib.SPMM_ERR_DEV_TIMEOUT
+        lib.spmm_set_wait_limit_ns(2_000_000_000)
+        assert np.array_equal(run_gpu_variant(lib, h, Bs, a["m"], N, "tf32"), want)
+    finally:
+        lib.spmm_set_wait_limit_ns(2_000_000_000)
+        lib.spmm_destroy(h)
