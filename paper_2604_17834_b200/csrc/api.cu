@@ -1065,14 +1065,18 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     return SPMM_OK;
 }
 
-// What spmm_run wants at a dense width, whatever the alignment of its operands.
+// What a run of the row kernel wants at any dense width up to N, whatever the alignment of its operands: the columns
+// that one launch covers, at most kRowsMaxTiles tiles of 32 lanes, and at most N and the lanes that the last vector and
+// an even cut into tiles leave over.  (The sum itself does not grow with N: 3976 columns take eight tiles of 31 lanes,
+// 4104 nine of 29.)
 size_t rows_workspace_bytes(const spmm_handle_s* h, int64_t N) {
-    size_t most = 0;
-    for (int wide = 0; wide < 2; ++wide) {
-        const RowsShape s = wcsr_rows_shape(N, h->es, wide != 0);
-        most = std::max(most, rows_partial_bytes(h, s, std::min(s.tiles, kRowsMaxTiles)));
-    }
-    return most;
+    const int64_t ve = 32 / h->es;
+    return static_cast<size_t>(h->rows.n_slots) * 4 * static_cast<size_t>(std::min<int64_t>(kRowsMaxTiles * 32 * ve, N + (kRowsMaxTiles + 1) * ve));
+}
+
+// The workspace of a run at dense width N, by the kernel it takes.
+size_t wcsr_run_bytes(const spmm_handle_s* h, int64_t N, bool rows) {
+    return rows ? rows_workspace_bytes(h, N) : static_cast<size_t>(wcsr_workspace_bytes(h, N));
 }
 
 int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, int64_t N, cudaStream_t stream) {
@@ -1126,13 +1130,12 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
     return e == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
 }
 
-// The handle's workspace for the partial tiles of split windows at dense width N (grown, never shrunk).  It outlives
+// The handle's workspace for partial tiles or partial rows (grown, never shrunk).  It outlives
 // the run and serves runs on any stream, so it is never a stream-ordered allocation of the run's own stream -- under
 // stream capture that would be a node of the graph, whose memory exists while the graph runs only.  A run that needs
 // to grow it under capture asks for memory outside the pool instead: refused (SPMM_ERR_ALLOC, nothing launched) in
 // the capture modes that forbid an allocation, lasting in the relaxed one.
-int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, bool rows, cudaStream_t stream) {
-    const size_t need = rows ? rows_workspace_bytes(h, N) : static_cast<size_t>(wcsr_workspace_bytes(h, N));
+int ensure_wcsr_workspace(spmm_handle_s* h, size_t need, cudaStream_t stream) {
     if (need <= h->partial_bytes) return SPMM_OK;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capture) != cudaSuccess) {    // (the legacy stream while a blocking one is captured)
@@ -1159,7 +1162,7 @@ int ensure_wcsr_workspace(spmm_handle_s* h, int64_t N, bool rows, cudaStream_t s
 
 // rows: use_rows for the whole operand of which these are N columns (the kernels add in different orders)
 int run_wcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, bool rows, cudaStream_t stream) {
-    if (int rc = ensure_wcsr_workspace(h, N, rows, stream)) return rc;
+    if (int rc = ensure_wcsr_workspace(h, wcsr_run_bytes(h, N, rows), stream)) return rc;
     if (rows) return launch_wcsr_rows_all(h, B, C, h->d_partial, h->partial_bytes, N, stream);
     return launch_wcsr_all(h, B, C, h->d_partial, N, stream);
 }
@@ -1292,7 +1295,9 @@ int spmm_prepare(spmm_handle_t h, int64_t N) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
     if (dev != h->device) return SPMM_ERR_INVALID_ARG;
-    return ensure_wcsr_workspace(h, N, use_rows(h, N), nullptr);
+    // for every width up to N: a handle with a row stream may take either kernel there
+    const size_t need = std::max(wcsr_run_bytes(h, N, false), wcsr_run_bytes(h, N, true));
+    return ensure_wcsr_workspace(h, need, nullptr);
 }
 
 int spmm_wcsr_run_static(spmm_handle_t h, const void* B_dev, void* C_dev, int64_t N, void* stream) {

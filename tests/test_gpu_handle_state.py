@@ -121,3 +121,45 @@ def test_destroying_a_handle_gives_its_memory_back(lib):
     left = free0 - torch.cuda.mem_get_info()[0]
     assert held > 700 << 20
     assert left <= (256 << 20) + (64 << 20), "%.0f MB still held" % (left / 2 ** 20)       # (64: the pool grows in steps)
+
+
+def _band_with_long_rows(dtype, m=50000, n_long=40):
+    """A band that condenses 1.5 values per padded column -- the row kernel's below 64 (TF32: 128) columns, the window
+    kernel's from there on -- and, far from it, rows of 1200 entries, which both kernels cut into parts."""
+    rng = np.random.default_rng(3)
+    band = np.sort(np.arange(m)[:, None] + rng.permuted(np.tile(np.arange(240), (m, 1)), axis=1)[:, :16], axis=1)
+    k = m + 240
+    cols = [band[i] for i in range(m)]
+    for r in range(n_long):
+        cols[r * 16] = np.sort(rng.choice(k, 1200, replace=False))
+    lens = np.array([c.size for c in cols])
+    rp = np.concatenate(([0], np.cumsum(lens))).astype(np.int64)
+    return {"m": m, "k": k, "row_ptr": rp, "col_idx": np.concatenate(cols).astype(np.int32),
+            "vals": wl.dense(5, 1, int(rp[-1]), ("normal", 0.0, 1.0), dtype).ravel()}
+
+
+@pytest.mark.parametrize("matrix,dtype,N,narrower", [
+    ("band", "fp16", 128, (128, 72, 64, 56, 32, 8)),       # window kernel at N, row kernel below 64
+    ("band", "tf32", 256, (256, 128, 124, 36, 4)),
+    ("long", "fp16", 4104, (4104, 4096, 3976, 1024, 8)),   # nine tiles of 29 lanes need less than eight of 31
+    ("long", "tf32", 2052, (2052, 1988, 96)),
+])
+def test_after_prepare_no_narrower_run_allocates(lib, matrix, dtype, N, narrower):
+    """spmm_prepare(h, N) covers every N' <= N: both kernels, and widths whose workspace is larger than N's own."""
+    import torch
+    a = _band_with_long_rows(dtype) if matrix == "band" else _long_rows(dtype, m=300, k=30000)
+    h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16)
+    try:
+        tdt = torch.float32 if dtype == "tf32" else torch.float16
+        B = torch.zeros((a["k"], N), dtype=tdt, device="cuda")
+        C = torch.empty((a["m"], N), dtype=torch.float32, device="cuda")
+        lib.spmm_prepare(h, N)
+        kernels = []
+        for n in narrower:
+            code, nodes = captured_run(lib, h, B, C, n)
+            assert code == lib.SPMM_OK and nodes and set(nodes) == {"kernel"}, "N' = %d: %s %s" % (n, code, nodes)
+            kernels.append(len(nodes))
+        if (matrix, dtype) == ("band", "fp16"):            # windows are cut: the window kernel is two launches, the row kernel one
+            assert kernels == [2, 2, 2, 1, 1, 1]
+    finally:
+        lib.spmm_destroy(h)
