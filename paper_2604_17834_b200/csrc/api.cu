@@ -28,6 +28,12 @@ struct NvtxRange {
     NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
+// A CUDA call of this library has failed: its error must not be found again by a later call's check of its launches.
+int cuda_error() {
+    cudaGetLastError();
+    return SPMM_ERR_CUDA;
+}
+
 std::atomic<uint64_t> g_wait_limit_ns{2000000000ull};
 
 inline int elem_size(int dtype) { return dtype == SPMM_TF32 ? 4 : (dtype == SPMM_FP8_E4M3 ? 1 : 2); }
@@ -60,7 +66,7 @@ inline CUtensorMapDataType tmap_dtype(int dtype) {
 int encode_2d(CUtensorMap* map, int dtype, const void* base, uint64_t rows, uint64_t cols,
                     uint32_t box_rows, uint32_t box_cols, CUtensorMapSwizzle swz) {
     EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return SPMM_ERR_CUDA;
+    if (!fn) return cuda_error();
     const uint64_t es = static_cast<uint64_t>(elem_size(dtype));
     const cuuint64_t dims[2] = {cols, rows};
     const cuuint64_t strides[1] = {cols * es};
@@ -69,7 +75,7 @@ int encode_2d(CUtensorMap* map, int dtype, const void* base, uint64_t rows, uint
     const CUtensorMapDataType dt = tmap_dtype(dtype);
     CUresult r = fn(map, dt, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                     swz, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? SPMM_OK : SPMM_ERR_CUDA;
+    return r == CUDA_SUCCESS ? SPMM_OK : cuda_error();
 }
 
 // Ready for every stream when it returns (a copy from pageable memory may still be on its way when cudaMemcpy does).
@@ -78,7 +84,7 @@ int upload(T** dptr, const void* src, size_t bytes) {
     *dptr = nullptr;
     if (!dev_alloc_ready_ok(dptr, bytes)) return SPMM_ERR_ALLOC;
     if (bytes && (cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess))
-        return SPMM_ERR_CUDA;
+        return cuda_error();
     return SPMM_OK;
 }
 
@@ -223,17 +229,17 @@ int device_setup(spmm_handle_s* h, const spmm_opts_t* opts, cudaStream_t stream)
         return SPMM_OK;
     }
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return cuda_error();
     int major = 0, sms = 0;
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return SPMM_ERR_CUDA;
+        return cuda_error();
     if (major != 10) return SPMM_ERR_UNSUPPORTED;   // sm_100a code only
     h->device = dev;
     h->sms = sms;
     h->n_ctas = (opts && opts->n_ctas > 0) ? opts->n_ctas : h->sms;
     if (!dev_alloc_ok(&h->d_status, 4 * sizeof(int), stream)) return SPMM_ERR_ALLOC;
-    if (cudaMemsetAsync(h->d_status, 0, 4 * sizeof(int), stream) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (cudaMemsetAsync(h->d_status, 0, 4 * sizeof(int), stream) != cudaSuccess) return cuda_error();
     return SPMM_OK;
 }
 
@@ -433,13 +439,13 @@ int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
     put(o_merge + 2 * nm, f.merge_nparts.data(), nm * 4);
     put(o_class, f.grp_class.data(), f.grp_class.size());
     if (!dev_alloc_ok(&h->d_plan, words * 4, stream)) return SPMM_ERR_ALLOC;
-    if (cudaMemcpyAsync(h->d_plan, w.data(), w.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (cudaMemcpyAsync(h->d_plan, w.data(), w.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess) return cuda_error();
     int32_t* fills = h->d_plan + o_fills;
     int32_t* fills_n = h->d_plan + o_fills_n;
     if (expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill, f.kt, fills, stream) != cudaSuccess ||
         (narrow && expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill_n,
                                      kWcsrNarrowCols, fills_n, stream) != cudaSuccess))
-        return SPMM_ERR_CUDA;
+        return cuda_error();
     h->n_merge = static_cast<int>(nm);
     h->d_tasks = reinterpret_cast<WcsrDevTask*>(h->d_plan + o_tasks);
     h->d_bin_ptr = h->d_plan + o_bin_ptr;
@@ -528,7 +534,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
             dev_free(d_ci, nullptr);
             dev_free(d_va, nullptr);
         }
-        if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = SPMM_ERR_CUDA;
+        if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = cuda_error();
         if (rc) { free_handle(h); return rc; }
         std::vector<uint8_t>().swap(h->wcsr.packed);
     }
@@ -557,7 +563,7 @@ int create_wcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
     } catch (const std::bad_alloc&) {
         rc = SPMM_ERR_ALLOC;
     }
-    if (!rc && cudaStreamSynchronize(stream) != cudaSuccess) rc = SPMM_ERR_CUDA;
+    if (!rc && cudaStreamSynchronize(stream) != cudaSuccess) rc = cuda_error();
     if (rc) { free_handle(h); return rc; }
     *out = h;
     return SPMM_OK;
@@ -581,7 +587,7 @@ int make_view(CsrView* v, int64_t m, int64_t k, const int64_t* row_ptr, const in
 // Map of B for the WCSR row gather: box = one row x 128 bytes.
 int encode_gather_map(CUtensorMap* map, int dtype, const void* base, uint64_t rows, uint64_t cols) {
     EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return SPMM_ERR_CUDA;
+    if (!fn) return cuda_error();
     const uint32_t es = static_cast<uint32_t>(elem_size(dtype));
     const cuuint64_t dims[2] = {cols, rows};
     const cuuint64_t strides[1] = {cols * es};
@@ -592,7 +598,7 @@ int encode_gather_map(CUtensorMap* map, int dtype, const void* base, uint64_t ro
     const CUtensorMapL2promotion promo = cols * es >= 128 ? CU_TENSOR_MAP_L2_PROMOTION_L2_128B : CU_TENSOR_MAP_L2_PROMOTION_NONE;
     CUresult r = fn(map, dt, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                     promo, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? SPMM_OK : SPMM_ERR_CUDA;
+    return r == CUDA_SUCCESS ? SPMM_OK : cuda_error();
 }
 
 int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
@@ -667,7 +673,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
 int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
     if (h->tmC_ptr == C && h->tmC_N == N) return SPMM_OK;
     EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return SPMM_ERR_CUDA;
+    if (!fn) return cuda_error();
     const uint32_t w = static_cast<uint32_t>(bcsr_epi_cols(h->bcsr.b, h->c16, h->col_major));
     const CUtensorMapDataType dt = !h->c16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : (h->dtype == SPMM_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16);
@@ -687,10 +693,22 @@ int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
         r = fn(&h->tmC, dt, 2, C, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
-    if (r != CUDA_SUCCESS) return SPMM_ERR_CUDA;
+    if (r != CUDA_SUCCESS) return cuda_error();
     h->tmC_ptr = C;
     h->tmC_N = N;
     return SPMM_OK;
+}
+
+// Gives the device arrays of the schedule back; no run may be using them.
+void drop_schedule(spmm_handle_s* h) {
+    int32_t** const arrays[] = {&h->d_tiles, &h->d_tile_recs, &h->d_rec_ptr, &h->d_cta_ptr, &h->d_stile_recs, &h->d_scta_ptr, &h->d_kmerge};
+    for (int32_t** a : arrays) {
+        dev_free(*a, nullptr);
+        *a = nullptr;
+    }
+    h->n_kmerge = 0;
+    h->tmP_ok = false;
+    h->sched.N = -1;
 }
 
 // Tile width, slab width and the tile schedule for dense width N (cached for the last N).
@@ -813,17 +831,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     sc.N = N;
     if (!h->host_only) {
         if (h->d_tiles) {   // a previous schedule may still be in use by a running kernel
-            if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
-            dev_free(h->d_tiles, nullptr);
-            dev_free(h->d_tile_recs, nullptr);
-            dev_free(h->d_rec_ptr, nullptr);
-            dev_free(h->d_cta_ptr, nullptr);
-            dev_free(h->d_stile_recs, nullptr);
-            dev_free(h->d_scta_ptr, nullptr);
-            dev_free(h->d_kmerge, nullptr);
-            h->d_tiles = h->d_tile_recs = h->d_rec_ptr = h->d_cta_ptr = h->d_stile_recs = h->d_scta_ptr = h->d_kmerge = nullptr;
-            h->n_kmerge = 0;
-            h->tmP_ok = false;
+            if (cudaDeviceSynchronize() != cudaSuccess) return cuda_error();
+            drop_schedule(h);
         }
         rc = upload(&h->d_tiles, sc.tiles.data(), sc.tiles.size() * 4);
         if (!rc) {
@@ -869,10 +878,12 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             rc = upload(&h->d_kmerge, mg.data(), mg.size() * 4);
             const size_t need = static_cast<size_t>(sc.n_slots) * f.b * static_cast<size_t>(N) * 4;
             if (!rc && need > h->partial_bytes) {
-                if (h->d_partial && cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
-                free_partial(h);
-                if (!dev_alloc_ready_ok(&h->d_partial, need)) rc = SPMM_ERR_ALLOC;
-                else h->partial_bytes = need;
+                if (h->d_partial) {
+                    if (cudaDeviceSynchronize() != cudaSuccess) rc = cuda_error();
+                    else free_partial(h);
+                }
+                if (!rc && !dev_alloc_ready_ok(&h->d_partial, need)) rc = SPMM_ERR_ALLOC;
+                if (!rc) h->partial_bytes = need;
             }
             if (!rc) {
                 EncodeTiledFn fn = get_encode_fn();
@@ -883,7 +894,7 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                 if (!fn || fn(&h->tmP, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->d_partial, dims, strides, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-                    rc = SPMM_ERR_CUDA;
+                    rc = cuda_error();
                 else
                     h->tmP_ok = true;
             }
@@ -903,7 +914,10 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             rc = upload(&h->d_stile_recs, recs.data(), recs.size() * 4);
             if (!rc) rc = upload(&h->d_scta_ptr, run.cta_ptr.data(), run.cta_ptr.size() * 4);
         }
-        if (rc) return rc;
+        if (rc) {
+            drop_schedule(h);            // the handle holds no schedule rather than half of one
+            return rc;
+        }
     }
     h->stack_groups = ss.tiles.empty() ? 0 : (narrow ? 1 : kStackGroups);
     h->tmB_N = -1;                   // (the stacked launch's map of B depends on its tile)
@@ -963,7 +977,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         p.overlap = 2;
         cudaError_t es = launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
                                              h->n_ctas, stream);
-        if (es != cudaSuccess) return SPMM_ERR_CUDA;
+        if (es != cudaSuccess) return cuda_error();
         if (h->sched.tiles.empty()) return SPMM_OK;
     }
     // dynamic: one CTA per tile, the schedule was built as a single list in the global order
@@ -973,7 +987,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     if (ksplit) p.overlap = 1;          // the merge kernel's CTAs may be placed while this grid runs
     cudaError_t e = launch_bcsr(h->dtype, f.b, h->sched.groups, h->c16, h->col_major, h->dynamic, tmA, h->tmB, h->tmB3,
                                 h->tmC, ksplit ? h->tmP : h->tmC, p, grid, stream);
-    if (e != cudaSuccess) return SPMM_ERR_CUDA;
+    if (e != cudaSuccess) return cuda_error();
     if (ksplit) {
         BcsrMergeParams mp;
         mp.row = h->d_kmerge;
@@ -985,7 +999,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         mp.N = N;
         mp.n = h->n_kmerge;
         mp.b = f.b;
-        if (launch_bcsr_merge(mp, stream) != cudaSuccess) return SPMM_ERR_CUDA;
+        if (launch_bcsr_merge(mp, stream) != cudaSuccess) return cuda_error();
     }
     return SPMM_OK;
 }
@@ -1061,7 +1075,7 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     if (rows_partial_bytes(h, s, step) > cap) return SPMM_ERR_TOO_LARGE;
     for (int t = 0; t < s.tiles; t += step)
         if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), stream) != cudaSuccess)
-            return SPMM_ERR_CUDA;
+            return cuda_error();
     return SPMM_OK;
 }
 
@@ -1115,7 +1129,7 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
         int rc = ensure_tmB(h, B, N, 1);
         if (rc) return rc;
         cudaError_t e = launch_wcsr(h->dtype, f.wh, h->c16, narrow ? 1 : 0, h->lsu_gather ? 1 : 0, h->tmB, p, h->sms, stream);
-        if (e != cudaSuccess) return SPMM_ERR_CUDA;
+        if (e != cudaSuccess) return cuda_error();
     }
     MergeParams mp;
     mp.window = h->d_merge;
@@ -1127,7 +1141,7 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
     mp.N = N;
     mp.n = h->n_merge;
     cudaError_t e = launch_wcsr_merge(mp, f.wh, h->c16 ? (h->dtype == SPMM_FP16 ? 1 : 2) : 0, stream);
-    return e == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
+    return e == cudaSuccess ? SPMM_OK : cuda_error();
 }
 
 // The handle's workspace for partial tiles or partial rows (grown, never shrunk).  It outlives
@@ -1143,7 +1157,7 @@ int ensure_wcsr_workspace(spmm_handle_s* h, size_t need, cudaStream_t stream) {
         capture = cudaStreamCaptureStatusActive;
     }
     if (h->d_partial) {
-        if (cudaDeviceSynchronize() != cudaSuccess) return SPMM_ERR_CUDA;
+        if (cudaDeviceSynchronize() != cudaSuccess) return cuda_error();
         free_partial(h);
     }
     if (capture == cudaStreamCaptureStatusNone) {
@@ -1172,7 +1186,7 @@ int check_run_args(spmm_handle_s* h, const void* B, const void* C, int64_t N) {
     if (h->host_only) return SPMM_ERR_HOST_ONLY;
     // the handle's arrays, tensor maps and kernel attributes belong to the device it was created on
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return cuda_error();
     if (dev != h->device) return SPMM_ERR_INVALID_ARG;
     // row-major B and C have N elements per row: rows must stay 16-byte aligned (column-major
     // operands have k and m elements per row, checked at creation)
@@ -1293,7 +1307,7 @@ int spmm_prepare(spmm_handle_t h, int64_t N) {
     if (N >= (int64_t{1} << 31)) return SPMM_ERR_TOO_LARGE;
     if (h->host_only) return SPMM_OK;
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (cudaGetDevice(&dev) != cudaSuccess) return cuda_error();
     if (dev != h->device) return SPMM_ERR_INVALID_ARG;
     // for every width up to N: a handle with a row stream may take either kernel there
     const size_t need = std::max(wcsr_run_bytes(h, N, false), wcsr_run_bytes(h, N, true));
@@ -1307,7 +1321,7 @@ int spmm_wcsr_run_static(spmm_handle_t h, const void* B_dev, void* C_dev, int64_
     if (h->format != 1) return SPMM_ERR_INVALID_ARG;
     float* scratch = nullptr;
     size_t cap = 0;
-    if (wcsr_static_scratch(&scratch, &cap) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (wcsr_static_scratch(&scratch, &cap) != cudaSuccess) return cuda_error();
     if (static_cast<size_t>(wcsr_workspace_bytes(h, N)) > cap) return SPMM_ERR_TOO_LARGE;
     if (use_rows(h, N) && rows_partial_bytes(h, rows_shape(h, B_dev, C_dev, N), 1) <= cap)
         return launch_wcsr_rows_all(h, B_dev, C_dev, scratch, cap, N, static_cast<cudaStream_t>(stream));
@@ -1320,7 +1334,7 @@ int spmm_run_host(spmm_handle_t h, const void* B_host, void* C_host, int64_t N, 
     if (h->host_only) return SPMM_ERR_HOST_ONLY;
     {
         int dev = -1;
-        if (cudaGetDevice(&dev) != cudaSuccess) return SPMM_ERR_CUDA;
+        if (cudaGetDevice(&dev) != cudaSuccess) return cuda_error();
         if (dev != h->device) return SPMM_ERR_INVALID_ARG;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1358,22 +1372,22 @@ int spmm_run_host(spmm_handle_t h, const void* B_host, void* C_host, int64_t N, 
         }
     }
     if (nchunks == 1) {
-        if (cudaMemcpyAsync(h->d_Bstage, B_host, bbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return SPMM_ERR_CUDA;
+        if (cudaMemcpyAsync(h->d_Bstage, B_host, bbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return cuda_error();
         int rc = spmm_run(h, h->d_Bstage, h->d_Cstage, N, stream);
         if (rc) return rc;
-        if (cudaMemcpyAsync(C_host, h->d_Cstage, cbytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) return SPMM_ERR_CUDA;
-        if (cudaStreamSynchronize(st) != cudaSuccess) return SPMM_ERR_CUDA;
+        if (cudaMemcpyAsync(C_host, h->d_Cstage, cbytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) return cuda_error();
+        if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_error();
         return SPMM_OK;
     }
     if (!h->s_in) {
         if (cudaStreamCreateWithFlags(&h->s_in, cudaStreamNonBlocking) != cudaSuccess ||
             cudaStreamCreateWithFlags(&h->s_out, cudaStreamNonBlocking) != cudaSuccess ||
             cudaEventCreateWithFlags(&h->ev_start, cudaEventDisableTiming) != cudaSuccess)
-            return SPMM_ERR_CUDA;
+            return cuda_error();
         for (int i = 0; i < spmm_handle_s::kMaxHostChunks; ++i)
             if (cudaEventCreateWithFlags(&h->ev_in[i], cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreateWithFlags(&h->ev_run[i], cudaEventDisableTiming) != cudaSuccess)
-                return SPMM_ERR_CUDA;
+                return cuda_error();
     }
     const int64_t nc = N / nchunks;
     const bool rows = h->format == 1 && use_rows(h, N);
@@ -1414,14 +1428,14 @@ int spmm_run_host(spmm_handle_t h, const void* B_host, void* C_host, int64_t N, 
     const bool s2 = cudaStreamSynchronize(st) == cudaSuccess;
     const bool s3 = cudaStreamSynchronize(h->s_out) == cudaSuccess;
     if (rc) return rc;
-    return (bad || !s1 || !s2 || !s3) ? SPMM_ERR_CUDA : SPMM_OK;
+    return (bad || !s1 || !s2 || !s3) ? cuda_error() : SPMM_OK;
 }
 
 int spmm_check(spmm_handle_t h) {
     if (!h) return SPMM_ERR_INVALID_ARG;
     if (h->host_only) return SPMM_ERR_HOST_ONLY;
     int st[4] = {0, 0, 0, 0};
-    if (cudaMemcpy(st, h->d_status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return SPMM_ERR_CUDA;
+    if (cudaMemcpy(st, h->d_status, sizeof(st), cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_error();
     if (st[0] != 0) {
         cudaMemset(h->d_status, 0, sizeof(st));
         cudaStreamSynchronize(nullptr);          // (the next run may come on a stream that does not wait for this one)
@@ -1557,7 +1571,7 @@ int spmm_export(spmm_handle_t h, int which, void* host_dst, size_t cap, size_t* 
         const uint8_t* packed = f.packed.data();
         if (!h->host_only) {
             packed_dl.resize(bytes);
-            if (cudaMemcpy(packed_dl.data(), h->d_vals, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return SPMM_ERR_CUDA;
+            if (cudaMemcpy(packed_dl.data(), h->d_vals, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_error();
             packed = packed_dl.data();
         }
         uint8_t* dst = static_cast<uint8_t*>(host_dst);
@@ -1579,7 +1593,7 @@ int spmm_export(spmm_handle_t h, int which, void* host_dst, size_t cap, size_t* 
             }
         } else {
             std::vector<WcsrDevTask> dt(f.tasks.size());
-            if (cudaMemcpy(dt.data(), h->d_tasks, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return SPMM_ERR_CUDA;
+            if (cudaMemcpy(dt.data(), h->d_tasks, bytes, cudaMemcpyDeviceToHost) != cudaSuccess) return cuda_error();
             for (size_t i = 0; i < dt.size(); ++i) {
                 dst[4 * i + 0] = dt[i].window;
                 dst[4 * i + 1] = dt[i].col_begin - f.window_row_ptr[dt[i].window];
@@ -1593,7 +1607,7 @@ int spmm_export(spmm_handle_t h, int which, void* host_dst, size_t cap, size_t* 
         std::memcpy(host_dst, host_src, bytes);
         return SPMM_OK;
     }
-    return cudaMemcpy(host_dst, dev_src, bytes, cudaMemcpyDeviceToHost) == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA;
+    return cudaMemcpy(host_dst, dev_src, bytes, cudaMemcpyDeviceToHost) == cudaSuccess ? SPMM_OK : cuda_error();
 }
 
 int spmm_destroy(spmm_handle_t h) {

@@ -286,6 +286,7 @@ int stack_bcsr_device(const uint8_t* d_blocks, const BcsrStack& st, int b, int e
                                                                    reinterpret_cast<uint4*>(*d_stacked), st.R, pieces, n_pieces);
         if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) rc = SPMM_ERR_CUDA;
     }
+    if (rc) cudaGetLastError();
     dev_free(d_src, nullptr);
     if (rc) { dev_free(*d_stacked, nullptr); *d_stacked = nullptr; }
     return rc;
@@ -311,6 +312,7 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     int* d_flags = nullptr;                     // [0] CSR error code (min), [1] scan overflow, [2] a bad entry
     int32_t* d_counts = nullptr;
     auto fail = [&](int code) {
+        cudaGetLastError();                  // (of a call that failed: not for a later check to find)
         dev_free(d_flags, st);
         dev_free(d_counts, st);
         dev_free(*d_block_row_ptr, st);
@@ -562,6 +564,7 @@ int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, int64_
     }
     dev_free(block, st);
     if (!ok) {
+        cudaGetLastError();
         dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
         return SPMM_ERR_CUDA;
@@ -609,6 +612,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     uint8_t* d_work = nullptr;                // keys, sorted keys, rows of the entries, window lengths and starts, column marks, CUB's
     auto release = [&]() { dev_free(d_flags, st); dev_free(d_work, st); };
     auto fail = [&](int code) {
+        cudaGetLastError();                  // (of a call that failed: not for a later check to find)
         release();
         dev_free(*d_window_row_ptr, st); dev_free(*d_window_col_idx, st); dev_free(*d_packed, st);
         *d_window_row_ptr = nullptr; *d_window_col_idx = nullptr; *d_packed = nullptr;
@@ -950,6 +954,7 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     int4 *d_size = nullptr, *d_start = nullptr;
     void* d_temp = nullptr;
     auto done = [&](int code) {
+        if (code) cudaGetLastError();
         void* const arrays[] = {d_cls, d_cls2, d_ids, d_counts, d_head, d_size, d_start, d_temp};
         for (void* ptr : arrays) dev_free(ptr, st);
         if (code) free_wcsr_rows(out, st);

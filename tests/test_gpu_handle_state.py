@@ -163,3 +163,43 @@ def test_after_prepare_no_narrower_run_allocates(lib, matrix, dtype, N, narrower
             assert kernels == [2, 2, 2, 1, 1, 1]
     finally:
         lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["bcsr", "bcsr_ksplit", "wcsr"])
+def test_a_refused_run_leaves_nothing_behind(lib, kind):
+    """A width that was not prepared is refused under capture, whatever the handle holds already; the prepared width,
+    new handles and new widths then work (no error of the refused call is found by a later one)."""
+    import torch
+    dtype = "fp16"
+
+    def make():
+        if kind == "wcsr":
+            a = _long_rows(dtype, seed=6)
+            return a, lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16)
+        a = wl.bcsr_sweep(93, m=1024, k=1024, b=64, density=0.05, dtype=dtype)
+        return a, lib.spmm_bcsr_create_csr(1024, 1024, a["row_ptr"], a["col_idx"], a["vals"], dtype, 64, k_split=1 if kind == "bcsr_ksplit" else 0)
+
+    def product(h, a, N):
+        Bs = wl.dense(95, a["k"], N, ("normal", 0.0, 1.0), dtype)
+        C = run_gpu(lib, h, Bs, a["m"], N)
+        assert_close(C, *reference(a, Bs, dtype), dtype, "%s N=%d" % (kind, N))
+        return C
+
+    a, h = make()
+    try:
+        first = product(h, a, 64)
+        B = torch.zeros((a["k"], 512), dtype=torch.float16, device="cuda")
+        C = torch.empty((a["m"], 512), dtype=torch.float32, device="cuda")
+        code, nodes = captured_run(lib, h, B, C, 512)
+        assert code in (lib.SPMM_ERR_ALLOC, lib.SPMM_ERR_CUDA) and nodes is None
+        a2, h2 = make()
+        try:
+            code, _ = captured_run(lib, h2, B, C, 512)          # a handle that holds nothing yet
+            assert code in (lib.SPMM_ERR_ALLOC, lib.SPMM_ERR_CUDA)
+            assert np.array_equal(product(h2, a2, 64), first)
+        finally:
+            lib.spmm_destroy(h2)
+        assert np.array_equal(product(h, a, 64), first)
+        product(h, a, 512)
+    finally:
+        lib.spmm_destroy(h)
