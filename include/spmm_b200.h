@@ -371,13 +371,13 @@ int spmm_run(spmm_handle_t h, const void *B_dev, void *C_dev, int64_t N, void *s
  * call: code that runs inside a framework whose memory pool already owns the device, or a
  * latency-critical loop that cannot afford the device-wide synchronisation an allocation
  * or a free can cause.
- *   - The partial tiles need n_slots * window_height * N * 4 bytes (spmm_get_info:
- *     workspace_bytes; a 64-row handle needs four times what a 16-row one does).  More than
- *     8 MiB returns SPMM_ERR_TOO_LARGE and nothing is launched; choose a larger split_cols at
- *     creation, a smaller N, or use spmm_run.
+ *   - The window kernel's partial tiles need n_slots * window_height * N * 4 bytes (n_slots of
+ *     spmm_get_info; a 64-row handle needs four times what a 16-row one does).  More than
+ *     8 MiB returns SPMM_ERR_TOO_LARGE and nothing is launched, whichever kernel spmm_run takes
+ *     at this N; choose a larger split_cols at creation, a smaller N, or use spmm_run.
  *   - The first call on each device looks up the scratch array's device address, and the
  *     first launch of each kernel variant (value type, window height, C type, N <= 64 or
- *     wider) on a device sets that kernel's attributes and may load its code.  Make one
+ *     wider; row kernel: operands aligned to 32 bytes with such rows, or not) on a device sets that kernel's attributes and may load its code.  Make one
  *     warm-up call per handle type and N class outside any stream capture and outside the
  *     loop that must not stall.  Later calls only launch kernels.
  *   - The array is shared by all handles and all calls and keeps the previous call's

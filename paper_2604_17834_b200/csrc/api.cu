@@ -1048,11 +1048,19 @@ RowsShape rows_shape(const spmm_handle_s* h, const void* B, const void* C, int64
     return wcsr_rows_shape(N, h->es, aligned32);
 }
 
-// partial: room for cap bytes of partial rows, one column tile's at least; the column tiles go in as few
-// launches as that and the counters allow.
+// partial: room for cap bytes of partial rows; the column tiles go in as few launches as that and the counters allow,
+// and are made narrower where it does not hold one (sums do not depend on the cut).  A tile of one vector takes
+// kRowsMaxSlots * 32 bytes at most, which the built-in scratch holds.
 int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partial, size_t cap, int64_t N, cudaStream_t stream) {
     const WcsrRowStream& r = h->rows;
-    const RowsShape s = rows_shape(h, B, C, N);
+    RowsShape s = rows_shape(h, B, C, N);
+    if (rows_partial_bytes(h, s, 1) > cap) {
+        const int64_t ve = s.vec / h->es, lanes = static_cast<int64_t>(cap / 4) / (static_cast<int64_t>(r.n_slots) * ve);
+        if (lanes < 1) return SPMM_ERR_TOO_LARGE;
+        s.lanes = static_cast<int>(std::min<int64_t>(lanes, s.lanes));
+        s.tiles = static_cast<int>((N + s.lanes * ve - 1) / (s.lanes * ve));
+        s.tile_cols = static_cast<int>(s.lanes * ve);
+    }
     WcsrRowsParams p;
     p.tasks = reinterpret_cast<const int4*>(r.d_tasks);
     p.parts = reinterpret_cast<const int4*>(r.d_parts);
@@ -1072,7 +1080,6 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     p.n_parts = r.n_parts;
     int step = std::min(s.tiles, kRowsMaxTiles);
     while (step > 1 && rows_partial_bytes(h, s, step) > cap) --step;
-    if (rows_partial_bytes(h, s, step) > cap) return SPMM_ERR_TOO_LARGE;
     for (int t = 0; t < s.tiles; t += step)
         if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), stream) != cudaSuccess)
             return cuda_error();
@@ -1323,7 +1330,7 @@ int spmm_wcsr_run_static(spmm_handle_t h, const void* B_dev, void* C_dev, int64_
     size_t cap = 0;
     if (wcsr_static_scratch(&scratch, &cap) != cudaSuccess) return cuda_error();
     if (static_cast<size_t>(wcsr_workspace_bytes(h, N)) > cap) return SPMM_ERR_TOO_LARGE;
-    if (use_rows(h, N) && rows_partial_bytes(h, rows_shape(h, B_dev, C_dev, N), 1) <= cap)
+    if (use_rows(h, N))
         return launch_wcsr_rows_all(h, B_dev, C_dev, scratch, cap, N, static_cast<cudaStream_t>(stream));
     return launch_wcsr_all(h, B_dev, C_dev, scratch, N, static_cast<cudaStream_t>(stream));
 }

@@ -180,3 +180,35 @@ def test_a_wait_limit_of_zero_does_not_change_the_kernel(lib):
     finally:
         lib.spmm_set_wait_limit_ns(2_000_000_000)
         lib.spmm_destroy(h)
+
+
+def test_static_run_takes_the_kernel_of_spmm_run(lib):
+    """Partial rows of more than the built-in scratch holds (14,208 of 160 columns, 9.1 MB): the static run goes
+    through it in narrower column tiles instead of taking another kernel, and stays bitwise equal to spmm_run."""
+    import torch
+    m, n, k, N, dtype = 7104, 1100, 400000, 160, "fp16"
+    g = torch.Generator(device="cuda").manual_seed(7)
+    step = k // n
+    start = torch.randint(0, step, (m, 1), generator=g, device="cuda")
+    ci = (torch.arange(n, device="cuda")[None, :] * step + start).to(torch.int32).contiguous()
+    rp = torch.arange(m + 1, device="cuda", dtype=torch.int64) * n
+    va = torch.randn(m * n, generator=g, device="cuda").to(torch.float16)
+    B = torch.randn((k, N), generator=g, device="cuda").to(torch.float16)
+    h = lib.spmm_wcsr_create_csr_device(m, k, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), dtype, 16)
+    try:
+        info = lib.spmm_get_info(h, N)
+        assert info["n_slots"] * 16 * N * 4 <= 8 << 20 and info["nnz"] * 16 <= 1.2 * info["stored_values"]
+        st = torch.cuda.current_stream().cuda_stream
+        want, got = (torch.full((m, N), float("nan"), device="cuda") for _ in range(2))
+        lib.spmm_run(h, B.data_ptr(), want.data_ptr(), N, st)
+        for _ in range(2):
+            lib.spmm_wcsr_run_static(h, B.data_ptr(), got.data_ptr(), N, st)
+            torch.cuda.synchronize()
+            lib.spmm_check(h)
+            assert torch.equal(got, want)
+        a = {"row_ptr": rp.cpu().numpy(), "col_idx": ci.cpu().numpy().ravel(), "vals": va.cpu().numpy()}
+        cols = np.array([0, 7, 8, 143, 144, 159])
+        Cr, S = reference(a, B.cpu().numpy(), dtype, cols=cols)
+        assert_close(want[:, torch.from_numpy(cols).cuda()].cpu().numpy(), Cr, S, dtype, "long rows")
+    finally:
+        lib.spmm_destroy(h)
