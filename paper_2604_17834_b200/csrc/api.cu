@@ -533,6 +533,10 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
             dev_free(d_rp, nullptr);
             dev_free(d_ci, nullptr);
             dev_free(d_va, nullptr);
+            if (rc == SPMM_ERR_ALLOC) {          // no room for the row stream: the window kernel serves the handle
+                free_wcsr_rows(&h->rows, nullptr);
+                rc = SPMM_OK;
+            }
         }
         if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = cuda_error();
         if (rc) { free_handle(h); return rc; }

@@ -712,7 +712,10 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     }
     release();                                // (ordered behind the kernels that use them)
     int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
-    if (!rc && rows && wcsr_wants_rows(es, m, nnz, P)) rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, st, rows);
+    if (!rc && rows && wcsr_wants_rows(es, m, nnz, P)) {
+        rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, st, rows);
+        if (rc == SPMM_ERR_ALLOC) rc = SPMM_OK;          // no room for it: the window kernel serves the handle
+    }
     // the split plan needs the window lengths only: the host makes it while the kernels above run
     if (!rc) {
         try {

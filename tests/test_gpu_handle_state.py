@@ -203,3 +203,66 @@ def test_a_refused_run_leaves_nothing_behind(lib, kind):
         product(h, a, 512)
     finally:
         lib.spmm_destroy(h)
+
+
+_SCARCE = r"""
+import sys
+import numpy as np, torch
+sys.path[:0] = [".", "tests"]
+from paper_2604_17834_b200 import binding as lib, workloads as wl
+from helpers import assert_close, reference
+left = int(sys.argv[1])
+m = k = 500000
+n, N, dtype = 16, 8, "fp16"
+step = k // n
+start = np.random.default_rng(1).integers(0, step, (m, 1))
+ci = (np.arange(n, dtype=np.int64)[None, :] * step + start).astype(np.int32).ravel()
+rp = np.arange(m + 1, dtype=np.int64) * n
+va = wl.dense(2, 1, m * n, ("normal", 0.0, 1.0), dtype).ravel()
+Bs = wl.dense(3, k, N, ("normal", 0.0, 1.0), dtype)
+B, C = torch.from_numpy(Bs).cuda(), torch.full((m, N), float("nan"), device="cuda")
+def make(rp, ci, va, m, **opt):
+    return lib.spmm_wcsr_create_csr(m, k, rp, ci, va, dtype, 16, **opt)
+st = torch.cuda.current_stream().cuda_stream
+small = (rp[:65], ci[:1024], va[:1024])
+for opt in ({}, dict(gather=lib.GATHER_TMA)):                      # loads the kernels
+    h = make(*small, 64, **opt)
+    lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, st)
+    torch.cuda.synchronize()
+    lib.spmm_destroy(h)
+free = torch.cuda.mem_get_info()[0]
+if left < 0:
+    h = make(rp, ci, va, m, gather=lib.GATHER_TMA)
+    print("window", free - torch.cuda.mem_get_info()[0])
+    h2 = make(rp, ci, va, m)
+    print("both", free - torch.cuda.mem_get_info()[0])
+else:
+    hog = torch.empty(free - left, dtype=torch.uint8, device="cuda")
+    h = make(rp, ci, va, m)
+    lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, st)
+    torch.cuda.synchronize()
+    lib.spmm_check(h)
+    Cr, S = reference(dict(row_ptr=rp, col_idx=ci, vals=va), Bs, dtype)
+    assert_close(C.cpu().numpy(), Cr, S, dtype, "without a row stream")
+    print("ran")
+"""
+
+
+def test_a_handle_does_without_its_row_stream_where_memory_is_short(lib):
+    """The private copy of the nonzeros only makes runs faster: where the format's own arrays fit and it does not,
+    the handle is created all the same and the window kernel serves it.  (In processes of their own, whose memory
+    is filled up to the window handle's need and a little more.)"""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+    def child(left):
+        r = subprocess.run([sys.executable, "-c", _SCARCE, str(left)], cwd=root, capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout[-500:] + r.stderr[-1500:]
+        return r.stdout.split()
+
+    said = child(-1)
+    window, both = int(said[1]), int(said[3])
+    assert both > 2 * window + (64 << 20)
+    assert child(window + (56 << 20)) == ["ran"]
