@@ -149,7 +149,7 @@ struct WcsrHost {
 //   entries    {column | sign bit on a row's last entry, value}; task t starts at the first multiple of
 //              four from (entries of the tasks before it) + 3 t on; padding and empty rows have column
 //              0x7fffffff.
-//   long rows  after the tasks' entries, each starting on a multiple of eight, no sign bits, cut into
+//   long rows  behind the last task's entries, each starting on a multiple of eight, no sign bits, cut into
 //              parts of part_len entries (one CTA each).
 struct WcsrRowStream {
     int pack = 0, task_max = 0, part_len = 0;

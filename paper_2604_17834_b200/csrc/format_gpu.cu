@@ -791,7 +791,7 @@ __global__ void rows_size_kernel(int64_t m, const int32_t* __restrict__ order, c
 // packed rows.
 struct RowsPlan {
     int64_t m;
-    int pack, part_len, long_base;       // long_base: the long rows' first entry
+    int pack, part_len;
     const int32_t* counts;
     const int4* start;                   // exclusive sums of rows_size_kernel's fields
     int n_classes;
@@ -807,6 +807,9 @@ struct RowsPlan {
         return i < p0 ? static_cast<int>(i) - nl : ns + (start[i].x - start[p0].x) / pack;
     }
     __device__ __forceinline__ int begin(int task, int first_entry) const { return (first_entry + 3 * task + 3) / 4 * 4; }
+    __device__ __forceinline__ int n_tasks(int nl, int ns) const { return nl < m ? task(m - 1, nl, ns) + 1 : 0; }
+    // the long rows' first entry: behind the last task
+    __device__ __forceinline__ int long_base(int nl, int ns) const { return (begin(n_tasks(nl, ns), start[m].x) + 7) / 8 * 8; }
 };
 
 // task heads; descriptors of the long rows and their parts; totals {tasks, parts, long rows, slots}
@@ -815,7 +818,7 @@ __global__ void rows_plan_kernel(const RowsPlan p, const int32_t* __restrict__ o
     const int nl = p.n_long(), ns = p.n_single();
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i <= p.m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         if (i == p.m) {
-            const int tasks = nl < p.m ? p.task(p.m - 1, nl, ns) + 1 : 0;
+            const int tasks = p.n_tasks(nl, ns);
             head[tasks] = static_cast<int32_t>(p.m);
             *total = make_int4(tasks, p.start[p.m].z, nl, p.start[p.m].w);
         } else if (i < nl) {
@@ -823,9 +826,10 @@ __global__ void rows_plan_kernel(const RowsPlan p, const int32_t* __restrict__ o
             const int np = p.start[i + 1].z - s.z;
             const int32_t r = order[i];
             const int n = static_cast<int>(row_ptr[r + 1] - row_ptr[r]);
+            const int base = p.long_base(nl, ns);
             longs[i] = make_int4(r, s.w, np, 0);
             for (int j = 0; j < np; ++j)
-                parts[s.z + j] = make_int4(p.long_base + s.y + j * p.part_len, min(p.part_len, n - j * p.part_len), static_cast<int>(i), j);
+                parts[s.z + j] = make_int4(base + s.y + j * p.part_len, min(p.part_len, n - j * p.part_len), static_cast<int>(i), j);
         } else {
             const int t = p.task(i, nl, ns);
             if (i == nl || t != p.task(i - 1, nl, ns)) head[t] = static_cast<int32_t>(i);
@@ -884,9 +888,11 @@ __global__ void rows_fill_long_kernel(const RowsPlan p, const int32_t* __restric
     const T* src = reinterpret_cast<const T*>(vals);
     T* dst = reinterpret_cast<T*>(val);
     const int nl = p.n_long();
+    if (static_cast<int>(blockIdx.x) >= nl) return;
+    const int base = p.long_base(nl, p.n_single());
     for (int i = blockIdx.x; i < nl; i += gridDim.x) {
         const int32_t r = order[i];
-        const int64_t s = row_ptr[r], n = row_ptr[r + 1] - s, at = p.long_base + p.start[i].y;
+        const int64_t s = row_ptr[r], n = row_ptr[r + 1] - s, at = base + p.start[i].y;
         for (int64_t j = threadIdx.x; j < (n + 7) / 8 * 8; j += blockDim.x) {
             col[at + j] = j < n ? col_idx[s + j] : 0x7fffffff;
             dst[at + j] = j < n ? src[s + j] : T(0);
@@ -944,12 +950,13 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     else { out->pack = 8; out->task_max = 32; out->part_len = 256; }
     // rows of more than one part have more than part_len nonzeros: at most kRowsMaxSlots parts
     out->part_len = static_cast<int>(std::max<int64_t>(out->part_len, (2 * nnz / kRowsMaxSlots + 127) / 128 * 128));
-    // upper bounds for the arrays, so that nothing has to be read back before the end
-    const int64_t max_tasks = 2 * ((nnz + m) / out->pack) + 2;
+    // Upper bounds for the arrays, so that nothing has to be read back before the end.  An entry is in a task or in a
+    // long row; a task of one row has more than `pack` entries, and the packed rows make a run per `pack` of theirs,
+    // the last one begun.
+    const int64_t max_tasks = (nnz + m) / out->pack + 2;
     const int64_t max_long = nnz / out->task_max + 1;
     const int64_t max_parts = max_long + nnz / out->part_len + 1;
-    const int64_t long_base = (nnz + m + 3 * max_tasks + 15) / 8 * 8;
-    const int64_t entries = long_base + nnz + 8 * max_long;
+    const int64_t entries = nnz + m + 3 * max_tasks + 8 * max_long + 16;
     if (entries >= (int64_t{1} << 31) || m >= (int64_t{1} << 31) - 1) return SPMM_OK;
 
     uint8_t *d_cls = nullptr, *d_cls2 = nullptr;
@@ -989,7 +996,6 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     p.m = m;
     p.pack = out->pack;
     p.part_len = out->part_len;
-    p.long_base = static_cast<int>(long_base);
     p.counts = d_counts;
     p.start = d_start;
     p.n_classes = 2;                                         // long, packed, and the classes between

@@ -265,4 +265,8 @@ def test_a_handle_does_without_its_row_stream_where_memory_is_short(lib):
     said = child(-1)
     window, both = int(said[1]), int(said[3])
     assert both > 2 * window + (64 << 20)
+    # ... and holds every nonzero once: 6 bytes an entry, at most 3 of padding per 16 entries, 16 bytes a task (the pool
+    # grows by 32 MB at a time for each of the larger arrays)
+    entries = 500000 * 17
+    assert both - 2 * window <= entries * (6 * (1 + 3 / 16) + 1) + (96 << 20)
     assert child(window + (56 << 20)) == ["ran"]
