@@ -198,16 +198,20 @@ typedef struct {
     int64_t n_tasks;         /* WCSR sub-tasks; BCSR: K-split units of the current plan (0 if no
                                 block-row is cut)                                             */
     int64_t n_split;         /* WCSR windows / BCSR block-rows cut into more than one part    */
-    int64_t n_slots;         /* partial-sum tiles (WCSR sub-tasks of split windows; BCSR parts) */
+    int64_t n_slots;         /* partial-sum tiles (WCSR sub-tasks of split windows; BCSR parts): with
+                                n_tasks, n_split and split_cols the window kernel's plan        */
     int32_t split_cols;      /* WCSR T in effect; BCSR: the K-split cap in stored blocks      */
     int32_t n_ctas;          /* grid size the schedule was built for                          */
     int64_t distinct_b_rows; /* rows of B that A touches (distinct stored columns)            */
-    /* bytes the roofline model charges for one spmm_run at the given N: */
+    /* bytes the roofline model charges for one spmm_run at the given N, as the format holds A (the
+       row kernel of a WCSR handle reads nnz values and columns instead of bytes_a + bytes_idx): */
     double  bytes_a, bytes_idx, bytes_b_touched, bytes_c;
     double  bytes_gather;    /* B bytes that must enter shared memory (no reuse assumed)      */
     double  flops_stored;    /* 2 * stored_values * N                                         */
-    int64_t workspace_bytes; /* device scratch spmm_run needs at this N (partial tiles; for BCSR
-                                at the planned N)                                             */
+    int64_t workspace_bytes; /* device scratch spmm_run needs at this N: partial tiles, or the row
+                                kernel's partial rows where a WCSR run takes it (known on the
+                                device: a host_only handle reports the window kernel's); for BCSR
+                                at the planned N                                              */
     /* BCSR tile schedule currently held (spmm_bcsr_plan or the last spmm_run); 0 if none:   */
     int64_t plan_n;          /* dense width it was built for                                  */
     int32_t plan_token_tile; /* columns of B per tile: 128, 256 or 512                        */

@@ -1514,7 +1514,7 @@ int spmm_get_info(spmm_handle_t h, int64_t N, spmm_info_t* info) {
         info->bytes_a = static_cast<double>(info->stored_values) * s;
         info->bytes_idx = static_cast<double>(f.nwin + 1 + f.P) * 4.0;
         info->bytes_gather = static_cast<double>(f.P) * n * s;
-        info->workspace_bytes = wcsr_workspace_bytes(h, N);
+        info->workspace_bytes = N > 0 ? static_cast<int64_t>(wcsr_run_bytes(h, N, use_rows(h, N))) : 0;
     }
     info->fill_ratio = info->stored_values ? static_cast<double>(h->nnz) / static_cast<double>(info->stored_values) : 0.0;
     info->bytes_b_touched = static_cast<double>(info->distinct_b_rows) * n * s;

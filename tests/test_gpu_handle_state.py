@@ -270,3 +270,24 @@ def test_a_handle_does_without_its_row_stream_where_memory_is_short(lib):
     entries = 500000 * 17
     assert both - 2 * window <= entries * (6 * (1 + 3 / 16) + 1) + (96 << 20)
     assert child(window + (56 << 20)) == ["ran"]
+
+
+@pytest.mark.parametrize("matrix,opt", [("long", {}), ("long", dict(gather=2)), ("band", {}), ("short", {}), ("short", dict(split_cols=64))])
+def test_workspace_bytes_is_what_a_run_allocates(lib, matrix, opt):
+    """spmm_get_info tells the workspace of the kernel that runs at N: a new handle's first run takes memory
+    (and is refused under capture) exactly where that is not zero."""
+    import torch
+    dtype = "fp16"
+    a = {"long": lambda: _long_rows(dtype, m=300, k=30000), "band": lambda: _band_with_long_rows(dtype, m=20000, n_long=0),
+         "short": lambda: wl.wcsr_irregular(seed=96, m=3000, dtype=dtype, max_len=200)}[matrix]()
+    for N in (32, 128, 512):
+        h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16, **opt)
+        try:
+            B = torch.zeros((a["k"], N), dtype=torch.float16, device="cuda")
+            C = torch.empty((a["m"], N), dtype=torch.float32, device="cuda")
+            need = lib.spmm_get_info(h, N)["workspace_bytes"]
+            code, _ = captured_run(lib, h, B, C, N)
+            assert code == (lib.SPMM_ERR_ALLOC if need else lib.SPMM_OK), (N, need)
+            assert lib.spmm_get_info(h, 0)["workspace_bytes"] == 0
+        finally:
+            lib.spmm_destroy(h)
