@@ -237,7 +237,9 @@ typedef enum {
                                        ascending                                              */
     SPMM_X_BCSR_STACK_TILE_PTR = 9, /* int32 [n_ctas+1]: per-CTA ranges of STACK_TILES (needs a
                                        plan)                                                  */
-    SPMM_X_BCSR_STACK_TILES = 20,   /* int32 [n][2]: row group, 256-column token tile; CTA-major */
+    SPMM_X_BCSR_STACK_TILES = 20,   /* int32 [n][2]: row group, token tile; CTA-major.  A tile is 256
+                                       columns, or 128 where a few long groups would hold up the
+                                       launch: n = groups * ceil(N / tile)                     */
     SPMM_X_BCSR_UNITS = 21,         /* int32 [n_units][4]: block-row, first stored block, end
                                        stored block, partial slot (-1: the unit is a whole block-row
                                        and writes C).  Empty unless the plan cut a block-row
@@ -319,7 +321,8 @@ int spmm_wcsr_create_coo(spmm_handle_t *out, int64_t m, int64_t k, int64_t nnz,
  * The schedule answers the load imbalance Sec. 3.5 and Sec. 4.2 (opt6) report for a persistent
  * kernel with a fixed tile order: tiles (block-row x token tile) are dealt to the CTAs ahead
  * of time, longest block-row first, each to the least loaded CTA.  A handle with row groups
- * (opts.stack_min_fill) gets two such lists: STACK_TILES for the groups (256-token tiles), whose
+ * (opts.stack_min_fill) gets two such lists: STACK_TILES for the groups (256-token tiles, or
+ * 128-token ones where the longest of those alone exceeds a CTA's share of the work by half), whose
  * launch goes first, and TILES for the other block-rows, dealt with the head start that the
  * j-th lightest CTA of the first launch leaves to CTA j of the second (loads counted in bytes
  * staged per block).  Works on host_only handles.

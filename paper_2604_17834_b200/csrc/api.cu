@@ -126,7 +126,6 @@ struct spmm_handle_s {
     int32_t* d_scta_ptr = nullptr;
     CUtensorMap tmAs;                // map of d_svals
     int stack_groups = 0;            // token groups of the stacked launch's tile (2, or 1: see ensure_schedule)
-    int32_t* d_rec_ptr = nullptr;    // ranges of d_tile_recs per CTA
     CUtensorMap tmB3s;               // whole-tile map of B for the stacked launch's token tile
     bool tmB3s_ok = false;
     int k_split = 0;                 // opts.k_split (1: cut outlier block-rows into parts)
@@ -202,7 +201,7 @@ void free_handle(spmm_handle_s* h) {
         void* const arrays[] = {
             h->d_ptr, h->d_idx, h->d_vals, h->d_order, h->d_tiles, h->d_tile_recs, h->d_cta_ptr, h->d_kmerge,
             h->d_sidx, h->d_srows, h->d_svals, h->d_stile_recs, h->d_scta_ptr, h->d_status,
-            h->d_plan, h->d_class, h->d_rec_ptr};
+            h->d_plan, h->d_class};
         for (void* ptr : arrays) dev_free(ptr, nullptr);
         free_partial(h);
         free_wcsr_rows(&h->rows, nullptr);
@@ -705,7 +704,7 @@ int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
 
 // Gives the device arrays of the schedule back; no run may be using them.
 void drop_schedule(spmm_handle_s* h) {
-    int32_t** const arrays[] = {&h->d_tiles, &h->d_tile_recs, &h->d_rec_ptr, &h->d_cta_ptr, &h->d_stile_recs, &h->d_scta_ptr, &h->d_kmerge};
+    int32_t** const arrays[] = {&h->d_tiles, &h->d_tile_recs, &h->d_cta_ptr, &h->d_stile_recs, &h->d_scta_ptr, &h->d_kmerge};
     for (int32_t** a : arrays) {
         dev_free(*a, nullptr);
         *a = nullptr;
@@ -737,8 +736,6 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     if (sw < 1) sw = 1;
     if (sw > n_tt) sw = n_tt;
     BcsrSchedule sc, ss;
-    BcsrSchedule kc, ks;             // what the kernels run where it is not the exported plan: narrower tiles of the row groups
-    bool narrow = false;
     const BcsrStack& st = h->stack;
     int rc;
     try {
@@ -811,7 +808,7 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                 for (int64_t g = 0; g < st.ng; ++g) longest = std::max<int64_t>(longest, st.ptr[g + 1] - st.ptr[g]);
                 longest = (longest + kStackTileFixedCost) * bcsr_stack_block_cost(kStackGroups);
                 if (!rc && N > 128 && 2 * longest * h->n_ctas > 3 * work) {
-                    narrow = true;
+                    BcsrSchedule kc, ks;
                     std::vector<int32_t> gu, gl;
                     for (int64_t g = 0; g < st.ng; ++g) {
                         gu.push_back(static_cast<int32_t>(g));
@@ -823,6 +820,12 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                         std::sort(loads.begin(), loads.end());
                         rc = build_tile_schedule(units, lens, kTileFixedCost, n_tt, static_cast<int>(sw), h->n_ctas, &kc,
                                                  bcsr_block_cost(f.b, groups), &loads);
+                    }
+                    if (!rc) {
+                        sc = std::move(kc);
+                        ss = std::move(ks);
+                        ss.groups = 1;
+                        ss.N = N;
                     }
                 }
             }
@@ -841,13 +844,12 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
         rc = upload(&h->d_tiles, sc.tiles.data(), sc.tiles.size() * 4);
         if (!rc) {
             // self-contained records, so that a role needs one load per tile (and can fetch it a tile ahead)
-            const BcsrSchedule& run = narrow ? kc : sc;
-            const size_t nt = run.tiles.size() / 2;
+            const size_t nt = sc.tiles.size() / 2;
             std::vector<int32_t> recs(4 * nt);
             for (size_t i = 0; i < nt; ++i) {
-                recs[4 * i + 1] = run.tiles[2 * i + 1];
-                if (run.units.empty()) {
-                    const int32_t I = run.tiles[2 * i];
+                recs[4 * i + 1] = sc.tiles[2 * i + 1];
+                if (sc.units.empty()) {
+                    const int32_t I = sc.tiles[2 * i];
                     recs[4 * i] = I;
                     recs[4 * i + 2] = f.block_row_ptr[I];
                     recs[4 * i + 3] = f.block_row_ptr[I + 1];
@@ -861,7 +863,6 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                 }
             }
             rc = upload(&h->d_tile_recs, recs.data(), recs.size() * 4);
-            if (!rc) rc = upload(&h->d_rec_ptr, run.cta_ptr.data(), run.cta_ptr.size() * 4);
         }
         if (!rc && sc.n_slots > 0) {
             // merge lists (split block-rows in ascending order: their slots are consecutive), the
@@ -905,25 +906,24 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
         }
         if (!rc) rc = upload(&h->d_cta_ptr, sc.cta_ptr.data(), sc.cta_ptr.size() * 4);
         if (!rc && !ss.tiles.empty()) {
-            const BcsrSchedule& run = narrow ? ks : ss;
-            const size_t nt = run.tiles.size() / 2;
+            const size_t nt = ss.tiles.size() / 2;
             std::vector<int32_t> recs(4 * nt);
             for (size_t i = 0; i < nt; ++i) {
-                const int32_t g = run.tiles[2 * i];
+                const int32_t g = ss.tiles[2 * i];
                 recs[4 * i] = g;
-                recs[4 * i + 1] = run.tiles[2 * i + 1];
+                recs[4 * i + 1] = ss.tiles[2 * i + 1];
                 recs[4 * i + 2] = st.ptr[g];
                 recs[4 * i + 3] = st.ptr[g + 1];
             }
             rc = upload(&h->d_stile_recs, recs.data(), recs.size() * 4);
-            if (!rc) rc = upload(&h->d_scta_ptr, run.cta_ptr.data(), run.cta_ptr.size() * 4);
+            if (!rc) rc = upload(&h->d_scta_ptr, ss.cta_ptr.data(), ss.cta_ptr.size() * 4);
         }
         if (rc) {
             drop_schedule(h);            // the handle holds no schedule rather than half of one
             return rc;
         }
     }
-    h->stack_groups = ss.tiles.empty() ? 0 : (narrow ? 1 : kStackGroups);
+    h->stack_groups = ss.tiles.empty() ? 0 : ss.groups;
     h->tmB_N = -1;                   // (the stacked launch's map of B depends on its tile)
     h->sched_stack = std::move(ss);
     h->sched = std::move(sc);
@@ -941,7 +941,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.block_row_ptr = h->d_ptr;
     p.block_col_idx = h->d_idx;
     p.tiles = reinterpret_cast<const int4*>(h->d_tile_recs);
-    p.cta_ptr = h->d_rec_ptr;
+    p.cta_ptr = h->d_cta_ptr;
     p.C = C;
     p.m = h->m;
     p.N = N;

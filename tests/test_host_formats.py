@@ -445,3 +445,43 @@ def test_wcsr_reuse_classes_of_the_gather_hints(lib):
     assert got.shape[0] == wcol.shape[0] // 4
     assert np.array_equal(got, per_col.max(axis=1).astype(np.uint8))
     assert got.max() == 7 and (got == 6).any() and (got == 0).any()
+
+
+@pytest.mark.parametrize("b,N", [(32, 256), (32, 392), (16, 256), (32, 2048), (32, 16384)])
+def test_bcsr_plan_of_a_few_long_row_groups_is_the_one_that_runs(lib, b, N):
+    """Where the longest 256-token tile of a row group alone exceeds a CTA's share of all work by half, the groups get
+    128-token tiles and both lists are dealt again: what spmm_export returns is that plan, the launches' own."""
+    m, k, n_ctas = 2048, 1536, 148
+    s = wl.bcsr_sweep(700 + b, m=m, k=k, b=b, density=0.05, dtype="fp16")
+    h = lib.spmm_bcsr_create_csr(m, k, s["row_ptr"], s["col_idx"], s["vals"], "fp16", b, host_only=True, n_ctas=n_ctas)
+    try:
+        f = F.bcsr_from_csr(m, k, s["row_ptr"], s["col_idx"], s["vals"], b)
+        brp = f["block_row_ptr"]
+        rows, ptr, _ = F.bcsr_row_groups(brp, f["block_col_idx"], b, {16: 30, 32: 45}[b])
+        lib.spmm_bcsr_plan(h, N)
+        info = lib.spmm_get_info(h, N)
+        bnt = info["plan_token_tile"]
+        n_tt = -(-N // bnt)
+        order = F.bcsr_row_order(brp)
+        rest = order[~np.isin(order, rows.reshape(-1))]
+
+        def plan(tile):
+            n_tt_g = -(-N // tile)
+            slab_g = max(1, min(-(-N // 256), (16 << 20) // (k * 2) // 256)) * (256 // tile)
+            gp, gt, loads = F.bcsr_tile_schedule(None, n_tt_g, slab_g, n_ctas, fixed_cost=8, units=np.arange(rows.shape[0]),
+                                                 lens=np.diff(ptr), unit_cost=2 * (tile + 128), return_loads=True)
+            tp, tt, total = F.bcsr_tile_schedule(None, n_tt, info["plan_slab_tiles"], n_ctas, units=rest, lens=np.diff(brp)[rest],
+                                                 unit_cost=2 * (bnt + b), initial=np.sort(loads), return_loads=True)
+            return gp, gt, tp, tt, int(total.sum())
+
+        wide = plan(256)
+        longest = (int(np.diff(ptr).max()) + 8) * 2 * (256 + 128)
+        narrow = 2 * longest * n_ctas > 3 * wide[4]
+        assert narrow == (N <= 2048)
+        want = plan(128) if narrow else wide
+        names = (lib.X_BCSR_STACK_TILE_PTR, lib.X_BCSR_STACK_TILES, lib.X_BCSR_TILE_PTR, lib.X_BCSR_TILES)
+        for which, w in zip(names, want):
+            assert np.array_equal(lib.spmm_export(h, which, np.int32), np.asarray(w).reshape(-1))
+        assert lib.spmm_export(h, lib.X_BCSR_STACK_TILES, np.int32).size // 2 == rows.shape[0] * -(-N // (128 if narrow else 256))
+    finally:
+        lib.spmm_destroy(h)
