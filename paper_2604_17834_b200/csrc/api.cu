@@ -519,7 +519,11 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
         rc = upload(&h->d_ptr, f.window_row_ptr.data(), f.window_row_ptr.size() * 4);
         if (!rc) rc = upload(&h->d_idx, f.window_col_idx.data(), f.window_col_idx.size() * 4);
         if (!rc) rc = upload(&h->d_vals, f.packed.data(), f.packed.size());
-        if (!rc) rc = upload_wcsr_plan(h, nullptr);
+        try {
+            if (!rc) rc = upload_wcsr_plan(h, nullptr);
+        } catch (const std::bad_alloc&) {
+            rc = SPMM_ERR_ALLOC;
+        }
         if (!rc && h->want_rows && wcsr_wants_rows(a.es, a.m, a.nnz, f.P)) {
             int64_t* d_rp = nullptr;
             int32_t* d_ci = nullptr;
@@ -714,6 +718,90 @@ void drop_schedule(spmm_handle_s* h) {
     h->sched.N = -1;
 }
 
+// The device arrays of a schedule (and of its row groups', where it has any).
+int upload_schedule(spmm_handle_s* h, const BcsrSchedule& sc, const BcsrSchedule& ss, int64_t N) {
+    const BcsrHost& f = h->bcsr;
+    const BcsrStack& st = h->stack;
+    int rc = upload(&h->d_tiles, sc.tiles.data(), sc.tiles.size() * 4);
+    if (!rc) {
+        // self-contained records, so that a role needs one load per tile (and can fetch it a tile ahead)
+        const size_t nt = sc.tiles.size() / 2;
+        std::vector<int32_t> recs(4 * nt);
+        for (size_t i = 0; i < nt; ++i) {
+            recs[4 * i + 1] = sc.tiles[2 * i + 1];
+            if (sc.units.empty()) {
+                const int32_t I = sc.tiles[2 * i];
+                recs[4 * i] = I;
+                recs[4 * i + 2] = f.block_row_ptr[I];
+                recs[4 * i + 3] = f.block_row_ptr[I + 1];
+            } else {
+                // K-split: the tile names a unit {block-row, first block, end block, slot}; a part
+                // carries -1 - slot in place of the block-row
+                const int32_t* u = &sc.units[4 * static_cast<size_t>(sc.tiles[2 * i])];
+                recs[4 * i] = u[3] < 0 ? u[0] : -1 - u[3];
+                recs[4 * i + 2] = u[1];
+                recs[4 * i + 3] = u[2];
+            }
+        }
+        rc = upload(&h->d_tile_recs, recs.data(), recs.size() * 4);
+    }
+    if (!rc && sc.n_slots > 0) {
+        // merge lists (split block-rows in ascending order: their slots are consecutive), the
+        // partial tiles' workspace and its store map
+        // (the parts of a block-row are consecutive units, in part order)
+        std::vector<int32_t> rows, firsts, parts;
+        for (size_t u = 0; u < sc.units.size() / 4; ++u) {
+            const int32_t I = sc.units[4 * u], slot = sc.units[4 * u + 3];
+            if (slot < 0) continue;
+            if (rows.empty() || rows.back() != I) { rows.push_back(I); firsts.push_back(slot); parts.push_back(0); }
+            parts.back()++;
+        }
+        std::vector<int32_t> mg;
+        mg.insert(mg.end(), rows.begin(), rows.end());
+        mg.insert(mg.end(), firsts.begin(), firsts.end());
+        mg.insert(mg.end(), parts.begin(), parts.end());
+        h->n_kmerge = static_cast<int>(rows.size());
+        rc = upload(&h->d_kmerge, mg.data(), mg.size() * 4);
+        const size_t need = static_cast<size_t>(sc.n_slots) * f.b * static_cast<size_t>(N) * 4;
+        if (!rc && need > h->partial_bytes) {
+            if (h->d_partial) {
+                if (cudaDeviceSynchronize() != cudaSuccess) rc = cuda_error();
+                else free_partial(h);
+            }
+            if (!rc && !dev_alloc_ready_ok(&h->d_partial, need)) rc = SPMM_ERR_ALLOC;
+            if (!rc) h->partial_bytes = need;
+        }
+        if (!rc) {
+            EncodeTiledFn fn = get_encode_fn();
+            const cuuint64_t dims[2] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(sc.n_slots) * f.b};
+            const cuuint64_t strides[1] = {static_cast<cuuint64_t>(N) * 4};
+            const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(bcsr_epi_cols(f.b, false, false))};
+            const cuuint32_t estr[2] = {1, 1};
+            if (!fn || fn(&h->tmP, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->d_partial, dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+                rc = cuda_error();
+            else
+                h->tmP_ok = true;
+        }
+    }
+    if (!rc) rc = upload(&h->d_cta_ptr, sc.cta_ptr.data(), sc.cta_ptr.size() * 4);
+    if (!rc && !ss.tiles.empty()) {
+        const size_t nt = ss.tiles.size() / 2;
+        std::vector<int32_t> recs(4 * nt);
+        for (size_t i = 0; i < nt; ++i) {
+            const int32_t g = ss.tiles[2 * i];
+            recs[4 * i] = g;
+            recs[4 * i + 1] = ss.tiles[2 * i + 1];
+            recs[4 * i + 2] = st.ptr[g];
+            recs[4 * i + 3] = st.ptr[g + 1];
+        }
+        rc = upload(&h->d_stile_recs, recs.data(), recs.size() * 4);
+        if (!rc) rc = upload(&h->d_scta_ptr, ss.cta_ptr.data(), ss.cta_ptr.size() * 4);
+    }
+    return rc;
+}
+
 // Tile width, slab width and the tile schedule for dense width N (cached for the last N).
 int ensure_schedule(spmm_handle_s* h, int64_t N) {
     if (h->sched.N == N) return SPMM_OK;
@@ -841,82 +929,10 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             if (cudaDeviceSynchronize() != cudaSuccess) return cuda_error();
             drop_schedule(h);
         }
-        rc = upload(&h->d_tiles, sc.tiles.data(), sc.tiles.size() * 4);
-        if (!rc) {
-            // self-contained records, so that a role needs one load per tile (and can fetch it a tile ahead)
-            const size_t nt = sc.tiles.size() / 2;
-            std::vector<int32_t> recs(4 * nt);
-            for (size_t i = 0; i < nt; ++i) {
-                recs[4 * i + 1] = sc.tiles[2 * i + 1];
-                if (sc.units.empty()) {
-                    const int32_t I = sc.tiles[2 * i];
-                    recs[4 * i] = I;
-                    recs[4 * i + 2] = f.block_row_ptr[I];
-                    recs[4 * i + 3] = f.block_row_ptr[I + 1];
-                } else {
-                    // K-split: the tile names a unit {block-row, first block, end block, slot}; a part
-                    // carries -1 - slot in place of the block-row
-                    const int32_t* u = &sc.units[4 * static_cast<size_t>(sc.tiles[2 * i])];
-                    recs[4 * i] = u[3] < 0 ? u[0] : -1 - u[3];
-                    recs[4 * i + 2] = u[1];
-                    recs[4 * i + 3] = u[2];
-                }
-            }
-            rc = upload(&h->d_tile_recs, recs.data(), recs.size() * 4);
-        }
-        if (!rc && sc.n_slots > 0) {
-            // merge lists (split block-rows in ascending order: their slots are consecutive), the
-            // partial tiles' workspace and its store map
-            // (the parts of a block-row are consecutive units, in part order)
-            std::vector<int32_t> rows, firsts, parts;
-            for (size_t u = 0; u < sc.units.size() / 4; ++u) {
-                const int32_t I = sc.units[4 * u], slot = sc.units[4 * u + 3];
-                if (slot < 0) continue;
-                if (rows.empty() || rows.back() != I) { rows.push_back(I); firsts.push_back(slot); parts.push_back(0); }
-                parts.back()++;
-            }
-            std::vector<int32_t> mg;
-            mg.insert(mg.end(), rows.begin(), rows.end());
-            mg.insert(mg.end(), firsts.begin(), firsts.end());
-            mg.insert(mg.end(), parts.begin(), parts.end());
-            h->n_kmerge = static_cast<int>(rows.size());
-            rc = upload(&h->d_kmerge, mg.data(), mg.size() * 4);
-            const size_t need = static_cast<size_t>(sc.n_slots) * f.b * static_cast<size_t>(N) * 4;
-            if (!rc && need > h->partial_bytes) {
-                if (h->d_partial) {
-                    if (cudaDeviceSynchronize() != cudaSuccess) rc = cuda_error();
-                    else free_partial(h);
-                }
-                if (!rc && !dev_alloc_ready_ok(&h->d_partial, need)) rc = SPMM_ERR_ALLOC;
-                if (!rc) h->partial_bytes = need;
-            }
-            if (!rc) {
-                EncodeTiledFn fn = get_encode_fn();
-                const cuuint64_t dims[2] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(sc.n_slots) * f.b};
-                const cuuint64_t strides[1] = {static_cast<cuuint64_t>(N) * 4};
-                const cuuint32_t box[2] = {32, static_cast<cuuint32_t>(bcsr_epi_cols(f.b, false, false))};
-                const cuuint32_t estr[2] = {1, 1};
-                if (!fn || fn(&h->tmP, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, h->d_partial, dims, strides, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-                    rc = cuda_error();
-                else
-                    h->tmP_ok = true;
-            }
-        }
-        if (!rc) rc = upload(&h->d_cta_ptr, sc.cta_ptr.data(), sc.cta_ptr.size() * 4);
-        if (!rc && !ss.tiles.empty()) {
-            const size_t nt = ss.tiles.size() / 2;
-            std::vector<int32_t> recs(4 * nt);
-            for (size_t i = 0; i < nt; ++i) {
-                const int32_t g = ss.tiles[2 * i];
-                recs[4 * i] = g;
-                recs[4 * i + 1] = ss.tiles[2 * i + 1];
-                recs[4 * i + 2] = st.ptr[g];
-                recs[4 * i + 3] = st.ptr[g + 1];
-            }
-            rc = upload(&h->d_stile_recs, recs.data(), recs.size() * 4);
-            if (!rc) rc = upload(&h->d_scta_ptr, ss.cta_ptr.data(), ss.cta_ptr.size() * 4);
+        try {
+            rc = upload_schedule(h, sc, ss, N);
+        } catch (const std::bad_alloc&) {
+            rc = SPMM_ERR_ALLOC;
         }
         if (rc) {
             drop_schedule(h);            // the handle holds no schedule rather than half of one

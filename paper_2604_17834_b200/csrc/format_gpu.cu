@@ -308,6 +308,7 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     out->b = b;
     out->nbr = nbr;
     out->nbc = nbc;
+    out->block_row_ptr.assign(static_cast<size_t>(nbr) + 1, 0);        // (may throw: before anything is held on the device)
 
     int* d_flags = nullptr;                     // [0] CSR error code (min), [1] scan overflow, [2] a bad entry
     int32_t* d_counts = nullptr;
@@ -353,7 +354,6 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     }
     if (nbr > 0) bcsr_count_kernel<<<static_cast<unsigned>(nbr), kThreads, smem, st>>>(m, b, words, d_row_ptr, d_col_idx, d_counts);
     exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_counts, nbr, *d_block_row_ptr, d_flags + 1);
-    out->block_row_ptr.assign(static_cast<size_t>(nbr) + 1, 0);
     if (cudaMemcpyAsync(out->block_row_ptr.data(), *d_block_row_ptr, static_cast<size_t>(nbr + 1) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return fail(SPMM_ERR_CUDA);
     if (cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
@@ -376,7 +376,11 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         else
             bcsr_fill_kernel<2><<<static_cast<unsigned>(nbr), kThreads, smem, st>>>(m, b, words, d_row_ptr, d_col_idx, d_vals, *d_block_row_ptr, *d_block_col_idx, *d_blocks);
     }
-    out->block_col_idx.assign(static_cast<size_t>(nnzb), 0);
+    try {
+        out->block_col_idx.assign(static_cast<size_t>(nnzb), 0);
+    } catch (const std::bad_alloc&) {
+        return fail(SPMM_ERR_ALLOC);
+    }
     if (nnzb && cudaMemcpyAsync(out->block_col_idx.data(), *d_block_col_idx, idx_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return fail(SPMM_ERR_CUDA);
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess) return fail(SPMM_ERR_CUDA);
@@ -595,6 +599,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     out->wh = wh;
     out->b_col = b_col;
     out->nwin = nwin;
+    out->window_row_ptr.assign(static_cast<size_t>(nwin) + 1, 0);      // (may throw: before anything is held on the device)
     *d_window_row_ptr = nullptr;
     *d_window_col_idx = nullptr;
     *d_packed = nullptr;
@@ -677,7 +682,6 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     wcsr_pad_kernel<<<static_cast<unsigned>(std::min<int64_t>((nwin + 255) / 256 + 1, 2048)), 256, 0, st>>>(d_ustart, nwin, b_col, d_len);
     exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_len, nwin, *d_window_row_ptr, &d_flags->overflow);
     if (k > 0) wcsr_sum_used_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 1024)), 256, 0, st>>>(d_used, k, &d_flags->distinct);
-    out->window_row_ptr.assign(static_cast<size_t>(nwin) + 1, 0);
     if (cudaMemcpyAsync(out->window_row_ptr.data(), *d_window_row_ptr, static_cast<size_t>(nwin + 1) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         !read_flags())
         return fail(SPMM_ERR_CUDA);
