@@ -96,8 +96,8 @@ def assert_close(C_gpu, C_ref, S, dtype, what=""):
     return float(np.max(err / bound))
 
 
-def captured_run(lib, h, B, C, N, relaxed=False, replay=False):
-    """One spmm_run inside a stream capture of its own stream.  -> (status code of the run, kinds of the captured
+def captured_run(lib, h, B, C, N, relaxed=False, replay=False, static=False):
+    """One spmm_run (static: spmm_wcsr_run_static) inside a stream capture of its own stream.  -> (status code of the run, kinds of the captured
     nodes, or None where the capture gave no graph).  replay: launch the graph once, unless the run was refused."""
     import torch
     from cuda.bindings import runtime as rt
@@ -107,7 +107,7 @@ def captured_run(lib, h, B, C, N, relaxed=False, replay=False):
     assert rt.cudaStreamBeginCapture(stream.cuda_stream, mode)[0] == rt.cudaError_t.cudaSuccess
     code = lib.SPMM_OK
     try:
-        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, stream.cuda_stream)
+        (lib.spmm_wcsr_run_static if static else lib.spmm_run)(h, B.data_ptr(), C.data_ptr(), N, stream.cuda_stream)
     except lib.SpmmError as e:
         code = e.code
     err, graph = rt.cudaStreamEndCapture(stream.cuda_stream)

@@ -35,13 +35,13 @@ def _sample_cols(N, seed):
     return np.array(sorted(cols), dtype=np.int64)
 
 
-def _run_and_check(lib, kind, a, dtype, size, N, Bs, cols=None, what="", c16=False, col_major=False):
+def _run_and_check(lib, kind, a, dtype, size, N, Bs, cols=None, what="", c16=False, col_major=False, **opt):
     """Bs is the k x N operand.  c16: C in the input's 16-bit type; col_major: the device gets
     X = B^T (N x k) and returns Y = C^T (N x m)."""
     import torch
     mk = lib.spmm_bcsr_create_csr if kind == "bcsr" else lib.spmm_wcsr_create_csr
     h = mk(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, size,
-           c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32, layout=lib.COLMAJOR if col_major else lib.ROWMAJOR)
+           c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32, layout=lib.COLMAJOR if col_major else lib.ROWMAJOR, **opt)
     try:
         Bd = to_device(Bs)
         if col_major:
@@ -77,6 +77,14 @@ def test_config1_wcsr_irregular_full(lib):
     a = wl.wcsr_irregular()
     Bs = wl.dense(1102, a["k"], 128, ("normal", 0.0, 1.0), "tf32")
     worst = _run_and_check(lib, "wcsr", a, "tf32", 16, 128, Bs, what="configs[1]")
+    assert worst < 1.0
+
+
+def test_config1_wcsr_irregular_full_window_kernel(lib):
+    """The same with the window kernel asked for (the default takes the row kernel on this matrix)."""
+    a = wl.wcsr_irregular()
+    Bs = wl.dense(1102, a["k"], 128, ("normal", 0.0, 1.0), "tf32")
+    worst = _run_and_check(lib, "wcsr", a, "tf32", 16, 128, Bs, what="configs[1], window kernel", gather=lib.GATHER_TMA)
     assert worst < 1.0
 
 
@@ -143,6 +151,15 @@ def test_config4_wcsr_rmat_full(lib, rmat_full, N):
     # a third of the sampled positions, and in any case one column of every 128-column token tile
     cols = np.unique(np.concatenate([_sample_cols(N, N)[::3], np.arange(5, N, 128)])) if N > 32 else np.arange(0, 32, 3)
     _run_and_check(lib, "wcsr", a, "fp16", 16, N, Bs, cols=cols, what="configs[4] N=%d" % N)
+
+
+@pytest.mark.parametrize("N", [32, 128])
+def test_config4_wcsr_rmat_full_window_kernel(lib, rmat_full, N):
+    """The same with the window kernel asked for (the default takes the row kernel on this matrix)."""
+    a = rmat_full
+    Bs = wl.dense(1105 + N, a["k"], N, ("normal", 0.0, 1.0), "fp16")
+    cols = _sample_cols(N, N)[::3] if N > 32 else np.arange(0, 32, 3)
+    _run_and_check(lib, "wcsr", a, "fp16", 16, N, Bs, cols=cols, what="configs[4] N=%d, window kernel" % N, gather=lib.GATHER_TMA)
 
 
 def test_config4_wcsr_rmat_fp16_output_full(lib, rmat_full):

@@ -199,7 +199,8 @@ def test_run_host_matches_device_run(lib):
     lib.spmm_destroy(h)
 
 
-@pytest.mark.parametrize("case", ["wcsr_tf32", "bcsr_fp16", "bcsr_bf16_colmajor_c16", "wcsr_fp16_c16"])
+@pytest.mark.parametrize("case", ["wcsr_tf32", "bcsr_fp16", "bcsr_bf16_colmajor_c16", "wcsr_fp16_c16", "wcsr_tf32_window",
+                                  "wcsr_fp16_window_c16"])
 def test_run_host_in_chunks_matches_device_run(lib, case):
     """Operands of 8 MB and more go through spmm_run_host in column chunks whose transfers overlap;
     the result is the one spmm_run gives on the whole operand, bit for bit, with pinned and with
@@ -212,6 +213,7 @@ def test_run_host_in_chunks_matches_device_run(lib, case):
         a = wl.wcsr_irregular(seed=77, m=24000, dtype=dtype)
         N = 128 if dtype == "tf32" else 256
         h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16,
+                                     gather=lib.GATHER_TMA if "window" in case else lib.GATHER_AUTO,
                                      c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
     else:
         dtype = "bf16" if "bf16" in case else "fp16"
@@ -263,7 +265,7 @@ def test_bad_run_arguments(lib):
     lib.spmm_destroy(h)
 
 
-@pytest.mark.parametrize("kind", ["bcsr", "wcsr", "bcsr_dynamic", "bcsr_row_groups"])
+@pytest.mark.parametrize("kind", ["bcsr", "wcsr", "wcsr_window", "bcsr_dynamic", "bcsr_row_groups"])
 def test_wait_that_runs_out_is_reported_and_the_context_survives(lib, kind):
     """Every wait inside the kernels is bounded.  With the bound set to zero the first wait
     for operands that are still on their way runs out: the kernel leaves early
@@ -283,6 +285,9 @@ def test_wait_that_runs_out_is_reported_and_the_context_survives(lib, kind):
     else:
         a, dtype, size, N = wl.wcsr_irregular(seed=405, m=20000, dtype="tf32"), "tf32", 16, 128
         mk = lib.spmm_wcsr_create_csr
+        if kind == "wcsr_window":        # (the default here is the row kernel, which has no waits and reports the same)
+            def mk(*args):
+                return lib.spmm_wcsr_create_csr(*args, gather=lib.GATHER_TMA)
     Bs = wl.dense(41, a["k"], N, ("normal", 0.0, 1.0), dtype)
     h = mk(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, size)
     try:

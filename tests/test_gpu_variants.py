@@ -8,7 +8,7 @@ import pytest
 
 from paper_2604_17834_b200 import workloads as wl
 
-from helpers import assert_close, reference, run_gpu, run_gpu_variant, to_device
+from helpers import assert_close, captured_run, reference, run_gpu, run_gpu_variant, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -451,7 +451,8 @@ def test_bcsr_row_groups_find_scattered_families(lib, b, dtype):
 def test_prepare_leaves_nothing_to_allocate_for_the_run(lib, kind):
     """After spmm_prepare(h, N) the first spmm_run at that width changes neither the free device
     memory nor the workspace the handle reports (one throw-away handle of the same kind runs first,
-    so that the kernel variant's code is already loaded)."""
+    so that the kernel variant's code is already loaded).  Free memory alone would not show an
+    allocation that the library's pool serves, so the run is captured first: nothing but kernels."""
     import torch
     dtype, N = "fp16", 512
     st = torch.cuda.current_stream().cuda_stream
@@ -478,6 +479,8 @@ def test_prepare_leaves_nothing_to_allocate_for_the_run(lib, kind):
         info = lib.spmm_get_info(h, N)
         if kind != "bcsr":
             assert info["workspace_bytes"] > 0, "the case must need a workspace"
+        code, nodes = captured_run(lib, h, Bd, C, N)
+        assert code == lib.SPMM_OK and nodes and set(nodes) == {"kernel"}
         C.fill_(float("nan"))
         torch.cuda.synchronize()
         free0 = torch.cuda.mem_get_info()[0]
@@ -678,3 +681,76 @@ def test_bcsr_tf32_row_groups_keep_non_finite_operands_to_their_rows(lib, b, col
     Cr, S = reference(a, np.where(finite, Bs, 0.0).astype(np.float32), "tf32")
     for C in outs:
         assert_close(np.where(hit, 0.0, C).astype(np.float32), np.where(hit, 0.0, Cr), S, "tf32", "non-finite B b=%d" % b)
+
+
+@pytest.mark.parametrize("dtype,wh,c16", [("tf32", 16, False), ("fp16", 16, False), ("bf16", 16, True), ("fp8", 16, False),
+                                          ("tf32", 64, False), ("fp16", 64, True), ("bf16", 64, False), ("fp8", 64, False)])
+@pytest.mark.parametrize("N,T", [(128, 0), (48, 128), (336, 128), (64, 0)])
+def test_wcsr_window_kernel_on_matrices_that_condense(lib, dtype, wh, c16, N, T):
+    """Windows that share columns (a third of the matrix is stored) are the window kernel's with every option at its
+    default: whole, split, ragged and empty windows, both window heights, one token tile to three, both types of C;
+    host- and GPU-built handles."""
+    import torch
+    m, k = 1003, 1500
+    a = wl.random_csr(58 + wh, m, k, 0.3, dtype, empty_rows=tuple(range(64, 192)))
+    Bs = wl.dense(20, k, N, ("normal", 0.0, 1.0), dtype)
+    Cr, S = reference(a, Bs, dtype)
+    dev = [to_device(a[x]) for x in ("row_ptr", "col_idx", "vals")]
+    opt = dict(split_cols=T, c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
+    outs = []
+    for h in (lib.spmm_wcsr_create_csr(m, k, a["row_ptr"], a["col_idx"], a["vals"], dtype, wh, **opt),
+              lib.spmm_wcsr_create_csr_device(m, k, *[d.data_ptr() for d in dev], dtype, wh, torch.cuda.current_stream().cuda_stream, **opt)):
+        try:
+            info = lib.spmm_get_info(h, N)
+            assert info["nnz"] > 1.75 * info["n_units"] and info["n_empty"] >= 2
+            assert (info["n_split"] > 0) or not T
+            outs.append(run_gpu_variant(lib, h, Bs, m, N, dtype, c16=c16))
+            assert_close(outs[-1], Cr, S, dtype, "window kernel %s wh=%d N=%d T=%d" % (dtype, wh, N, T))
+        finally:
+            lib.spmm_destroy(h)
+    assert np.array_equal(outs[0], outs[1])
+
+
+def test_runs_of_different_kinds_that_feed_one_another(lib):
+    """The chain of the test above across kinds: the grid whose CTAs are cancelled, a plan with a merge kernel, the row
+    kernel in several launches of several column tiles, the window kernel with its merge, and two handles in
+    turn.  Without a synchronise the chain gives the bits it gives with one after every run."""
+    import torch
+    n, N = 1024, 2176                      # TF32, row kernel: 2176 columns are nine tiles, two launches
+    st = torch.cuda.current_stream().cuda_stream
+    scaled = lambda a, dtype, x: wl.to_storage(wl.widen(a["vals"], dtype) * x, dtype)  # noqa: E731
+    b1 = wl.bcsr_sweep(621, m=n, k=n, b=64, density=0.1, dtype="fp16")
+    b2 = wl.bcsr_sweep(622, m=n, k=n, b=32, density=0.02, dtype="tf32")
+    w = wl.wcsr_irregular(seed=623, m=n, dtype="tf32", max_len=700)
+    w2 = wl.wcsr_irregular(seed=624, m=n, dtype="tf32", max_len=300)
+    hs = [lib.spmm_bcsr_create_csr(n, n, b1["row_ptr"], b1["col_idx"], scaled(b1, "fp16", 1 / 16), "fp16", 64, schedule=lib.SCHED_DYNAMIC),
+          lib.spmm_bcsr_create_csr(n, n, b2["row_ptr"], b2["col_idx"], scaled(b2, "tf32", 1 / 8), "tf32", 32, stack_min_fill=-1, k_split=1),
+          lib.spmm_wcsr_create_csr(n, n, w["row_ptr"], w["col_idx"], scaled(w, "tf32", 1 / 2), "tf32", 16),
+          lib.spmm_wcsr_create_csr(n, n, w["row_ptr"], w["col_idx"], scaled(w, "tf32", 1 / 2), "tf32", 16, split_cols=64),
+          lib.spmm_wcsr_create_csr(n, n, w2["row_ptr"], w2["col_idx"], scaled(w2, "tf32", 1 / 2), "tf32", 16)]
+    try:
+        x0 = to_device(wl.dense(625, n, N, ("normal", 0.0, 1.0), "fp16"))
+        bufs = [torch.empty((n, N), dtype=torch.float32, device="cuda") for _ in range(2)]
+        outs = []
+        for sync in (True, True, False, False):
+            x = x0.clone()
+            for _ in range(3):
+                src = x
+                for i, j in enumerate((0, 1, 2, 4, 2, 3, 4)):
+                    lib.spmm_run(hs[j], src.data_ptr(), bufs[i % 2].data_ptr(), N, st)
+                    src = bufs[i % 2]
+                    if sync:
+                        torch.cuda.synchronize()
+                x = (src / src.abs().max()).to(torch.float16)
+                if sync:
+                    torch.cuda.synchronize()
+            torch.cuda.synchronize()
+            for h in hs:
+                lib.spmm_check(h)
+            outs.append(x)
+        assert lib.spmm_get_info(hs[1], N)["n_split"] > 0 and lib.spmm_get_info(hs[3], N)["n_split"] > 0
+        assert bool(torch.isfinite(outs[0].float()).all()) and float(outs[0].float().abs().max()) == 1.0
+        assert all(torch.equal(outs[0], x) for x in outs[1:])
+    finally:
+        for h in hs:
+            lib.spmm_destroy(h)

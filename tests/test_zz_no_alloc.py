@@ -15,7 +15,7 @@ import pytest
 
 from paper_2604_17834_b200 import workloads as wl
 
-from helpers import assert_close, reference, run_gpu, to_device
+from helpers import assert_close, captured_run, reference, run_gpu, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -83,7 +83,8 @@ def test_static_scratch_refuses_what_does_not_fit(lib):
 def test_static_scratch_run_leaves_device_memory_alone(lib):
     """The point of the entry point: on a warmed handle a call neither takes nor returns device
     memory.  Free memory as the driver reports it is read before and after calls whose output
-    buffer already exists, and the handle's own workspace is never created by this path."""
+    buffer already exists, and the handle's own workspace is never created by this path.  An
+    allocation that the library's own pool serves does not show there: a captured call does."""
     import torch
     a = wl.wcsr_irregular(seed=79, m=6000, dtype="fp16")
     N = 128
@@ -101,6 +102,11 @@ def test_static_scratch_run_leaves_device_memory_alone(lib):
         torch.cuda.synchronize()
         lib.spmm_check(h)
         assert torch.cuda.mem_get_info()[0] == free0
+        code, nodes = captured_run(lib, h, Bd, C, N, static=True)
+        assert code == lib.SPMM_OK and nodes == ["kernel", "kernel"]
+        # the workspace was never created: spmm_run, which needs it, is refused under capture
+        code, _ = captured_run(lib, h, Bd, C, N)
+        assert code == lib.SPMM_ERR_ALLOC
     finally:
         lib.spmm_destroy(h)
 
