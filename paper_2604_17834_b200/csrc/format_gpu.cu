@@ -351,6 +351,7 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         cudaFuncSetAttribute(bcsr_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         cudaFuncSetAttribute(bcsr_fill_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
         cudaFuncSetAttribute(bcsr_fill_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        cudaFuncSetAttribute(bcsr_fill_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     }
     if (nbr > 0) bcsr_count_kernel<<<static_cast<unsigned>(nbr), kThreads, smem, st>>>(m, b, words, d_row_ptr, d_col_idx, d_counts);
     exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_counts, nbr, *d_block_row_ptr, d_flags + 1);

@@ -267,6 +267,28 @@ def test_wcsr_built_on_the_gpu_is_bit_exact(lib, dtype, wh, m, k, dens):
         lib.spmm_destroy(h0)
 
 
+@pytest.mark.parametrize("dtype", ["tf32", "fp16", "fp8"])
+def test_bcsr_gpu_builder_with_many_block_columns(lib, dtype):
+    """More than 196,608 block columns: the builder's bitmap takes more than 48 KB of shared memory."""
+    import torch
+    from oracle import formats as F
+    m, k, b = 70, 7_000_000, 32
+    rng = np.random.default_rng(9)
+    lens = rng.integers(0, 40, m)
+    rp = np.concatenate(([0], np.cumsum(lens))).astype(np.int64)
+    ci = np.concatenate([np.sort(rng.choice(k, n, replace=False)) for n in lens]).astype(np.int32)
+    va = wl.dense(10, 1, int(rp[-1]), ("normal", 0.0, 1.0), dtype).ravel()
+    dev = [to_device(x) for x in (rp, ci, va)]
+    h = lib.spmm_bcsr_create_csr_device(m, k, *[d.data_ptr() for d in dev], dtype, b, torch.cuda.current_stream().cuda_stream)
+    try:
+        f = F.bcsr_from_csr(m, k, rp, ci, va, b)
+        assert np.array_equal(lib.spmm_export(h, lib.X_BCSR_BLOCK_COL_IDX, np.int32), f["block_col_idx"])
+        bits = {4: np.uint32, 2: np.uint16, 1: np.uint8}[va.itemsize]
+        assert np.array_equal(lib.spmm_export(h, lib.X_BCSR_BLOCKS, bits), f["blocks"].view(bits).ravel())
+    finally:
+        lib.spmm_destroy(h)
+
+
 def test_bcsr_gpu_builder_rejects_malformed_csr(lib):
     import torch
     vals = to_device(wl.to_storage(np.ones(4), "fp16"))
