@@ -111,13 +111,24 @@ def workload_table():
         "cfg5_wcsr_rmat_n128": ("configs[4] WCSR R-MAT 2^21 deg 16 fp16 wh=16, N=128", cfg5(128)),
         "cfg5_wcsr_rmat_n256": ("configs[4] WCSR R-MAT 2^21 deg 16 fp16 wh=16, N=256", cfg5(256)),
     }
-    def tall(base):
-        """Same matrix with the paper's own 64-row WCSR windows (Sec. 4.1) instead of 16."""
+    def window(base):
+        """Same workload on the window kernel (TMA row gather): by default these matrices, whose windows condense
+        almost nothing, run on the row kernel."""
         def f():
             w = base()
+            w["opts"] = dict(w.get("opts", {}), gather=2)
+            return w
+        return f
+    def tall(base):
+        """Same matrix with the paper's own 64-row WCSR windows (Sec. 4.1) instead of 16, on the window kernel."""
+        def f():
+            w = window(base)()
             w["size"] = 64
             return w
         return f
+    t["cfg2_wcsr_irregular_window"] = ("configs[1] on the window kernel", window(cfg2))
+    for N in (32, 128, 256):
+        t["cfg5_wcsr_rmat_n%d_window" % N] = ("configs[4] N=%d on the window kernel" % N, window(cfg5(N)))
     def plain(base):
         """Same workload with the BCSR row groups (stacked 128-row blocks) switched off."""
         def f():
@@ -216,7 +227,9 @@ ALL_OTHERS = DEFAULT_OTHERS + [
     "cfg4_bcsr_sweep_b64_d0.05", "cfg4_bcsr_sweep_b64_d0.01", "cfg4_bcsr_flat_b64_d0.05", "cfg4_bcsr_flat_b64_d0.01",
     "cfg3_bcsr_llm_gate_c16", "cfg3_bcsr_llm_gate_cm", "cfg3_bcsr_llm_gate_cm_c16",
     "cfg3_bcsr_llm_down_cm_c16", "cfg5_wcsr_rmat_n128_c16",
-    "cfg3_bcsr_llm_gate_cm_fp8", "cfg3_bcsr_llm_down_cm_fp8", "cfg3_bcsr_llm_gate_fp8", "cfg2_wcsr_irregular_wh64", "cfg5_wcsr_rmat_n128_wh64",
+    "cfg3_bcsr_llm_gate_cm_fp8", "cfg3_bcsr_llm_down_cm_fp8", "cfg3_bcsr_llm_gate_fp8",
+    "cfg2_wcsr_irregular_window", "cfg5_wcsr_rmat_n32_window", "cfg5_wcsr_rmat_n128_window", "cfg5_wcsr_rmat_n256_window",
+    "cfg2_wcsr_irregular_wh64", "cfg5_wcsr_rmat_n128_wh64",
     "cfg2_wcsr_irregular_lsu_gather", "cfg5_wcsr_rmat_n128_lsu_gather",
     "cfg4_bcsr_sweep_b64_d0.1_dyn", "cfg4_bcsr_sweep_b16_d0.1_plain", "cfg4_bcsr_sweep_b32_d0.1_plain",
     "cfg4_bcsr_sweep_b16_d0.5", "cfg4_bcsr_sweep_b32_d0.5",
@@ -228,11 +241,11 @@ ALL_OTHERS = DEFAULT_OTHERS + [
 # DRAM bytes (read + write) of one launch of the dominant kernel, from the ncu captures whose
 # summaries are under profiles/ (absent where no capture of that exact launch exists).
 NCU_DRAM_TRAFFIC = {
-    "cfg2_wcsr_irregular": 118.5e6,     # profiles/wcsr_spmm_cfg2_ncu.md
-    "cfg5_wcsr_rmat_n128": 3.525e9,     # profiles/wcsr_spmm_cfg5_n128_dram.md
-    "cfg5_wcsr_rmat_n256": 7.186e9,     # the same file, N = 256
+    "cfg2_wcsr_irregular_window": 118.5e6,
+    "cfg5_wcsr_rmat_n128_window": 3.525e9,
+    "cfg5_wcsr_rmat_n256_window": 7.186e9,
     # captured at N = 16,384 (1.409 GB) and scaled by 4 to N = 65,536: one L2 slab is 2048
-    # tokens, so traffic grows in proportion to N (profiles/bcsr_spmm_cfg3_n8192_ncu.md)
+    # tokens, so traffic grows in proportion to N
     "cfg3_bcsr_llm_gate": 5.64e9,
 }
 
@@ -322,21 +335,53 @@ def device_B(torch, w, seed=7):
     return B
 
 
-def roofline_of(info, ms, pk, name=None):
+def launched_kernels(lib, h, B, C, N):
+    """Names of the kernels one spmm_run launches, from a stream capture of it (nothing is executed)."""
+    import torch
+    from cuda.bindings import driver as drv
+    from cuda.bindings import runtime as rt
+    stream = torch.cuda.Stream()
+    if rt.cudaStreamBeginCapture(stream.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)[0]:
+        raise RuntimeError("stream capture failed")
+    try:
+        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, stream.cuda_stream)
+    finally:
+        err, graph = rt.cudaStreamEndCapture(stream.cuda_stream)
+    n = rt.cudaGraphGetNodes(graph, 0)[-1]
+    names = []
+    for node in rt.cudaGraphGetNodes(graph, n)[1] if n else []:
+        err, p = drv.cuGraphKernelNodeGetParams(drv.CUgraphNode(int(node)))
+        err, name = drv.cuKernelGetName(p.kern) if int(p.kern) else drv.cuFuncGetName(p.func)
+        names.append(name.decode())
+    rt.cudaGraphDestroy(graph)
+    return names
+
+
+def model_of(info, kernels):
+    """-> (bytes, flops) of one spmm_run.  Bytes: A values + indices + distinct B rows touched + C; the row kernel of
+    a WCSR handle reads the nonzeros with their columns instead of the packed windows, and multiplies those only."""
+    shared = info["bytes_b_touched"] + info["bytes_c"]
+    if any("wcsr_rows_kernel" in k for k in kernels):
+        es = {2: 4, 3: 1}.get(info["dtype"], 2)
+        return info["nnz"] * (es + 4.0) + (info["m"] + 1) * 4.0 + shared, info["flops_stored"] * info["fill_ratio"]
+    return info["bytes_a"] + info["bytes_idx"] + shared, info["flops_stored"]
+
+
+def roofline_of(info, ms, pk, kernels, name=None):
     """Roofline of one spmm_run: slower of tensor time for the stored flops and HBM time for the
-    model bytes (A values + indices + distinct B rows touched + C).  `traffic` is the DRAM
-    traffic ncu measured for the same launch, where a capture exists."""
-    model_bytes = info["bytes_a"] + info["bytes_idx"] + info["bytes_b_touched"] + info["bytes_c"]
+    model bytes (model_of).  `traffic` is the DRAM traffic ncu measured for the same launch,
+    where a capture exists."""
+    model_bytes, flops = model_of(info, kernels)
     # TF32 = half, 8-bit = twice the measured bf16 rate (nominal ratios)
     tc_peak = pk["bf16_tflops"] * {2: 0.5, 3: 2.0}.get(info["dtype"], 1.0)
     t_hbm = model_bytes / (pk["hbm_gbs"] * 1e9)
-    t_tc = info["flops_stored"] / (tc_peak * 1e12)
+    t_tc = flops / (tc_peak * 1e12)
     t = ms * 1e-3
     if t_hbm >= t_tc:
         ach = model_bytes / t / 1e9
         r = {"bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s", "frac": ach / pk["hbm_gbs"]}
     else:
-        ach = info["flops_stored"] / t / 1e12
+        ach = flops / t / 1e12
         r = {"bound": "tensor", "achieved": ach, "peak": tc_peak, "unit": "TFLOP/s", "frac": ach / tc_peak}
     r.update({"traffic": NCU_DRAM_TRAFFIC.get(name), "peak_source": pk["source"], "model_bytes": model_bytes,
               "t_roof_us": max(t_hbm, t_tc) * 1e6})
@@ -385,15 +430,9 @@ def time_workload(torch, lib, w, steps, warmup, flush):
             wevs.append((e0, e1))
         torch.cuda.synchronize()
         ms_warm = float(np.mean([a.elapsed_time(b) for a, b in wevs]))
-        launches = 1 + (1 if (w["kind"] == "wcsr" and (info["n_split"] + info["n_empty"]) > 0) else 0)
-        if w["kind"] == "bcsr" and info["n_slots"] > 0:
-            launches = 2                                   # K-split: the SpMM kernel and the merge of the parts
-        if w["kind"] == "bcsr" and info["n_stacked_rows"] > 0:
-            # row groups: their own launch, then the remaining block-rows (if any)
-            if lib.spmm_export(h, lib.X_BCSR_STACK_TILES, np.int32).size > 0:
-                launches = 2 if lib.spmm_export(h, lib.X_BCSR_TILES, np.int32).size > 0 else 1
+        kernels = launched_kernels(lib, h, B, C, N)
         return dict(info=info, ms_mean=float(ms.mean()), ms_median=float(np.median(ms)), ms_min=float(ms.min()), ms_warm=ms_warm,
-                    create_ms=create_ms, launches_per_step=launches, B=B, C=C)
+                    create_ms=create_ms, launches_per_step=len(kernels), kernels=kernels, B=B, C=C)
     finally:
         lib.spmm_destroy(h)
 
@@ -445,14 +484,16 @@ def dense_context(torch, flush, m=18944, k=3584, N=65536, steps=5):
 def summarize(name, desc, res, pk, N):
     info = res["info"]
     ms = res["ms_mean"]
-    gf = info["flops_stored"] / (ms * 1e-3) / 1e9
+    gf = model_of(info, res["kernels"])[1] / (ms * 1e-3) / 1e9      # over the stored values that the kernel multiplies
+    rows = any("wcsr_rows_kernel" in k for k in res["kernels"])
     return {
         "workload": name, "description": desc, "ms_per_step": ms, "ms_median": res["ms_median"], "ms_min": res["ms_min"],
         "ms_warm_l2": res["ms_warm"],
+        "kernel": "rows" if rows else ("window" if info["format"] else "bcsr"),
         "gflops_stored": gf, "gflops_useful": 2.0 * info["nnz"] * N / (ms * 1e-3) / 1e9,
         "fill_ratio": info["fill_ratio"], "stored_values": info["stored_values"], "n_units": info["n_units"],
         "create_ms": res["create_ms"], "launches_per_step": res["launches_per_step"],
-        "roofline": roofline_of(info, ms, pk, name),
+        "roofline": roofline_of(info, ms, pk, res["kernels"], name),
     }
 
 
