@@ -78,15 +78,16 @@ int encode_2d(CUtensorMap* map, int dtype, const void* base, uint64_t rows, uint
     return r == CUDA_SUCCESS ? SPMM_OK : cuda_error();
 }
 
-// Ready for every stream when it returns (a copy from pageable memory may still be on its way when cudaMemcpy does).
+// In the order of the default stream: finish_uploads makes what was uploaded ready for every stream (a copy from
+// pageable memory may still be on its way when cudaMemcpy returns).
 template <class T>
 int upload(T** dptr, const void* src, size_t bytes) {
     *dptr = nullptr;
-    if (!dev_alloc_ready_ok(dptr, bytes)) return SPMM_ERR_ALLOC;
-    if (bytes && (cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess))
-        return cuda_error();
+    if (!dev_alloc_ok(dptr, bytes, nullptr)) return SPMM_ERR_ALLOC;
+    if (bytes && cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice) != cudaSuccess) return cuda_error();
     return SPMM_OK;
 }
+int finish_uploads() { return cudaStreamSynchronize(nullptr) == cudaSuccess ? SPMM_OK : cuda_error(); }
 
 }  // namespace
 
@@ -357,6 +358,7 @@ int create_bcsr(spmm_handle_t* out, const CsrView& a, int dtype, int block, cons
     } catch (const std::bad_alloc&) {
         rc = SPMM_ERR_ALLOC;
     }
+    if (!rc && !h->host_only) rc = finish_uploads();
     if (rc) { free_handle(h); return rc; }
     *out = h;
     return SPMM_OK;
@@ -386,6 +388,7 @@ int create_bcsr_device(spmm_handle_t* out, int64_t m, int64_t k, const int64_t* 
             rc = SPMM_ERR_ALLOC;
         }
     }
+    if (!rc) rc = finish_uploads();
     if (rc) { free_handle(h); return rc; }
     *out = h;
     return SPMM_OK;
@@ -541,7 +544,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
                 rc = SPMM_OK;
             }
         }
-        if (!rc && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = cuda_error();
+        if (!rc) rc = finish_uploads();
         if (rc) { free_handle(h); return rc; }
         std::vector<uint8_t>().swap(h->wcsr.packed);
     }
@@ -768,7 +771,7 @@ int upload_schedule(spmm_handle_s* h, const BcsrSchedule& sc, const BcsrSchedule
                 if (cudaDeviceSynchronize() != cudaSuccess) rc = cuda_error();
                 else free_partial(h);
             }
-            if (!rc && !dev_alloc_ready_ok(&h->d_partial, need)) rc = SPMM_ERR_ALLOC;
+            if (!rc && !dev_alloc_ok(&h->d_partial, need, nullptr)) rc = SPMM_ERR_ALLOC;
             if (!rc) h->partial_bytes = need;
         }
         if (!rc) {
@@ -799,7 +802,7 @@ int upload_schedule(spmm_handle_s* h, const BcsrSchedule& sc, const BcsrSchedule
         rc = upload(&h->d_stile_recs, recs.data(), recs.size() * 4);
         if (!rc) rc = upload(&h->d_scta_ptr, ss.cta_ptr.data(), ss.cta_ptr.size() * 4);
     }
-    return rc;
+    return rc ? rc : finish_uploads();
 }
 
 // Tile width, slab width and the tile schedule for dense width N (cached for the last N).
@@ -1171,11 +1174,11 @@ int launch_wcsr_all(spmm_handle_s* h, const void* B, void* C, float* partial, in
     return e == cudaSuccess ? SPMM_OK : cuda_error();
 }
 
-// The handle's workspace for partial tiles or partial rows (grown, never shrunk).  It outlives
-// the run and serves runs on any stream, so it is never a stream-ordered allocation of the run's own stream -- under
-// stream capture that would be a node of the graph, whose memory exists while the graph runs only.  A run that needs
-// to grow it under capture asks for memory outside the pool instead: refused (SPMM_ERR_ALLOC, nothing launched) in
-// the capture modes that forbid an allocation, lasting in the relaxed one.
+// The handle's workspace for partial tiles or partial rows (grown, never shrunk).  It outlives the run and serves runs
+// on any stream, so it is ready for all of them when this returns, and never an allocation on a stream that is
+// captured: that would be a node of the graph, whose memory exists while the graph runs only.  A run that needs to grow
+// it under capture asks for memory outside the pool instead: refused (SPMM_ERR_ALLOC, nothing launched) in the capture
+// modes that forbid an allocation, lasting in the relaxed one.
 int ensure_wcsr_workspace(spmm_handle_s* h, size_t need, cudaStream_t stream) {
     if (need <= h->partial_bytes) return SPMM_OK;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -1188,7 +1191,7 @@ int ensure_wcsr_workspace(spmm_handle_s* h, size_t need, cudaStream_t stream) {
         free_partial(h);
     }
     if (capture == cudaStreamCaptureStatusNone) {
-        if (!dev_alloc_ready_ok(&h->d_partial, need)) return SPMM_ERR_ALLOC;
+        if (!dev_alloc_ready_ok(&h->d_partial, need, stream)) return SPMM_ERR_ALLOC;
     } else {
         if (cudaMalloc(reinterpret_cast<void**>(&h->d_partial), need) != cudaSuccess) {
             cudaGetLastError();

@@ -8,33 +8,27 @@ namespace spmm {
 
 namespace {
 
-struct Pool {
-    cudaMemPool_t pool = nullptr;
-    cudaStream_t service = nullptr;      // carries allocations only (dev_alloc_ready): never waits for a user's work
-};
-
-cudaError_t device_pool(Pool* pool) {
+cudaError_t device_pool(cudaMemPool_t* pool) {
     static std::mutex mu;
-    static Pool pools[kMaxDevices];
+    static cudaMemPool_t pools[kMaxDevices] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
-    if (!pools[dev].pool) {
+    if (!pools[dev]) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
         props.handleTypes = cudaMemHandleTypeNone;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
-        Pool p;
-        e = cudaMemPoolCreate(&p.pool, &props);
+        cudaMemPool_t p = nullptr;
+        e = cudaMemPoolCreate(&p, &props);
         if (e != cudaSuccess) return e;
         unsigned long long keep = kPoolKeepBytes;
-        e = cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p.service, cudaStreamNonBlocking);
+        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
         if (e != cudaSuccess) {
-            cudaMemPoolDestroy(p.pool);
+            cudaMemPoolDestroy(p);
             return e;
         }
         pools[dev] = p;
@@ -43,23 +37,19 @@ cudaError_t device_pool(Pool* pool) {
     return cudaSuccess;
 }
 
-// `stream` null with `ready`: the service stream, waited for.
-cudaError_t alloc_from_pool(void** ptr, size_t bytes, cudaStream_t stream, bool ready) {
+}  // namespace
+
+cudaError_t dev_alloc(void** ptr, size_t bytes, cudaStream_t stream) {
     *ptr = nullptr;
-    Pool pool;
+    cudaMemPool_t pool = nullptr;
     cudaError_t e = device_pool(&pool);
     if (e != cudaSuccess) return e;
-    if (ready) stream = pool.service;
     if (bytes == 0) bytes = 16;
-    e = cudaMallocFromPoolAsync(ptr, bytes, pool.pool, stream);
+    e = cudaMallocFromPoolAsync(ptr, bytes, pool, stream);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        cudaMemPoolTrimTo(pool.pool, 0);
-        e = cudaMallocFromPoolAsync(ptr, bytes, pool.pool, stream);
-    }
-    if (e == cudaSuccess && ready) {
-        e = cudaStreamSynchronize(stream);
-        if (e != cudaSuccess) cudaFreeAsync(*ptr, stream);
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(ptr, bytes, pool, stream);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -68,24 +58,30 @@ cudaError_t alloc_from_pool(void** ptr, size_t bytes, cudaStream_t stream, bool 
     return e;
 }
 
-}  // namespace
-
-cudaError_t dev_alloc(void** ptr, size_t bytes, cudaStream_t stream) { return alloc_from_pool(ptr, bytes, stream, false); }
-
-cudaError_t dev_alloc_ready(void** ptr, size_t bytes) { return alloc_from_pool(ptr, bytes, nullptr, true); }
+cudaError_t dev_alloc_ready(void** ptr, size_t bytes, cudaStream_t stream) {
+    cudaError_t e = dev_alloc(ptr, bytes, stream);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamSynchronize(stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        dev_free(*ptr, stream);
+        *ptr = nullptr;
+    }
+    return e;
+}
 
 void dev_free(void* ptr, cudaStream_t stream) {
     if (ptr) cudaFreeAsync(ptr, stream);
 }
 
 void dev_give_back(size_t keep) {
-    Pool pool;
+    cudaMemPool_t pool = nullptr;
     unsigned long long reserved = 0;
     if (device_pool(&pool) != cudaSuccess ||
-        cudaMemPoolGetAttribute(pool.pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess || reserved <= keep)
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess || reserved <= keep)
         return;
     cudaStreamSynchronize(nullptr);              // the frees count once they are known to have happened
-    cudaMemPoolTrimTo(pool.pool, keep);
+    cudaMemPoolTrimTo(pool, keep);
 }
 
 cudaError_t dev_malloc(void** ptr, size_t bytes) {

@@ -17,9 +17,10 @@ constexpr size_t kPoolKeepBytes = size_t{256} << 20;
 // Like cudaMalloc for use on `stream` (after it has been synchronised: anywhere); bytes = 0 gives a valid
 // small allocation.  The current device's pool.
 cudaError_t dev_alloc(void** ptr, size_t bytes, cudaStream_t stream);
-// The same, ready for every stream when the call returns (as after cudaMalloc): for memory that a handle keeps, whose
-// runs may come on any stream.
-cudaError_t dev_alloc_ready(void** ptr, size_t bytes);
+// The same, and `stream` is synchronised: ready for every stream when the call returns (as after cudaMalloc), for
+// memory that a handle keeps, whose runs may come on any stream.  (A stream of the library's own in its place need
+// not wait for the caller's work, but does not reuse what was freed on the others.)
+cudaError_t dev_alloc_ready(void** ptr, size_t bytes, cudaStream_t stream);
 // Null is accepted.  The memory must not be in use by work outside `stream`'s order.
 void dev_free(void* ptr, cudaStream_t stream);
 // After frees on the default stream: what the pool holds beyond kPoolKeepBytes and nobody uses goes back to the
@@ -34,8 +35,8 @@ inline bool dev_alloc_ok(T** ptr, size_t bytes, cudaStream_t stream) {
 }
 
 template <class T>
-inline bool dev_alloc_ready_ok(T** ptr, size_t bytes) {
-    return dev_alloc_ready(reinterpret_cast<void**>(ptr), bytes) == cudaSuccess;
+inline bool dev_alloc_ready_ok(T** ptr, size_t bytes, cudaStream_t stream) {
+    return dev_alloc_ready(reinterpret_cast<void**>(ptr), bytes, stream) == cudaSuccess;
 }
 
 }  // namespace spmm
