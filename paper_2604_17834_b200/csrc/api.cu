@@ -1075,6 +1075,7 @@ RowsShape rows_shape(const spmm_handle_s* h, const void* B, const void* C, int64
 // and are made narrower where it does not hold one (sums do not depend on the cut).  A tile of one vector takes
 // kRowsMaxSlots * 32 bytes at most, which the built-in scratch holds.
 int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partial, size_t cap, int64_t N, cudaStream_t stream) {
+    if (g_wait_limit_ns.load() == 0) return launch_wcsr_rows_give_up(h->d_status, stream) == cudaSuccess ? SPMM_OK : cuda_error();
     const WcsrRowStream& r = h->rows;
     RowsShape s = rows_shape(h, B, C, N);
     if (rows_partial_bytes(h, s, 1) > cap) {
@@ -1097,8 +1098,6 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     p.B = B;
     p.C = C;
     p.N = N;
-    p.status = h->d_status;
-    p.give_up = g_wait_limit_ns.load() == 0 ? 1 : 0;
     p.n_tasks = r.n_tasks;
     p.n_parts = r.n_parts;
     int step = std::min(s.tiles, kRowsMaxTiles);

@@ -486,10 +486,11 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     int32_t crow = static_cast<int32_t>(row0) + c0;
                     if constexpr (H != B) crow = __shfl_sync(0xffffffffu, member, c0 / B) * B + (c0 % B);
                     if constexpr (H != B && FMT == 2) {
-                        bool nan = false;
+                        float most = 0.f;                     // NaN if any value is
 #pragma unroll
-                        for (int j = 0; j < W; ++j) nan |= __uint_as_float(v[j]) != __uint_as_float(v[j]);
-                        if (__any_sync(0xffffffffu, nan)) {
+                        for (int j = 0; j < W; j += 2)
+                            asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(most) : "f"(__uint_as_float(v[j])), "f"(__uint_as_float(v[j + 1])));
+                        if (__any_sync(0xffffffffu, most != most)) {
 #pragma unroll
                             for (int j = 0; j < W; ++j)
                                 if (__uint_as_float(v[j]) != __uint_as_float(v[j]) && crow + j < p.m && nw + lane < N)

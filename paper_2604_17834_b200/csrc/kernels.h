@@ -188,8 +188,6 @@ struct WcsrRowsParams {
     const void* B;
     void* C;
     int64_t N;
-    int* status;
-    int32_t give_up;             // the wait limit is zero: leave at once and report a wait that ran out (below)
     int32_t n_tasks, n_parts;
     int32_t lanes, groups, tile0;    // set by launch_wcsr_rows
 };
@@ -201,6 +199,10 @@ struct RowsShape { int vec, lanes, tiles, tile_cols; };
 RowsShape wcsr_rows_shape(int64_t N, int es, bool aligned32);
 // bf16, fp16, tf32.  Column tiles [tile0, tile0 + tiles), at most kRowsMaxTiles of them.
 cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, cudaStream_t stream);
+
+// In the row kernel's place where the wait limit is zero, which makes the kernels that wait give up at their first wait:
+// the row kernel waits for nothing, and this reports to `status` what they would.
+cudaError_t launch_wcsr_rows_give_up(int* status, cudaStream_t stream);
 
 // Device address and size in bytes of the library's built-in partial-tile scratch on the
 // current device (resolved on the first call per device).

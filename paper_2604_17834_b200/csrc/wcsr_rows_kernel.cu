@@ -34,7 +34,6 @@ namespace {
 
 constexpr int kWarps = kRowsThreads / 32;
 constexpr int kStrands = 16;            // partial sums of a part: strand = (entry / 8) % kStrands, whatever the dense width
-constexpr int kGiveUpSite = 31;         // in the status word, where other kernels name the wait that ran out
 constexpr int kNoCol = 0x7fffffff;      // an entry without a gather: row without nonzeros, or padding
 
 template <int VB> struct Vec { uint32_t w[VB / 4]; };
@@ -152,16 +151,6 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     __shared__ unsigned arrived;
 
     grid_trigger();
-    // This kernel waits for nothing of its own.  With a wait limit of zero, which makes the kernels that do wait give
-    // up at their first wait, it does what they do: it leaves early and says so.
-    if (p.give_up) {
-        grid_wait();
-        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && atomicCAS(p.status, 0, 1) == 0) {
-            p.status[1] = kGiveUpSite;
-            p.status[2] = 0;
-        }
-        return;
-    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane / p.lanes, l = lane - g * p.lanes;
     const int tile = p.tile0 + blockIdx.y;
@@ -283,6 +272,15 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     }
 }
 
+__global__ void wcsr_rows_give_up_kernel(int* status) {
+    grid_trigger();
+    grid_wait();
+    if (atomicCAS(status, 0, 1) == 0) {
+        status[1] = 31;                                   // (where other kernels name the wait that ran out)
+        status[2] = 0;
+    }
+}
+
 template <int VB>
 cudaError_t launch_vb(int dtype, int c16, const WcsrRowsParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
     auto go = [&](auto kfn) { return launch_dependent(kfn, grid, kRowsThreads, smem, stream, p); };
@@ -311,6 +309,10 @@ RowsShape wcsr_rows_shape(int64_t N, int es, bool aligned32) {
     s.tiles = static_cast<int>((vecs + s.lanes - 1) / s.lanes);
     s.tile_cols = s.lanes * (s.vec / es);
     return s;
+}
+
+cudaError_t launch_wcsr_rows_give_up(int* status, cudaStream_t stream) {
+    return launch_dependent(wcsr_rows_give_up_kernel, dim3(1), 1, 0, stream, status);
 }
 
 cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, cudaStream_t stream) {
