@@ -250,7 +250,7 @@ typedef enum {
     SPMM_X_WCSR_VALUES = 12,        /* dtype [h][P] row-major                                 */
     SPMM_X_WCSR_TASKS = 13,         /* int32 [n_tasks][4]: window, first col in window,
                                        column count, partial slot (-1 = writes C directly)    */
-    SPMM_X_WCSR_BIN_PTR = 14,       /* int32 [n_bins+1]: ranges of BIN_TASKS, n_bins = 2*n_ctas */
+    SPMM_X_WCSR_BIN_PTR = 14,       /* int32 [n_bins+1]: ranges of BIN_TASKS (n_bins of spmm_info_t) */
     SPMM_X_WCSR_BIN_TASKS = 15,     /* int32 [n_tasks]: task indices bin by bin (the static
                                        schedule: CTA c runs bins c, c + grid, ...)            */
     SPMM_X_WCSR_GROUP_CLASS = 16    /* uint8 [P / 4]: reuse class of every four padded columns
@@ -334,8 +334,8 @@ int spmm_bcsr_plan(spmm_handle_t h, int64_t N);
 /*
  * Both formats (an addition of this library): do ahead of time what the first spmm_run with a
  * new dense width N would do besides launching -- BCSR: spmm_bcsr_plan (schedule, its device
- * arrays, the workspace of a K-split plan); WCSR: grow the handle's partial-tile workspace to
- * what N needs.  May allocate and synchronise the device.  Afterwards spmm_run(h, ., ., N', .)
+ * arrays, the workspace of a K-split plan); WCSR: grow the handle's workspace to what either
+ * kernel needs at any width up to N.  May allocate and synchronise the device.  Afterwards spmm_run(h, ., ., N', .)
  * with N' = N (BCSR) or N' <= N (WCSR) makes no allocating or synchronising call of its own
  * (the CUDA runtime may still load a kernel variant's code on that variant's first launch).
  * Same argument rules as spmm_run for N; a host_only WCSR handle returns SPMM_OK and does nothing.

@@ -8,7 +8,7 @@
 // round trip of a stage.  With about one nonzero per column the same gathers can go straight into
 // registers: no stage, no hand-shake, no padded values, and a product of a row of B with one scalar.
 // What bounds this kernel is the latency and the L1 data path of the gathered rows (long-scoreboard
-// stalls, L1 data pipe 65 % busy on an R-MAT graph of 2^19 rows, fp16, N = 128; DRAM 23 %).
+// stalls, L1 data pipe 67 % busy on an R-MAT graph of 2^19 rows, fp16, N = 128; DRAM 23 %).
 //
 // Work split.  A column tile is `lanes` vectors of VB bytes of B; a warp holds 32 / lanes groups.
 // One group takes one task (whole rows) and walks its nonzeros four at a time: the columns and
