@@ -337,23 +337,37 @@ def device_B(torch, w, seed=7):
 
 def launched_kernels(lib, h, B, C, N):
     """Names of the kernels one spmm_run launches, from a stream capture of it (nothing is executed)."""
+    import ctypes
     import torch
-    from cuda.bindings import driver as drv
-    from cuda.bindings import runtime as rt
+
+    class KernelNodeParams(ctypes.Structure):        # CUDA_KERNEL_NODE_PARAMS_v2
+        _fields_ = [("func", ctypes.c_void_p), ("dims", ctypes.c_uint * 7), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                    ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+    cu = ctypes.CDLL("libcuda.so.1")
     stream = torch.cuda.Stream()
-    if rt.cudaStreamBeginCapture(stream.cuda_stream, rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)[0]:
+    st, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    if cu.cuStreamBeginCapture_v2(st, 2):            # CU_STREAM_CAPTURE_MODE_RELAXED
         raise RuntimeError("stream capture failed")
     try:
         lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, stream.cuda_stream)
     finally:
-        err, graph = rt.cudaStreamEndCapture(stream.cuda_stream)
-    n = rt.cudaGraphGetNodes(graph, 0)[-1]
+        cu.cuStreamEndCapture(st, ctypes.byref(graph))
+    cu.cuGraphGetNodes(graph, None, ctypes.byref(n))
+    nodes = (ctypes.c_void_p * n.value)()
+    if n.value:
+        cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n))
     names = []
-    for node in rt.cudaGraphGetNodes(graph, n)[1] if n else []:
-        err, p = drv.cuGraphKernelNodeGetParams(drv.CUgraphNode(int(node)))
-        err, name = drv.cuKernelGetName(p.kern) if int(p.kern) else drv.cuFuncGetName(p.func)
-        names.append(name.decode())
-    rt.cudaGraphDestroy(graph)
+    for x in nodes:
+        p, name = KernelNodeParams(), ctypes.c_char_p()
+        if cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(x), ctypes.byref(p)):
+            continue                                 # (not a kernel)
+        if p.kern:
+            cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern))
+        elif p.func:
+            cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func))
+        names.append((name.value or b"").decode())
+    cu.cuGraphDestroy(graph)
     return names
 
 

@@ -99,30 +99,34 @@ def assert_close(C_gpu, C_ref, S, dtype, what=""):
 def captured_run(lib, h, B, C, N, relaxed=False, replay=False, static=False):
     """One spmm_run (static: spmm_wcsr_run_static) inside a stream capture of its own stream.  -> (status code of the run, kinds of the captured
     nodes, or None where the capture gave no graph).  replay: launch the graph once, unless the run was refused."""
+    import ctypes
     import torch
-    from cuda.bindings import runtime as rt
+    cu = ctypes.CDLL("libcuda.so.1")
     torch.cuda.synchronize()
     stream = torch.cuda.Stream()
-    mode = rt.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed if relaxed else rt.cudaStreamCaptureMode.cudaStreamCaptureModeGlobal
-    assert rt.cudaStreamBeginCapture(stream.cuda_stream, mode)[0] == rt.cudaError_t.cudaSuccess
+    st, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    assert cu.cuStreamBeginCapture_v2(st, 2 if relaxed else 0) == 0          # CU_STREAM_CAPTURE_MODE_RELAXED / _GLOBAL
     code = lib.SPMM_OK
     try:
         (lib.spmm_wcsr_run_static if static else lib.spmm_run)(h, B.data_ptr(), C.data_ptr(), N, stream.cuda_stream)
     except lib.SpmmError as e:
         code = e.code
-    err, graph = rt.cudaStreamEndCapture(stream.cuda_stream)
-    rt.cudaGetLastError()
-    if err != rt.cudaError_t.cudaSuccess or int(graph) == 0:
+    if cu.cuStreamEndCapture(st, ctypes.byref(graph)) != 0 or not graph.value:
         return code, None
-    n = rt.cudaGraphGetNodes(graph, 0)[-1]
-    nodes = rt.cudaGraphGetNodes(graph, n)[1] if n else []
-    kinds = [str(rt.cudaGraphNodeGetType(x)[1]).split(".")[-1].split("NodeType")[-1].split(":")[0].strip().lower() for x in nodes]
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert n.value == 0 or cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)) == 0
+    kinds = []
+    for x in nodes:
+        t = ctypes.c_int(-1)
+        assert cu.cuGraphNodeGetType(ctypes.c_void_p(x), ctypes.byref(t)) == 0
+        kinds.append("kernel" if t.value == 0 else "type %d" % t.value)      # CU_GRAPH_NODE_TYPE_KERNEL
     if replay and code == lib.SPMM_OK:
-        err, ex = rt.cudaGraphInstantiate(graph, 0)
-        assert err == rt.cudaError_t.cudaSuccess
-        assert rt.cudaGraphLaunch(ex, stream.cuda_stream)[0] == rt.cudaError_t.cudaSuccess
+        ex = ctypes.c_void_p()
+        assert cu.cuGraphInstantiateWithFlags(ctypes.byref(ex), graph, ctypes.c_ulonglong(0)) == 0
+        assert cu.cuGraphLaunch(ex, st) == 0
         stream.synchronize()
         lib.spmm_check(h)
-        rt.cudaGraphExecDestroy(ex)
-    rt.cudaGraphDestroy(graph)
+        cu.cuGraphExecDestroy(ex)
+    cu.cuGraphDestroy(graph)
     return code, kinds

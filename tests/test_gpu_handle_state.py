@@ -55,14 +55,19 @@ def test_a_run_under_capture_never_takes_its_workspace_from_the_graph(lib, kind)
         lib.spmm_destroy(h)
 
 
-@pytest.mark.parametrize("kind", ["rows", "window"])
+@pytest.mark.parametrize("kind", ["rows", "window", "bcsr", "bcsr_ksplit"])
 def test_a_relaxed_capture_allocates_outside_the_graph(lib, kind):
-    """cudaStreamCaptureModeRelaxed allows allocations: the workspace is then ordinary memory that outlives the graph."""
+    """cudaStreamCaptureModeRelaxed allows allocations: workspaces and schedules are then ordinary memory that
+    outlives the graph."""
     import torch
     dtype, N = "fp16", 96
-    a = _long_rows(dtype, seed=4) if kind == "rows" else wl.random_csr(52, 1000, 900, 0.3, dtype)
-    h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16,
-                                 **({} if kind == "rows" else dict(split_cols=64)))
+    if kind.startswith("bcsr"):
+        a = wl.bcsr_sweep(97, m=1024, k=1024, b=64, density=0.05, dtype=dtype)
+        h = lib.spmm_bcsr_create_csr(1024, 1024, a["row_ptr"], a["col_idx"], a["vals"], dtype, 64, k_split=1 if kind == "bcsr_ksplit" else 0)
+    else:
+        a = _long_rows(dtype, seed=4) if kind == "rows" else wl.random_csr(52, 1000, 900, 0.3, dtype)
+        h = lib.spmm_wcsr_create_csr(a["m"], a["k"], a["row_ptr"], a["col_idx"], a["vals"], dtype, 16,
+                                     **({} if kind == "rows" else dict(split_cols=64)))
     try:
         Bs = wl.dense(9, a["k"], N, ("normal", 0.0, 1.0), dtype)
         B = to_device(Bs)
