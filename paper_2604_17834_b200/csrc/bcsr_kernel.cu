@@ -227,8 +227,12 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // The row groups' launch (overlap = 1): the launch of the remaining block-rows runs beside this one (the two
     // write disjoint rows of C), so it is let go only when the operands are ready.
     if (p.overlap != 1) grid_trigger();
-    if (p.overlap != 2) grid_wait();
-    if (p.overlap == 1) grid_trigger();
+    // What a role does before this is with the handle's own data only (complete on every stream once the handle
+    // exists): the producers request their first stored blocks, see below.
+    auto operands_ready = [&]() {
+        if (p.overlap != 2) grid_wait();
+        if (p.overlap == 1) grid_trigger();
+    };
     // Next tile of this warp's walk; nth = number of tiles it has taken so far.  A tile's record
     // {block-row, token tile, first stored block, end block} is all a role needs to know about
     // it; with the static schedule the following tile's record is requested one tile ahead
@@ -285,6 +289,47 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int4 tcd, tcd_next;
             int Jl_next = 0;                 // block columns of the next tile's first 32 blocks, fetched a tile ahead
             bool have_next = false;
+            // the stage of unit it: its byte count, then its stored blocks q .. q + nb - 1 (columns kx .. of them)
+            auto request_blocks = [&](uint32_t it, int q, int kx, int nb, int nvalid) {
+                const int s = it % STAGES;
+                const uint32_t sb = smem_base + s * Cfg::kStageBytes;
+                const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
+                // the A request always brings kBps blocks (the box of the tensor map)
+                const uint32_t dense_tx = CM ? ((p.use_3d && nvalid == Cfg::kBnT) ? Cfg::kDenseBytes : ((nvalid + 127) >> 7) * (128 * Cfg::kBB))
+                                             : nbox * Cfg::kBoxBytes;
+                // (stacked blocks: one request per block, a box holds at most 256 rows)
+                if (lane == 0) mbar_arrive_expect_tx(full_bar(s), (H == B ? Cfg::kBps : nb) * Cfg::kABytes + nb * dense_tx);
+                __syncwarp();
+                if constexpr (H == B) {
+                    if (lane == 8) {
+                        tma_load_2d_hint(sb + Cfg::kAOff, &tmA, full_bar(s), kx, q * B, keep);
+                    } else if (Cfg::kBB > 128 && lane == 9) {
+                        tma_load_2d_hint(sb + Cfg::kAOff + B * 128, &tmA, full_bar(s), 128 / ES, q * B, keep);
+                    }
+                } else {
+                    if (lane >= 8 && lane < 8 + nb)
+                        tma_load_2d_hint(sb + Cfg::kAOff + (lane - 8) * Cfg::kABytes, &tmA, full_bar(s), 0, (q + lane - 8) * H, keep);
+                }
+            };
+            // The first tile's first units: their block columns and stored blocks belong to the handle and are
+            // fetched while the launch before this one may still be running (a short launch is a chain of index,
+            // request, MMA and store latencies, and the weights of a decode step come from HBM); the units' B tiles
+            // follow in the loop below, whose waits for these fresh stages cannot run out.  Back to back, us: 512 x
+            // 512, N = 256 4.13 -> 3.82; both projections 18944 x 3584, bf16, N = 128 19.4 -> 17.7; 8192 x 8192,
+            // b = 16, N = 4096 222 -> 216; prefill shapes unchanged.
+            uint32_t early = 0;
+            if (!DYN && tile_begin < tile_end && rec0.w > rec0.z) {
+                Jl_next = (rec0.z + lane < rec0.w) ? __ldg(p.block_col_idx + rec0.z + lane) : 0;
+                have_next = true;
+                const int nq = min(32, rec0.w - rec0.z);
+                early = min(STAGES, (nq + Cfg::kBps - 1) / Cfg::kBps * Cfg::kKS);
+                const int nvalid = static_cast<int>(min_i64(Cfg::kBnT, N - rec0.y * Cfg::kBnT));
+                for (uint32_t u = pw; u < early; u += NP) {
+                    const int jq = static_cast<int>(u) / Cfg::kKS * Cfg::kBps;
+                    request_blocks(u, rec0.z + jq, static_cast<int>(u) % Cfg::kKS * Cfg::kKB, min(Cfg::kBps, nq - jq), nvalid);
+                }
+            }
+            operands_ready();
             for (uint32_t nth = 0; ok && next_tile(nth, &tcd, &tcd_next, &ok); ++nth) {
                 const int n0 = tcd.y * Cfg::kBnT;
                 const int nvalid = static_cast<int>(min_i64(Cfg::kBnT, N - n0));
@@ -312,12 +357,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const uint32_t ph = (it / STAGES) & 1u;
                         if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, ctl, 1))) { ok = false; break; }
                         const uint32_t sb = smem_base + s * Cfg::kStageBytes;
-                        // the A request always brings kBps blocks (the box of the tensor map)
-                        const uint32_t dense_tx = CM ? (whole_tile ? Cfg::kDenseBytes : ((nvalid + 127) >> 7) * (128 * Cfg::kBB))
-                                                     : nbox * Cfg::kBoxBytes;
-                        // (stacked blocks: one request per block, a box holds at most 256 rows)
-                        if (lane == 0) mbar_arrive_expect_tx(full_bar(s), (H == B ? Cfg::kBps : nb) * Cfg::kABytes + nb * dense_tx);
-                        __syncwarp();
+                        if (it >= early) request_blocks(it, q, kx, nb, nvalid);
                         if constexpr (CM) {
                             // X as [N / 128][128][k]: box = GROUPS x 128 tokens x min(b, 64) elements
                             // of block column J (b = 128: lanes nb.. fetch the second K half)
@@ -349,16 +389,6 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                     tma_load_2d_hint(sb + i * Cfg::kDenseBytes + lane * Cfg::kBoxBytes, &tmB, full_bar(s),
                                                      n0 + lane * Cfg::kTokBox, J * B + kx, keep);
                             }
-                        }
-                        if constexpr (H == B) {
-                            if (lane == 8) {
-                                tma_load_2d_hint(sb + Cfg::kAOff, &tmA, full_bar(s), kx, q * B, keep);
-                            } else if (Cfg::kBB > 128 && lane == 9) {
-                                tma_load_2d_hint(sb + Cfg::kAOff + B * 128, &tmA, full_bar(s), 128 / ES, q * B, keep);
-                            }
-                        } else {
-                            if (lane >= 8 && lane < 8 + nb)
-                                tma_load_2d_hint(sb + Cfg::kAOff + (lane - 8) * Cfg::kABytes, &tmA, full_bar(s), 0, (q + lane - 8) * H, keep);
                         }
                     }
                 }
@@ -448,6 +478,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         uint32_t chunk = 0;                         // staging tiles this warp has filled so far
         const uint32_t stg0 = smem_base + STAGES * Cfg::kStageBytes + (warp - 2) * (Cfg::kEpiBufs * Cfg::kEpiTileBytes);
         bool ok = true;
+        operands_ready();
         int4 tcd, tcd_next;
         for (; ok && next_tile(tile_i, &tcd, &tcd_next, &ok); ++tile_i) {
             const int tI = tcd.x;
