@@ -682,6 +682,10 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
 // Store map of C for the BCSR epilogue (shared-memory staging tile -> TMA store).
 int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
     if (h->tmC_ptr == C && h->tmC_N == N) return SPMM_OK;
+    if (h->col_major && h->c16) {            // stored without a map; the kernel is given a valid one all the same
+        h->tmC = h->tmB;
+        return SPMM_OK;
+    }
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return cuda_error();
     const uint32_t w = static_cast<uint32_t>(bcsr_epi_cols(h->bcsr.b, h->c16, h->col_major));

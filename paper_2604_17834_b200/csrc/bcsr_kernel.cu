@@ -21,7 +21,8 @@
 //               per warp as fit beside the stage ring, so that the warp fills the next tile
 //               while earlier TMA stores are still reading theirs) -> one TMA store per tile,
 //               which also clips at the edges of C (zeros for empty block-rows); overlaps the
-//               next tile's MMAs thanks to the second TMEM buffer.
+//               next tile's MMAs thanks to the second TMEM buffer.  (Column-major 16-bit results:
+//               straight from the registers, see BcsrCfg::kDirect.)
 // Value types (FMT): fp16, bf16 (K = 16 per MMA), TF32 (fp32 storage, K = 8; the token tile then
 // uses the 128-byte swizzle with 32-byte atoms, and blocks wider than 32 columns pass through the
 // ring in 32-column slices), E4M3 (K = 32): a K step is 32 bytes of an operand row in all of them.
@@ -33,7 +34,7 @@
 //            linear layer Y = X W^T, Sec. 4.4): B is given as X[N][k] (one row per token, k
 //            contiguous) and C as Y[N][m].  The token tile is then a K-major MMA operand
 //            (rows of min(b, 64) elements, swizzle = row bytes; b = 128 as two K halves), and
-//            the staging tile is [32 tokens][16 or 32 columns of Y].
+//            the staging tile is [32 tokens][16 columns of Y] (fp32).
 //   DYN = 1  dynamic tile scheduling with Cluster Launch Control (the direction Sec. 5 points
 //            to after the paper's atomic-counter scheduler lost to the hardware block
 //            scheduler, Sec. 3.6): the grid has one CTA per tile, in the schedule's global order
@@ -91,11 +92,17 @@ struct BcsrCfg {
     // operand stream comes first: a deeper stage ring gains more than more staging), at most
     // eight.  With more than one tile a warp fills the next tile while earlier TMA stores are
     // still reading theirs.
+    // Column-major 16-bit results leave straight from the registers instead: a lane holds consecutive elements of its
+    // token's row of Y, whole 128-byte lines of it at b >= 64, and does not wait for a staging tile (the 512-token
+    // shapes have room for one per warp).  Up-projection 18944 x 3584, density 0.1, bf16, N = 9001: 195.6 -> 176.6 us
+    // (3584 x 18944, eight times the blocks per tile, 151 either way).  fp32 results keep the staging tiles: E4M3,
+    // N = 2048, 44.0 us with them, 45.5 without.
+    static constexpr bool kDirect = CM != 0 && CS == 2;
     static constexpr int kEpiCols = bcsr_epi_cols(B, CS == 2, CM != 0);
     static constexpr int kEpiTileBytes = kEpiCols * 32 * CS;
     static constexpr int kEpiRoom = (227 * 1024 - 1024 /*align*/ - kBarrierBytes - STAGES * kStageBytes) / (4 * kEpiTileBytes);
     static constexpr int kEpiBufs = kEpiRoom < 8 ? kEpiRoom : 8;
-    static constexpr int kStagingBytes = 4 * kEpiBufs * kEpiTileBytes;
+    static constexpr int kStagingBytes = kDirect ? 0 : 4 * kEpiBufs * kEpiTileBytes;
     static constexpr int kSmemBytes = STAGES * kStageBytes + kStagingBytes + 1024 /*align*/ + kBarrierBytes;
     static_assert(kEpiBufs >= 1 && kEpiBufs <= 8, "no room for the epilogue's staging tiles");
     static_assert(kEpiCols <= B && H % kEpiCols == 0, "a staging tile never straddles two block-rows");
@@ -478,6 +485,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         uint32_t chunk = 0;                         // staging tiles this warp has filled so far
         const uint32_t stg0 = smem_base + STAGES * Cfg::kStageBytes + (warp - 2) * (Cfg::kEpiBufs * Cfg::kEpiTileBytes);
         bool ok = true;
+        [[maybe_unused]] const bool wide = ((reinterpret_cast<uintptr_t>(p.C) | static_cast<uintptr_t>(p.m * sizeof(CElem))) & 31) == 0;
         operands_ready();
         int4 tcd, tcd_next;
         for (; ok && next_tile(tile_i, &tcd, &tcd_next, &ok); ++tile_i) {
@@ -498,7 +506,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const bool part = tI < 0;
             const int64_t row0 = static_cast<int64_t>(part ? -1 - tI : tI) * B;
             const CUtensorMap* tm_out = part ? &tmP : &tmC;
-            constexpr int W = Cfg::kEpiCols;                // accumulator columns per staging tile
+            constexpr int W = Cfg::kDirect ? (B < 64 ? B : 64) : Cfg::kEpiCols;     // accumulator columns at a time
             for (int g = 0; g < ngrp; ++g) {
                 const int nw = n0 + g * 128 + qd * 32;          // first token of this warp
                 if (nw >= N) break;                             // the whole warp is beyond the last token
@@ -530,6 +538,31 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             __syncwarp();
                         }
                     }
+                    if constexpr (Cfg::kDirect) {
+                        // this lane's token: W consecutive columns of its row of Y, straight from the registers in
+                        // pieces of 32 bytes (16 where a row or the end of Y does not allow it)
+                        constexpr int kPer = 32 / static_cast<int>(sizeof(CElem));
+                        if (nw + lane < N) {
+                            CElem* dst = static_cast<CElem*>(p.C) + (nw + lane) * p.m + crow;
+#pragma unroll
+                            for (int c = 0; c < W; c += kPer) {
+                                uint32_t w8[8];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    const CElem lo = from_f32<CElem>(__uint_as_float(v[c + 2 * i]));
+                                    const CElem hi = from_f32<CElem>(__uint_as_float(v[c + 2 * i + 1]));
+                                    w8[i] = static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&lo)) |
+                                            (static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&hi)) << 16);
+                                }
+                                if (wide && crow + c + kPer <= p.m) {
+                                    st_global_v8(dst + c, w8);
+                                } else {
+                                    if (crow + c + kPer / 2 <= p.m) st_global_v4(dst + c, w8);
+                                    if (crow + c + kPer <= p.m) st_global_v4(dst + c + kPer / 2, w8 + 4);
+                                }
+                            }
+                        }
+                    } else {
                     // registers -> the next tile of this warp's staging ring -> one TMA store.  The
                     // store that used this tile kEpiBufs chunks ago must have read it first.
                     const uint32_t stg = stg0 + (chunk % Cfg::kEpiBufs) * Cfg::kEpiTileBytes;
@@ -549,29 +582,13 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             }
                         }
                     } else {
-                        // tile [32 tokens][W elements]: this lane's row, in 16-byte chunks; 64-byte
-                        // rows are stored with the tensor map's 64-byte swizzle (chunk index XOR
-                        // (row / 2) % 4), which also keeps the warp's stores off each other's banks
-                        constexpr int kChunks = W * static_cast<int>(sizeof(CElem)) / 16;     // 2 or 4
-                        constexpr int kPer = 16 / static_cast<int>(sizeof(CElem));            // elements per chunk
+                        // tile [32 tokens][16 fp32]: this lane's row, in 16-byte chunks; its 64 bytes are stored with
+                        // the tensor map's 64-byte swizzle (chunk index XOR (row / 2) % 4), which also keeps the
+                        // warp's stores off each other's banks
+                        static_assert(W == 16 && sizeof(CElem) == 4, "64-byte rows");
 #pragma unroll
-                        for (int c = 0; c < kChunks; ++c) {
-                            uint32_t w4[4];
-                            if constexpr (sizeof(CElem) == 4) {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) w4[i] = v[c * kPer + i];
-                            } else {
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) {
-                                    const CElem lo = from_f32<CElem>(__uint_as_float(v[c * kPer + 2 * i]));
-                                    const CElem hi = from_f32<CElem>(__uint_as_float(v[c * kPer + 2 * i + 1]));
-                                    w4[i] = static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&lo)) |
-                                            (static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&hi)) << 16);
-                                }
-                            }
-                            const int cs = kChunks == 4 ? (c ^ ((lane >> 1) & 3)) : c;
-                            st_shared_v4(stg + lane * (kChunks * 16) + (cs << 4), w4[0], w4[1], w4[2], w4[3]);
-                        }
+                        for (int c = 0; c < 4; ++c)
+                            st_shared_v4(stg + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
@@ -581,6 +598,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         if constexpr (!CM) tma_store_2d(tm_out, stg, nw, crow);
                         else tma_store_2d(tm_out, stg, crow, nw);
                         bulk_commit_group();
+                    }
                     }
                 }
             }

@@ -62,8 +62,8 @@ struct BcsrParams {
 // (col_major): tmB = X as [N][k], box 128 tokens x min(kb * es, 128) bytes; tmB3 = X as
 // [N / 128][128][k], box groups x 128 x the same; both with the swizzle of that row length.
 // tmA: the stored blocks as [blocks * b][b], box (b * blocks per stage) rows x min(kb * es, 128) bytes.
-// tmC: C as [m][N], box 32 x bcsr_epi_cols, no swizzle; or Y as [N][m], box bcsr_epi_cols x 32,
-// 64-byte swizzle when a box row is 64 bytes.
+// tmC: C as [m][N], box 32 x bcsr_epi_cols, no swizzle; or fp32 Y as [N][m], box 16 x 32, 64-byte swizzle (16-bit Y:
+// any valid map, it is stored without one).
 // dynamic: the grid is one CTA per tile (grid = number of tiles, p.tiles in the schedule's global
 // order, p.cta_ptr unused) and CTAs steal tiles through Cluster Launch Control; fp32 row-major only.
 cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA,
@@ -94,7 +94,7 @@ int bcsr_token_groups_max(int dtype, int b, int c16, int col_major);
 // Accumulator columns (= rows of A's block) an epilogue warp handles at a time: it stages them
 // in a 2 KB (1 KB for b = 16 with 16-bit C) shared-memory tile and stores the tile with one TMA
 // request whose box is 32 tokens x this many rows (row-major C) or this many columns x 32 tokens
-// (column-major Y).  Larger tiles (up to 64 rows) were measured slower: the stage ring needs the room.
+// (column-major fp32 Y).  Larger tiles (up to 64 rows) were measured slower: the stage ring needs the room.
 constexpr int bcsr_epi_cols(int b, bool c16, bool col_major) { return (b < 32 || !c16) ? 16 : 32; }
 // stored blocks that share one pipeline stage (and one A request): 4 / 2 for b = 16 / 32
 constexpr int bcsr_blocks_per_stage(int b) { return b == 16 ? 4 : (b == 32 ? 2 : 1); }
