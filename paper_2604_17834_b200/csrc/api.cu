@@ -534,7 +534,7 @@ int create_wcsr(spmm_handle_t* out, const CsrView& a, int dtype, int wh, const s
             rc = upload(&d_rp, a.row_ptr, static_cast<size_t>(a.m + 1) * 8);
             if (!rc) rc = upload(&d_ci, a.col_idx, static_cast<size_t>(a.nnz) * 4);
             if (!rc) rc = upload(&d_va, a.vals, static_cast<size_t>(a.nnz) * a.es);
-            if (!rc) rc = build_wcsr_rows_device(a.m, a.nnz, d_rp, d_ci, d_va, a.es, h->sms, nullptr, &h->rows);
+            if (!rc) rc = build_wcsr_rows_device(a.m, a.nnz, d_rp, d_ci, d_va, a.es, h->sms, nullptr, nullptr, &h->rows);
             if (!rc) rc = finish_wcsr_rows(&h->rows, nullptr);
             dev_free(d_rp, nullptr);
             dev_free(d_ci, nullptr);

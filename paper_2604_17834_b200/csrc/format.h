@@ -171,9 +171,9 @@ inline int64_t wcsr_rows_load(int64_t m, int64_t nnz, int sms) { return (nnz + m
 constexpr int kRowsMaxSlots = 65536;    // partial rows of long rows cut into parts
 // Builds the stream on the GPU from a (validated) CSR matrix in device memory, in the order of `stream`; leaves
 // *out empty when the matrix has no rows or is too large for 32-bit entry positions, and when it fails.  A handle
-// does without the stream where there is no memory for it (SPMM_ERR_ALLOC).
+// does without the stream where there is no memory for it (SPMM_ERR_ALLOC).  d_row_of: the row of every entry, or null.
 int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
-                           int es, int sms, cudaStream_t stream, WcsrRowStream* out);
+                           int es, int sms, const int32_t* d_row_of, cudaStream_t stream, WcsrRowStream* out);
 // Reads the counts the launches need; synchronises `stream`.  Until then n_tasks = n_parts = 0.
 int finish_wcsr_rows(WcsrRowStream* s, cudaStream_t stream);
 void free_wcsr_rows(WcsrRowStream* s, cudaStream_t stream);

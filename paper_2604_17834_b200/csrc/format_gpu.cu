@@ -14,16 +14,14 @@
 // A bitmap needs 2 * ceil(k / b) / 8 bytes of shared memory (bits + word prefix), at most 200 KB:
 // k / b <= 819,200.
 //
-// WCSR (window condensation of Sec. 2.3): every stored entry becomes the 64-bit key
-// (window << 32 | column); a radix sort and a unique pass (CUB primitives) leave, window after
-// window, the ascending union of each window's columns; where the window changes gives each window's
-// place in the key list, a prefix sum window_row_ptr (lengths padded to b_col);
-// window_col_idx is those columns over a -1 fill, and every value finds its condensed column by
-// binary search in its window's list and goes straight into the packed tile layout.
-#include <cub/cub.cuh>
-
+// WCSR (window condensation of Sec. 2.3): a window's entries are one contiguous range of the CSR arrays, wh ascending
+// runs.  One CTA merges them pair by pair in shared memory; where the merged column changes, a new condensed column
+// begins, so that an entry's rank gives its place in the window (windows too long for that: a bitmap of columns, as
+// above).  A prefix sum of the lengths padded to b_col is window_row_ptr; a last pass, entry by entry, writes the
+// columns over a -1 fill and the values straight into the packed tile layout.
 #include <cstring>
 #include <numeric>
+#include <type_traits>
 #include <algorithm>
 #include <new>
 
@@ -127,42 +125,59 @@ bcsr_count_kernel(int64_t m, int b, int words, const int64_t* row_ptr, const int
     if (threadIdx.x == 0) counts[blockIdx.x] = total;
 }
 
-// out[0] = 0, out[i + 1] = counts[0] + ... + counts[i]; *overflow set if the total passes int32.
-__global__ void __launch_bounds__(1024)
-exclusive_scan_kernel(const int32_t* counts, int64_t n, int32_t* out, int* overflow) {
-    __shared__ long long warp_sum[32];
-    __shared__ long long carry;
-    if (threadIdx.x == 0) { carry = 0; out[0] = 0; }
-    __syncthreads();
+// Exclusive sums over a CTA of 1024 threads, one value each; *total gets the sum of all.  scratch: 33 values.
+__device__ __forceinline__ long long block_exclusive_sum(long long v, long long* scratch, long long* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int64_t base = 0; base < n; base += blockDim.x) {
-        const int64_t i = base + threadIdx.x;
-        long long v = i < n ? counts[i] : 0;
-        long long x = v;
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) warp_sum[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            long long s = warp_sum[lane];
-            for (int o = 1; o < 32; o <<= 1) {
-                const long long y = __shfl_up_sync(0xffffffffu, s, o);
-                if (lane >= o) s += y;
-            }
-            warp_sum[lane] = s;
-        }
-        __syncthreads();
-        const long long incl = carry + (warp ? warp_sum[warp - 1] : 0) + x;
-        if (i < n) {
-            if (incl >= (1ll << 31)) *overflow = 1;
-            out[i + 1] = static_cast<int32_t>(incl);
-        }
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) carry = incl;
-        __syncthreads();
+    long long x = v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
     }
+    __syncthreads();                         // (the scratch may still be read from the call before)
+    if (lane == 31) scratch[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        long long t = scratch[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const long long y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        scratch[lane] = t;
+    }
+    __syncthreads();
+    *total = scratch[31];
+    return (warp ? scratch[warp - 1] : 0) + x - v;
+}
+
+// out[0] = 0, out[i + 1] = c[0] + ... + c[i] with every count rounded up to a multiple of `unit`; *overflow set if the
+// total passes int32.  One CTA of 1024 threads, eight counts a thread and step.
+__device__ __forceinline__ void scan_counts(const int32_t* counts, int64_t n, int unit, int32_t* out, int* overflow) {
+    __shared__ long long scratch[32];
+    constexpr int kPer = 8;
+    long long carry = 0;
+    if (threadIdx.x == 0) out[0] = 0;
+    for (int64_t base = 0; base < n; base += 1024 * kPer) {
+        const int64_t i0 = base + static_cast<int64_t>(threadIdx.x) * kPer;
+        int c[kPer];
+        long long sum = 0, total;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            c[j] = i0 + j < n ? (counts[i0 + j] + unit - 1) / unit * unit : 0;
+            sum += c[j];
+        }
+        long long at = carry + block_exclusive_sum(sum, scratch, &total);
+        carry += total;
+        if (at + sum >= (1ll << 31)) *overflow = 1;
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            at += c[j];
+            if (i0 + j < n) out[i0 + j + 1] = static_cast<int32_t>(at);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(1024) exclusive_scan_kernel(const int32_t* counts, int64_t n, int32_t* out, int* overflow) {
+    scan_counts(counts, n, 1, out, overflow);
 }
 
 template <int ES>
@@ -393,87 +408,213 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
 
 namespace {
 
-// Entry by entry (a warp per row took four times as long: a row of 5000 entries was one warp's work): the row of
-// every entry, looked up in row_ptr, and its key = window << cb | column, cb = bits of a column: no empty bits for
-// the radix sort to pass over.
-// An entry out of range or not ascending in its row sets *bad and counts as column 0.
-__global__ void wcsr_keys_kernel(int64_t m, int64_t k, int wh, int cb, const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                                 uint64_t* __restrict__ keys, int32_t* __restrict__ row_of, int* bad) {
-    const int64_t nnz = row_ptr[m];
-    for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        int64_t lo = 0, hi = m - 1;                       // last row that starts at or before p
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) >> 1;
-            if (row_ptr[mid] <= p) lo = mid; else hi = mid - 1;
+// ---- window condensation
+// Per entry: its row, and its place among the window's condensed columns; per window: how many it has; per column: how
+// many windows hold it.  An entry out of range or not ascending in its row sets *bad and counts as column 0; nothing
+// below leaves its arrays then, and the results are not used.
+struct CondenseParams {
+    int64_t m, k, nwin;
+    const int64_t* row_ptr;
+    const int32_t* col_idx;
+    int32_t* row_of;                         // [nnz]
+    int32_t* pos_of;                         // [nnz]
+    int32_t* ucount;                         // [nwin]
+    int32_t* refs;                           // [k], zero before
+    int* bad;
+    int32_t* big;                            // windows left to the second kernel, and how many
+    int* n_big;
+};
+
+// Entries whose wh runs are merged in shared memory by one CTA: at most kSmallWindow by 128 threads (20 KB, a dozen CTAs
+// per SM), kLargeWindow by 1024 (205 KB).  Against radix sort of 64-bit keys, unique and lookups, 60,000 power-law rows
+// (0.8 M entries): 115 us of kernels for the same arrays, @@.
+constexpr int kSmallWindow = 2048, kLargeWindow = 20480;
+
+__device__ __forceinline__ int32_t checked_column(const CondenseParams& p, int64_t at, int64_t row_start) {
+    const int32_t c = p.col_idx[at];
+    if (c < 0 || c >= p.k || (at > row_start && p.col_idx[at - 1] >= c)) {
+        *p.bad = 1;
+        return 0;
+    }
+    return c;
+}
+
+// off[0 .. rows]: where the rows of the window start, relative to its first entry.
+template <int WH>
+__device__ __forceinline__ int row_in_window(const int* off, int j) {
+    int r = 0;                               // the last row that starts at or before entry j
+#pragma unroll
+    for (int step = WH / 2; step > 0; step >>= 1)
+        if (off[r + step] <= j) r += step;
+    return r;
+}
+
+// n entries from p0 on: keys[2][cap], rank[cap] in shared memory; off has WH + 1 entries.
+template <int WH, int THREADS>
+__device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, int32_t* keys, int cap, uint16_t* rank) {
+    __shared__ int warp_sum[THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int j = threadIdx.x; j < n; j += THREADS) {
+        const int r = row_in_window<WH>(off, j);
+        keys[j] = checked_column(p, p0 + j, p0 + off[r]);
+        rank[j] = static_cast<uint16_t>(j);
+        p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
+    }
+    __syncthreads();
+    int32_t *src = keys, *dst = keys + cap;
+    // runs of 2^level rows: an entry's rank in the merged pair of runs = its place in its own + the entries of the other
+    // that go before it (equal ones: the earlier run first)
+    for (int span = 1; span < WH; span *= 2) {
+        for (int j = threadIdx.x; j < n; j += THREADS) {
+            const int g = row_in_window<WH>(off, j) & ~(span - 1);       // first row of this entry's run
+            const bool right = (g & span) != 0;
+            const int sib = right ? g - span : g + span;
+            const int at = rank[j];
+            const int32_t c = src[at];
+            const int s0 = off[sib];
+            int lo = s0, hi = off[sib + span];
+            const int32_t bound = right ? c : c - 1;                     // entries of the other run up to here go before
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (src[mid] <= bound) lo = mid + 1; else hi = mid;
+            }
+            const int to = at + (right ? lo - off[g] : lo - s0);
+            dst[to] = c;
+            rank[j] = static_cast<uint16_t>(to);
         }
-        int64_t c = col_idx[p];
-        if (c < 0 || c >= k || (p > row_ptr[lo] && col_idx[p - 1] >= c)) {
-            *bad = 1;
-            c = 0;
+        __syncthreads();
+        int32_t* t = src;
+        src = dst;
+        dst = t;
+    }
+    // dst[r] = condensed columns up to and with rank r
+    int carry = 0;
+    for (int base = 0; base < n; base += THREADS) {
+        const int r = base + threadIdx.x;
+        const bool first = r < n && (r == 0 || src[r] != src[r - 1]);
+        if (first && static_cast<uint32_t>(src[r]) < static_cast<uint32_t>(p.k)) atomicAdd(p.refs + src[r], 1);     // (any value, after a bad entry)
+        const unsigned ball = __ballot_sync(0xffffffffu, first);
+        if (lane == 0) warp_sum[warp] = __popc(ball);
+        __syncthreads();
+        int before = carry, all = carry;
+        for (int i = 0; i < THREADS / 32; ++i) {
+            const int x = warp_sum[i];
+            if (i < warp) before += x;
+            all += x;
         }
-        row_of[p] = static_cast<int32_t>(lo);
-        keys[p] = static_cast<uint64_t>(lo / wh) << cb | static_cast<uint64_t>(c);
+        if (r < n) dst[r] = before + __popc(ball & ((2u << lane) - 1u));
+        carry = all;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) p.ucount[w] = carry;
+    for (int j = threadIdx.x; j < n; j += THREADS) p.pos_of[p0 + j] = dst[rank[j]] - 1;
+}
+
+template <int WH>
+__device__ __forceinline__ void load_offsets(const CondenseParams& p, int64_t w, int* off) {
+    const int64_t r0 = w * WH;
+    const int64_t p0 = p.row_ptr[r0];
+    for (int i = threadIdx.x; i <= WH; i += blockDim.x) off[i] = static_cast<int>(p.row_ptr[min(r0 + i, p.m)] - p0);
+}
+
+template <int WH>
+__global__ void __launch_bounds__(128) wcsr_condense_kernel(const CondenseParams p) {
+    __shared__ int32_t keys[2 * kSmallWindow];
+    __shared__ uint16_t rank[kSmallWindow];
+    __shared__ int off[WH + 1];
+    const int64_t w = blockIdx.x;
+    load_offsets<WH>(p, w, off);
+    __syncthreads();
+    const int n = off[WH];
+    if (n > kSmallWindow) {
+        if (threadIdx.x == 0) p.big[atomicAdd(p.n_big, 1)] = static_cast<int32_t>(w);
+        return;
+    }
+    merge_window<WH, 128>(p, w, p.row_ptr[w * WH], n, off, keys, kSmallWindow, rank);
+}
+
+// Windows of more than kLargeWindow entries: bits of the columns [c0, c0 + 32 words) and the set bits before each word.
+template <int WH>
+__device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, uint32_t* bits, int max_words) {
+    __shared__ long long scratch[32];
+    uint32_t* prefix = bits + max_words;
+    int found = 0;                           // condensed columns before c0
+    for (int64_t c0 = 0; c0 < p.k; c0 += int64_t{32} * max_words) {
+        const int words = static_cast<int>(min(static_cast<int64_t>(max_words), (p.k - c0 + 31) / 32));
+        __syncthreads();
+        for (int i = threadIdx.x; i < words; i += 1024) bits[i] = 0u;
+        __syncthreads();
+        for (int j = threadIdx.x; j < n; j += 1024) {
+            const int r = row_in_window<WH>(off, j);
+            const int64_t c = checked_column(p, p0 + j, p0 + off[r]) - c0;
+            if (c0 == 0) p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
+            if (c >= 0 && c < int64_t{32} * words) atomicOr(&bits[c >> 5], 1u << (c & 31));
+        }
+        __syncthreads();
+        long long carry = found;
+        for (int base = 0; base < words; base += 1024) {
+            const int i = base + threadIdx.x;
+            long long total;
+            const long long before = carry + block_exclusive_sum(i < words ? __popc(bits[i]) : 0, scratch, &total);
+            if (i < words) prefix[i] = static_cast<uint32_t>(before);
+            carry += total;
+        }
+        __syncthreads();
+        found = static_cast<int>(carry);
+        for (int j = threadIdx.x; j < n; j += 1024) {
+            const int r = row_in_window<WH>(off, j);
+            const int64_t c = checked_column(p, p0 + j, p0 + off[r]) - c0;
+            if (c < 0 || c >= int64_t{32} * words) continue;
+            p.pos_of[p0 + j] = static_cast<int32_t>(prefix[c >> 5] + __popc(bits[c >> 5] & ((1u << (c & 31)) - 1u)));
+        }
+        for (int i = threadIdx.x; i < words; i += 1024)
+            for (uint32_t x = bits[i]; x; x &= x - 1) atomicAdd(p.refs + c0 + 32 * int64_t{i} + (__ffs(x) - 1), 1);
+    }
+    if (threadIdx.x == 0) p.ucount[w] = found;
+}
+
+constexpr int kLargeSmem = kLargeWindow * 10;                 // two key arrays and the ranks; or bits and their prefixes
+template <int WH>
+__global__ void __launch_bounds__(1024) wcsr_condense_large_kernel(const CondenseParams p) {
+    extern __shared__ int32_t dyn[];
+    __shared__ int off[WH + 1];
+    for (int i = blockIdx.x; i < *p.n_big; i += gridDim.x) {
+        const int64_t w = p.big[i];
+        __syncthreads();
+        load_offsets<WH>(p, w, off);
+        __syncthreads();
+        const int n = off[WH];
+        if (n <= kLargeWindow)
+            merge_window<WH, 1024>(p, w, p.row_ptr[w * WH], n, off, dyn, kLargeWindow, reinterpret_cast<uint16_t*>(dyn + 2 * kLargeWindow));
+        else
+            bitmap_window<WH>(p, w, p.row_ptr[w * WH], n, off, reinterpret_cast<uint32_t*>(dyn), kLargeSmem / 8);
     }
 }
 
-// The unique keys ascend, so a window's keys are a run: where each run starts (ustart[nwin] = their number);
-// per column: is it referenced at all
-__global__ void wcsr_starts_kernel(const uint64_t* __restrict__ ukeys, const int* __restrict__ n_unique, int64_t nwin, int cb,
-                                   int32_t* __restrict__ ustart, uint8_t* __restrict__ used) {
-    const int64_t n = *n_unique;
-    const uint64_t col_mask = (uint64_t{1} << cb) - 1;
-    for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j <= n; j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t w = j < n ? static_cast<int64_t>(ukeys[j] >> cb) : nwin;
-        const int64_t before = j > 0 ? static_cast<int64_t>(ukeys[j - 1] >> cb) : -1;
-        for (int64_t x = before + 1; x <= w; ++x) ustart[x] = static_cast<int32_t>(j);
-        if (j < n) used[ukeys[j] & col_mask] = 1;
+// CTA 0: window_row_ptr; the others: how many columns are referenced at all
+__global__ void __launch_bounds__(1024) wcsr_row_ptr_kernel(const int32_t* ucount, int64_t nwin, int b_col, int32_t* window_row_ptr, int* overflow,
+                                                            const int32_t* __restrict__ refs, int64_t k, unsigned long long* distinct) {
+    if (blockIdx.x == 0) {
+        scan_counts(ucount, nwin, b_col, window_row_ptr, overflow);
+        return;
     }
-}
-
-__global__ void wcsr_pad_kernel(const int32_t* __restrict__ ustart, int64_t nwin, int b_col, int32_t* __restrict__ len) {
-    for (int64_t w = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; w < nwin;
-         w += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        len[w] = (ustart[w + 1] - ustart[w] + b_col - 1) / b_col * b_col;
-}
-
-__global__ void wcsr_sum_used_kernel(const uint8_t* used, int64_t k, unsigned long long* total) {
     unsigned long long n = 0;
-    for (int64_t c = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; c < k;
-         c += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        n += used[c];
+    for (int64_t c = (blockIdx.x - 1) * int64_t{1024} + threadIdx.x; c < k; c += (gridDim.x - 1) * int64_t{1024}) n += refs[c] > 0;
     for (int o = 16; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
-    if ((threadIdx.x & 31) == 0 && n) atomicAdd(total, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(distinct, n);
 }
 
-__global__ void wcsr_cols_kernel(const uint64_t* ukeys, const int* n_unique, int cb, const int32_t* ustart,
-                                 const int32_t* window_row_ptr, int32_t* window_col_idx) {
-    const int64_t n = *n_unique;
-    const uint64_t col_mask = (uint64_t{1} << cb) - 1;
-    for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < n;
-         j += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const uint64_t key = ukeys[j];
-        const int64_t w = static_cast<int64_t>(key >> cb);
-        window_col_idx[window_row_ptr[w] + (j - ustart[w])] = static_cast<int32_t>(key & col_mask);
-    }
-}
-
-// One thread per entry: its column's place in its window's list, by binary search.
+// One thread per entry: its column and its value to their places (entries that share a condensed column write the same).
 template <int ES>
-__global__ void wcsr_values_kernel(int64_t nnz, int wh, int b_col, const int32_t* __restrict__ row_of, const int32_t* __restrict__ col_idx,
-                                   const uint8_t* __restrict__ vals, const int32_t* __restrict__ ustart, const int32_t* __restrict__ window_row_ptr,
-                                   const int32_t* __restrict__ window_col_idx, uint8_t* __restrict__ packed) {
+__global__ void wcsr_place_kernel(int64_t nnz, int wh, int b_col, const int32_t* __restrict__ row_of, const int32_t* __restrict__ pos_of,
+                                  const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ vals, const int32_t* __restrict__ window_row_ptr,
+                                  int32_t* __restrict__ window_col_idx, uint8_t* __restrict__ packed) {
     for (int64_t p = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         const int i = row_of[p];
         const int w = i / wh, r = i - w * wh;
-        const int64_t base = window_row_ptr[w];
-        const int32_t* seg = window_col_idx + base;
-        const int32_t c = col_idx[p];
-        int lo = 0, hi = ustart[w + 1] - ustart[w];      // first position with seg[pos] >= c; c is in the list
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (seg[mid] < c) lo = mid + 1; else hi = mid;
-        }
-        uint8_t* dst = packed + wcsr_packed_offset(wh, b_col, ES, r, base + lo);
+        const int64_t at = static_cast<int64_t>(window_row_ptr[w]) + pos_of[p];
+        window_col_idx[at] = col_idx[p];
+        uint8_t* dst = packed + wcsr_packed_offset(wh, b_col, ES, r, at);
         const uint8_t* src = vals + static_cast<size_t>(p) * ES;
         if constexpr (ES == 1) *dst = *src;
         else if constexpr (ES == 2) *reinterpret_cast<uint16_t*>(dst) = *reinterpret_cast<const uint16_t*>(src);
@@ -496,29 +637,111 @@ __global__ void wcsr_fills_kernel(int64_t n_items, const WcsrDevTask* __restrict
 }
 
 // ---- reuse classes of the column groups (gather hints; the host rule of wcsr_reuse_classes)
+// The class of a row of B is its rank by gather count (ties: the lower index first) against the limits 16 Ki, 32 Ki, ...,
+// so no sort is needed: a histogram of the counts says at which count each limit falls and how many of the rows with just
+// that count are still inside; only those rows' order among themselves has to be found.
 
-__global__ void wcsr_refs_kernel(const int32_t* __restrict__ col_idx, int64_t P, int32_t* __restrict__ refs) {
-    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < P; q += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int32_t c = col_idx[q];
-        if (c >= 0) atomicAdd(refs + c, 1);
+constexpr int kLimits = 7;                   // classes 7 .. 1
+struct ClassCut { int32_t count[kLimits]; int32_t quota[kLimits]; };   // inside limit i: more than count[i] gathers, or one of the first quota[i] rows with just as many
+
+constexpr int kSmallCounts = 1024;
+__global__ void __launch_bounds__(256) wcsr_count_hist_kernel(const int32_t* __restrict__ refs, int64_t k, int32_t* __restrict__ hist) {
+    __shared__ int32_t small[kSmallCounts];
+    for (int i = threadIdx.x; i < kSmallCounts; i += 256) small[i] = 0;
+    __syncthreads();
+    for (int64_t c = blockIdx.x * int64_t{256} + threadIdx.x; c < k; c += gridDim.x * int64_t{256}) {
+        const int n = refs[c];
+        if (n > 1) atomicAdd(n < kSmallCounts ? &small[n] : hist + n, 1);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kSmallCounts; i += 256)
+        if (small[i]) atomicAdd(hist + i, small[i]);
+}
+
+// one CTA: from the highest count down; top = the highest one possible
+__global__ void __launch_bounds__(1024) wcsr_class_cut_kernel(const int32_t* __restrict__ hist, int64_t top, ClassCut* cut) {
+    __shared__ long long scratch[32];
+    if (threadIdx.x < kLimits) {             // (a limit that is not reached: every row gathered more than once is inside)
+        cut->count[threadIdx.x] = 1;
+        cut->quota[threadIdx.x] = 0;
+    }
+    long long above = 0;
+    for (int64_t base = top; base >= 2 && above < (static_cast<long long>(kWcsrTopClassRows) << (kLimits - 1)); base -= 1024) {
+        const int64_t v = base - threadIdx.x;
+        const long long h = v >= 2 ? hist[v] : 0;
+        long long total;
+        const long long before = above + block_exclusive_sum(h, scratch, &total);
+#pragma unroll
+        for (int i = 0; i < kLimits; ++i) {
+            const long long lim = static_cast<long long>(kWcsrTopClassRows) << i;
+            if (before < lim && lim <= before + h) {
+                cut->count[i] = static_cast<int32_t>(v);
+                cut->quota[i] = static_cast<int32_t>(lim - before);
+            }
+        }
+        above += total;
     }
 }
 
-__global__ void iota_kernel(int32_t* __restrict__ x, int64_t n) {
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += static_cast<int64_t>(gridDim.x) * blockDim.x)
-        x[i] = static_cast<int32_t>(i);
+// rows whose count is the one of limit i, per chunk of columns: at [block][i]
+__global__ void __launch_bounds__(256) wcsr_cut_rows_kernel(const int32_t* __restrict__ refs, int64_t k, int64_t chunk, const ClassCut* __restrict__ cut,
+                                                            int32_t* __restrict__ n_rows) {
+    __shared__ int n[kLimits];
+    if (threadIdx.x < kLimits) n[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t c1 = min(k, (blockIdx.x + 1) * chunk);
+    for (int64_t c = blockIdx.x * chunk + threadIdx.x; c < c1; c += 256) {
+        const int x = refs[c];
+        if (x > 1)
+#pragma unroll
+            for (int i = 0; i < kLimits; ++i)
+                if (x == cut->count[i]) atomicAdd(&n[i], 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < kLimits) n_rows[blockIdx.x * kLimits + threadIdx.x] = n[threadIdx.x];
 }
 
-// rows in descending order of their gather count (stable: ties by index): rank r -> class
-__global__ void wcsr_class_kernel(const int32_t* __restrict__ sorted_refs, const int32_t* __restrict__ order, int64_t k,
-                                  uint8_t* __restrict__ cls) {
-    for (int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; r < k; r += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        int level = 0;
-        if (sorted_refs[r] > 1) {
-            level = 7;
-            for (int64_t lim = kWcsrTopClassRows; level > 0 && r >= lim; lim *= 2) --level;
+__global__ void __launch_bounds__(256) wcsr_class_kernel(const int32_t* __restrict__ refs, int64_t k, int64_t chunk, const ClassCut* __restrict__ cut,
+                                                         const int32_t* __restrict__ n_rows, uint8_t* __restrict__ cls) {
+    __shared__ int before[kLimits];          // rows with the count of limit i in the columns before this step's
+    __shared__ int in_warp[8][kLimits];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < kLimits) before[threadIdx.x] = 0;
+    __syncthreads();
+    for (int j = threadIdx.x; j < static_cast<int>(blockIdx.x) * kLimits; j += 256)
+        if (n_rows[j]) atomicAdd(&before[j % kLimits], n_rows[j]);
+    __syncthreads();
+    const int64_t c1 = min(k, (blockIdx.x + 1) * chunk);
+    for (int64_t base = blockIdx.x * chunk; base < c1; base += 256) {
+        const int64_t c = base + threadIdx.x;
+        const int x = c < c1 ? refs[c] : 0;
+        unsigned at_limit = 0;
+        int ordinal[kLimits];
+#pragma unroll
+        for (int i = 0; i < kLimits; ++i) {
+            const unsigned b = __ballot_sync(0xffffffffu, x > 1 && x == cut->count[i]);
+            ordinal[i] = __popc(b & ((1u << lane) - 1u));
+            if (b >> lane & 1u) at_limit |= 1u << i;
+            if (lane == 0) in_warp[warp][i] = __popc(b);
         }
-        cls[order[r]] = static_cast<uint8_t>(level);
+        __syncthreads();
+        int level = 0;
+        if (x > 1)
+#pragma unroll
+            for (int i = kLimits - 1; i >= 0; --i) {
+                bool inside = x > cut->count[i];
+                if (at_limit >> i & 1u) {
+                    int n = before[i] + ordinal[i];
+                    for (int v = 0; v < warp; ++v) n += in_warp[v][i];
+                    inside = n < cut->quota[i];
+                }
+                if (inside) level = kLimits - i;
+            }
+        if (c < c1) cls[c] = static_cast<uint8_t>(level);
+        __syncthreads();
+        if (threadIdx.x < kLimits)
+            for (int v = 0; v < 8; ++v) before[threadIdx.x] += in_warp[v][threadIdx.x];
+        __syncthreads();
     }
 }
 
@@ -535,41 +758,36 @@ __global__ void wcsr_group_class_kernel(const int32_t* __restrict__ col_idx, int
     }
 }
 
-// Allocates and fills *d_grp_class [P / 4] from the device copy of window_col_idx, in the order of `st`.
-int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, int64_t k, int64_t nwin, cudaStream_t st, uint8_t** d_grp_class) {
+// Allocates and fills *d_grp_class [P / 4] from the device copy of window_col_idx and the gather counts refs [k] (each at
+// most nwin), in the order of `st`.
+int wcsr_reuse_classes_device(const int32_t* d_window_col_idx, int64_t P, const int32_t* refs, int64_t k, int64_t nwin, cudaStream_t st,
+                              uint8_t** d_grp_class) {
     *d_grp_class = nullptr;
     if (P <= 0 || k <= 0) return SPMM_OK;
-    int count_bits = 1;                       // a row of B is gathered by nwin windows at most
-    while (count_bits < 31 && (int64_t{1} << count_bits) <= nwin) ++count_bits;
-    int32_t *refs = nullptr, *refs_sorted = nullptr, *ids = nullptr, *order = nullptr;
-    size_t tb = 0;
-    cub::DeviceRadixSort::SortPairsDescending(nullptr, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st);
-    const size_t kb = static_cast<size_t>(k) * 4, step = (kb + 255) / 256 * 256;
-    uint8_t* block = nullptr;                 // refs | sorted refs | ids | order | classes | CUB's
-    if (!dev_alloc_ok(&block, 5 * step + tb, st) || !dev_alloc_ok(d_grp_class, static_cast<size_t>(P / 4), st)) {
+    const int64_t chunk = std::max<int64_t>(256, (k + 1023) / 1024);          // at most 1024 of them
+    const unsigned chunks = static_cast<unsigned>((k + chunk - 1) / chunk);
+    const int64_t counts = std::max<int64_t>(nwin + 1, kSmallCounts);
+    auto up = [](int64_t bytes) { return (bytes + 255) / 256 * 256; };
+    const int64_t o_hist = up(k), o_cut = o_hist + up(counts * 4), o_rows = o_cut + 256, bytes = o_rows + int64_t{chunks} * kLimits * 4;
+    uint8_t* block = nullptr;                 // classes | histogram of the counts | cuts | rows at the cuts
+    if (!dev_alloc_ok(&block, static_cast<size_t>(bytes), st) || !dev_alloc_ok(d_grp_class, static_cast<size_t>(P / 4), st)) {
         dev_free(block, st);
         dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
         return SPMM_ERR_ALLOC;
     }
-    refs = reinterpret_cast<int32_t*>(block);
-    refs_sorted = reinterpret_cast<int32_t*>(block + step);
-    ids = reinterpret_cast<int32_t*>(block + 2 * step);
-    order = reinterpret_cast<int32_t*>(block + 3 * step);
-    uint8_t* cls = block + 4 * step;
-    void* temp = block + 5 * step;
-    cudaMemsetAsync(refs, 0, kb, st);
-    wcsr_refs_kernel<<<2048, 256, 0, st>>>(d_window_col_idx, P, refs);
-    iota_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 2048)), 256, 0, st>>>(ids, k);
-    bool ok = cub::DeviceRadixSort::SortPairsDescending(temp, tb, refs, refs_sorted, ids, order, static_cast<int>(k), 0, count_bits, st) == cudaSuccess;
-    if (ok) {
-        wcsr_class_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 2048)), 256, 0, st>>>(refs_sorted, order, k, cls);
-        wcsr_group_class_kernel<<<2048, 256, 0, st>>>(d_window_col_idx, P / 4, cls, *d_grp_class);
-        ok = cudaGetLastError() == cudaSuccess;
-    }
+    int32_t* hist = reinterpret_cast<int32_t*>(block + o_hist);
+    ClassCut* cut = reinterpret_cast<ClassCut*>(block + o_cut);
+    int32_t* n_rows = reinterpret_cast<int32_t*>(block + o_rows);
+    cudaMemsetAsync(hist, 0, static_cast<size_t>(counts) * 4, st);
+    wcsr_count_hist_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 1023) / 1024, 1024)), 256, 0, st>>>(refs, k, hist);
+    wcsr_class_cut_kernel<<<1, 1024, 0, st>>>(hist, nwin, cut);
+    wcsr_cut_rows_kernel<<<chunks, 256, 0, st>>>(refs, k, chunk, cut, n_rows);
+    wcsr_class_kernel<<<chunks, 256, 0, st>>>(refs, k, chunk, cut, n_rows, block);
+    wcsr_group_class_kernel<<<static_cast<unsigned>(std::min<int64_t>((P / 4 + 255) / 256, 2048)), 256, 0, st>>>(d_window_col_idx, P / 4, block, *d_grp_class);
+    const bool ok = cudaGetLastError() == cudaSuccess;
     dev_free(block, st);
     if (!ok) {
-        cudaGetLastError();
         dev_free(*d_grp_class, st);
         *d_grp_class = nullptr;
         return SPMM_ERR_CUDA;
@@ -586,6 +804,17 @@ cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_
         n_items, static_cast<const WcsrDevTask*>(d_tasks), d_bin_tasks, d_item_fill, kt, reinterpret_cast<int2*>(d_fills));
     return cudaGetLastError();
 }
+
+namespace {
+
+template <int WH>
+void condense(const CondenseParams& p, int sms, cudaStream_t st) {
+    wcsr_condense_kernel<WH><<<static_cast<unsigned>(p.nwin), 128, 0, st>>>(p);
+    cudaFuncSetAttribute(wcsr_condense_large_kernel<WH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLargeSmem);
+    wcsr_condense_large_kernel<WH><<<static_cast<unsigned>(sms), 1024, kLargeSmem, st>>>(p);
+}
+
+}  // namespace
 
 int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
                       int es, int wh, int b_col, int T, int n_bins, int sms, cudaStream_t st, WcsrHost* out, int64_t* nnz_out,
@@ -609,13 +838,13 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     struct Flags {
         int err;                              // CSR error code
         int overflow;                         // of the scan
-        int n_unique;                         // unique keys
+        int n_big;                            // windows of the second condensation kernel
         int bad;                              // an entry out of range or not ascending
         int64_t nnz;
         unsigned long long distinct;          // columns that are referenced
     } flags = {};
     Flags* d_flags = nullptr;
-    uint8_t* d_work = nullptr;                // keys, sorted keys, rows of the entries, window lengths and starts, column marks, CUB's
+    uint8_t* d_work = nullptr;                // the entries' rows and places, window lengths, long windows, gather counts
     auto release = [&]() { dev_free(d_flags, st); dev_free(d_work, st); };
     auto fail = [&](int code) {
         cudaGetLastError();                  // (of a call that failed: not for a later check to find)
@@ -640,49 +869,39 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     if (nnz >= (int64_t{1} << 31)) return fail(SPMM_ERR_TOO_LARGE);
     *nnz_out = nnz;
 
-    // keys -> sorted -> unique
-    const int n = static_cast<int>(nnz);
-    const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 16384));
-    int cb = 1;
-    while ((int64_t{1} << cb) < k) ++cb;
-    int end_bit = cb + 1;
-    while ((int64_t{1} << (end_bit - cb)) < nwin) ++end_bit;
-    uint64_t *d_keys = nullptr, *d_keys2 = nullptr;
-    size_t t1 = 0, t2 = 0;
-    if (n > 0) {
-        cub::DeviceRadixSort::SortKeys(nullptr, t1, d_keys, d_keys2, n, 0, end_bit, st);
-        cub::DeviceSelect::Unique(nullptr, t2, d_keys2, d_keys, &d_flags->n_unique, n, st);
-    }
-    size_t work_bytes = 0, tb = std::max(t1, t2);
+    size_t work_bytes = 256;
     auto section = [&](size_t bytes) {
         const size_t at = work_bytes;
         work_bytes += (bytes + 255) / 256 * 256;
         return at;
     };
-    const size_t o_keys = section(static_cast<size_t>(nnz) * 8), o_keys2 = section(static_cast<size_t>(nnz) * 8);
-    const size_t o_row_of = section(static_cast<size_t>(nnz) * 4), o_len = section(static_cast<size_t>(nwin + 1) * 4);
-    const size_t o_ustart = section(static_cast<size_t>(nwin + 1) * 4), o_used = section(static_cast<size_t>(k)), o_temp = section(tb);
+    const size_t o_row_of = section(static_cast<size_t>(nnz) * 4), o_pos_of = section(static_cast<size_t>(nnz) * 4);
+    const size_t o_big = section(static_cast<size_t>(nwin) * 4), o_ucount = section(static_cast<size_t>(nwin) * 4), o_refs = section(static_cast<size_t>(k) * 4);
     if (!alloc(reinterpret_cast<void**>(&d_work), work_bytes) ||
         !alloc(reinterpret_cast<void**>(d_window_row_ptr), static_cast<size_t>(nwin + 1) * 4))
         return fail(SPMM_ERR_ALLOC);
-    d_keys = reinterpret_cast<uint64_t*>(d_work + o_keys);
-    d_keys2 = reinterpret_cast<uint64_t*>(d_work + o_keys2);
-    int32_t* d_row_of = reinterpret_cast<int32_t*>(d_work + o_row_of);
-    int32_t* d_len = reinterpret_cast<int32_t*>(d_work + o_len);
-    int32_t* d_ustart = reinterpret_cast<int32_t*>(d_work + o_ustart);
-    uint8_t* d_used = d_work + o_used;
-    void* d_temp = d_work + o_temp;
-    cudaMemsetAsync(d_ustart, 0, o_temp - o_ustart, st);       // the starts and the marks behind them
-    if (n > 0) {
-        wcsr_keys_kernel<<<entry_grid, 256, 0, st>>>(m, k, wh, cb, d_row_ptr, d_col_idx, d_keys, d_row_of, &d_flags->bad);
-        if (cub::DeviceRadixSort::SortKeys(d_temp, tb, d_keys, d_keys2, n, 0, end_bit, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        if (cub::DeviceSelect::Unique(d_temp, tb, d_keys2, d_keys, &d_flags->n_unique, n, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
-        // d_keys now holds the unique keys
-        wcsr_starts_kernel<<<2048, 256, 0, st>>>(d_keys, &d_flags->n_unique, nwin, cb, d_ustart, d_used);
+    CondenseParams cp;
+    cp.m = m;
+    cp.k = k;
+    cp.nwin = nwin;
+    cp.row_ptr = d_row_ptr;
+    cp.col_idx = d_col_idx;
+    cp.row_of = reinterpret_cast<int32_t*>(d_work + o_row_of);
+    cp.pos_of = reinterpret_cast<int32_t*>(d_work + o_pos_of);
+    cp.ucount = reinterpret_cast<int32_t*>(d_work + o_ucount);
+    cp.refs = reinterpret_cast<int32_t*>(d_work + o_refs);
+    cp.bad = &d_flags->bad;
+    cp.big = reinterpret_cast<int32_t*>(d_work + o_big);
+    cp.n_big = &d_flags->n_big;
+    const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 16384));
+    if (cudaMemsetAsync(cp.ucount, 0, work_bytes - o_ucount, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);     // and the gather counts behind it
+    if (nnz > 0 && k > 0) {
+        if (wh == 16) condense<16>(cp, sms, st);
+        else condense<64>(cp, sms, st);
     }
-    wcsr_pad_kernel<<<static_cast<unsigned>(std::min<int64_t>((nwin + 255) / 256 + 1, 2048)), 256, 0, st>>>(d_ustart, nwin, b_col, d_len);
-    exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_len, nwin, *d_window_row_ptr, &d_flags->overflow);
-    if (k > 0) wcsr_sum_used_kernel<<<static_cast<unsigned>(std::min<int64_t>((k + 255) / 256, 1024)), 256, 0, st>>>(d_used, k, &d_flags->distinct);
+    if (nnz > 0 && k == 0) return fail(SPMM_ERR_OUT_OF_RANGE);
+    wcsr_row_ptr_kernel<<<1 + static_cast<unsigned>(std::min<int64_t>((k + 1023) / 1024, 128)), 1024, 0, st>>>(
+        cp.ucount, nwin, b_col, *d_window_row_ptr, &d_flags->overflow, cp.refs, k, &d_flags->distinct);
     if (cudaMemcpyAsync(out->window_row_ptr.data(), *d_window_row_ptr, static_cast<size_t>(nwin + 1) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         !read_flags())
         return fail(SPMM_ERR_CUDA);
@@ -706,21 +925,20 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         cudaMemsetAsync(*d_window_col_idx, 0xFF, static_cast<size_t>(P) * 4, st);
         cudaMemsetAsync(*d_packed, 0, packed_bytes, st);
     }
-    if (n > 0) {
-        wcsr_cols_kernel<<<2048, 256, 0, st>>>(d_keys, &d_flags->n_unique, cb, d_ustart, *d_window_row_ptr, *d_window_col_idx);
+    if (nnz > 0) {
         if (es == 1)
-            wcsr_values_kernel<1><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
+            wcsr_place_kernel<1><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, cp.row_of, cp.pos_of, d_col_idx, d_vals, *d_window_row_ptr, *d_window_col_idx, *d_packed);
         else if (es == 2)
-            wcsr_values_kernel<2><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
+            wcsr_place_kernel<2><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, cp.row_of, cp.pos_of, d_col_idx, d_vals, *d_window_row_ptr, *d_window_col_idx, *d_packed);
         else
-            wcsr_values_kernel<4><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, d_row_of, d_col_idx, d_vals, d_ustart, *d_window_row_ptr, *d_window_col_idx, *d_packed);
+            wcsr_place_kernel<4><<<entry_grid, 256, 0, st>>>(nnz, wh, b_col, cp.row_of, cp.pos_of, d_col_idx, d_vals, *d_window_row_ptr, *d_window_col_idx, *d_packed);
     }
-    release();                                // (ordered behind the kernels that use them)
-    int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
+    int rc = cudaGetLastError() == cudaSuccess ? wcsr_reuse_classes_device(*d_window_col_idx, P, cp.refs, k, nwin, st, d_grp_class) : SPMM_ERR_CUDA;
     if (!rc && rows && wcsr_wants_rows(es, m, nnz, P)) {
-        rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, st, rows);
+        rc = build_wcsr_rows_device(m, nnz, d_row_ptr, d_col_idx, d_vals, es, sms, cp.row_of, st, rows);
         if (rc == SPMM_ERR_ALLOC) rc = SPMM_OK;          // no room for it: the window kernel serves the handle
     }
+    release();                                // (ordered behind the kernels that use them)
     // the split plan needs the window lengths only: the host makes it while the kernels above run
     if (!rc) {
         try {
@@ -752,43 +970,147 @@ __device__ __forceinline__ int row_class(int64_t len, int pack, int task_max) {
     return c;
 }
 
-__global__ void rows_class_kernel(int64_t m, const int64_t* __restrict__ row_ptr, int pack, int task_max, uint8_t* __restrict__ cls,
-                                  int32_t* __restrict__ ids, int32_t* __restrict__ counts) {
-    __shared__ int n[kRowClasses];
-    if (threadIdx.x < kRowClasses) n[threadIdx.x] = 0;
-    __syncthreads();
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int c = row_class(row_ptr[i + 1] - row_ptr[i], pack, task_max);
-        cls[i] = static_cast<uint8_t>(c);
-        ids[i] = static_cast<int32_t>(i);
-        atomicAdd(&n[c], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x < kRowClasses && n[threadIdx.x]) atomicAdd(&counts[threadIdx.x], n[threadIdx.x]);
+// Rows are put in the order of their classes (stable) in three passes over chunks of kRowsChunk rows: what each chunk
+// has of every class, exclusive sums of that over (class, chunk), and every row to its place.
+constexpr int kRowsChunk = 1024;
+
+// What a row adds to the sums over rows in order: x entries (an empty row counts one; a long row none here), y padded
+// entries of a long row, z its parts, w its partial slots.
+__device__ __forceinline__ int4 row_size(int64_t len, int task_max, int part_len) {
+    if (len <= task_max) return make_int4(len > 0 ? static_cast<int>(len) : 1, 0, 0, 0);
+    const int parts = static_cast<int>((len + part_len - 1) / part_len);
+    return make_int4(0, static_cast<int>((len + 7) / 8 * 8), parts, parts > 1 ? parts : 0);
 }
 
-struct Int4Sum {
-    __host__ __device__ int4 operator()(const int4& a, const int4& b) const { return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
-};
+struct ClassSum { int rows, x, y, z, w; };
+__device__ __forceinline__ void add_sum(ClassSum* to, const ClassSum& v) {
+    if (v.rows) atomicAdd(&to->rows, v.rows);
+    if (v.x) atomicAdd(&to->x, v.x);
+    if (v.y) atomicAdd(&to->y, v.y);
+    if (v.z) atomicAdd(&to->z, v.z);
+    if (v.w) atomicAdd(&to->w, v.w);
+}
 
-// Per position of `order`: {entries (an empty row counts one; a long row none here), padded entries of a long row,
-// its parts, its partial slots}; position m closes the scan.
-__global__ void rows_size_kernel(int64_t m, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr, int task_max, int part_len,
-                                 int4* __restrict__ size) {
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i <= m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        int4 s = make_int4(0, 0, 0, 0);
-        if (i < m) {
-            const int32_t r = order[i];
-            const int n = static_cast<int>(row_ptr[r + 1] - row_ptr[r]);
-            if (n <= task_max) {
-                s.x = n > 0 ? n : 1;
-            } else {
-                s.y = (n + 7) / 8 * 8;
-                s.z = (n + part_len - 1) / part_len;
-                s.w = s.z > 1 ? s.z : 0;
-            }
+__global__ void __launch_bounds__(256) rows_count_kernel(int64_t m, const int64_t* __restrict__ row_ptr, int pack, int task_max, int part_len, int chunks,
+                                                         ClassSum* __restrict__ sums) {
+    __shared__ ClassSum n[kRowClasses];
+    if (threadIdx.x < kRowClasses) n[threadIdx.x] = ClassSum{0, 0, 0, 0, 0};
+    __syncthreads();
+    for (int j = threadIdx.x; j < kRowsChunk; j += 256) {
+        const int64_t i = static_cast<int64_t>(blockIdx.x) * kRowsChunk + j;
+        if (i >= m) break;
+        const int64_t len = row_ptr[i + 1] - row_ptr[i];
+        const int4 s = row_size(len, task_max, part_len);
+        add_sum(&n[row_class(len, pack, task_max)], ClassSum{1, s.x, s.y, s.z, s.w});
+    }
+    __syncthreads();
+    if (threadIdx.x < kRowClasses) sums[threadIdx.x * chunks + blockIdx.x] = n[threadIdx.x];
+}
+
+// One CTA: exclusive sums in place, class by class and chunk by chunk; the classes' rows; the sums over all rows behind the last.
+__global__ void __launch_bounds__(1024) rows_sums_kernel(int chunks, ClassSum* __restrict__ sums, int32_t* __restrict__ counts) {
+    __shared__ ClassSum warp_sum[32];
+    __shared__ int class_start[kRowClasses + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = chunks * kRowClasses;
+    ClassSum carry = {0, 0, 0, 0, 0};
+    auto plus = [](ClassSum a, const ClassSum& b) { a.rows += b.rows; a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; return a; };
+    auto scan = [&](ClassSum v) {            // inclusive, over a warp
+        for (int o = 1; o < 32; o <<= 1) {
+            const ClassSum u = {__shfl_up_sync(0xffffffffu, v.rows, o), __shfl_up_sync(0xffffffffu, v.x, o), __shfl_up_sync(0xffffffffu, v.y, o),
+                                __shfl_up_sync(0xffffffffu, v.z, o), __shfl_up_sync(0xffffffffu, v.w, o)};
+            if (lane >= o) v = plus(v, u);
         }
-        size[i] = s;
+        return v;
+    };
+    for (int base = 0; base < n; base += 1024) {
+        const int i = base + threadIdx.x;
+        const ClassSum v = i < n ? sums[i] : ClassSum{0, 0, 0, 0, 0};
+        const ClassSum in = scan(v);
+        if (lane == 31) warp_sum[warp] = in;
+        __syncthreads();
+        if (warp == 0) warp_sum[lane] = scan(warp_sum[lane]);
+        __syncthreads();
+        ClassSum ex = {in.rows - v.rows, in.x - v.x, in.y - v.y, in.z - v.z, in.w - v.w};
+        ex = plus(ex, carry);
+        if (warp) ex = plus(ex, warp_sum[warp - 1]);
+        if (i < n) sums[i] = ex;
+        if (i < n && i % chunks == 0) class_start[i / chunks] = ex.rows;
+        carry = plus(carry, warp_sum[31]);
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        sums[n] = carry;
+        class_start[kRowClasses] = carry.rows;
+    }
+    __syncthreads();
+    if (threadIdx.x < kRowClasses) counts[threadIdx.x] = class_start[threadIdx.x + 1] - class_start[threadIdx.x];
+}
+
+// order[position] = row, start[position] = sums over the rows before it; position m closes both.
+__global__ void __launch_bounds__(256) rows_order_kernel(int64_t m, const int64_t* __restrict__ row_ptr, int pack, int task_max, int part_len, int chunks,
+                                                         const ClassSum* __restrict__ sums, int32_t* __restrict__ order, int4* __restrict__ start) {
+    __shared__ ClassSum before[kRowClasses];              // of the rows of the class before this step's
+    __shared__ ClassSum in_warp[8][kRowClasses];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < kRowClasses) before[threadIdx.x] = sums[threadIdx.x * chunks + blockIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const ClassSum& t = sums[chunks * kRowClasses];
+        order[m] = 0;
+        start[m] = make_int4(t.x, t.y, t.z, t.w);
+    }
+    for (int j = 0; j < kRowsChunk; j += 256) {
+        const int64_t i = static_cast<int64_t>(blockIdx.x) * kRowsChunk + j + threadIdx.x;
+        const bool on = i < m;
+        const int64_t len = on ? row_ptr[i + 1] - row_ptr[i] : 0;
+        const int c = on ? row_class(len, pack, task_max) : -1;
+        const int4 s = on ? row_size(len, task_max, part_len) : make_int4(0, 0, 0, 0);
+        ClassSum mine = {0, 0, 0, 0, 0};                  // of the rows of this class before this one in the warp
+#pragma unroll
+        for (int q = 0; q < kRowClasses; ++q) {
+            const unsigned same = __ballot_sync(0xffffffffu, c == q);
+            ClassSum all = {__popc(same), 0, 0, 0, 0}, ex = {__popc(same & ((1u << lane) - 1u)), 0, 0, 0, 0};
+            auto field = [&](int v, int* a, int* e) {
+                int x = c == q ? v : 0;
+                const int own = x;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, x, o);
+                    if (lane >= o) x += y;
+                }
+                *a = __shfl_sync(0xffffffffu, x, 31);
+                *e = x - own;
+            };
+            if (same) {                                   // (uniform)
+                if (q == 0) {
+                    field(s.y, &all.y, &ex.y);
+                    field(s.z, &all.z, &ex.z);
+                    field(s.w, &all.w, &ex.w);
+                } else {
+                    field(s.x, &all.x, &ex.x);
+                }
+            }
+            if (c == q) mine = ex;
+            if (lane == 0) in_warp[warp][q] = all;
+        }
+        __syncthreads();
+        if (on) {
+            ClassSum at = before[c];
+            for (int v = 0; v < warp; ++v) {
+                const ClassSum& u = in_warp[v][c];
+                at.rows += u.rows; at.x += u.x; at.y += u.y; at.z += u.z; at.w += u.w;
+            }
+            at.rows += mine.rows; at.x += mine.x; at.y += mine.y; at.z += mine.z; at.w += mine.w;
+            order[at.rows] = static_cast<int32_t>(i);
+            start[at.rows] = make_int4(at.x, at.y, at.z, at.w);
+        }
+        __syncthreads();
+        if (threadIdx.x < kRowClasses)
+            for (int v = 0; v < 8; ++v) {
+                const ClassSum& u = in_warp[v][threadIdx.x];
+                ClassSum& t = before[threadIdx.x];
+                t.rows += u.rows; t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+            }
+        __syncthreads();
     }
 }
 
@@ -798,7 +1120,7 @@ struct RowsPlan {
     int64_t m;
     int pack, part_len;
     const int32_t* counts;
-    const int4* start;                   // exclusive sums of rows_size_kernel's fields
+    const int4* start;                   // exclusive sums of row_size's fields
     int n_classes;
     __device__ __forceinline__ int n_long() const { return counts[0]; }
     __device__ __forceinline__ int n_single() const {
@@ -817,91 +1139,89 @@ struct RowsPlan {
     __device__ __forceinline__ int long_base(int nl, int ns) const { return (begin(n_tasks(nl, ns), start[m].x) + 7) / 8 * 8; }
 };
 
-// task heads; descriptors of the long rows and their parts; totals {tasks, parts, long rows, slots}
-__global__ void rows_plan_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr, int32_t* __restrict__ head,
-                                 int4* __restrict__ parts, int4* __restrict__ longs, int4* __restrict__ total) {
-    const int nl = p.n_long(), ns = p.n_single();
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i <= p.m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        if (i == p.m) {
-            const int tasks = p.n_tasks(nl, ns);
-            head[tasks] = static_cast<int32_t>(p.m);
-            *total = make_int4(tasks, p.start[p.m].z, nl, p.start[p.m].w);
-        } else if (i < nl) {
-            const int4 s = p.start[i];
-            const int np = p.start[i + 1].z - s.z;
-            const int32_t r = order[i];
-            const int n = static_cast<int>(row_ptr[r + 1] - row_ptr[r]);
-            const int base = p.long_base(nl, ns);
-            longs[i] = make_int4(r, s.w, np, 0);
-            for (int j = 0; j < np; ++j)
-                parts[s.z + j] = make_int4(base + s.y + j * p.part_len, min(p.part_len, n - j * p.part_len), static_cast<int>(i), j);
-        } else {
-            const int t = p.task(i, nl, ns);
-            if (i == nl || t != p.task(i - 1, nl, ns)) head[t] = static_cast<int32_t>(i);
-        }
-    }
-}
-
 template <int ES> struct RowsValue { using type = uint16_t; };
 template <> struct RowsValue<4> { using type = uint32_t; };
 
-// eight lanes per position: a row's nonzeros to their place in its task, the task's descriptor and padding
+// By position: where the row's entries go (at[row]) and what is not an entry of the matrix (the empty rows, the padding);
+// the tasks, the long rows and their parts; totals {tasks, parts, long rows, slots}.
 template <int ES>
-__global__ void rows_fill_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int32_t* __restrict__ head,
-                                 const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ vals,
-                                 int4* __restrict__ tasks, int32_t* __restrict__ col, uint8_t* __restrict__ val) {
+__global__ void rows_plan_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr, int32_t* __restrict__ at,
+                                 int4* __restrict__ tasks, int4* __restrict__ parts, int4* __restrict__ longs, int4* __restrict__ total,
+                                 int32_t* __restrict__ col, uint8_t* __restrict__ val) {
     using T = typename RowsValue<ES>::type;
-    const T* src = reinterpret_cast<const T*>(vals);
     T* dst = reinterpret_cast<T*>(val);
     const int nl = p.n_long(), ns = p.n_single();
-    const int sub = threadIdx.x & 7;
-    for (int64_t i = nl + ((static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 3); i < p.m;
-         i += (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 3) {
-        const int t = p.task(i, nl, ns);
-        const int h = head[t], h1 = head[t + 1];
-        const int first = p.start[h].x;
-        const int64_t base = p.begin(t, first);
-        const int64_t at = base + (p.start[i].x - first);
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i <= p.m; i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        if (i == p.m) {
+            *total = make_int4(p.n_tasks(nl, ns), p.start[p.m].z, nl, p.start[p.m].w);
+            continue;
+        }
         const int32_t r = order[i];
-        const int64_t s = row_ptr[r];
-        const int n = static_cast<int>(row_ptr[r + 1] - s);
-        if (n == 0 && sub == 0) {
-            col[at] = -1;                                  // the sign bit and no gather
-            dst[at] = 0;
-        }
-        for (int j = sub; j < n; j += 8) {
-            col[at + j] = col_idx[s + j] | (j == n - 1 ? static_cast<int32_t>(0x80000000u) : 0);
-            dst[at + j] = src[s + j];
-        }
-        if (i == h) {
-            const int len = p.start[h1].x - first;
-            if (sub == 0) tasks[t] = make_int4(static_cast<int>(base), len, h, 0);
-            if (sub < 4 && len + sub < (len + 3) / 4 * 4) {
-                col[base + len + sub] = 0x7fffffff;
-                dst[base + len + sub] = 0;
+        const int n = static_cast<int>(row_ptr[r + 1] - row_ptr[r]);
+        if (i < nl) {
+            const int4 s = p.start[i];
+            const int np = p.start[i + 1].z - s.z;
+            const int base = p.long_base(nl, ns) + s.y;
+            at[r] = base;
+            longs[i] = make_int4(r, s.w, np, 0);
+            for (int j = 0; j < np; ++j)
+                parts[s.z + j] = make_int4(base + j * p.part_len, min(p.part_len, n - j * p.part_len), static_cast<int>(i), j);
+            for (int j = n; j < (n + 7) / 8 * 8; ++j) {
+                col[base + j] = 0x7fffffff;
+                dst[base + j] = 0;
+            }
+        } else {
+            // (a task of packed rows holds at most `pack` of them: the steps to its first one are few)
+            const int t = p.task(i, nl, ns);
+            int64_t h = i;
+            while (h > nl && p.task(h - 1, nl, ns) == t) --h;
+            const int first = p.start[h].x;
+            const int base = p.begin(t, first);
+            const int to = base + (p.start[i].x - first);
+            at[r] = to;
+            if (n == 0) {
+                col[to] = -1;                              // the sign bit and no gather
+                dst[to] = 0;
+            }
+            if (i == h) {
+                int64_t h1 = i + 1;
+                while (h1 < p.m && p.task(h1, nl, ns) == t) ++h1;
+                const int len = p.start[h1].x - first;
+                tasks[t] = make_int4(base, len, static_cast<int>(i), 0);
+                for (int j = len; j < (len + 3) / 4 * 4; ++j) {
+                    col[base + j] = 0x7fffffff;
+                    dst[base + j] = 0;
+                }
             }
         }
     }
 }
 
-// one CTA per long row
+// One thread per entry of the matrix (a CTA per long row took 19 us for 60,000 power-law rows, this 6 for all rows).
 template <int ES>
-__global__ void rows_fill_long_kernel(const RowsPlan p, const int32_t* __restrict__ order, const int64_t* __restrict__ row_ptr,
-                                      const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ vals, int32_t* __restrict__ col,
-                                      uint8_t* __restrict__ val) {
+__global__ void rows_fill_kernel(int64_t nnz, int task_max, const int32_t* __restrict__ row_of, const int64_t* __restrict__ row_ptr,
+                                 const int32_t* __restrict__ at, const int32_t* __restrict__ col_idx, const uint8_t* __restrict__ vals,
+                                 int32_t* __restrict__ col, uint8_t* __restrict__ val) {
     using T = typename RowsValue<ES>::type;
-    const T* src = reinterpret_cast<const T*>(vals);
-    T* dst = reinterpret_cast<T*>(val);
-    const int nl = p.n_long();
-    if (static_cast<int>(blockIdx.x) >= nl) return;
-    const int base = p.long_base(nl, p.n_single());
-    for (int i = blockIdx.x; i < nl; i += gridDim.x) {
-        const int32_t r = order[i];
-        const int64_t s = row_ptr[r], n = row_ptr[r + 1] - s, at = base + p.start[i].y;
-        for (int64_t j = threadIdx.x; j < (n + 7) / 8 * 8; j += blockDim.x) {
-            col[at + j] = j < n ? col_idx[s + j] : 0x7fffffff;
-            dst[at + j] = j < n ? src[s + j] : T(0);
+    for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int32_t r = row_of[p];
+        const int64_t s = row_ptr[r], e = row_ptr[r + 1];
+        const int64_t to = at[r] + (p - s);
+        const bool last = p == e - 1 && e - s <= task_max;
+        col[to] = col_idx[p] | (last ? static_cast<int32_t>(0x80000000u) : 0);
+        reinterpret_cast<T*>(val)[to] = reinterpret_cast<const T*>(vals)[p];
+    }
+}
+
+// the row of every entry, looked up in row_ptr
+__global__ void rows_of_entries_kernel(int64_t m, int64_t nnz, const int64_t* __restrict__ row_ptr, int32_t* __restrict__ row_of) {
+    for (int64_t p = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; p < nnz; p += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        int64_t lo = 0, hi = m - 1;                       // last row that starts at or before p
+        while (lo < hi) {
+            const int64_t mid = (lo + hi + 1) >> 1;
+            if (row_ptr[mid] <= p) lo = mid; else hi = mid - 1;
         }
+        row_of[p] = static_cast<int32_t>(lo);
     }
 }
 
@@ -930,7 +1250,7 @@ int finish_wcsr_rows(WcsrRowStream* s, cudaStream_t st) {
 }
 
 int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, const int32_t* d_col_idx, const uint8_t* d_vals,
-                           int es, int sms, cudaStream_t st, WcsrRowStream* out) {
+                           int es, int sms, const int32_t* d_row_of, cudaStream_t st, WcsrRowStream* out) {
     *out = WcsrRowStream();
     if (m <= 0 || (es != 2 && es != 4)) return SPMM_OK;
     // Task sizes by the entries there are per SM and 128 groups: small matrices need short tasks and parts to fill
@@ -964,39 +1284,39 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     const int64_t entries = nnz + m + 3 * max_tasks + 8 * max_long + 16;
     if (entries >= (int64_t{1} << 31) || m >= (int64_t{1} << 31) - 1) return SPMM_OK;
 
-    uint8_t *d_cls = nullptr, *d_cls2 = nullptr;
-    int32_t *d_ids = nullptr, *d_counts = nullptr, *d_head = nullptr;
-    int4 *d_size = nullptr, *d_start = nullptr;
-    void* d_temp = nullptr;
+    const int64_t chunks = (m + kRowsChunk - 1) / kRowsChunk;
+    auto up = [](int64_t bytes) { return (bytes + 255) / 256 * 256; };
+    // places by row | sums by position | sums by class and chunk | rows by class | rows of the entries, where not given
+    const int64_t o_start = up(m * 4), o_sums = o_start + up((m + 1) * 16), o_counts = o_sums + up((chunks * kRowClasses + 1) * sizeof(ClassSum));
+    const int64_t o_row_of = o_counts + 256, work_bytes = o_row_of + (d_row_of ? 0 : nnz * 4);
+    uint8_t* d_work = nullptr;
     auto done = [&](int code) {
         if (code) cudaGetLastError();
-        void* const arrays[] = {d_cls, d_cls2, d_ids, d_counts, d_head, d_size, d_start, d_temp};
-        for (void* ptr : arrays) dev_free(ptr, st);
+        dev_free(d_work, st);
         if (code) free_wcsr_rows(out, st);
         return code;
     };
     auto alloc = [&](auto** ptr, int64_t bytes) { return dev_alloc_ok(ptr, static_cast<size_t>(bytes), st); };
-    size_t t1 = 0, t2 = 0;
-    const int4 zero = make_int4(0, 0, 0, 0);
-    cub::DeviceRadixSort::SortPairs(nullptr, t1, d_cls, d_cls2, d_ids, out->d_order, static_cast<int>(m), 0, 3, st);
-    cub::DeviceScan::ExclusiveScan(nullptr, t2, d_size, d_start, Int4Sum(), zero, static_cast<int>(m + 1), st);
-    size_t tb = std::max(t1, t2);
     const int64_t counter_bytes = 32 + max_long * kRowsMaxTiles * 4;
-    if (!alloc(&d_cls, m) || !alloc(&d_cls2, m) || !alloc(&d_ids, m * 4) || !alloc(&d_counts, kRowClasses * 4) || !alloc(&d_head, (max_tasks + 1) * 4) ||
-        !alloc(&d_size, (m + 1) * 16) || !alloc(&d_start, (m + 1) * 16) || !alloc(&d_temp, static_cast<int64_t>(tb)) ||
+    if (!alloc(&d_work, work_bytes) ||
         !alloc(&out->d_order, (m + 1) * 4) || !alloc(&out->d_tasks, max_tasks * 16) || !alloc(&out->d_parts, max_parts * 16) ||
         !alloc(&out->d_longs, max_long * 16) || !alloc(&out->d_col, entries * 4) || !alloc(&out->d_val, entries * es) ||
         !alloc(&out->d_counters, counter_bytes) || !alloc(&out->d_total, 16))
         return done(SPMM_ERR_ALLOC);
-    cudaMemsetAsync(d_counts, 0, kRowClasses * 4, st);
-    cudaMemsetAsync(out->d_order + m, 0, 4, st);
+    int32_t* d_at = reinterpret_cast<int32_t*>(d_work);
+    int4* d_start = reinterpret_cast<int4*>(d_work + o_start);
+    ClassSum* d_sums = reinterpret_cast<ClassSum*>(d_work + o_sums);
+    int32_t* d_counts = reinterpret_cast<int32_t*>(d_work + o_counts);
     cudaMemsetAsync(out->d_counters, 0, static_cast<size_t>(counter_bytes), st);
-    rows_class_kernel<<<grid_for(m, 256), 256, 0, st>>>(m, d_row_ptr, out->pack, out->task_max, d_cls, d_ids, d_counts);
-    if (cub::DeviceRadixSort::SortPairs(d_temp, tb, d_cls, d_cls2, d_ids, out->d_order, static_cast<int>(m), 0, 3, st) != cudaSuccess)
-        return done(SPMM_ERR_CUDA);
-    rows_size_kernel<<<grid_for(m + 1, 256), 256, 0, st>>>(m, out->d_order, d_row_ptr, out->task_max, out->part_len, d_size);
-    if (cub::DeviceScan::ExclusiveScan(d_temp, tb, d_size, d_start, Int4Sum(), zero, static_cast<int>(m + 1), st) != cudaSuccess)
-        return done(SPMM_ERR_CUDA);
+    if (!d_row_of && nnz > 0) {
+        int32_t* own = reinterpret_cast<int32_t*>(d_work + o_row_of);
+        rows_of_entries_kernel<<<grid_for(nnz, 256), 256, 0, st>>>(m, nnz, d_row_ptr, own);
+        d_row_of = own;
+    }
+    const int nc = static_cast<int>(chunks);
+    rows_count_kernel<<<static_cast<unsigned>(chunks), 256, 0, st>>>(m, d_row_ptr, out->pack, out->task_max, out->part_len, nc, d_sums);
+    rows_sums_kernel<<<1, 1024, 0, st>>>(nc, d_sums, d_counts);
+    rows_order_kernel<<<static_cast<unsigned>(chunks), 256, 0, st>>>(m, d_row_ptr, out->pack, out->task_max, out->part_len, nc, d_sums, out->d_order, d_start);
     RowsPlan p;
     p.m = m;
     p.pack = out->pack;
@@ -1006,16 +1326,17 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
     p.n_classes = 2;                                         // long, packed, and the classes between
     for (int lim = out->task_max / 2; lim >= out->pack; lim /= 2) ++p.n_classes;
     int4* tasks = reinterpret_cast<int4*>(out->d_tasks);
-    rows_plan_kernel<<<grid_for(m + 1, 256), 256, 0, st>>>(p, out->d_order, d_row_ptr, d_head, reinterpret_cast<int4*>(out->d_parts),
-                                                          reinterpret_cast<int4*>(out->d_longs), reinterpret_cast<int4*>(out->d_total));
-    const unsigned lg = static_cast<unsigned>(std::min<int64_t>(max_long, 8192));
-    if (es == 2) {
-        rows_fill_kernel<2><<<grid_for(m * 8, 256), 256, 0, st>>>(p, out->d_order, d_head, d_row_ptr, d_col_idx, d_vals, tasks, out->d_col, out->d_val);
-        rows_fill_long_kernel<2><<<lg, 256, 0, st>>>(p, out->d_order, d_row_ptr, d_col_idx, d_vals, out->d_col, out->d_val);
-    } else {
-        rows_fill_kernel<4><<<grid_for(m * 8, 256), 256, 0, st>>>(p, out->d_order, d_head, d_row_ptr, d_col_idx, d_vals, tasks, out->d_col, out->d_val);
-        rows_fill_long_kernel<4><<<lg, 256, 0, st>>>(p, out->d_order, d_row_ptr, d_col_idx, d_vals, out->d_col, out->d_val);
-    }
+    int4* parts = reinterpret_cast<int4*>(out->d_parts);
+    int4* longs = reinterpret_cast<int4*>(out->d_longs);
+    int4* total = reinterpret_cast<int4*>(out->d_total);
+    auto plan = [&](auto bytes) {
+        constexpr int ES = decltype(bytes)::value;
+        rows_plan_kernel<ES><<<grid_for(m + 1, 256), 256, 0, st>>>(p, out->d_order, d_row_ptr, d_at, tasks, parts, longs, total, out->d_col, out->d_val);
+        if (nnz > 0)
+            rows_fill_kernel<ES><<<grid_for(nnz, 256), 256, 0, st>>>(nnz, out->task_max, d_row_of, d_row_ptr, d_at, d_col_idx, d_vals, out->d_col, out->d_val);
+    };
+    if (es == 2) plan(std::integral_constant<int, 2>());
+    else plan(std::integral_constant<int, 4>());
     return done(cudaGetLastError() == cudaSuccess ? SPMM_OK : SPMM_ERR_CUDA);
 }
 
