@@ -15,9 +15,9 @@
 // k / b <= 819,200.
 //
 // WCSR (window condensation of Sec. 2.3): a window's entries are one contiguous range of the CSR arrays, wh ascending
-// runs.  One CTA merges them pair by pair in shared memory; where the merged column changes, a new condensed column
-// begins, so that an entry's rank gives its place in the window (windows too long for that: a bitmap of columns, as
-// above).  A prefix sum of the lengths padded to b_col is window_row_ptr; a last pass, entry by entry, writes the
+// runs.  A short window is sorted by one warp in registers, a longer one goes through a bitmap of its columns or, where
+// the matrix is too wide for that, is merged run by run in shared memory; each way an entry gets its place among the
+// window's distinct columns.  A prefix sum of the lengths padded to b_col is window_row_ptr; a last pass, entry by entry, writes the
 // columns over a -1 fill and the values straight into the packed tile layout.
 #include <cstring>
 #include <numeric>
@@ -28,6 +28,7 @@
 #include "device_memory.h"
 #include "format.h"
 #include "kernels.h"
+#include "ptx.cuh"
 #include "spmm_b200.h"
 
 namespace spmm {
@@ -36,17 +37,42 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Which of its kernels condenses a window of n entries (below: sort_window, bitmap_window, merge_window).  The bitmap of a
+// window costs about a word per 32 columns of the matrix, so short windows of a wide matrix are merged instead, up to
+// what fits shared memory.
+constexpr int kWarpWindow = 256, kMergeWindow = 2048, kLargeWindow = 18432;
+constexpr int kColumnsPerEntry = 256;        // a bitmap from one entry per that many columns on
+enum { kListBitmap, kListMerge, kListLarge, kLists };
+struct WindowLists {
+    int wh;                                  // 0: no lists are wanted
+    int64_t k;
+    int32_t* list[kLists];
+    int* count;                              // [kLists], zero before
+    __device__ __forceinline__ int which(int64_t n) const {
+        if (n <= kWarpWindow) return -1;
+        if (n > kLargeWindow || n * kColumnsPerEntry >= k) return kListBitmap;
+        return n <= kMergeWindow ? kListMerge : kListLarge;
+    }
+};
+
 // Validation in two passes, so that the second one never reads past the arrays: once row_ptr is
 // known to start at 0 and to be monotone, every position below row_ptr[m] lies inside col_idx.
-// (nnz: receives row_ptr[m] where the caller reads it together with *err; may be null)
-__global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* err, int64_t* nnz) {
+// (nnz: receives row_ptr[m] where the caller reads it together with *err; may be null.  longer, where not null: lists
+// of the windows of wh rows that one warp does not condense, see WindowLists.)
+__global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* err, int64_t* nnz, const WindowLists longer) {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (row_ptr[0] != 0) atomicMin(err, SPMM_ERR_INVALID_ARG);
         if (nnz) *nnz = row_ptr[m];
     }
     for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < m;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
         if (row_ptr[i + 1] < row_ptr[i]) atomicMin(err, SPMM_ERR_INVALID_ARG);
+        if (longer.wh && i % longer.wh == 0) {
+            const int64_t n = row_ptr[min(i + longer.wh, m)] - row_ptr[i];
+            const int which = longer.which(n);
+            if (which >= 0) longer.list[which][atomicAdd(longer.count + which, 1)] = static_cast<int32_t>(i / longer.wh);
+        }
+    }
 }
 
 __global__ void csr_check_cols_kernel(int64_t m, int64_t k, const int64_t* row_ptr, const int32_t* col_idx, int* err) {
@@ -125,7 +151,8 @@ bcsr_count_kernel(int64_t m, int b, int words, const int64_t* row_ptr, const int
     if (threadIdx.x == 0) counts[blockIdx.x] = total;
 }
 
-// Exclusive sums over a CTA of 1024 threads, one value each; *total gets the sum of all.  scratch: 33 values.
+// Exclusive sums over a CTA of THREADS threads, one value each; *total gets the sum of all.  scratch: 32 values.
+template <int THREADS = 1024>
 __device__ __forceinline__ long long block_exclusive_sum(long long v, long long* scratch, long long* total) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     long long x = v;
@@ -137,7 +164,7 @@ __device__ __forceinline__ long long block_exclusive_sum(long long v, long long*
     if (lane == 31) scratch[warp] = x;
     __syncthreads();
     if (warp == 0) {
-        long long t = scratch[lane];
+        long long t = lane < THREADS / 32 ? scratch[lane] : 0;
         for (int o = 1; o < 32; o <<= 1) {
             const long long y = __shfl_up_sync(0xffffffffu, t, o);
             if (lane >= o) t += y;
@@ -349,7 +376,7 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     int flags[2] = {0, 0};
     const unsigned check_grid = static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048));
     if (m > 0) {
-        csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, d_flags, nullptr);
+        csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, d_flags, nullptr, WindowLists{});
         if (cudaMemcpyAsync(&nnz, d_row_ptr + m, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
     }
     if (cudaMemcpyAsync(flags, d_flags, sizeof(flags), cudaMemcpyDeviceToHost, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
@@ -421,14 +448,8 @@ struct CondenseParams {
     int32_t* ucount;                         // [nwin]
     int32_t* refs;                           // [k], zero before
     int* bad;
-    int32_t* big;                            // windows left to the second kernel, and how many
-    int* n_big;
+    const int32_t* list;                     // the windows of this launch, where it does not go over all
 };
-
-// Entries whose wh runs are merged in shared memory by one CTA: at most kSmallWindow by 128 threads (20 KB, a dozen CTAs
-// per SM), kLargeWindow by 1024 (205 KB).  Against radix sort of 64-bit keys, unique and lookups, 60,000 power-law rows
-// (0.8 M entries): 115 us of kernels for the same arrays, @@.
-constexpr int kSmallWindow = 2048, kLargeWindow = 20480;
 
 __device__ __forceinline__ int32_t checked_column(const CondenseParams& p, int64_t at, int64_t row_start) {
     const int32_t c = p.col_idx[at];
@@ -449,15 +470,94 @@ __device__ __forceinline__ int row_in_window(const int* off, int j) {
     return r;
 }
 
+// One warp: at most 32 * ITEMS entries, sorted in registers by a bitonic network over positions lane * ITEMS + i; the
+// distinct ones then lie ascending in cols (padded to 256 with the largest int), where every entry looks its own up.
+// For 60,000 power-law rows the network takes about four warp instructions per entry, merging in shared memory 44.
+template <int WH, int ITEMS>
+__device__ __forceinline__ void sort_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, int32_t* own, int32_t* cols) {
+    constexpr int kPad = 0x7fffffff;
+    constexpr int N = 32 * ITEMS;
+    const int lane = threadIdx.x & 31;
+    int32_t key[ITEMS];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int j = i * 32 + lane;
+        key[i] = kPad;
+        if (j < n) {
+            const int r = row_in_window<WH>(off, j);
+            key[i] = checked_column(p, p0 + j, p0 + off[r]);
+            p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
+        }
+        own[j] = key[i];
+        cols[j] = kPad;
+    }
+#pragma unroll
+    for (int size = 2; size <= N; size *= 2)
+#pragma unroll
+        for (int stride = size / 2; stride > 0; stride /= 2) {
+            if (stride >= ITEMS) {
+                // partner in another lane; ascending where the position's `size` bit is clear
+                const bool up = size >= N || ((lane * ITEMS) & size) == 0;
+                const bool low = (lane & (stride / ITEMS)) == 0;
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i) {
+                    const int32_t other = __shfl_xor_sync(0xffffffffu, key[i], stride / ITEMS);
+                    key[i] = up == low ? min(key[i], other) : max(key[i], other);
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i) {
+                    if (i & stride) continue;
+                    const bool up = size >= N || ((lane * ITEMS + i) & size) == 0;
+                    const int32_t a = min(key[i], key[i | stride]), b = max(key[i], key[i | stride]);
+                    key[i] = up ? a : b;
+                    key[i | stride] = up ? b : a;
+                }
+            }
+        }
+    const int32_t before = __shfl_up_sync(0xffffffffu, key[ITEMS - 1], 1);
+    unsigned first = 0;                      // bit i: the first of its column
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const bool f = key[i] != kPad && ((lane == 0 && i == 0) || key[i] != (i ? key[i - 1] : before));
+        first |= static_cast<unsigned>(f) << i;
+    }
+    int at = __popc(first);
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += y;
+    }
+    if (lane == 31) p.ucount[w] = at;
+    at -= __popc(first);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (first >> i & 1u) {
+            cols[at++] = key[i];
+            atomicAdd(p.refs + key[i], 1);
+        }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int j = i * 32 + lane;
+        const int32_t c = own[j];
+        int pos = 0;
+#pragma unroll
+        for (int step = N / 2; step > 0; step /= 2)
+            if (cols[pos + step - 1] < c) pos += step;
+        if (j < n) p.pos_of[p0 + j] = pos;
+    }
+}
+
 // n entries from p0 on: keys[2][cap], rank[cap] in shared memory; off has WH + 1 entries.
 template <int WH, int THREADS>
-__device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, int32_t* keys, int cap, uint16_t* rank) {
+__device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, int32_t* keys, int cap, uint32_t* rank) {
     __shared__ int warp_sum[THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j < n; j += THREADS) {
         const int r = row_in_window<WH>(off, j);
         keys[j] = checked_column(p, p0 + j, p0 + off[r]);
-        rank[j] = static_cast<uint16_t>(j);
+        rank[j] = static_cast<uint32_t>(j) | static_cast<uint32_t>(r) << 16;     // the row stays beside the rank
         p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
     }
     __syncthreads();
@@ -466,21 +566,22 @@ __device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w,
     // that go before it (equal ones: the earlier run first)
     for (int span = 1; span < WH; span *= 2) {
         for (int j = threadIdx.x; j < n; j += THREADS) {
-            const int g = row_in_window<WH>(off, j) & ~(span - 1);       // first row of this entry's run
+            const uint32_t row = rank[j] >> 16;
+            const int g = static_cast<int>(row) & ~(span - 1);                   // first row of this entry's run
             const bool right = (g & span) != 0;
             const int sib = right ? g - span : g + span;
-            const int at = rank[j];
+            const int at = static_cast<int>(rank[j] & 0xffffu);
             const int32_t c = src[at];
             const int s0 = off[sib];
             int lo = s0, hi = off[sib + span];
-            const int32_t bound = right ? c : c - 1;                     // entries of the other run up to here go before
+            const int32_t bound = right ? c : c - 1;                             // entries of the other run up to here go before
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
                 if (src[mid] <= bound) lo = mid + 1; else hi = mid;
             }
             const int to = at + (right ? lo - off[g] : lo - s0);
             dst[to] = c;
-            rank[j] = static_cast<uint16_t>(to);
+            rank[j] = static_cast<uint32_t>(to) | row << 16;
         }
         __syncthreads();
         int32_t* t = src;
@@ -507,44 +608,65 @@ __device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w,
         __syncthreads();
     }
     if (threadIdx.x == 0) p.ucount[w] = carry;
-    for (int j = threadIdx.x; j < n; j += THREADS) p.pos_of[p0 + j] = dst[rank[j]] - 1;
+    for (int j = threadIdx.x; j < n; j += THREADS) p.pos_of[p0 + j] = dst[rank[j] & 0xffffu] - 1;
 }
 
+// One warp per window; the last of the launches that run side by side, it ends after the others.
+constexpr int kSortWarps = 4;
 template <int WH>
+__global__ void __launch_bounds__(32 * kSortWarps) wcsr_sort_windows_kernel(const CondenseParams p) {
+    __shared__ int32_t own[kSortWarps][kWarpWindow], cols[kSortWarps][kWarpWindow];
+    __shared__ int offs[kSortWarps][WH + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t w = blockIdx.x * int64_t{kSortWarps} + warp;
+    if (w < p.nwin) {
+        const int64_t r0 = w * WH, p0 = p.row_ptr[r0];
+        int* off = offs[warp];
+        for (int i = lane; i <= WH; i += 32) off[i] = static_cast<int>(p.row_ptr[min(r0 + i, p.m)] - p0);
+        __syncwarp();
+        const int n = off[WH];
+        if (n <= 64) sort_window<WH, 2>(p, w, p0, n, off, own[warp], cols[warp]);
+        else if (n <= 128) sort_window<WH, 4>(p, w, p0, n, off, own[warp], cols[warp]);
+        else if (n <= kWarpWindow) sort_window<WH, 8>(p, w, p0, n, off, own[warp], cols[warp]);
+    }
+    grid_wait();
+}
+
+template <int WH, int THREADS>
 __device__ __forceinline__ void load_offsets(const CondenseParams& p, int64_t w, int* off) {
     const int64_t r0 = w * WH;
     const int64_t p0 = p.row_ptr[r0];
-    for (int i = threadIdx.x; i <= WH; i += blockDim.x) off[i] = static_cast<int>(p.row_ptr[min(r0 + i, p.m)] - p0);
-}
-
-template <int WH>
-__global__ void __launch_bounds__(128) wcsr_condense_kernel(const CondenseParams p) {
-    __shared__ int32_t keys[2 * kSmallWindow];
-    __shared__ uint16_t rank[kSmallWindow];
-    __shared__ int off[WH + 1];
-    const int64_t w = blockIdx.x;
-    load_offsets<WH>(p, w, off);
+    for (int i = threadIdx.x; i <= WH; i += THREADS) off[i] = static_cast<int>(p.row_ptr[min(r0 + i, p.m)] - p0);
     __syncthreads();
-    const int n = off[WH];
-    if (n > kSmallWindow) {
-        if (threadIdx.x == 0) p.big[atomicAdd(p.n_big, 1)] = static_cast<int32_t>(w);
-        return;
-    }
-    merge_window<WH, 128>(p, w, p.row_ptr[w * WH], n, off, keys, kSmallWindow, rank);
 }
 
-// Windows of more than kLargeWindow entries: bits of the columns [c0, c0 + 32 words) and the set bits before each word.
+// One CTA per listed window.  shared memory: two key arrays and the ranks.
+template <int WH, int THREADS>
+__global__ void __launch_bounds__(THREADS) wcsr_merge_windows_kernel(const CondenseParams p) {
+    constexpr int kCap = THREADS == 1024 ? kLargeWindow : kMergeWindow;
+    extern __shared__ int32_t dyn[];
+    __shared__ int off[WH + 1];
+    grid_trigger();
+    const int64_t w = p.list[blockIdx.x];
+    load_offsets<WH, THREADS>(p, w, off);
+    merge_window<WH, THREADS>(p, w, p.row_ptr[w * WH], off[WH], off, dyn, kCap, reinterpret_cast<uint32_t*>(dyn + 2 * kCap));
+    grid_wait();
+}
+
+// Bits of the columns [c0, c0 + 32 words) and the set bits before each word, as many at a time as there is room for.
+constexpr int kBitmapThreads = 512;
 template <int WH>
 __device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, uint32_t* bits, int max_words) {
     __shared__ long long scratch[32];
+    constexpr int T = kBitmapThreads;
     uint32_t* prefix = bits + max_words;
     int found = 0;                           // condensed columns before c0
     for (int64_t c0 = 0; c0 < p.k; c0 += int64_t{32} * max_words) {
         const int words = static_cast<int>(min(static_cast<int64_t>(max_words), (p.k - c0 + 31) / 32));
         __syncthreads();
-        for (int i = threadIdx.x; i < words; i += 1024) bits[i] = 0u;
+        for (int i = threadIdx.x; i < words; i += T) bits[i] = 0u;
         __syncthreads();
-        for (int j = threadIdx.x; j < n; j += 1024) {
+        for (int j = threadIdx.x; j < n; j += T) {
             const int r = row_in_window<WH>(off, j);
             const int64_t c = checked_column(p, p0 + j, p0 + off[r]) - c0;
             if (c0 == 0) p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
@@ -552,43 +674,37 @@ __device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w
         }
         __syncthreads();
         long long carry = found;
-        for (int base = 0; base < words; base += 1024) {
+        for (int base = 0; base < words; base += T) {
             const int i = base + threadIdx.x;
             long long total;
-            const long long before = carry + block_exclusive_sum(i < words ? __popc(bits[i]) : 0, scratch, &total);
+            const long long before = carry + block_exclusive_sum<T>(i < words ? __popc(bits[i]) : 0, scratch, &total);
             if (i < words) prefix[i] = static_cast<uint32_t>(before);
             carry += total;
         }
         __syncthreads();
         found = static_cast<int>(carry);
-        for (int j = threadIdx.x; j < n; j += 1024) {
+        for (int j = threadIdx.x; j < n; j += T) {
             const int r = row_in_window<WH>(off, j);
             const int64_t c = checked_column(p, p0 + j, p0 + off[r]) - c0;
             if (c < 0 || c >= int64_t{32} * words) continue;
             p.pos_of[p0 + j] = static_cast<int32_t>(prefix[c >> 5] + __popc(bits[c >> 5] & ((1u << (c & 31)) - 1u)));
         }
-        for (int i = threadIdx.x; i < words; i += 1024)
+        for (int i = threadIdx.x; i < words; i += T)
             for (uint32_t x = bits[i]; x; x &= x - 1) atomicAdd(p.refs + c0 + 32 * int64_t{i} + (__ffs(x) - 1), 1);
     }
     if (threadIdx.x == 0) p.ucount[w] = found;
 }
 
-constexpr int kLargeSmem = kLargeWindow * 10;                 // two key arrays and the ranks; or bits and their prefixes
+constexpr int kMostBitmap = 216 * 1024;                       // bits and their prefixes, 8 bytes per 32 columns
 template <int WH>
-__global__ void __launch_bounds__(1024) wcsr_condense_large_kernel(const CondenseParams p) {
+__global__ void __launch_bounds__(kBitmapThreads) wcsr_bitmap_windows_kernel(const CondenseParams p, int max_words) {
     extern __shared__ int32_t dyn[];
     __shared__ int off[WH + 1];
-    for (int i = blockIdx.x; i < *p.n_big; i += gridDim.x) {
-        const int64_t w = p.big[i];
-        __syncthreads();
-        load_offsets<WH>(p, w, off);
-        __syncthreads();
-        const int n = off[WH];
-        if (n <= kLargeWindow)
-            merge_window<WH, 1024>(p, w, p.row_ptr[w * WH], n, off, dyn, kLargeWindow, reinterpret_cast<uint16_t*>(dyn + 2 * kLargeWindow));
-        else
-            bitmap_window<WH>(p, w, p.row_ptr[w * WH], n, off, reinterpret_cast<uint32_t*>(dyn), kLargeSmem / 8);
-    }
+    grid_trigger();
+    const int64_t w = p.list[blockIdx.x];
+    load_offsets<WH, kBitmapThreads>(p, w, off);
+    bitmap_window<WH>(p, w, p.row_ptr[w * WH], off[WH], off, reinterpret_cast<uint32_t*>(dyn), max_words);
+    grid_wait();
 }
 
 // CTA 0: window_row_ptr; the others: how many columns are referenced at all
@@ -807,11 +923,27 @@ cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_
 
 namespace {
 
+// Every window by its kernel.  The launches touch disjoint data and run side by side, each ending behind the one before
+// it (grid_wait); the first starts when the stream gets there.
 template <int WH>
-void condense(const CondenseParams& p, int sms, cudaStream_t st) {
-    wcsr_condense_kernel<WH><<<static_cast<unsigned>(p.nwin), 128, 0, st>>>(p);
-    cudaFuncSetAttribute(wcsr_condense_large_kernel<WH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLargeSmem);
-    wcsr_condense_large_kernel<WH><<<static_cast<unsigned>(sms), 1024, kLargeSmem, st>>>(p);
+bool condense(CondenseParams p, const WindowLists& lists, const int* count, cudaStream_t st) {
+    bool first = true;
+    auto launch = [&](auto kernel, int64_t grid, int threads, size_t smem, const auto&... args) {
+        if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) return false;
+        if (!first) return launch_dependent(kernel, dim3(static_cast<unsigned>(grid)), threads, smem, st, p, args...) == cudaSuccess;
+        first = false;
+        kernel<<<static_cast<unsigned>(grid), threads, smem, st>>>(p, args...);
+        return cudaGetLastError() == cudaSuccess;
+    };
+    auto list = [&](int which, auto kernel, int threads, size_t smem, const auto&... args) {
+        p.list = lists.list[which];
+        return count[which] == 0 || launch(kernel, count[which], threads, smem, args...);
+    };
+    const int words = static_cast<int>(std::min<int64_t>((p.k + 31) / 32, kMostBitmap / 8));
+    return list(kListBitmap, wcsr_bitmap_windows_kernel<WH>, kBitmapThreads, static_cast<size_t>(words) * 8, words) &&
+           list(kListLarge, wcsr_merge_windows_kernel<WH, 1024>, 1024, size_t{kLargeWindow} * 12) &&
+           list(kListMerge, wcsr_merge_windows_kernel<WH, 256>, 256, size_t{kMergeWindow} * 12) &&
+           launch(wcsr_sort_windows_kernel<WH>, (p.nwin + kSortWarps - 1) / kSortWarps, 32 * kSortWarps, 0);
 }
 
 }  // namespace
@@ -838,14 +970,15 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     struct Flags {
         int err;                              // CSR error code
         int overflow;                         // of the scan
-        int n_big;                            // windows of the second condensation kernel
+        int n_listed[kLists];                 // windows of the condensation kernels that go by lists
         int bad;                              // an entry out of range or not ascending
         int64_t nnz;
         unsigned long long distinct;          // columns that are referenced
     } flags = {};
     Flags* d_flags = nullptr;
-    uint8_t* d_work = nullptr;                // the entries' rows and places, window lengths, long windows, gather counts
-    auto release = [&]() { dev_free(d_flags, st); dev_free(d_work, st); };
+    int32_t* d_lists = nullptr;               // those windows
+    uint8_t* d_work = nullptr;                // the entries' rows and places, window lengths, gather counts
+    auto release = [&]() { dev_free(d_flags, st); dev_free(d_lists, st); dev_free(d_work, st); };
     auto fail = [&](int code) {
         cudaGetLastError();                  // (of a call that failed: not for a later check to find)
         release();
@@ -855,13 +988,15 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     };
     auto alloc = [&](void** ptr, size_t bytes) { return dev_alloc(ptr, bytes, st) == cudaSuccess; };
 
-    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags))) return fail(SPMM_ERR_ALLOC);
+    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags)) || !alloc(reinterpret_cast<void**>(&d_lists), static_cast<size_t>(kLists * nwin + 1) * 4))
+        return fail(SPMM_ERR_ALLOC);
     if (cudaMemsetAsync(d_flags, 0, sizeof(Flags), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
     auto read_flags = [&]() {
         return cudaMemcpyAsync(&flags, d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
     };
     const unsigned check_grid = static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048));
-    if (m > 0) csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, &d_flags->err, &d_flags->nnz);
+    const WindowLists lists = {wh, k, {d_lists, d_lists + nwin, d_lists + 2 * nwin}, d_flags->n_listed};
+    if (m > 0) csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, &d_flags->err, &d_flags->nnz, lists);
     if (!read_flags()) return fail(SPMM_ERR_CUDA);
     if (flags.err != 0) return fail(flags.err);
     const int64_t nnz = flags.nnz;
@@ -876,7 +1011,7 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         return at;
     };
     const size_t o_row_of = section(static_cast<size_t>(nnz) * 4), o_pos_of = section(static_cast<size_t>(nnz) * 4);
-    const size_t o_big = section(static_cast<size_t>(nwin) * 4), o_ucount = section(static_cast<size_t>(nwin) * 4), o_refs = section(static_cast<size_t>(k) * 4);
+    const size_t o_ucount = section(static_cast<size_t>(nwin) * 4), o_refs = section(static_cast<size_t>(k) * 4);
     if (!alloc(reinterpret_cast<void**>(&d_work), work_bytes) ||
         !alloc(reinterpret_cast<void**>(d_window_row_ptr), static_cast<size_t>(nwin + 1) * 4))
         return fail(SPMM_ERR_ALLOC);
@@ -891,15 +1026,11 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     cp.ucount = reinterpret_cast<int32_t*>(d_work + o_ucount);
     cp.refs = reinterpret_cast<int32_t*>(d_work + o_refs);
     cp.bad = &d_flags->bad;
-    cp.big = reinterpret_cast<int32_t*>(d_work + o_big);
-    cp.n_big = &d_flags->n_big;
+    cp.list = nullptr;
     const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 16384));
     if (cudaMemsetAsync(cp.ucount, 0, work_bytes - o_ucount, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);     // and the gather counts behind it
-    if (nnz > 0 && k > 0) {
-        if (wh == 16) condense<16>(cp, sms, st);
-        else condense<64>(cp, sms, st);
-    }
     if (nnz > 0 && k == 0) return fail(SPMM_ERR_OUT_OF_RANGE);
+    if (nnz > 0 && !(wh == 16 ? condense<16>(cp, lists, flags.n_listed, st) : condense<64>(cp, lists, flags.n_listed, st))) return fail(SPMM_ERR_CUDA);
     wcsr_row_ptr_kernel<<<1 + static_cast<unsigned>(std::min<int64_t>((k + 1023) / 1024, 128)), 1024, 0, st>>>(
         cp.ucount, nwin, b_col, *d_window_row_ptr, &d_flags->overflow, cp.refs, k, &d_flags->distinct);
     if (cudaMemcpyAsync(out->window_row_ptr.data(), *d_window_row_ptr, static_cast<size_t>(nwin + 1) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||

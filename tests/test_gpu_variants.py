@@ -267,6 +267,42 @@ def test_wcsr_built_on_the_gpu_is_bit_exact(lib, dtype, wh, m, k, dens):
         lib.spmm_destroy(h0)
 
 
+@pytest.mark.parametrize("dtype,wh,k", [("fp16", 16, 30000), ("tf32", 16, 5_000_000), ("bf16", 64, 884_737), ("fp8", 64, 60000)])
+def test_wcsr_gpu_builder_by_window_size(lib, dtype, wh, k):
+    """Windows at the edges of the builder's kernels (up to 64, 128, 256 entries one warp; from an entry per 256 columns on,
+    and above 18,432 entries, a bitmap of 884,736 columns at a time; up to 2048 and 18,432 entries merged), empty ones, rows
+    that hold everything; more columns than the first reuse class has room for, with many ties: the same arrays as the
+    host builder's."""
+    import torch
+    rng = np.random.default_rng(wh + k)
+    lens = []
+    for total, rows in ((64, wh), (65, 2), (128, wh), (129, 1), (256, wh), (257, wh), (2048, wh), (2049, 3), (0, wh), (1, 1), (3456, 5), (3457, wh),
+                        (18432, wh), (18433, 2), (25000, wh), (200, 3), (40, wh), (5000, 1)):
+        cut = np.sort(rng.integers(0, total + 1, rows - 1))
+        part = np.diff(np.concatenate(([0], cut, [total])))
+        lens += list(rng.permutation(np.concatenate((part, np.zeros(wh - rows, np.int64)))))
+    lens = np.asarray(lens[:-(wh // 2)], np.int64)                     # a ragged last window
+    m = lens.size
+    rp = np.concatenate(([0], np.cumsum(lens))).astype(np.int64)
+    ci = np.concatenate([np.sort(rng.choice(k, n, replace=False)) for n in lens] + [np.zeros(0, np.int64)]).astype(np.int32)
+    vals = wl.to_storage(rng.uniform(-1, 1, ci.size), dtype)
+    d = [torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), to_device(vals)]
+    h = lib.spmm_wcsr_create_csr_device(m, k, *[x.data_ptr() for x in d], dtype, wh)
+    h0 = lib.spmm_wcsr_create_csr(m, k, rp, ci, vals, dtype, wh)
+    try:
+        bits = {4: np.uint32, 2: np.uint16, 1: np.uint8}[wl.elem_size(dtype)]
+        for which, t in ((lib.X_WCSR_WINDOW_ROW_PTR, np.int32), (lib.X_WCSR_WINDOW_COL_IDX, np.int32), (lib.X_WCSR_VALUES, bits),
+                         (lib.X_WCSR_GROUP_CLASS, np.uint8), (lib.X_WCSR_TASKS, np.int32), (lib.X_WCSR_BIN_PTR, np.int32), (lib.X_WCSR_BIN_TASKS, np.int32)):
+            assert np.array_equal(lib.spmm_export(h, which, t), lib.spmm_export(h0, which, t)), which
+        assert lib.spmm_get_info(h, 64) == lib.spmm_get_info(h0, 64)
+        N = 16 // wl.elem_size(dtype)
+        Bs = wl.dense(3, k, N, ("normal", 0.0, 1.0), dtype)
+        assert np.array_equal(run_gpu(lib, h, Bs, m, N), run_gpu(lib, h0, Bs, m, N))
+    finally:
+        lib.spmm_destroy(h)
+        lib.spmm_destroy(h0)
+
+
 @pytest.mark.parametrize("dtype", ["tf32", "fp16", "fp8"])
 def test_bcsr_gpu_builder_with_many_block_columns(lib, dtype):
     """More than 196,608 block columns: the builder's bitmap takes more than 48 KB of shared memory."""
