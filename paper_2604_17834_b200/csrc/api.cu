@@ -6,6 +6,7 @@
 #include <atomic>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -411,7 +412,8 @@ int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
     const size_t o_item_fill = section(f.item_fill.size()), o_bin_fill = section(f.bin_fill.size());
     const size_t o_item_fill_n = section(f.item_fill_narrow.size()), o_bin_fill_n = section(f.bin_fill_narrow.size());
     const size_t o_merge = section(3 * nm), o_class = section((f.grp_class.size() + 3) / 4);
-    std::vector<int32_t> w(words, 0);
+    const size_t n_words = words;
+    const std::unique_ptr<int32_t[]> w(new int32_t[n_words]);          // (what lies between the sections is never read)
     // the fills themselves are written on the GPU, behind what is copied
     const size_t o_fills = section(2 * static_cast<size_t>(f.item_fill.empty() ? 0 : f.item_fill.back()));
     const size_t o_fills_n = section(2 * static_cast<size_t>(narrow ? f.item_fill_narrow.back() : 0));
@@ -426,6 +428,7 @@ int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
         w[o_items + 4 * i] = t.window;
         w[o_items + 4 * i + 1] = t.slot;
         w[o_items + 4 * i + 2] = t.count;
+        w[o_items + 4 * i + 3] = 0;
     }
     auto put = [&](size_t at, const void* src, size_t bytes) {
         if (bytes) std::memcpy(&w[at], src, bytes);
@@ -441,7 +444,7 @@ int upload_wcsr_plan(spmm_handle_s* h, cudaStream_t stream) {
     put(o_merge + 2 * nm, f.merge_nparts.data(), nm * 4);
     put(o_class, f.grp_class.data(), f.grp_class.size());
     if (!dev_alloc_ok(&h->d_plan, words * 4, stream)) return SPMM_ERR_ALLOC;
-    if (cudaMemcpyAsync(h->d_plan, w.data(), w.size() * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess) return cuda_error();
+    if (cudaMemcpyAsync(h->d_plan, w.get(), n_words * 4, cudaMemcpyHostToDevice, stream) != cudaSuccess) return cuda_error();
     int32_t* fills = h->d_plan + o_fills;
     int32_t* fills_n = h->d_plan + o_fills_n;
     if (expand_wcsr_fills(static_cast<int64_t>(ni), h->d_plan + o_tasks, h->d_plan + o_bin_tasks, h->d_plan + o_item_fill, f.kt, fills, stream) != cudaSuccess ||

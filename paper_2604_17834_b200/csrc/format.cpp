@@ -446,15 +446,18 @@ public:
     }
     // takes the lightest bin and gives it back with `cost` units more
     int32_t add(int64_t cost) {
-        while (bits_[at_] == 0) ++at_;
+        while (bits_[at_] == 0) {
+            ++at_;
+            if (++word_ == per_) word_ = 0;
+        }
         const int32_t bit = __builtin_ctzll(bits_[at_]);
         bits_[at_] &= bits_[at_] - 1;
         bits_[at_ + static_cast<size_t>(cost) * per_] |= uint64_t{1} << bit;
-        return static_cast<int32_t>(at_ % per_) * 64 + bit;
+        return static_cast<int32_t>(word_) * 64 + bit;
     }
 
 private:
-    size_t per_, at_ = 0;           // words per load; the word that holds the lightest bin, or one before it
+    size_t per_, at_ = 0, word_ = 0;  // words per load; the word that holds the lightest bin, or one before it; its place in its load
     std::vector<uint64_t> bits_;
 };
 
@@ -513,7 +516,12 @@ static int64_t lpt_max_load(const std::vector<int32_t>& window_row_ptr, int64_t 
 }
 
 int default_split_cols(const std::vector<int32_t>& window_row_ptr, int64_t nwin, int64_t P, int n_bins) {
-    // candidates: one bin's share of the padded columns and its half, quarter and eighth
+    // candidates: one bin's share of the padded columns and its half, quarter and eighth.  Whatever the size, the bins
+    // hold all columns and a fixed cost per window: a load within 2 % of their average needs no comparison with the sizes
+    // that have not been tried (usually the first one: 60,000 power-law rows, the four evaluations 50 us, one 13).
+    int64_t least = P;
+    for (int64_t w = 0; w < nwin; ++w) least += window_row_ptr[w + 1] > window_row_ptr[w] ? kTaskFixedCost : 0;
+    least = cdiv(least, n_bins);
     int cand[4];
     int64_t load[4], best = INT64_MAX;
     for (int i = 0; i < 4; ++i) {
@@ -521,9 +529,12 @@ int default_split_cols(const std::vector<int32_t>& window_row_ptr, int64_t nwin,
         cand[i] = static_cast<int>(std::min<int64_t>(65536, std::max<int64_t>(128, t)));
         load[i] = (i > 0 && cand[i] == cand[i - 1]) ? load[i - 1] : lpt_max_load(window_row_ptr, nwin, cand[i], n_bins);
         best = std::min(best, load[i]);
+        const int64_t bound = i < 3 ? std::min(best, least) : best;      // no later size can do better than this
+        for (int j = 0; j <= i; ++j) {
+            if (load[j] * 100 <= bound * 102) return cand[j];
+            if (load[j] * 100 <= best * 102) break;                      // open until the later ones are known
+        }
     }
-    for (int i = 0; i < 4; ++i)
-        if (load[i] * 100 <= best * 102) return cand[i];
     return cand[3];
 }
 
@@ -540,28 +551,33 @@ int plan_wcsr(WcsrHost* out, int T, int n_bins, int es) {
     out->merge_nparts.clear();
     out->n_empty = out->n_split = out->n_slots = 0;
     std::vector<int32_t> empty_windows;
+    const int32_t* ptr = out->window_row_ptr.data();
+    int64_t n_tasks = 0, n_slots = 0;
     for (int64_t w = 0; w < nwin; ++w) {
-        const int32_t len = out->window_row_ptr[w + 1] - out->window_row_ptr[w];
-        if (len == 0) {
-            empty_windows.push_back(static_cast<int32_t>(w));
-            continue;
-        }
-        const int32_t nchunk = len <= T ? 1 : static_cast<int32_t>(cdiv(len, T));
-        if (nchunk > 1) {
-            out->merge_window.push_back(static_cast<int32_t>(w));
-            out->merge_first.push_back(static_cast<int32_t>(out->n_slots));
+        const int32_t len = ptr[w + 1] - ptr[w];
+        n_tasks += len <= T ? (len > 0) : cdiv(len, T);
+    }
+    out->tasks.resize(static_cast<size_t>(n_tasks));
+    WcsrTask* next = out->tasks.data();
+    int32_t most = 0;
+    for (int64_t w = 0; w < nwin; ++w) {
+        const int32_t len = ptr[w + 1] - ptr[w], window = static_cast<int32_t>(w);
+        if (len > 0 && len <= T) {
+            most = std::max(most, len);
+            *next++ = WcsrTask{window, 0, len, -1};
+        } else if (len == 0) {
+            empty_windows.push_back(window);
+        } else {
+            const int32_t nchunk = static_cast<int32_t>(cdiv(len, T));
+            most = T;
+            out->merge_window.push_back(window);
+            out->merge_first.push_back(static_cast<int32_t>(n_slots));
             out->merge_nparts.push_back(nchunk);
             out->n_split++;
-        }
-        for (int32_t c = 0; c < nchunk; ++c) {
-            WcsrTask t;
-            t.window = static_cast<int32_t>(w);
-            t.q0 = c * T;
-            t.count = std::min(T, len - c * T);
-            t.slot = nchunk > 1 ? static_cast<int32_t>(out->n_slots++) : -1;
-            out->tasks.push_back(t);
+            for (int32_t c = 0; c < nchunk; ++c) *next++ = WcsrTask{window, c * T, std::min(T, len - c * T), static_cast<int32_t>(n_slots++)};
         }
     }
+    out->n_slots = n_slots;
     out->n_empty = static_cast<int64_t>(empty_windows.size());
     for (int32_t w : empty_windows) {
         out->merge_window.push_back(w);
@@ -573,10 +589,8 @@ int plan_wcsr(WcsrHost* out, int T, int n_bins, int es) {
     const int64_t ntasks = static_cast<int64_t>(out->tasks.size());
     std::vector<int32_t> order(static_cast<size_t>(ntasks));
     {   // heaviest first, equal ones in task order: a counting sort
-        int32_t most = 0;
-        for (const WcsrTask& t : out->tasks) most = std::max(most, t.count);
-        std::vector<int32_t> at(static_cast<size_t>(most / out->b_col) + 2, 0);
-        auto key = [&](int64_t t) { return static_cast<size_t>((most - out->tasks[t].count) / out->b_col); };
+        std::vector<int32_t> at(static_cast<size_t>(most / kLoadUnit) + 2, 0);
+        auto key = [&](int64_t t) { return static_cast<unsigned>(most - out->tasks[t].count) / kLoadUnit; };
         for (int64_t t = 0; t < ntasks; ++t) at[key(t) + 1]++;
         for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
         for (int64_t t = 0; t < ntasks; ++t) order[at[key(t)]++] = static_cast<int32_t>(t);

@@ -154,6 +154,7 @@ struct WcsrHost {
 struct WcsrRowStream {
     int pack = 0, task_max = 0, part_len = 0;
     int32_t n_tasks = 0, n_parts = 0, n_long = 0, n_slots = 0;
+    uint8_t* d_block = nullptr;      // one allocation, in which the arrays below lie
     int32_t* d_order = nullptr;      // [m + 1]
     int32_t* d_tasks = nullptr;      // int4 [n_tasks]
     int32_t* d_parts = nullptr;      // int4 [n_parts]

@@ -1361,8 +1361,7 @@ unsigned grid_for(int64_t n, int per) { return static_cast<unsigned>(std::max<in
 }  // namespace
 
 void free_wcsr_rows(WcsrRowStream* s, cudaStream_t st) {
-    void* const arrays[] = {s->d_order, s->d_tasks, s->d_parts, s->d_longs, s->d_col, s->d_val, s->d_counters, s->d_total};
-    for (void* ptr : arrays) dev_free(ptr, st);
+    dev_free(s->d_block, st);
     *s = WcsrRowStream();
 }
 
@@ -1371,7 +1370,6 @@ int finish_wcsr_rows(WcsrRowStream* s, cudaStream_t st) {
     int32_t total[4] = {0, 0, 0, 0};
     if (cudaMemcpyAsync(total, s->d_total, sizeof(total), cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
         return SPMM_ERR_CUDA;
-    dev_free(s->d_total, st);
     s->d_total = nullptr;
     s->n_tasks = total[0];
     s->n_parts = total[1];
@@ -1427,13 +1425,20 @@ int build_wcsr_rows_device(int64_t m, int64_t nnz, const int64_t* d_row_ptr, con
         if (code) free_wcsr_rows(out, st);
         return code;
     };
-    auto alloc = [&](auto** ptr, int64_t bytes) { return dev_alloc_ok(ptr, static_cast<size_t>(bytes), st); };
     const int64_t counter_bytes = 32 + max_long * kRowsMaxTiles * 4;
-    if (!alloc(&d_work, work_bytes) ||
-        !alloc(&out->d_order, (m + 1) * 4) || !alloc(&out->d_tasks, max_tasks * 16) || !alloc(&out->d_parts, max_parts * 16) ||
-        !alloc(&out->d_longs, max_long * 16) || !alloc(&out->d_col, entries * 4) || !alloc(&out->d_val, entries * es) ||
-        !alloc(&out->d_counters, counter_bytes) || !alloc(&out->d_total, 16))
+    const int64_t o_order = 0, o_tasks = o_order + up((m + 1) * 4), o_parts = o_tasks + up(max_tasks * 16), o_longs = o_parts + up(max_parts * 16);
+    const int64_t o_col = o_longs + up(max_long * 16), o_val = o_col + up(entries * 4), o_counters = o_val + up(entries * es);
+    const int64_t o_total = o_counters + up(counter_bytes);
+    if (!dev_alloc_ok(&d_work, static_cast<size_t>(work_bytes), st) || !dev_alloc_ok(&out->d_block, static_cast<size_t>(o_total + 16), st))
         return done(SPMM_ERR_ALLOC);
+    out->d_order = reinterpret_cast<int32_t*>(out->d_block + o_order);
+    out->d_tasks = reinterpret_cast<int32_t*>(out->d_block + o_tasks);
+    out->d_parts = reinterpret_cast<int32_t*>(out->d_block + o_parts);
+    out->d_longs = reinterpret_cast<int32_t*>(out->d_block + o_longs);
+    out->d_col = reinterpret_cast<int32_t*>(out->d_block + o_col);
+    out->d_val = out->d_block + o_val;
+    out->d_counters = reinterpret_cast<unsigned*>(out->d_block + o_counters);
+    out->d_total = reinterpret_cast<int32_t*>(out->d_block + o_total);
     int32_t* d_at = reinterpret_cast<int32_t*>(d_work);
     int4* d_start = reinterpret_cast<int4*>(d_work + o_start);
     ClassSum* d_sums = reinterpret_cast<ClassSum*>(d_work + o_sums);
