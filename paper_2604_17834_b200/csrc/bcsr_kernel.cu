@@ -425,6 +425,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             uint32_t it = 0, tile_i = 0;
             bool ready = false;
             bool ok = true;
+            operands_ready();               // (the time its waits may take is not to include the launch before this one)
             int4 tcd, tcd_next;
             for (; ok && next_tile(tile_i, &tcd, &tcd_next, &ok); ++tile_i) {
                 const int n0 = tcd.y * Cfg::kBnT;

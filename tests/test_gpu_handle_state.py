@@ -296,3 +296,29 @@ def test_workspace_bytes_is_what_a_run_allocates(lib, matrix, opt):
             assert lib.spmm_get_info(h, 0)["workspace_bytes"] == 0
         finally:
             lib.spmm_destroy(h)
+
+
+def test_waits_do_not_count_the_launch_before(lib):
+    """One block-row of 2048 blocks: a launch of a millisecond on a few SMs.  The next one starts beside it on the others and
+    waits for its end; that time is no part of its bounded waits, whose limit is a third of it here."""
+    import torch
+    m, k, N = 128, 262144, 128
+    rp = torch.arange(m + 1, dtype=torch.int64, device="cuda") * k
+    ci = torch.arange(k, dtype=torch.int32, device="cuda").repeat(m)
+    va = torch.ones(m * k, dtype=torch.bfloat16, device="cuda")
+    h = lib.spmm_bcsr_create_csr_device(m, k, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), "bf16", 128)
+    try:
+        B = torch.ones((k, N), dtype=torch.bfloat16, device="cuda")
+        C = torch.zeros((m, N), dtype=torch.float32, device="cuda")
+        st = torch.cuda.current_stream().cuda_stream
+        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, st)
+        torch.cuda.synchronize()
+        lib.spmm_set_wait_limit_ns(300_000)
+        for _ in range(4):
+            lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, st)
+        torch.cuda.synchronize()
+        lib.spmm_check(h)
+        assert bool(torch.all(C == k))
+    finally:
+        lib.spmm_set_wait_limit_ns(2_000_000_000)
+        lib.spmm_destroy(h)
