@@ -128,6 +128,10 @@ struct spmm_handle_s {
     int32_t* d_scta_ptr = nullptr;
     CUtensorMap tmAs;                // map of d_svals
     int stack_groups = 0;            // token groups of the stacked launch's tile (2, or 1: see ensure_schedule)
+    // launches by half tiles (see ensure_schedule), and their maps: boxes of 64 rows of stacked blocks, of 64 tokens of X, of
+    // 16 tokens of C or Y
+    bool split = false, stack_split = false;
+    CUtensorMap tmAsh, tmBh, tmCh;
     CUtensorMap tmB3s;               // whole-tile map of B for the stacked launch's token tile
     bool tmB3s_ok = false;
     int k_split = 0;                 // opts.k_split (1: cut outlier block-rows into parts)
@@ -289,19 +293,23 @@ int new_bcsr_handle(spmm_handle_s** hp, int64_t m, int64_t k, int dtype, int blo
     return SPMM_OK;
 }
 
-// Tensor map of the stored blocks: box rows of min(b * es, 128) bytes, swizzle = the row bytes.
+// Map of stored blocks: box of `rows` rows of min(b * es, 128) bytes (a stage unit's: the whole block row, or one column
+// slice of it, at most 128 bytes per piece), swizzle = the row bytes.
+int encode_blocks(const spmm_handle_s* h, CUtensorMap* map, const void* blocks, int64_t total_rows, int rows) {
+    const int b = h->bcsr.b;
+    const int unit_bytes = b / bcsr_k_split(b, h->es) * h->es;
+    const int row_bytes = unit_bytes < 128 ? unit_bytes : 128;
+    const CUtensorMapSwizzle swz = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                  : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
+    return encode_2d(map, h->dtype, blocks, static_cast<uint64_t>(total_rows), b, static_cast<uint32_t>(rows), row_bytes / h->es, swz);
+}
+
+// Tensor map of the stored blocks.
 int encode_tmA(spmm_handle_s* h) {
     const BcsrHost& f = h->bcsr;
     if (f.nnzb <= 0) return SPMM_OK;
     if (static_cast<int64_t>(f.nnzb) * f.b >= (int64_t{1} << 31)) return SPMM_ERR_TOO_LARGE;
-    // (a stage unit's rows: the whole block row, or one column slice of it, at most 128 bytes per piece)
-    const int unit_bytes = f.b / bcsr_k_split(f.b, h->es) * h->es;
-    const int row_bytes = unit_bytes < 128 ? unit_bytes : 128;
-    const int bw = row_bytes / h->es;
-    const CUtensorMapSwizzle swz = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                  : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
-    int rc = encode_2d(&h->tmA, h->dtype, h->d_vals, static_cast<uint64_t>(f.nnzb) * f.b, f.b,
-                             static_cast<uint32_t>(f.b * bcsr_blocks_per_stage(f.b)), bw, swz);
+    const int rc = encode_blocks(h, &h->tmA, h->d_vals, f.nnzb * f.b, f.b * bcsr_blocks_per_stage(f.b));
     h->tmA_ok = rc == SPMM_OK;
     return rc;
 }
@@ -322,10 +330,8 @@ int setup_stack(spmm_handle_s* h) {
     if (!rc) rc = upload(&h->d_srows, st.rows.data(), st.rows.size() * 4);
     if (rc) return rc;
     std::vector<int32_t>().swap(h->stack.src);        // only needed to build the values
-    const int row_bytes = f.b * h->es;                // <= 128 for b <= 64
-    const CUtensorMapSwizzle swz = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
-                                  : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
-    return encode_2d(&h->tmAs, h->dtype, h->d_svals, static_cast<uint64_t>(st.ns) * kStackRows, f.b, kStackRows, f.b, swz);
+    rc = encode_blocks(h, &h->tmAs, h->d_svals, st.ns * kStackRows, kStackRows);         // (block rows of at most 128 bytes)
+    return rc ? rc : encode_blocks(h, &h->tmAsh, h->d_svals, st.ns * kStackRows, kStackRows / 2);
 }
 
 int create_bcsr(spmm_handle_t* out, const CsrView& a, int dtype, int block, const spmm_opts_t* opts) {
@@ -630,6 +636,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
         const CUtensorMapSwizzle swz = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                       : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
         rc = encode_2d(&h->tmB, h->dtype, B, static_cast<uint64_t>(N), static_cast<uint64_t>(h->k), 128, bw, swz);
+        if (!rc) rc = encode_2d(&h->tmBh, h->dtype, B, static_cast<uint64_t>(N), static_cast<uint64_t>(h->k), 64, bw, swz);
         EncodeTiledFn fn = get_encode_fn();
         auto whole_tile_map = [&](int g, CUtensorMap* out, bool* ok) {
             *ok = false;
@@ -656,6 +663,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
         const uint32_t kb = static_cast<uint32_t>(h->bcsr.b / bcsr_k_split(h->bcsr.b, h->es));
         const CUtensorMapSwizzle swz = h->es == 4 ? CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B : CU_TENSOR_MAP_SWIZZLE_128B;
         rc = encode_2d(&h->tmB, h->dtype, B, static_cast<uint64_t>(h->k), static_cast<uint64_t>(N), kb, tok, swz);
+        h->tmBh = h->tmB;
         // the same memory as [N / tok][k][tok]: one request then brings a whole token tile
         // (es * groups boxes); only full groups of tok tokens are covered, a ragged tail uses tmB
         EncodeTiledFn fn = get_encode_fn();
@@ -686,7 +694,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
 int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
     if (h->tmC_ptr == C && h->tmC_N == N) return SPMM_OK;
     if (h->col_major && h->c16) {            // stored without a map; the kernel is given a valid one all the same
-        h->tmC = h->tmB;
+        h->tmC = h->tmCh = h->tmB;
         return SPMM_OK;
     }
     EncodeTiledFn fn = get_encode_fn();
@@ -695,21 +703,22 @@ int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
     const CUtensorMapDataType dt = !h->c16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : (h->dtype == SPMM_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16);
     const cuuint32_t estr[2] = {1, 1};
-    CUresult r;
-    if (h->col_major) {
-        const cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->m), static_cast<cuuint64_t>(N)};
-        const cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->m) * h->cs};
-        const cuuint32_t box[2] = {w, 32};
-        const CUtensorMapSwizzle swz = w * h->cs == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE;
-        r = fn(&h->tmC, dt, 2, C, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    } else {
+    auto encode = [&](CUtensorMap* map, cuuint32_t tokens) {
+        if (h->col_major) {                  // (fp32: box rows of 64 bytes)
+            const cuuint64_t dims[2] = {static_cast<cuuint64_t>(h->m), static_cast<cuuint64_t>(N)};
+            const cuuint64_t strides[1] = {static_cast<cuuint64_t>(h->m) * h->cs};
+            const cuuint32_t box[2] = {w, tokens};
+            return fn(map, dt, 2, C, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        }
         const cuuint64_t dims[2] = {static_cast<cuuint64_t>(N), static_cast<cuuint64_t>(h->m)};
         const cuuint64_t strides[1] = {static_cast<cuuint64_t>(N) * h->cs};
-        const cuuint32_t box[2] = {32, w};
-        r = fn(&h->tmC, dt, 2, C, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-               CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    }
+        const cuuint32_t box[2] = {tokens, w};
+        return fn(map, dt, 2, C, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    CUresult r = encode(&h->tmC, 32);
+    if (r == CUDA_SUCCESS) r = encode(&h->tmCh, 16);
     if (r != CUDA_SUCCESS) return cuda_error();
     h->tmC_ptr = C;
     h->tmC_N = N;
@@ -812,6 +821,9 @@ int upload_schedule(spmm_handle_s* h, const BcsrSchedule& sc, const BcsrSchedule
     return rc ? rc : finish_uploads();
 }
 
+// Bytes that the longest tile of a launch brings into shared memory, from which on it runs by half tiles.
+constexpr int64_t kSplitMinBytes = 768 << 10;
+
 // Tile width, slab width and the tile schedule for dense width N (cached for the last N).
 int ensure_schedule(spmm_handle_s* h, int64_t N) {
     if (h->sched.N == N) return SPMM_OK;
@@ -836,6 +848,25 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     BcsrSchedule sc, ss;
     const BcsrStack& st = h->stack;
     int rc;
+    // Where the 128-token tiles of a launch are half as many as the CTAs or fewer, each is computed by two CTAs: half of
+    // its tokens in either, or, where 128-row stacked blocks are multiplied, half of their rows.  An SM's load rate and its
+    // tensor core bound such a launch; an SM then loads two thirds to three quarters as much.  The sums are the same.  Only
+    // from kSplitMinBytes in the longest tile on (shorter ones are latencies, and two CTAs fetch the blocks, or the tokens,
+    // twice); row groups only where their longest tile, not the work as a whole, decides when the last CTA ends.  us:
+    //   1500 x 9000, b = 64, 10 % full rows, fp16, N = 200 (3.4 MB a tile)   35.0 -> 22.5
+    //   3000 x 16000, b = 16, 10 % full rows, bf16, N = 256 (8 MB, grouped)  93.2 -> 75.3
+    //   600 x 6000, b = 16, 10 % full rows, TF32, N = 200 (6 MB, grouped)    55.2 -> 44.0
+    //   3000 x 6000, b = 32, 10 % full rows, fp16, N = 512 (3 MB, grouped)   25.9 -> 26.6: left alone
+    //   3584 x 18944, b = 64, density 0.1, bf16, N = 128 (1 MB)              9.6 -> 9.4
+    //   1024 x 4096 and back, b = 64, density 0.2, N = 300 (0.3 MB)          10.7 -> 11.0: left alone
+    //   6000 x 5000, b = 32, TF32, N = 1500 (5 MB; 3.7 MB of work per CTA)   48.8 -> 60.7: left alone
+    // (One MMA of two CTAs, cta_group::2, in their place: 16.3 for the fourth, 70 for the last: with N = 64 or 128 its
+    // exchange of the other half's block rows takes longer than the product.)
+    bool split = false, stack_split = false;
+    auto split_fits = [&](int64_t n_tiles, int64_t longest, int64_t rows) {
+        return N > 64 && 2 * n_tiles <= h->n_ctas && longest * (128 + rows) * f.b * h->es >= kSplitMinBytes && !h->dynamic &&
+               !(h->dtype == SPMM_FP8_E4M3 && !h->col_major);
+    };
     try {
         // dynamic scheduling: one list in the global order (slab by slab, longest block-row first)
         // b = 64 gains little per stacked block (its MMAs, not the operand traffic, bound it), so
@@ -860,6 +891,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                 rc = build_tile_schedule(order, lens, kTileFixedCost, n_tt, static_cast<int>(sw), h->n_ctas, &sc);
             } else if (!rc) {
                 rc = build_bcsr_schedule(f, n_tt, static_cast<int>(sw), h->dynamic ? 1 : h->n_ctas, &sc);
+                const int32_t I = f.nbr > 0 ? f.row_order[0] : 0;
+                split = !rc && groups == 1 && f.nbr > 0 && split_fits(f.nbr * n_tt, f.block_row_ptr[I + 1] - f.block_row_ptr[I], f.b);
             }
         } else {
             // The row groups get a launch and a schedule of their own; the launch of the remaining
@@ -901,11 +934,13 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                 // b = 32, N = 1500 (24 tiles of 157 stacked blocks, an 80 us launch whose CTAs were busy for 18 us on
                 // average) 79.6 -> 50.4; 8192 x 8192 fp16, b = 32, N = 504 78.7 -> 53.0; with the share exceeded by
                 // 15 % only (b = 16, N = 1000) 99.7 -> 103.6, the stacked blocks being fetched twice as often.
-                int64_t work = 0, longest = 0;
+                int64_t work = 0, rest = 0, most = 0;
                 for (int64_t x : totals) work += x;
-                for (int64_t g = 0; g < st.ng; ++g) longest = std::max<int64_t>(longest, st.ptr[g + 1] - st.ptr[g]);
-                longest = (longest + kStackTileFixedCost) * bcsr_stack_block_cost(kStackGroups);
-                if (!rc && N > 128 && 2 * longest * h->n_ctas > 3 * work) {
+                rest = work;
+                for (int64_t x : loads) rest -= x;
+                for (int64_t g = 0; g < st.ng; ++g) most = std::max<int64_t>(most, st.ptr[g + 1] - st.ptr[g]);
+                const int64_t longest = (most + kStackTileFixedCost) * bcsr_stack_block_cost(kStackGroups);
+                if (!rc && N > 64 && 2 * longest * h->n_ctas > 3 * work) {
                     BcsrSchedule kc, ks;
                     std::vector<int32_t> gu, gl;
                     for (int64_t g = 0; g < st.ng; ++g) {
@@ -914,6 +949,11 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                     }
                     rc = build_tile_schedule(gu, gl, kStackTileFixedCost, static_cast<int>((N + 127) / 128), static_cast<int>(2 * sws), h->n_ctas, &ks,
                                              bcsr_stack_block_cost(1), nullptr, &loads);
+                    // (in halves of 64 rows a stacked block costs 2 (128 + 64) instead of 2 (128 + 128); the other launch is
+                    // dealt for one CTA per tile, so that some of its lists start when the halves are done and count twice)
+                    const int64_t n_tiles = static_cast<int64_t>(ks.tiles.size() / 2);
+                    const int64_t whole = (most + kStackTileFixedCost) * bcsr_stack_block_cost(1);
+                    stack_split = !rc && split_fits(n_tiles, most, kStackRows) && (whole * 3 / 4 + 2 * rest / (h->n_ctas - n_tiles)) * 10 < whole * 9;
                     if (!rc) {
                         std::sort(loads.begin(), loads.end());
                         rc = build_tile_schedule(units, lens, kTileFixedCost, n_tt, static_cast<int>(sw), h->n_ctas, &kc,
@@ -950,6 +990,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
         }
     }
     h->stack_groups = ss.tiles.empty() ? 0 : ss.groups;
+    h->split = split;
+    h->stack_split = stack_split;
     h->tmB_N = -1;                   // (the stacked launch's map of B depends on its tile)
     h->sched_stack = std::move(ss);
     h->sched = std::move(sc);
@@ -1005,14 +1047,22 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         ps.use_3d = h->tmB3s_ok ? 1 : 0;
         ps.overlap = 1;
         p.overlap = 2;
-        cudaError_t es = launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
-                                             h->n_ctas, stream);
+        const int n_tiles = static_cast<int>(h->sched_stack.tiles.size() / 2);
+        cudaError_t es = h->stack_split ? launch_bcsr_stacked(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, h->tmAsh, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
+                                                             n_tiles, stream)
+                                       : launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
+                                                             h->n_ctas, stream);
         if (es != cudaSuccess) return cuda_error();
         if (h->sched.tiles.empty()) return SPMM_OK;
     }
     // dynamic: one CTA per tile, the schedule was built as a single list in the global order
     const int grid = h->dynamic ? static_cast<int>(h->sched.tiles.size() / 2) : h->n_ctas;
     if (grid <= 0) return SPMM_OK;
+    if (h->split) {
+        const cudaError_t eh = launch_bcsr(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, 0, tmA, h->tmBh, h->tmB3, h->tmCh, h->tmCh, p,
+                                           static_cast<int>(h->sched.tiles.size() / 2), stream);
+        return eh == cudaSuccess ? SPMM_OK : cuda_error();
+    }
     const bool ksplit = h->sched.n_slots > 0 && h->tmP_ok;
     if (ksplit) p.overlap = 1;          // the merge kernel's CTAs may be placed while this grid runs
     cudaError_t e = launch_bcsr(h->dtype, f.b, h->sched.groups, h->c16, h->col_major, h->dynamic, tmA, h->tmB, h->tmB3,

@@ -61,18 +61,24 @@ namespace {
 // A pipeline stage holds one "unit": kBps whole blocks (small b), or one of the kKS column
 // slices a block is cut into where its rows are longer than 128 bytes of 4-byte elements
 // (b = 64 / 128 with TF32: units of 32 columns, so that a stage stays a fraction of shared memory).
-template <int B, int H, int GROUPS, int STAGES, int ES, int CS, int CM>
+// SPLIT = 1: a tile of 128 tokens is computed by two CTAs: 64 tokens in either (MMA M = 64), or, with stacked blocks, 64 of
+// their 128 rows (MMA N = 64).
+template <int B, int H, int GROUPS, int STAGES, int ES, int CS, int CM, int SPLIT>
 struct BcsrCfg {
     static constexpr int kKS = (H == B) ? bcsr_k_split(B, ES) : 1;     // stage units per block
     static constexpr int kKB = B / kKS;                      // columns of A (= rows of B) per unit
     static constexpr int kBB = kKB * ES;                     // bytes of one unit row (its K extent)
     static constexpr int kKSteps = kBB / 32;                 // MMAs per unit and token group (32 bytes of K each)
     static constexpr int kBnT = 128 * GROUPS;
+    static constexpr bool kHalfTok = SPLIT && H == B, kHalfRows = SPLIT && H != B;
+    static constexpr int kTok = kHalfTok ? 64 : kBnT;        // tokens and block rows that this CTA stages
+    static constexpr int kRows = kHalfRows ? H / 2 : H;
+    static constexpr int kWarpTok = kHalfTok ? 16 : 32;      // tokens of an epilogue warp (M = 64: a quarter of them in 16 of its lanes)
     static constexpr int kTokBox = 128 / ES;                 // tokens per 128-byte box row (row-major B)
-    static constexpr int kNBox = GROUPS * (128 / kTokBox);   // boxes per unit (row-major B)
+    static constexpr int kNBox = kTok / kTokBox;             // boxes per unit (row-major B)
     static constexpr int kBoxBytes = kKB * 128;              // kKB k-rows x 128 B (row-major B)
-    static constexpr int kDenseBytes = kBnT * kBB;           // B tile of one unit
-    static constexpr int kABytes = H * kBB;
+    static constexpr int kDenseBytes = kTok * kBB;           // B tile of one unit
+    static constexpr int kABytes = kRows * kBB;
     // Small blocks carry too little work for the fixed cost of a pipeline stage (barrier
     // round trip, request issue, MMA hand-off): a stage holds several consecutive stored
     // blocks of the block-row, their B tiles first, then their A blocks (one request).
@@ -83,8 +89,8 @@ struct BcsrCfg {
     static constexpr uint32_t kASwizzle = kARowBytes == 128 ? SWZ_128B : (kARowBytes == 64 ? SWZ_64B : SWZ_32B);
     // column-major operands: a token group's tile is 128 rows x kXRowBytes, K-major
     static constexpr int kXRowBytes = kARowBytes;
-    static constexpr int kXGroupBytes = 128 * kXRowBytes;    // one K half of one token group
-    static constexpr int kAccCols = GROUPS * H;
+    static constexpr int kXGroupBytes = (kHalfTok ? 64 : 128) * kXRowBytes;    // one K half of one token group
+    static constexpr int kAccCols = GROUPS * kRows;
     static constexpr int kTmemCols = (2 * kAccCols <= 32) ? 32 : (2 * kAccCols <= 64 ? 64 : (2 * kAccCols <= 128 ? 128 : (2 * kAccCols <= 256 ? 256 : 512)));
     static constexpr int kBarrierBytes = 512;                // mbarriers, TMEM slot, flags, tile-index ring
     // Epilogue staging: a tile is kEpiCols accumulator columns (rows of C) x 32 tokens.  Every
@@ -99,7 +105,7 @@ struct BcsrCfg {
     // N = 2048, 44.0 us with them, 45.5 without.
     static constexpr bool kDirect = CM != 0 && CS == 2;
     static constexpr int kEpiCols = bcsr_epi_cols(B, CS == 2, CM != 0);
-    static constexpr int kEpiTileBytes = kEpiCols * 32 * CS;
+    static constexpr int kEpiTileBytes = kEpiCols * kWarpTok * CS;
     static constexpr int kEpiRoom = (227 * 1024 - 1024 /*align*/ - kBarrierBytes - STAGES * kStageBytes) / (4 * kEpiTileBytes);
     static constexpr int kEpiBufs = kEpiRoom < 8 ? kEpiRoom : 8;
     static constexpr int kStagingBytes = kDirect ? 0 : 4 * kEpiBufs * kEpiTileBytes;
@@ -109,6 +115,7 @@ struct BcsrCfg {
     static_assert(2 * kAccCols <= 512, "accumulators exceed TMEM");
     static_assert(kSmemBytes <= 227 * 1024, "stage ring exceeds shared memory");
     static_assert((2 * STAGES + 7 + 8) * 8 + 64 + 32 <= kBarrierBytes, "barrier area");
+    static_assert(!SPLIT || (GROUPS == 1 && (CM || kNBox >= 1)), "half of a 128-token tile");
     static_assert(kBps == 1 || (B <= 32 && kKS == 1), "multi-block stages are for the small block sizes");
     static_assert(kKS == 1 || kBB <= 128, "a column slice is at most one 128-byte row piece");
     static_assert(kBB % 32 == 0, "a block row must hold whole K steps");
@@ -117,9 +124,9 @@ struct BcsrCfg {
 
 // Ring depth for a shape: CAP stages, fewer where they would leave no room for one staging tile
 // per epilogue warp.
-template <int B, int H, int GROUPS, int CAP, int ES, int CS, int CM>
+template <int B, int H, int GROUPS, int CAP, int ES, int CS, int CM, int SPLIT>
 constexpr int bcsr_fit_stages() {
-    using C1 = BcsrCfg<B, H, GROUPS, 1, ES, CS, CM>;
+    using C1 = BcsrCfg<B, H, GROUPS, 1, ES, CS, CM, SPLIT>;
     const int s = (227 * 1024 - 1024 - C1::kBarrierBytes - 4 * C1::kEpiTileBytes) / C1::kStageBytes;
     return s > CAP ? CAP : (s < 2 ? 2 : s);
 }
@@ -166,7 +173,7 @@ __device__ __noinline__ float plain_product(const int32_t* block_row_ptr, const 
     return s;
 }
 
-template <int B, int H, int GROUPS, int STAGES, int FMT, int CT, int CM, int DYN>
+template <int B, int H, int GROUPS, int STAGES, int FMT, int CT, int CM, int DYN, int SPLIT>
 __global__ void __launch_bounds__((BcsrProducers<B, GROUPS, STAGES, FMT == 3 ? 1 : (FMT == 2 ? 4 : 2), DYN>::kThreads), 1)
 bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmB3, const __grid_constant__ CUtensorMap tmC,
@@ -175,7 +182,8 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     static_assert(FMT != 2 || (!CT && !DYN && (H == B || B <= 32)), "TF32: fp32 C, static schedule, row groups of rows up to 128 bytes");
     static_assert(H == B || !DYN, "stacked blocks: static schedule only");
     using CElem = typename CType<FMT, CT>::type;
-    using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, static_cast<int>(sizeof(CElem)), CM>;
+    using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, static_cast<int>(sizeof(CElem)), CM, SPLIT>;
+    static_assert(!SPLIT || !DYN, "half tiles: static schedule only");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem_al = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -196,6 +204,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t sched_resp = (bar0 + 8u * (2 * STAGES + 7 + 2 * kSchedDepth) + 15u) & ~15u;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int half = SPLIT ? blockIdx.x & 1 : 0;          // which half of the tile's tokens or of the blocks' rows
     WaitCtl ctl{abort_flag, p.status, p.wait_limit_ns};
 
     if (threadIdx.x == 0) {
@@ -227,8 +236,9 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     int tile_begin = 0, tile_end = 0;
     int4 rec0 = make_int4(0, 0, 0, 0);               // record of this CTA's first tile
     if constexpr (!DYN) {
-        tile_begin = __ldg(p.cta_ptr + blockIdx.x);
-        tile_end = __ldg(p.cta_ptr + blockIdx.x + 1);
+        const int list = SPLIT ? blockIdx.x / 2 : blockIdx.x;
+        tile_begin = __ldg(p.cta_ptr + list);
+        tile_end = __ldg(p.cta_ptr + list + 1);
         if (tile_begin < tile_end) rec0 = __ldg(p.tiles + tile_begin);
     }
     // The row groups' launch (overlap = 1): the launch of the remaining block-rows runs beside this one (the two
@@ -296,13 +306,19 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             int4 tcd, tcd_next;
             int Jl_next = 0;                 // block columns of the next tile's first 32 blocks, fetched a tile ahead
             bool have_next = false;
+            // tokens of this CTA's part of the tile that exist
+            auto valid_tokens = [&](int n0) -> int {
+                if constexpr (Cfg::kHalfTok) return static_cast<int>(min_i64(Cfg::kTok, N > n0 + half * Cfg::kTok ? N - n0 - half * Cfg::kTok : 0));
+                return static_cast<int>(min_i64(Cfg::kBnT, N - n0));
+            };
             // the stage of unit it: its byte count, then its stored blocks q .. q + nb - 1 (columns kx .. of them)
             auto request_blocks = [&](uint32_t it, int q, int kx, int nb, int nvalid) {
                 const int s = it % STAGES;
                 const uint32_t sb = smem_base + s * Cfg::kStageBytes;
                 const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
                 // the A request always brings kBps blocks (the box of the tensor map)
-                const uint32_t dense_tx = CM ? ((p.use_3d && nvalid == Cfg::kBnT) ? Cfg::kDenseBytes : ((nvalid + 127) >> 7) * (128 * Cfg::kBB))
+                const uint32_t dense_tx = CM ? (Cfg::kHalfTok ? (nvalid > 0 ? Cfg::kDenseBytes : 0)
+                                                              : ((p.use_3d && nvalid == Cfg::kBnT) ? Cfg::kDenseBytes : ((nvalid + 127) >> 7) * (128 * Cfg::kBB)))
                                              : nbox * Cfg::kBoxBytes;
                 // (stacked blocks: one request per block, a box holds at most 256 rows)
                 if (lane == 0) mbar_arrive_expect_tx(full_bar(s), (H == B ? Cfg::kBps : nb) * Cfg::kABytes + nb * dense_tx);
@@ -315,13 +331,13 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     }
                 } else {
                     if (lane >= 8 && lane < 8 + nb)
-                        tma_load_2d_hint(sb + Cfg::kAOff + (lane - 8) * Cfg::kABytes, &tmA, full_bar(s), 0, (q + lane - 8) * H, keep);
+                        tma_load_2d_hint(sb + Cfg::kAOff + (lane - 8) * Cfg::kABytes, &tmA, full_bar(s), 0, (q + lane - 8) * H + half * (H - Cfg::kRows), keep);
                 }
             };
             // The first tile's first units: their block columns and stored blocks belong to the handle and are
             // fetched while the launch before this one may still be running (a short launch is a chain of index,
             // request, MMA and store latencies, and the weights of a decode step come from HBM); the units' B tiles
-            // follow in the loop below, whose waits for these fresh stages cannot run out.  Back to back, us: 512 x
+            // follow in the loop below.  Back to back, us: 512 x
             // 512, N = 256 4.13 -> 3.82; both projections 18944 x 3584, bf16, N = 128 19.4 -> 17.7; 8192 x 8192,
             // b = 16, N = 4096 222 -> 216; prefill shapes unchanged.
             uint32_t early = 0;
@@ -330,7 +346,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 have_next = true;
                 const int nq = min(32, rec0.w - rec0.z);
                 early = min(STAGES, (nq + Cfg::kBps - 1) / Cfg::kBps * Cfg::kKS);
-                const int nvalid = static_cast<int>(min_i64(Cfg::kBnT, N - rec0.y * Cfg::kBnT));
+                const int nvalid = valid_tokens(rec0.y * Cfg::kBnT);
                 for (uint32_t u = pw; u < early; u += NP) {
                     const int jq = static_cast<int>(u) / Cfg::kKS * Cfg::kBps;
                     request_blocks(u, rec0.z + jq, static_cast<int>(u) % Cfg::kKS * Cfg::kKB, min(Cfg::kBps, nq - jq), nvalid);
@@ -338,10 +354,10 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             }
             operands_ready();
             for (uint32_t nth = 0; ok && next_tile(nth, &tcd, &tcd_next, &ok); ++nth) {
-                const int n0 = tcd.y * Cfg::kBnT;
-                const int nvalid = static_cast<int>(min_i64(Cfg::kBnT, N - n0));
+                const int nvalid = valid_tokens(tcd.y * Cfg::kBnT);
+                const int n0 = tcd.y * Cfg::kBnT + (Cfg::kHalfTok ? half * Cfg::kTok : 0);         // this CTA's first token
                 const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
-                const bool whole_tile = p.use_3d && nvalid == Cfg::kBnT;
+                const bool whole_tile = !Cfg::kHalfTok && p.use_3d && nvalid == Cfg::kBnT;
                 const int pb = tcd.z, pe = tcd.w;
                 const int Jl_first = have_next ? Jl_next : ((pb + lane < pe) ? __ldg(p.block_col_idx + pb + lane) : 0);
                 if constexpr (!DYN) {
@@ -362,7 +378,8 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const int nb = min(Cfg::kBps, nq - jq);          // stored blocks in this stage
                         const int s = it % STAGES;
                         const uint32_t ph = (it / STAGES) & 1u;
-                        if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, ctl, 1))) { ok = false; break; }
+                        // (an early unit's stage is fresh; it may even have been used already, where it has no tokens)
+                        if (it >= early && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, ctl, 1))) { ok = false; break; }
                         const uint32_t sb = smem_base + s * Cfg::kStageBytes;
                         if (it >= early) request_blocks(it, q, kx, nb, nvalid);
                         if constexpr (CM) {
@@ -376,7 +393,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                     tma_load_3d_hint(sb + blk * Cfg::kDenseBytes + hf * (GROUPS * Cfg::kXGroupBytes), &tmB3,
                                                      full_bar(s), J * B + kx + hf * (128 / ES), 0, n0 >> 7, keep);
                             } else {
-                                // ragged tile: one request per 128-token group, rows >= N are zero filled
+                                // ragged tile, or half of one: one request per token group, rows >= N are zero filled
                                 const int ngrp = (nvalid + 127) >> 7;
                                 for (int g = 0; g < ngrp; ++g)
                                     if (blk < nb && hf < kHalves)
@@ -408,7 +425,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         // elected lane issues the tcgen05 instructions.
         {
             // 8-bit floats: format code 0 = E4M3 in both operand fields
-            constexpr uint32_t idesc = make_idesc(FMT == 3 ? 0 : FMT, 128, H, CM ? 0 : 1, 0);
+            constexpr uint32_t idesc = make_idesc(FMT == 3 ? 0 : FMT, Cfg::kHalfTok ? 64 : 128, Cfg::kRows, CM ? 0 : 1, 0);
             // row-major B: the token tile is MN-major; 4-byte elements need the 128-byte swizzle with
             // 32-byte atoms (a pattern of 4 k-rows), 2-byte elements the plain one (8 k-rows)
             const uint64_t adesc0 = CM ? make_smem_desc(0, 16, 8 * Cfg::kXRowBytes, Cfg::kASwizzle)
@@ -462,7 +479,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                                 for (int g = 0; g < GROUPS; ++g)
                                     if (leader && g < ngrp)
-                                        umma_kind<FMT == 3 ? 2 : (FMT == 2 ? 1 : 0)>(d0 + g * H,
+                                        umma_kind<FMT == 3 ? 2 : (FMT == 2 ? 1 : 0)>(d0 + g * Cfg::kRows,
                                                        a0 + ((CM ? (Cfg::kBB <= 128 ? g * Cfg::kXGroupBytes + ks * 32
                                                                             : (ks >> 2) * (GROUPS * Cfg::kXGroupBytes) + g * Cfg::kXGroupBytes + (ks & 3) * 32)
                                                                  : g * (Cfg::kNBox / GROUPS) * Cfg::kBoxBytes + ks * kStepBytes) >> 4),
@@ -482,6 +499,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     } else if (warp < 6) {
         // ------------------------------------------------------------------ epilogue warps
         const int qd = warp & 3;                    // TMEM lane quarter this warp may read
+        const bool mine = lane < Cfg::kWarpTok;     // this lane holds a token
         uint32_t tile_i = 0;
         uint32_t chunk = 0;                         // staging tiles this warp has filled so far
         const uint32_t stg0 = smem_base + STAGES * Cfg::kStageBytes + (warp - 2) * (Cfg::kEpiBufs * Cfg::kEpiTileBytes);
@@ -509,14 +527,14 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             const CUtensorMap* tm_out = part ? &tmP : &tmC;
             constexpr int W = Cfg::kDirect ? (B < 64 ? B : 64) : Cfg::kEpiCols;     // accumulator columns at a time
             for (int g = 0; g < ngrp; ++g) {
-                const int nw = n0 + g * 128 + qd * 32;          // first token of this warp
+                const int nw = n0 + g * 128 + (Cfg::kHalfTok ? half * 64 : 0) + qd * Cfg::kWarpTok;          // first token of this warp
                 if (nw >= N) break;                             // the whole warp is beyond the last token
 #pragma unroll 1
-                for (int c0 = 0; c0 < H; c0 += W) {
+                for (int c0 = 0; c0 < Cfg::kRows; c0 += W) {
                     uint32_t v[W];
                     if (has_blocks) {
                         const uint32_t ta = tmem_base + (static_cast<uint32_t>(qd * 32) << 16) +
-                                            acc * Cfg::kAccCols + g * H + c0;
+                                            acc * Cfg::kAccCols + g * Cfg::kRows + c0;
                         tmem_ld_cols<W>(ta, v);
                         tmem_ld_wait();
                     } else {
@@ -524,16 +542,16 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         for (int j = 0; j < W; ++j) v[j] = 0u;
                     }
                     int32_t crow = static_cast<int32_t>(row0) + c0;
-                    if constexpr (H != B) crow = __shfl_sync(0xffffffffu, member, c0 / B) * B + (c0 % B);
+                    if constexpr (H != B) crow = __shfl_sync(0xffffffffu, member, (half * (H - Cfg::kRows) + c0) / B) * B + (c0 % B);
                     if constexpr (H != B && FMT == 2) {
                         float most = 0.f;                     // NaN if any value is
 #pragma unroll
                         for (int j = 0; j < W; j += 2)
                             asm("max.NaN.f32 %0, %0, %1, %2;" : "+f"(most) : "f"(__uint_as_float(v[j])), "f"(__uint_as_float(v[j + 1])));
-                        if (__any_sync(0xffffffffu, most != most)) {
+                        if (__any_sync(0xffffffffu, mine && most != most)) {
 #pragma unroll
                             for (int j = 0; j < W; ++j)
-                                if (__uint_as_float(v[j]) != __uint_as_float(v[j]) && crow + j < p.m && nw + lane < N)
+                                if (__uint_as_float(v[j]) != __uint_as_float(v[j]) && mine && crow + j < p.m && nw + lane < N)
                                     v[j] = __float_as_uint(plain_product<B, CM>(p.block_row_ptr, p.plain_col_idx, p.plain_vals, p.B, p.k, N,
                                                                                crow + j, nw + lane));
                             __syncwarp();
@@ -543,7 +561,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         // this lane's token: W consecutive columns of its row of Y, straight from the registers in
                         // pieces of 32 bytes (16 where a row or the end of Y does not allow it)
                         constexpr int kPer = 32 / static_cast<int>(sizeof(CElem));
-                        if (nw + lane < N) {
+                        if (mine && nw + lane < N) {
                             CElem* dst = static_cast<CElem*>(p.C) + (nw + lane) * p.m + crow;
 #pragma unroll
                             for (int c = 0; c < W; c += kPer) {
@@ -576,10 +594,10 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 #pragma unroll
                         for (int j = 0; j < W; ++j) {
                             if constexpr (sizeof(CElem) == 4) {
-                                st_shared_u32(stg + j * 128 + lane * 4, v[j]);
+                                if (mine) st_shared_u32(stg + (j * Cfg::kWarpTok + lane) * 4, v[j]);
                             } else {
                                 const CElem h = from_f32<CElem>(__uint_as_float(v[j]));
-                                st_shared_u16(stg + j * 64 + lane * 2, *reinterpret_cast<const unsigned short*>(&h));
+                                if (mine) st_shared_u16(stg + (j * Cfg::kWarpTok + lane) * 2, *reinterpret_cast<const unsigned short*>(&h));
                             }
                         }
                     } else {
@@ -589,7 +607,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         static_assert(W == 16 && sizeof(CElem) == 4, "64-byte rows");
 #pragma unroll
                         for (int c = 0; c < 4; ++c)
-                            st_shared_v4(stg + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                            if (mine) st_shared_v4(stg + lane * 64 + ((c ^ ((lane >> 1) & 3)) << 4), v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
@@ -668,15 +686,15 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
 // CAP = the deepest ring the shape is given; the ring actually used also leaves room for the
 // epilogue's staging tiles (bcsr_fit_stages).
-template <int B, int H, int GROUPS, int CAP, int FMT, int CT, int CM, int DYN>
+template <int B, int H, int GROUPS, int CAP, int FMT, int CT, int CM, int DYN, int SPLIT = 0>
 cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
                        int grid, cudaStream_t stream) {
     constexpr int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2);
     constexpr int CS = static_cast<int>(sizeof(typename CType<FMT, CT>::type));
-    constexpr int STAGES = bcsr_fit_stages<B, H, GROUPS, CAP, ES, CS, CM>();
-    using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, CS, CM>;
+    constexpr int STAGES = bcsr_fit_stages<B, H, GROUPS, CAP, ES, CS, CM, SPLIT>();
+    using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, CS, CM, SPLIT>;
     constexpr int kThreads = BcsrProducers<B, GROUPS, STAGES, ES, DYN>::kThreads;
-    auto kfn = bcsr_spmm_kernel<B, H, GROUPS, STAGES, FMT, CT, CM, DYN>;
+    auto kfn = bcsr_spmm_kernel<B, H, GROUPS, STAGES, FMT, CT, CM, DYN, SPLIT>;
     // the attribute belongs to the (function, device) pair: set it once per device
     static std::mutex mu;
     static bool attr_done[kMaxDevices] = {};
@@ -696,7 +714,7 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
         kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmB, tmB3, tmC, tmP, p);
         return cudaGetLastError();
     } else {
-        return launch_dependent(kfn, dim3(static_cast<unsigned>(grid)), kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmB3, tmC, tmP, p);
+        return launch_dependent(kfn, dim3(static_cast<unsigned>(SPLIT ? 2 * grid : grid)), kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmB3, tmC, tmP, p);
     }
 }
 
@@ -715,8 +733,18 @@ cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtens
         case 644: return launch_one<64, 64, 4, 3, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 1281: return launch_one<128, 128, 1, 3, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 1282: return launch_one<128, 128, 2, 2, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        default: return cudaErrorInvalidValue;
+        default: break;
     }
+    if constexpr (!DYN) {
+        switch (b * 10 + groups) {
+            case 160: return launch_one<16, 16, 1, 16, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 32, 1, 16, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 640: return launch_one<64, 64, 1, 10, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 1280: return launch_one<128, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            default: break;
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
 // Stacked blocks (row groups): 128 rows x b; token tile 256 and four stages of 48 KB, or 128 and six of 32 KB.
@@ -728,6 +756,8 @@ cudaError_t launch_stack_shape(int b, int groups, const CUtensorMap& tmA, const 
         case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 160: return launch_one<16, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 320: return launch_one<32, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: break;
     }
     if constexpr (FMT != 2) {
@@ -763,8 +793,17 @@ cudaError_t launch_fp8(int b, int groups, const CUtensorMap& tmA, const CUtensor
         case 644: return launch_one<64, 64, 4, 5, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 1281: return launch_one<128, 128, 1, 6, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 1282: return launch_one<128, 128, 2, 4, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        default: return cudaErrorInvalidValue;
+        default: break;
     }
+    if constexpr (CM) {
+        switch (b * 10 + groups) {
+            case 320: return launch_one<32, 32, 1, 16, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 640: return launch_one<64, 64, 1, 16, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 1280: return launch_one<128, 128, 1, 8, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            default: break;
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
 // TF32 (fp32 storage): fp32 C, static schedule; the deepest rings the stage sizes allow.
@@ -781,6 +820,10 @@ cudaError_t launch_tf32(int b, int groups, const CUtensorMap& tmA, const CUtenso
         case 644: return launch_one<64, 64, 4, 3, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 1281: return launch_one<128, 128, 1, 6, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 1282: return launch_one<128, 128, 2, 4, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 160: return launch_one<16, 16, 1, 10, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 320: return launch_one<32, 32, 1, 8, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 640: return launch_one<64, 64, 1, 10, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1280: return launch_one<128, 128, 1, 8, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -841,6 +884,7 @@ cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_m
             case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
             case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
             case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 128, 1, 12, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
             default: break;
         }
     }

@@ -72,6 +72,10 @@ cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, in
 // Row groups: the same kernel with 128 x b stacked blocks (MMA N = 128) and a 256-token tile (groups = 2), or a
 // 128-token one (groups = 1; see ensure_schedule).
 // tmA: the stacked values as [blocks * 128][b], box 128 x b; tmB3 built for `groups`; b = 16, 32, 64 (tf32: 16, 32).
+// `groups` of a launch by half tiles (both kinds of launch): the lists of a 128-token schedule, two CTAs to each, with 64 of
+// its tiles' tokens in either (tmC: boxes of 16 tokens instead of 32; column-major tmB: box of 64 tokens; E4M3: column-major
+// operands only) or, for stacked blocks of b = 16 and 32, 64 of their rows (tmA: box of 64 rows).
+constexpr int kSplitGroups = 0;
 constexpr int kStackRows = 128;
 constexpr int kStackGroups = 2;
 cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,

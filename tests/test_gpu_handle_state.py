@@ -299,26 +299,29 @@ def test_workspace_bytes_is_what_a_run_allocates(lib, matrix, opt):
 
 
 def test_waits_do_not_count_the_launch_before(lib):
-    """One block-row of 2048 blocks: a launch of a millisecond on a few SMs.  The next one starts beside it on the others and
-    waits for its end; that time is no part of its bounded waits, whose limit is a third of it here."""
+    """One block-row of 2048 blocks: a launch of a millisecond on a few SMs.  The next one, of a matrix of 8 blocks, starts
+    beside it on the others and waits for its end; that time is no part of its bounded waits, whose limit is shorter."""
     import torch
-    m, k, N = 128, 262144, 128
-    rp = torch.arange(m + 1, dtype=torch.int64, device="cuda") * k
-    ci = torch.arange(k, dtype=torch.int32, device="cuda").repeat(m)
-    va = torch.ones(m * k, dtype=torch.bfloat16, device="cuda")
-    h = lib.spmm_bcsr_create_csr_device(m, k, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), "bf16", 128)
+    m, N = 128, 128
+    hs, ks = [], (262144, 1024)
     try:
-        B = torch.ones((k, N), dtype=torch.bfloat16, device="cuda")
-        C = torch.zeros((m, N), dtype=torch.float32, device="cuda")
+        for k in ks:
+            rp = torch.arange(m + 1, dtype=torch.int64, device="cuda") * k
+            ci = torch.arange(k, dtype=torch.int32, device="cuda").repeat(m)
+            va = torch.ones(m * k, dtype=torch.bfloat16, device="cuda")
+            hs.append(lib.spmm_bcsr_create_csr_device(m, k, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), "bf16", 128))
+        B = torch.ones((ks[0], N), dtype=torch.bfloat16, device="cuda")
+        C = torch.zeros((2, m, N), dtype=torch.float32, device="cuda")
         st = torch.cuda.current_stream().cuda_stream
-        lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, st)
+        for limit in (2_000_000_000, 300_000, 300_000):            # (the first pass: kernels loaded, plans made)
+            for i in range(2):
+                lib.spmm_set_wait_limit_ns(limit if i else 2_000_000_000)
+                lib.spmm_run(hs[i], B.data_ptr(), C[i].data_ptr(), N, st)
         torch.cuda.synchronize()
-        lib.spmm_set_wait_limit_ns(300_000)
-        for _ in range(4):
-            lib.spmm_run(h, B.data_ptr(), C.data_ptr(), N, st)
-        torch.cuda.synchronize()
-        lib.spmm_check(h)
-        assert bool(torch.all(C == k))
+        for i in range(2):
+            lib.spmm_check(hs[i])
+            assert bool(torch.all(C[i] == ks[i]))
     finally:
         lib.spmm_set_wait_limit_ns(2_000_000_000)
-        lib.spmm_destroy(h)
+        for h in hs:
+            lib.spmm_destroy(h)

@@ -303,6 +303,47 @@ def test_wcsr_gpu_builder_by_window_size(lib, dtype, wh, k):
         lib.spmm_destroy(h0)
 
 
+@pytest.mark.parametrize("dtype,b,dens,layout,c16", [
+    ("bf16", 64, 0.7, "row", False), ("fp16", 64, 0.7, "row", True), ("bf16", 64, 0.7, "col", True), ("fp16", 64, 0.7, "col", False),
+    ("tf32", 64, 0.7, "row", False), ("tf32", 64, 0.7, "col", False), ("fp8", 64, 0.7, "col", False),
+    ("fp16", 128, 0.8, "row", False), ("bf16", 128, 0.8, "col", True), ("tf32", 128, 0.8, "row", False), ("fp8", 128, 0.8, "col", False),
+    ("fp16", 16, 0.2, "row", False), ("bf16", 32, 0.3, "col", True), ("tf32", 16, 0.2, "col", False), ("tf32", 32, 0.3, "row", False),
+    ("bf16", 16, 0.2, "row", True), ("fp8", 32, 0.3, "col", False), ("fp16", 16, 1.0, "row", False), ("bf16", 16, 1.0, "col", True),
+    ("tf32", 16, 1.0, "row", False), ("bf16", 32, 1.0, "row", True), ("tf32", 32, 1.0, "row", False), ("tf32", 32, 1.0, "col", False),
+    ("fp8", 32, 1.0, "col", False)])
+def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16):
+    """Launches with at most half as many 128-token tiles as CTAs, each of 768 KB and more: two CTAs to a tile (halves of its
+    tokens for plain blocks, of the stacked blocks' rows for row groups).  The same bits as with one CTA per tile (a grid too
+    small for two), and the oracle's result; token counts around the halves of a tile, an empty block-row, ragged last rows."""
+    m = 328 if dens < 1 else 264
+    need = (768 << 10) // ((128 + (b if dens < 1 else 128)) * b * wl.elem_size(dtype)) + 2       # blocks of the longest tile
+    k = (need * b + 8) // 16 * 16
+    rng = np.random.default_rng(b)
+    nbr, nbc = -(-m // b), -(-k // b)
+    mask = rng.random((nbr, nbc)) < dens
+    mask[0, :] = True
+    if dens < 1:
+        mask[1, :] = False
+    full = np.kron(mask, np.ones((b, b), bool))[:m, :k]
+    rp = np.concatenate(([0], np.cumsum(full.sum(1)))).astype(np.int64)
+    ci = np.nonzero(full)[1].astype(np.int32)
+    vals = wl.to_storage(rng.uniform(-1, 1, ci.size), dtype)
+    a = {"m": m, "k": k, "row_ptr": rp, "col_idx": ci, "vals": vals}
+    opt = dict(layout=lib.COLMAJOR if layout == "col" else lib.ROWMAJOR, c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
+    for N in ((128, 129, 200, 321) if layout == "col" else (72, 96, 128, 136, 256)):
+        h = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, **opt)
+        h1 = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, n_ctas=3, **opt)
+        try:
+            Bs = wl.dense(7 + N, k, N, ("uniform", -1.0, 1.0), dtype)
+            C, C1 = (run_gpu_variant(lib, x, Bs, m, N, dtype, c16=c16, col_major=layout == "col") for x in (h, h1))
+            Cr, S = reference(a, Bs, dtype)
+            assert_close(C, Cr, S, dtype, "half tiles b=%d N=%d" % (b, N))
+            assert np.array_equal(C, C1), N
+        finally:
+            lib.spmm_destroy(h)
+            lib.spmm_destroy(h1)
+
+
 @pytest.mark.parametrize("dtype", ["tf32", "fp16", "fp8"])
 def test_bcsr_gpu_builder_with_many_block_columns(lib, dtype):
     """More than 196,608 block columns: the builder's bitmap takes more than 48 KB of shared memory."""
