@@ -1128,6 +1128,21 @@ RowsShape rows_shape(const spmm_handle_s* h, const void* B, const void* C, int64
     return wcsr_rows_shape(N, h->es, aligned32);
 }
 
+// Threads of a CTA of the row kernel.  A long row's part is 16 strands, which the CTA's groups sum one after the other
+// where there are fewer groups than that.  A launch that is over when its slowest part is gains from twice the warps; in
+// larger ones a CTA then holds its slot for its slowest warp.  The line, by entries per SM and 128 groups (load) and groups
+// per warp, from us with 128 / 256 threads (512: 0.6 - 1.07 of the speed of 256):
+//   power-law rows, 4000 (load 3)    TF32 N = 36 6.6 / 5.6   N = 128 8.9 / 6.4    bf16 N = 320 13.6 / 9.8
+//                   12,000 (6)       7.3 / 6.4               9.4 / 7.8            16.2 / 11.6
+//                   9000 (8)         7.6 / 8.1               9.8 / 9.8            17.4 / 14.3
+//   R-MAT 2^13, 4 a row (2)          6.1 / 5.4               8.5 / 6.5            13.0 / 8.3
+//         2^13, 16 a row (7)         7.0 / 8.8               9.0 / 10.5           15.8 / 14.2
+//         2^15, 4 a row (8)          7.2 / 7.5               9.9 / 10.6           21.2 / 21.9
+int wcsr_rows_threads(const spmm_handle_s* h, const RowsShape& s) {
+    const int groups = 32 / s.lanes;
+    return h->rows.n_parts > 0 && groups < 4 && wcsr_rows_load(h->m, h->nnz, h->sms) < (groups == 1 ? 8 : 7) ? 256 : kRowsThreads;
+}
+
 // partial: room for cap bytes of partial rows; the column tiles go in as few launches as that and the counters allow,
 // and are made narrower where it does not hold one (sums do not depend on the cut).  A tile of one vector takes
 // kRowsMaxSlots * 32 bytes at most, which the built-in scratch holds.
@@ -1157,10 +1172,11 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     p.N = N;
     p.n_tasks = r.n_tasks;
     p.n_parts = r.n_parts;
+    const int threads = wcsr_rows_threads(h, s);
     int step = std::min(s.tiles, kRowsMaxTiles);
     while (step > 1 && rows_partial_bytes(h, s, step) > cap) --step;
     for (int t = 0; t < s.tiles; t += step)
-        if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), stream) != cudaSuccess)
+        if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), threads, stream) != cudaSuccess)
             return cuda_error();
     return SPMM_OK;
 }

@@ -32,7 +32,6 @@ namespace spmm {
 
 namespace {
 
-constexpr int kWarps = kRowsThreads / 32;
 constexpr int kStrands = 16;            // partial sums of a part: strand = (entry / 8) % kStrands, whatever the dense width
 constexpr int kNoCol = 0x7fffffff;      // an entry without a gather: row without nonzeros, or padding
 
@@ -140,10 +139,13 @@ __device__ __forceinline__ void store_c(uint8_t* dst, const float (&acc)[VE]) {
 }
 
 // Resident CTAs per SM: registers cap the bytes in flight.  Wide vectors: 7 (72 registers) measured 805 us
-// on R-MAT 2^21 fp16 N = 128, 5 CTAs 858, 8 CTAs 893; 16-byte vectors: 8.
-template <int FMT, int CT, int VB>
-__global__ void __launch_bounds__(kRowsThreads, VB == 32 ? 7 : 8)
+// on R-MAT 2^21 fp16 N = 128, 5 CTAs 858, 8 CTAs 893; 16-byte vectors: 6 (30,000 power-law rows fp16 N = 48 8.8 us with 8,
+// 8.4 with 6, 9.3 with 10).
+// THREADS: kRowsThreads, or 256 (wcsr_rows_threads in api.cu).
+template <int FMT, int CT, int VB, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS > kRowsThreads ? 3 : (VB == 32 ? 7 : 6))
 wcsr_rows_kernel(const WcsrRowsParams p) {
+    constexpr int kWarps = THREADS / 32;
     constexpr int ES = FMT == 2 ? 4 : 2;
     constexpr int VE = VB / ES;                           // dense columns per lane
     using CElem = typename CType<FMT, CT>::type;
@@ -240,7 +242,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     CElem* Crow = static_cast<CElem*>(p.C) + lr.x * p.N + n_tile;
     const int64_t slot_pitch = static_cast<int64_t>(gridDim.y) * tile_cols;
     float* part0 = p.partial + static_cast<int64_t>(lr.y) * slot_pitch + static_cast<int64_t>(blockIdx.y) * tile_cols;
-    for (int t = threadIdx.x; t < tile_cols; t += kRowsThreads) {
+    for (int t = threadIdx.x; t < tile_cols; t += THREADS) {
         float s = 0.f;
 #pragma unroll
         for (int i = 0; i < kStrands; ++i) s += red[i * (p.lanes * (VE + 1)) + t + t / VE];
@@ -259,7 +261,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     __syncthreads();
     if (arrived != static_cast<unsigned>(lr.z) - 1u) return;
     __threadfence();
-    for (int t = threadIdx.x; t < tile_cols; t += kRowsThreads) {
+    for (int t = threadIdx.x; t < tile_cols; t += THREADS) {
         if (n_tile + t >= p.N) break;
         float s = 0.f;
         int i = 0;
@@ -284,12 +286,12 @@ __global__ void wcsr_rows_give_up_kernel(int* status) {
     }
 }
 
-template <int VB>
+template <int VB, int THREADS>
 cudaError_t launch_vb(int dtype, int c16, const WcsrRowsParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
-    auto go = [&](auto kfn) { return launch_dependent(kfn, grid, kRowsThreads, smem, stream, p); };
-    if (dtype == 2) return go(wcsr_rows_kernel<2, 0, VB>);
-    if (dtype == 1) return c16 ? go(wcsr_rows_kernel<0, 1, VB>) : go(wcsr_rows_kernel<0, 0, VB>);
-    if (dtype == 0) return c16 ? go(wcsr_rows_kernel<1, 1, VB>) : go(wcsr_rows_kernel<1, 0, VB>);
+    auto go = [&](auto kfn) { return launch_dependent(kfn, grid, THREADS, smem, stream, p); };
+    if (dtype == 2) return go(wcsr_rows_kernel<2, 0, VB, THREADS>);
+    if (dtype == 1) return c16 ? go(wcsr_rows_kernel<0, 1, VB, THREADS>) : go(wcsr_rows_kernel<0, 0, VB, THREADS>);
+    if (dtype == 0) return c16 ? go(wcsr_rows_kernel<1, 1, VB, THREADS>) : go(wcsr_rows_kernel<1, 0, VB, THREADS>);
     return cudaErrorInvalidValue;
 }
 
@@ -318,16 +320,17 @@ cudaError_t launch_wcsr_rows_give_up(int* status, cudaStream_t stream) {
     return launch_dependent(wcsr_rows_give_up_kernel, dim3(1), 1, 0, stream, status);
 }
 
-cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, cudaStream_t stream) {
+cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, int threads, cudaStream_t stream) {
     p.lanes = s.lanes;
     p.groups = 32 / s.lanes;
     p.tile0 = tile0;
-    const int per_cta = kWarps * p.groups;
+    const int per_cta = threads / 32 * p.groups;
     const int64_t ctas = p.n_parts + (static_cast<int64_t>(p.n_tasks) + per_cta - 1) / per_cta;
     if (ctas <= 0 || tiles <= 0) return cudaSuccess;
     const dim3 grid(static_cast<unsigned>(ctas), static_cast<unsigned>(tiles));
     const size_t smem = p.n_parts > 0 ? static_cast<size_t>(kStrands) * (s.tile_cols + s.lanes) * 4 : 0;     // at most 34 KB
-    return s.vec == 32 ? launch_vb<32>(dtype, c16, p, grid, smem, stream) : launch_vb<16>(dtype, c16, p, grid, smem, stream);
+    if (threads == 256) return s.vec == 32 ? launch_vb<32, 256>(dtype, c16, p, grid, smem, stream) : launch_vb<16, 256>(dtype, c16, p, grid, smem, stream);
+    return s.vec == 32 ? launch_vb<32, kRowsThreads>(dtype, c16, p, grid, smem, stream) : launch_vb<16, kRowsThreads>(dtype, c16, p, grid, smem, stream);
 }
 
 }  // namespace spmm

@@ -212,3 +212,21 @@ def test_static_run_takes_the_kernel_of_spmm_run(lib):
         assert_close(want[:, torch.from_numpy(cols).cuda()].cpu().numpy(), Cr, S, dtype, "long rows")
     finally:
         lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("dtype,widths", [("tf32", (36, 64, 128, 320)), ("fp16", (72, 128, 320, 520))])
+def test_the_sums_do_not_depend_on_the_cta_size(lib, dtype, widths):
+    """A small launch takes CTAs of 128 or 256 threads by the groups that its dense width leaves a warp (8 to 1 of them
+    here); a column's sums are those of the widest run, bit by bit."""
+    m, k = 3001, 20000
+    a = _matrix(m, k, 16, dtype)
+    Bs = wl.dense(64, k, widths[-1], ("uniform", -1.0, 1.0), dtype)
+    h = lib.spmm_wcsr_create_csr(m, k, a["row_ptr"], a["col_idx"], a["vals"], dtype, 16)
+    try:
+        want = run_gpu_variant(lib, h, Bs, m, widths[-1], dtype)
+        Cr, S = reference(a, Bs, dtype)
+        assert_close(want, Cr, S, dtype, "rows N=%d" % widths[-1])
+        for N in (16,) + widths[:-1]:
+            assert np.array_equal(run_gpu_variant(lib, h, np.ascontiguousarray(Bs[:, :N]), m, N, dtype), want[:, :N]), N
+    finally:
+        lib.spmm_destroy(h)
