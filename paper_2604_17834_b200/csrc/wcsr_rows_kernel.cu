@@ -139,11 +139,11 @@ __device__ __forceinline__ void store_c(uint8_t* dst, const float (&acc)[VE]) {
 }
 
 // Resident CTAs per SM: registers cap the bytes in flight.  Wide vectors: 7 (72 registers) measured 805 us
-// on R-MAT 2^21 fp16 N = 128, 5 CTAs 858, 8 CTAs 893; 16-byte vectors: 6 (30,000 power-law rows fp16 N = 48 8.8 us with 8,
-// 8.4 with 6, 9.3 with 10).
+// on R-MAT 2^21 fp16 N = 128, 5 CTAs 858, 8 CTAs 893; 16-byte vectors: 8 (with 6: R-MAT 2^20 TF32 N = 76 645 -> 703, 2^17 bf16
+// N = 40 38.4 -> 40.2, of 45,000 rows fp16 N = 48 12.9 -> 11.5; with 10: 30,000 rows fp16 N = 48 8.8 -> 9.3).
 // THREADS: kRowsThreads, or 256 (wcsr_rows_threads in api.cu).
 template <int FMT, int CT, int VB, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS > kRowsThreads ? 3 : (VB == 32 ? 7 : 6))
+__global__ void __launch_bounds__(THREADS, THREADS > kRowsThreads ? 3 : (VB == 32 ? 7 : 8))
 wcsr_rows_kernel(const WcsrRowsParams p) {
     constexpr int kWarps = THREADS / 32;
     constexpr int ES = FMT == 2 ? 4 : 2;
