@@ -61,23 +61,35 @@ __device__ __forceinline__ void st_vec(uint8_t* p, const uint32_t* w) {
 
 // acc[e] += a * b[e] over one vector of B.  16-bit types: the product of two 16-bit values is exact in
 // fp32, so the mixed-precision FMA rounds once, like an FMA of the widened values.  (Widening first and
-// a packed fma.rn.f32x2 measured 9 % slower.)
+// a packed fma.rn.f32x2 measured 9 % slower.)  fp32 goes two columns at a time: R-MAT 2^17, 16 a row, N = 200
+// 120.9 -> 118.6 us, 200,000 power-law rows N = 64 47.2 -> 46.2.
 template <int FMT, int VB, int VE>
 __device__ __forceinline__ void fma_vec(float (&acc)[VE], uint32_t a, const Vec<VB>& b) {
+    if constexpr (FMT == 2) {
+#pragma unroll
+        for (int i = 0; i < VE; i += 2)
+            asm("{\n\t"
+                ".reg .b64 d, x, y;\n\t"
+                "mov.b64 d, {%0, %1};\n\t"
+                "mov.b64 x, {%3, %4};\n\t"
+                "mov.b64 y, {%2, %2};\n\t"
+                "fma.rn.f32x2 d, x, y, d;\n\t"
+                "mov.b64 {%0, %1}, d;\n\t"
+                "}\n"
+                : "+f"(acc[i]), "+f"(acc[i + 1])
+                : "r"(a), "r"(b.w[i]), "r"(b.w[i + 1]));
+        return;
+    }
 #pragma unroll
     for (int i = 0; i < VB / 4; ++i) {
-        if constexpr (FMT == 2) {
-            acc[i] = fmaf(__uint_as_float(a), __uint_as_float(b.w[i]), acc[i]);
-        } else {
-            const unsigned short av = static_cast<unsigned short>(a);
-            const unsigned short lo = static_cast<unsigned short>(b.w[i]), hi = static_cast<unsigned short>(b.w[i] >> 16);
-            if constexpr (FMT == 0) {
-                asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(acc[2 * i]) : "h"(av), "h"(lo));
-                asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(acc[2 * i + 1]) : "h"(av), "h"(hi));
-            } else {
-                asm("fma.rn.f32.bf16 %0, %1, %2, %0;" : "+f"(acc[2 * i]) : "h"(av), "h"(lo));
-                asm("fma.rn.f32.bf16 %0, %1, %2, %0;" : "+f"(acc[2 * i + 1]) : "h"(av), "h"(hi));
-            }
+        const unsigned short av = static_cast<unsigned short>(a);
+        const unsigned short lo = static_cast<unsigned short>(b.w[i]), hi = static_cast<unsigned short>(b.w[i] >> 16);
+        if constexpr (FMT == 0) {
+            asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(acc[2 * i]) : "h"(av), "h"(lo));
+            asm("fma.rn.f32.f16 %0, %1, %2, %0;" : "+f"(acc[2 * i + 1]) : "h"(av), "h"(hi));
+        } else if constexpr (FMT == 1) {
+            asm("fma.rn.f32.bf16 %0, %1, %2, %0;" : "+f"(acc[2 * i]) : "h"(av), "h"(lo));
+            asm("fma.rn.f32.bf16 %0, %1, %2, %0;" : "+f"(acc[2 * i + 1]) : "h"(av), "h"(hi));
         }
     }
 }
