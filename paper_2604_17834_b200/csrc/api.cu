@@ -164,7 +164,7 @@ struct spmm_handle_s {
     bool partial_pooled = true;      // false: from cudaMalloc (see ensure_wcsr_workspace)
 
     // BCSR tensor maps
-    CUtensorMap tmA;
+    CUtensorMap tmA, tmA1;           // (tmA1: for tiles of 128 tokens, whose stages hold more blocks)
     bool tmA_ok = false;
     CUtensorMap tmB;
     CUtensorMap tmB3;                // BCSR: B as [N / 64][k][64] for whole-tile loads
@@ -304,12 +304,13 @@ int encode_blocks(const spmm_handle_s* h, CUtensorMap* map, const void* blocks, 
     return encode_2d(map, h->dtype, blocks, static_cast<uint64_t>(total_rows), b, static_cast<uint32_t>(rows), row_bytes / h->es, swz);
 }
 
-// Tensor map of the stored blocks.
+// Tensor maps of the stored blocks.
 int encode_tmA(spmm_handle_s* h) {
     const BcsrHost& f = h->bcsr;
     if (f.nnzb <= 0) return SPMM_OK;
     if (static_cast<int64_t>(f.nnzb) * f.b >= (int64_t{1} << 31)) return SPMM_ERR_TOO_LARGE;
-    const int rc = encode_blocks(h, &h->tmA, h->d_vals, f.nnzb * f.b, f.b * bcsr_blocks_per_stage(f.b));
+    int rc = encode_blocks(h, &h->tmA, h->d_vals, f.nnzb * f.b, f.b * bcsr_blocks_per_stage(f.b, h->es, 2));
+    if (!rc) rc = encode_blocks(h, &h->tmA1, h->d_vals, f.nnzb * f.b, f.b * bcsr_blocks_per_stage(f.b, h->es, 1));
     h->tmA_ok = rc == SPMM_OK;
     return rc;
 }
@@ -1021,11 +1022,12 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.B = nullptr;
     p.k = h->k;
     p.overlap = 0;
-    CUtensorMap tmA = h->tmA;
+    CUtensorMap tmA = h->sched.groups <= 1 ? h->tmA1 : h->tmA, tmA0 = h->tmA;
     if (!h->tmA_ok) {
         // no stored block at all: the kernel never touches A, any valid map will do
         rc = encode_2d(&tmA, h->dtype, h->d_vals, 8, 8, 8, 8, CU_TENSOR_MAP_SWIZZLE_NONE);
         if (rc) return rc;
+        tmA0 = tmA;
     }
     rc = ensure_tmB(h, B, N, h->sched.groups);
     if (rc) return rc;
@@ -1048,9 +1050,9 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         ps.overlap = 1;
         p.overlap = 2;
         const int n_tiles = static_cast<int>(h->sched_stack.tiles.size() / 2);
-        cudaError_t es = h->stack_split ? launch_bcsr_stacked(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, h->tmAsh, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
+        cudaError_t es = h->stack_split ? launch_bcsr_stacked(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, h->tmAsh, h->tmAsh, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
                                                              n_tiles, stream)
-                                       : launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
+                                       : launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
                                                              h->n_ctas, stream);
         if (es != cudaSuccess) return cuda_error();
         if (h->sched.tiles.empty()) return SPMM_OK;
@@ -1059,13 +1061,13 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     const int grid = h->dynamic ? static_cast<int>(h->sched.tiles.size() / 2) : h->n_ctas;
     if (grid <= 0) return SPMM_OK;
     if (h->split) {
-        const cudaError_t eh = launch_bcsr(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, 0, tmA, h->tmBh, h->tmB3, h->tmCh, h->tmCh, p,
+        const cudaError_t eh = launch_bcsr(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, 0, tmA, tmA0, h->tmBh, h->tmB3, h->tmCh, h->tmCh, p,
                                            static_cast<int>(h->sched.tiles.size() / 2), stream);
         return eh == cudaSuccess ? SPMM_OK : cuda_error();
     }
     const bool ksplit = h->sched.n_slots > 0 && h->tmP_ok;
     if (ksplit) p.overlap = 1;          // the merge kernel's CTAs may be placed while this grid runs
-    cudaError_t e = launch_bcsr(h->dtype, f.b, h->sched.groups, h->c16, h->col_major, h->dynamic, tmA, h->tmB, h->tmB3,
+    cudaError_t e = launch_bcsr(h->dtype, f.b, h->sched.groups, h->c16, h->col_major, h->dynamic, tmA, tmA0, h->tmB, h->tmB3,
                                 h->tmC, ksplit ? h->tmP : h->tmC, p, grid, stream);
     if (e != cudaSuccess) return cuda_error();
     if (ksplit) {

@@ -81,8 +81,16 @@ struct BcsrCfg {
     static constexpr int kABytes = kRows * kBB;
     // Small blocks carry too little work for the fixed cost of a pipeline stage (barrier
     // round trip, request issue, MMA hand-off): a stage holds several consecutive stored
-    // blocks of the block-row, their B tiles first, then their A blocks (one request).
-    static constexpr int kBps = H == B ? bcsr_blocks_per_stage(B) : bcsr_stacked_per_stage(B, ES);
+    // blocks of the block-row, their B tiles first, then their A blocks (one request).  So do
+    // blocks of 32 and 64 in tiles of 128 tokens, where the issuer's part of a stage (about 170
+    // cycles) is as long as a block's four MMAs of 48: twice as many blocks per stage, half as many
+    // stages, so that the staging tiles keep their room.  Down-projection 3584 x 18944, density
+    // 0.1, N = 128, bf16 9.5 -> 7.9 us; N = 2048, E4M3 34.4 -> 31.6; b = 32, 2048 x 8192 both ways,
+    // N = 700, bf16 25.2 -> 23.9.  Not for b = 16, whose stages already hold four blocks: with eight,
+    // 50 blocks a row 11.1 -> 10.7, but two blocks a row 6.8 -> 7.2 (half as many tiles in flight).
+    // A stage that is at most half full asks for half of the A blocks (tmA0): kFew.
+    static constexpr int kBps = H == B ? bcsr_blocks_per_stage(B, ES, GROUPS) : bcsr_stacked_per_stage(B, ES);
+    static constexpr int kFew = H == B ? bcsr_blocks_per_stage(B, ES, 2) : kBps;
     static constexpr int kStageBytes = ((kBps * (kDenseBytes + kABytes) + 1023) / 1024) * 1024;
     static constexpr int kAOff = kBps * kDenseBytes;         // A blocks inside the stage
     static constexpr int kARowBytes = kBB < 128 ? kBB : 128;
@@ -116,7 +124,7 @@ struct BcsrCfg {
     static_assert(kSmemBytes <= 227 * 1024, "stage ring exceeds shared memory");
     static_assert((2 * STAGES + 7 + 8) * 8 + 64 + 32 <= kBarrierBytes, "barrier area");
     static_assert(!SPLIT || (GROUPS == 1 && (CM || kNBox >= 1)), "half of a 128-token tile");
-    static_assert(kBps == 1 || (B <= 32 && kKS == 1), "multi-block stages are for the small block sizes");
+    static_assert(kBps == 1 || (B <= 64 && kKS == 1), "multi-block stages are for the small block sizes");
     static_assert(kKS == 1 || kBB <= 128, "a column slice is at most one 128-byte row piece");
     static_assert(kBB % 32 == 0, "a block row must hold whole K steps");
     static_assert(H == B || (H == 128 && B < 128), "stacked blocks are 128 rows high");
@@ -175,7 +183,7 @@ __device__ __noinline__ float plain_product(const int32_t* block_row_ptr, const 
 
 template <int B, int H, int GROUPS, int STAGES, int FMT, int CT, int CM, int DYN, int SPLIT>
 __global__ void __launch_bounds__((BcsrProducers<B, GROUPS, STAGES, FMT == 3 ? 1 : (FMT == 2 ? 4 : 2), DYN>::kThreads), 1)
-bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmB3, const __grid_constant__ CUtensorMap tmC,
                  const __grid_constant__ CUtensorMap tmP, const BcsrParams p) {
     constexpr int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2);
@@ -217,6 +225,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         *abort_flag = 0;
         fence_mbar_init();
         prefetch_tmap(&tmA);
+        if (Cfg::kFew < Cfg::kBps) prefetch_tmap(&tmA0);
         prefetch_tmap(&tmB);
         prefetch_tmap(&tmB3);
         prefetch_tmap(&tmC);
@@ -316,16 +325,17 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const int s = it % STAGES;
                 const uint32_t sb = smem_base + s * Cfg::kStageBytes;
                 const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
-                // the A request always brings kBps blocks (the box of the tensor map)
+                // the A request always brings kBps or kFew blocks (the boxes of the tensor maps)
+                const bool few = Cfg::kFew < Cfg::kBps && nb <= Cfg::kFew;
                 const uint32_t dense_tx = CM ? (Cfg::kHalfTok ? (nvalid > 0 ? Cfg::kDenseBytes : 0)
                                                               : ((p.use_3d && nvalid == Cfg::kBnT) ? Cfg::kDenseBytes : ((nvalid + 127) >> 7) * (128 * Cfg::kBB)))
                                              : nbox * Cfg::kBoxBytes;
                 // (stacked blocks: one request per block, a box holds at most 256 rows)
-                if (lane == 0) mbar_arrive_expect_tx(full_bar(s), (H == B ? Cfg::kBps : nb) * Cfg::kABytes + nb * dense_tx);
+                if (lane == 0) mbar_arrive_expect_tx(full_bar(s), (H == B ? (few ? Cfg::kFew : Cfg::kBps) : nb) * Cfg::kABytes + nb * dense_tx);
                 __syncwarp();
                 if constexpr (H == B) {
                     if (lane == 8) {
-                        tma_load_2d_hint(sb + Cfg::kAOff, &tmA, full_bar(s), kx, q * B, keep);
+                        tma_load_2d_hint(sb + Cfg::kAOff, few ? &tmA0 : &tmA, full_bar(s), kx, q * B, keep);
                     } else if (Cfg::kBB > 128 && lane == 9) {
                         tma_load_2d_hint(sb + Cfg::kAOff + B * 128, &tmA, full_bar(s), 128 / ES, q * B, keep);
                     }
@@ -687,7 +697,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // CAP = the deepest ring the shape is given; the ring actually used also leaves room for the
 // epilogue's staging tiles (bcsr_fit_stages).
 template <int B, int H, int GROUPS, int CAP, int FMT, int CT, int CM, int DYN, int SPLIT = 0>
-cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
+cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
                        int grid, cudaStream_t stream) {
     constexpr int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2);
     constexpr int CS = static_cast<int>(sizeof(typename CType<FMT, CT>::type));
@@ -711,36 +721,36 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmB, const CUt
         }
     }
     if constexpr (DYN) {        // (its grid is a queue of CTAs that running ones cancel: launched when the stream gets there)
-        kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmB, tmB3, tmC, tmP, p);
+        kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmA0, tmB, tmB3, tmC, tmP, p);
         return cudaGetLastError();
     } else {
-        return launch_dependent(kfn, dim3(static_cast<unsigned>(SPLIT ? 2 * grid : grid)), kThreads, Cfg::kSmemBytes, stream, tmA, tmB, tmB3, tmC, tmP, p);
+        return launch_dependent(kfn, dim3(static_cast<unsigned>(SPLIT ? 2 * grid : grid)), kThreads, Cfg::kSmemBytes, stream, tmA, tmA0, tmB, tmB3, tmC, tmP, p);
     }
 }
 
 template <int FMT, int CT, int CM, int DYN>
-cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                          const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 161: return launch_one<16, 16, 1, 10, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 162: return launch_one<16, 16, 2, 5, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 164: return launch_one<16, 16, 4, 3, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 321: return launch_one<32, 32, 1, 10, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 32, 2, 5, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 324: return launch_one<32, 32, 4, 3, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 641: return launch_one<64, 64, 1, 8, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 642: return launch_one<64, 64, 2, 5, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 644: return launch_one<64, 64, 4, 3, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1281: return launch_one<128, 128, 1, 3, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1282: return launch_one<128, 128, 2, 2, FMT, CT, CM, DYN>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 161: return launch_one<16, 16, 1, 10, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 162: return launch_one<16, 16, 2, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 164: return launch_one<16, 16, 4, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 321: return launch_one<32, 32, 1, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 322: return launch_one<32, 32, 2, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 324: return launch_one<32, 32, 4, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 641: return launch_one<64, 64, 1, 4, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 642: return launch_one<64, 64, 2, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 644: return launch_one<64, 64, 4, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1281: return launch_one<128, 128, 1, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1282: return launch_one<128, 128, 2, 2, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: break;
     }
     if constexpr (!DYN) {
         switch (b * 10 + groups) {
-            case 160: return launch_one<16, 16, 1, 16, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 320: return launch_one<32, 32, 1, 16, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 640: return launch_one<64, 64, 1, 10, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 1280: return launch_one<128, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 160: return launch_one<16, 16, 1, 16, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 32, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 640: return launch_one<64, 64, 1, 5, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 1280: return launch_one<128, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
             default: break;
         }
     }
@@ -749,57 +759,57 @@ cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtens
 
 // Stacked blocks (row groups): 128 rows x b; token tile 256 and four stages of 48 KB, or 128 and six of 32 KB.
 template <int FMT, int CT, int CM>
-cudaError_t launch_stack_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_stack_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                                const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 161: return launch_one<16, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 160: return launch_one<16, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 320: return launch_one<32, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 161: return launch_one<16, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 160: return launch_one<16, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 320: return launch_one<32, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: break;
     }
     if constexpr (FMT != 2) {
-        if (b == 64 && groups == 1) return launch_one<64, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        if (b == 64 && groups == 2) return launch_one<64, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        if (b == 64 && groups == 1) return launch_one<64, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        if (b == 64 && groups == 2) return launch_one<64, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
     }
     return cudaErrorInvalidValue;
 }
 
 template <int FMT>
-cudaError_t launch_stack_fmt(int b, int groups, int c16, int cm, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_stack_fmt(int b, int groups, int c16, int cm, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                              const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
     if constexpr (FMT != 2) {
-        if (c16) return cm ? launch_stack_shape<FMT, 1, 1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-                           : launch_stack_shape<FMT, 1, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        if (c16) return cm ? launch_stack_shape<FMT, 1, 1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
+                           : launch_stack_shape<FMT, 1, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
     }
     if (c16) return cudaErrorInvalidValue;
-    return cm ? launch_stack_shape<FMT, 0, 1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-              : launch_stack_shape<FMT, 0, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+    return cm ? launch_stack_shape<FMT, 0, 1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
+              : launch_stack_shape<FMT, 0, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
 }
 
 // E4M3 inputs: fp32 C, static schedule; b = 32, 64 or 128 (a block row must hold at least one
 // 32-element K step).  Stages are half the bytes of the 16-bit ones.
 template <int CM>
-cudaError_t launch_fp8(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_fp8(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                        const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 321: return launch_one<32, 32, 1, 10, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 32, 2, 10, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 324: return launch_one<32, 32, 4, 6, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 641: return launch_one<64, 64, 1, 10, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 642: return launch_one<64, 64, 2, 10, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 644: return launch_one<64, 64, 4, 5, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1281: return launch_one<128, 128, 1, 6, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1282: return launch_one<128, 128, 2, 4, 3, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 321: return launch_one<32, 32, 1, 8, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 322: return launch_one<32, 32, 2, 10, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 324: return launch_one<32, 32, 4, 6, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 641: return launch_one<64, 64, 1, 7, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 642: return launch_one<64, 64, 2, 10, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 644: return launch_one<64, 64, 4, 5, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1281: return launch_one<128, 128, 1, 6, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1282: return launch_one<128, 128, 2, 4, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: break;
     }
     if constexpr (CM) {
         switch (b * 10 + groups) {
-            case 320: return launch_one<32, 32, 1, 16, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 640: return launch_one<64, 64, 1, 16, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 1280: return launch_one<128, 128, 1, 8, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 32, 1, 8, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 640: return launch_one<64, 64, 1, 8, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 1280: return launch_one<128, 128, 1, 8, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
             default: break;
         }
     }
@@ -808,35 +818,35 @@ cudaError_t launch_fp8(int b, int groups, const CUtensorMap& tmA, const CUtensor
 
 // TF32 (fp32 storage): fp32 C, static schedule; the deepest rings the stage sizes allow.
 template <int CM>
-cudaError_t launch_tf32(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmB3,
+cudaError_t launch_tf32(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
                         const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 161: return launch_one<16, 16, 1, 5, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 162: return launch_one<16, 16, 2, 3, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 321: return launch_one<32, 32, 1, 5, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 32, 2, 3, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 641: return launch_one<64, 64, 1, 8, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 642: return launch_one<64, 64, 2, 5, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 644: return launch_one<64, 64, 4, 3, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1281: return launch_one<128, 128, 1, 6, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1282: return launch_one<128, 128, 2, 4, 2, 0, CM, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 160: return launch_one<16, 16, 1, 10, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 320: return launch_one<32, 32, 1, 8, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 640: return launch_one<64, 64, 1, 10, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1280: return launch_one<128, 128, 1, 8, 2, 0, CM, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 161: return launch_one<16, 16, 1, 5, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 162: return launch_one<16, 16, 2, 3, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 321: return launch_one<32, 32, 1, 5, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 322: return launch_one<32, 32, 2, 3, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 641: return launch_one<64, 64, 1, 8, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 642: return launch_one<64, 64, 2, 5, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 644: return launch_one<64, 64, 4, 3, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1281: return launch_one<128, 128, 1, 6, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1282: return launch_one<128, 128, 2, 4, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 160: return launch_one<16, 16, 1, 10, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 320: return launch_one<32, 32, 1, 8, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 640: return launch_one<64, 64, 1, 10, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 1280: return launch_one<128, 128, 1, 8, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <int FMT>
-cudaError_t launch_fmt(int b, int groups, int c16, int cm, int dyn, const CUtensorMap& tmA, const CUtensorMap& tmB,
+cudaError_t launch_fmt(int b, int groups, int c16, int cm, int dyn, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB,
                        const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
     // dynamic scheduling is built for the default output (fp32, row-major) only
-    if (dyn) return (c16 || cm) ? cudaErrorInvalidValue : launch_shape<FMT, 0, 0, 1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-    if (cm) return c16 ? launch_shape<FMT, 1, 1, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-                       : launch_shape<FMT, 0, 1, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-    return c16 ? launch_shape<FMT, 1, 0, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-               : launch_shape<FMT, 0, 0, 0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+    if (dyn) return (c16 || cm) ? cudaErrorInvalidValue : launch_shape<FMT, 0, 0, 1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+    if (cm) return c16 ? launch_shape<FMT, 1, 1, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
+                       : launch_shape<FMT, 0, 1, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+    return c16 ? launch_shape<FMT, 1, 0, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
+               : launch_shape<FMT, 0, 0, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
 }
 
 }  // namespace
@@ -853,38 +863,38 @@ int bcsr_token_groups_max(int dtype, int b, int c16, int col_major) {
     return (b == 64 && !c16 && !col_major) ? 2 : 4;
 }
 
-cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA,
+cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA, const CUtensorMap& tmA0,
                         const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
                         int grid, cudaStream_t stream) {
-    if (dtype == 1) return launch_fmt<0>(b, groups, c16, col_major, dynamic, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
-    if (dtype == 0) return launch_fmt<1>(b, groups, c16, col_major, dynamic, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
+    if (dtype == 1) return launch_fmt<0>(b, groups, c16, col_major, dynamic, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
+    if (dtype == 0) return launch_fmt<1>(b, groups, c16, col_major, dynamic, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
     if (dtype == 3) {
         if (c16 || dynamic) return cudaErrorInvalidValue;
-        return col_major ? launch_fp8<1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-                         : launch_fp8<0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        return col_major ? launch_fp8<1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
+                         : launch_fp8<0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
     }
     if (dtype == 2) {
         if (c16 || dynamic) return cudaErrorInvalidValue;
-        return col_major ? launch_tf32<1>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream)
-                         : launch_tf32<0>(b, groups, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+        return col_major ? launch_tf32<1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
+                         : launch_tf32<0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,
+cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB,
                                 const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid,
                                 cudaStream_t stream) {
-    if (dtype == 1) return launch_stack_fmt<0>(b, groups, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
-    if (dtype == 0) return launch_stack_fmt<1>(b, groups, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
-    if (dtype == 2) return launch_stack_fmt<2>(b, groups, c16, col_major, tmA, tmB, tmB3, tmC, tmP, p, grid, stream);   // TF32: b = 16, 32
+    if (dtype == 1) return launch_stack_fmt<0>(b, groups, c16, col_major, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
+    if (dtype == 0) return launch_stack_fmt<1>(b, groups, c16, col_major, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
+    if (dtype == 2) return launch_stack_fmt<2>(b, groups, c16, col_major, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // TF32: b = 16, 32
     if (dtype == 3 && !c16 && col_major) {
         // E4M3: half the bytes per stage, deeper rings
         switch (b * 10 + groups) {
-            case 321: return launch_one<32, 128, 1, 10, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 320: return launch_one<32, 128, 1, 12, 3, 0, 1, 0, 1>(tmA, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 321: return launch_one<32, 128, 1, 10, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 128, 1, 12, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
             default: break;
         }
     }

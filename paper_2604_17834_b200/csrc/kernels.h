@@ -61,12 +61,13 @@ struct BcsrParams {
 // (es * groups) x kb x t; 128-byte swizzle (with 32-byte atoms for es = 4).  Column-major operands
 // (col_major): tmB = X as [N][k], box 128 tokens x min(kb * es, 128) bytes; tmB3 = X as
 // [N / 128][128][k], box groups x 128 x the same; both with the swizzle of that row length.
-// tmA: the stored blocks as [blocks * b][b], box (b * blocks per stage) rows x min(kb * es, 128) bytes.
+// tmA0: tmA as wider tiles have it, fewer blocks to a box (stacked blocks: not used).
+// tmA: the stored blocks as [blocks * b][b], box (b * bcsr_blocks_per_stage) rows x min(kb * es, 128) bytes.
 // tmC: C as [m][N], box 32 x bcsr_epi_cols, no swizzle; or fp32 Y as [N][m], box 16 x 32, 64-byte swizzle (16-bit Y:
 // any valid map, it is stored without one).
 // dynamic: the grid is one CTA per tile (grid = number of tiles, p.tiles in the schedule's global
 // order, p.cta_ptr unused) and CTAs steal tiles through Cluster Launch Control; fp32 row-major only.
-cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA,
+cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA, const CUtensorMap& tmA0,
                         const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP,
                         const BcsrParams& p, int grid, cudaStream_t stream);
 // Row groups: the same kernel with 128 x b stacked blocks (MMA N = 128) and a 256-token tile (groups = 2), or a
@@ -78,7 +79,7 @@ cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, in
 constexpr int kSplitGroups = 0;
 constexpr int kStackRows = 128;
 constexpr int kStackGroups = 2;
-cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmB,
+cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB,
                                 const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
                                 int grid, cudaStream_t stream);
 // K-split: tmP = the partial tiles as [slots * b][N] fp32, box as tmC's (the tile record of a
@@ -100,10 +101,13 @@ int bcsr_token_groups_max(int dtype, int b, int c16, int col_major);
 // request whose box is 32 tokens x this many rows (row-major C) or this many columns x 32 tokens
 // (column-major fp32 Y).  Larger tiles (up to 64 rows) were measured slower: the stage ring needs the room.
 constexpr int bcsr_epi_cols(int b, bool c16, bool col_major) { return (b < 32 || !c16) ? 16 : 32; }
-// stored blocks that share one pipeline stage (and one A request): 4 / 2 for b = 16 / 32
-constexpr int bcsr_blocks_per_stage(int b) { return b == 16 ? 4 : (b == 32 ? 2 : 1); }
+// stored blocks that share one pipeline stage (and one A request): 4 / 2 / 1 for b = 16 / 32 / 64 and more; twice as many
+// for b = 32 and 64 with tiles of 128 tokens (groups <= 1) and up to 2-byte values, see BcsrCfg::kBps
+constexpr int bcsr_blocks_per_stage(int b, int es, int groups) {
+    return (b == 16 ? 4 : (b == 32 ? 2 : 1)) * (groups <= 1 && es <= 2 && (b == 32 || b == 64) ? 2 : 1);
+}
 // stacked blocks (row groups) per stage: 4 / 2 / 1 blocks; 4-byte values are twice as wide
-constexpr int bcsr_stacked_per_stage(int b, int es) { return es == 4 ? bcsr_blocks_per_stage(b) / 2 : bcsr_blocks_per_stage(b); }
+constexpr int bcsr_stacked_per_stage(int b, int es) { return bcsr_blocks_per_stage(b, es, 2) / (es == 4 ? 2 : 1); }
 // Column slices a stored block is cut into, one pipeline stage each: blocks of 4-byte elements
 // with rows longer than 128 bytes (TF32, b = 64 / 128) go through the ring 32 columns at a time;
 // every other block is one unit.
