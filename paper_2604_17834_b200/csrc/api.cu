@@ -855,8 +855,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     // from kSplitMinBytes in the longest tile on (shorter ones are latencies, and two CTAs fetch the blocks, or the tokens,
     // twice); row groups only where their longest tile, not the work as a whole, decides when the last CTA ends.  us:
     //   1500 x 9000, b = 64, 10 % full rows, fp16, N = 200 (3.4 MB a tile)   35.0 -> 22.5
-    //   3000 x 16000, b = 16, 10 % full rows, bf16, N = 256 (8 MB, grouped)  93.2 -> 75.3
-    //   600 x 6000, b = 16, 10 % full rows, TF32, N = 200 (6 MB, grouped)    55.2 -> 44.0
+    //   3000 x 16000, b = 16, 10 % full rows, bf16, N = 256 (8 MB, grouped)  93.2 -> 67.9
+    //   600 x 6000, b = 16, 10 % full rows, TF32, N = 200 (6 MB, grouped)    55.2 -> 41.6
     //   3000 x 6000, b = 32, 10 % full rows, fp16, N = 512 (3 MB, grouped)   25.9 -> 26.6: left alone
     //   3584 x 18944, b = 64, density 0.1, bf16, N = 128 (1 MB)              9.6 -> 9.4
     //   1024 x 4096 and back, b = 64, density 0.2, N = 300 (0.3 MB)          10.7 -> 11.0: left alone

@@ -88,8 +88,11 @@ struct BcsrCfg {
     // 0.1, N = 128, bf16 9.5 -> 7.9 us; N = 2048, E4M3 34.4 -> 31.6; b = 32, 2048 x 8192 both ways,
     // N = 700, bf16 25.2 -> 23.9.  Not for b = 16, whose stages already hold four blocks: with eight,
     // 50 blocks a row 11.1 -> 10.7, but two blocks a row 6.8 -> 7.2 (half as many tiles in flight).
+    // Halves of stacked rows, whose MMAs are half as long, have twice the blocks as well: 3000 x
+    // 16000, b = 16, 10 % full rows, bf16, N = 256 75.3 -> 67.8, 600 x 6000 TF32, N = 200 44.0 ->
+    // 41.1 (whole stacked blocks, three stages of 64 KB for six of 32: 49.0 -> 50.5 on 6000 x 5000).
     // A stage that is at most half full asks for half of the A blocks (tmA0): kFew.
-    static constexpr int kBps = H == B ? bcsr_blocks_per_stage(B, ES, GROUPS) : bcsr_stacked_per_stage(B, ES);
+    static constexpr int kBps = H == B ? bcsr_blocks_per_stage(B, ES, GROUPS) : bcsr_stacked_per_stage(B, ES) * (SPLIT ? 2 : 1);
     static constexpr int kFew = H == B ? bcsr_blocks_per_stage(B, ES, 2) : kBps;
     static constexpr int kStageBytes = ((kBps * (kDenseBytes + kABytes) + 1023) / 1024) * 1024;
     static constexpr int kAOff = kBps * kDenseBytes;         // A blocks inside the stage
@@ -766,8 +769,8 @@ cudaError_t launch_stack_shape(int b, int groups, const CUtensorMap& tmA, const 
         case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 160: return launch_one<16, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 320: return launch_one<32, 128, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 160: return launch_one<16, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 320: return launch_one<32, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
         default: break;
     }
     if constexpr (FMT != 2) {
@@ -894,7 +897,7 @@ cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_m
             case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
             case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
             case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 320: return launch_one<32, 128, 1, 12, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 128, 1, 6, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
             default: break;
         }
     }
