@@ -999,6 +999,25 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     return SPMM_OK;
 }
 
+// Which request of a stage goes first, its stored blocks or its B tiles: the one that is longer on its way.  Many
+// block-rows share a token tile, which is then close by in L2, and the blocks go first; where few do, the tiles do.  The line, by
+// block-rows (148 CTAs), from the speed with the tiles first over that with the blocks first, geometric mean (and range) of
+// products of random sizes, 0.3 - 5 ms, N = 300 - 50,000, row-major:
+//   block-rows    under 10            10 - 20             20 - 30             30 - 50             60 - 100            100 - 200
+//   b = 128 TF32  1.016 (0.97 - 1.04) 1.011 (0.96 - 1.06) 1.008 (0.96 - 1.23) 1.003 (0.97 - 1.05) 0.983 (0.92 - 1.09) 0.951 (0.92 - 1.00)
+//           bf16  1.015 (0.92 - 1.05) 1.014 (0.95 - 1.07) 1.005 (0.93 - 1.11) 0.997 (0.87 - 1.10) 0.961 (0.89 - 1.02) 0.977 (0.91 - 1.02)
+//   b = 64  TF32  1.014 (1.00 - 1.02) 1.006 (0.98 - 1.04) 1.007 (0.98 - 1.02) 1.007 (0.98 - 1.06) 1.000 (0.96 - 1.07) 0.995 (0.95 - 1.06), under 16 blocks a row
+//           bf16  1.007 (1.00 - 1.03) 1.006 (0.99 - 1.03) 1.002 (0.94 - 1.04) 0.998 (0.98 - 1.04) 0.996 (0.94 - 1.02) 0.99  (0.96 - 1.02)
+// b <= 32 (and stacked blocks) do not gain on either side.  TF32 at b = 64 has the longest B tiles beside its blocks (32 KB to
+// 8): long tiles, 32 blocks a row and more, gain at any number of block-rows, 1.009 (0.96 - 1.08); not in decode steps (0.97
+// - 0.99 with N under 200).
+bool bcsr_tiles_first(const spmm_handle_s* h, int groups) {
+    const BcsrHost& f = h->bcsr;
+    if (f.b < 64) return false;
+    if (h->es == 4 && f.b == 64 && groups > 1) return 3 * f.nbr < h->n_ctas || f.nnzb >= 32 * f.nbr;
+    return 5 * f.nbr < h->n_ctas;
+}
+
 int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t stream) {
     const BcsrHost& f = h->bcsr;
     // the box of the dense operand is 64 tokens wide (128 with column-major operands or 1-byte values)
@@ -1022,6 +1041,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.B = nullptr;
     p.k = h->k;
     p.overlap = 0;
+    p.tiles_first = bcsr_tiles_first(h, h->sched.groups) ? 1 : 0;
     CUtensorMap tmA = h->sched.groups <= 1 ? h->tmA1 : h->tmA, tmA0 = h->tmA;
     if (!h->tmA_ok) {
         // no stored block at all: the kernel never touches A, any valid map will do

@@ -45,6 +45,7 @@
 // The host deals tiles to CTAs ahead of time: slab by slab (a slab = token tiles whose B rows
 // fit in L2), longest block-row first, each tile to the least loaded CTA; CTA c walks its list.
 #include <mutex>
+#include <type_traits>
 
 #include "kernels.h"
 #include "ptx.cuh"
@@ -323,22 +324,26 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 if constexpr (Cfg::kHalfTok) return static_cast<int>(min_i64(Cfg::kTok, N > n0 + half * Cfg::kTok ? N - n0 - half * Cfg::kTok : 0));
                 return static_cast<int>(min_i64(Cfg::kBnT, N - n0));
             };
-            // the stage of unit it: its byte count, then its stored blocks q .. q + nb - 1 (columns kx .. of them)
-            auto request_blocks = [&](uint32_t it, int q, int kx, int nb, int nvalid) {
-                const int s = it % STAGES;
-                const uint32_t sb = smem_base + s * Cfg::kStageBytes;
+            // the A request always brings kBps or kFew blocks (the boxes of the tensor maps)
+            auto few_blocks = [&](int nb) { return Cfg::kFew < Cfg::kBps && nb <= Cfg::kFew; };
+            // the stage of unit it, nb stored blocks: its byte count, before any of its requests
+            auto expect_stage = [&](uint32_t it, int nb, int nvalid) {
                 const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
-                // the A request always brings kBps or kFew blocks (the boxes of the tensor maps)
-                const bool few = Cfg::kFew < Cfg::kBps && nb <= Cfg::kFew;
                 const uint32_t dense_tx = CM ? (Cfg::kHalfTok ? (nvalid > 0 ? Cfg::kDenseBytes : 0)
                                                               : ((p.use_3d && nvalid == Cfg::kBnT) ? Cfg::kDenseBytes : ((nvalid + 127) >> 7) * (128 * Cfg::kBB)))
                                              : nbox * Cfg::kBoxBytes;
                 // (stacked blocks: one request per block, a box holds at most 256 rows)
-                if (lane == 0) mbar_arrive_expect_tx(full_bar(s), (H == B ? (few ? Cfg::kFew : Cfg::kBps) : nb) * Cfg::kABytes + nb * dense_tx);
+                if (lane == 0)
+                    mbar_arrive_expect_tx(full_bar(it % STAGES), (H == B ? (few_blocks(nb) ? Cfg::kFew : Cfg::kBps) : nb) * Cfg::kABytes + nb * dense_tx);
                 __syncwarp();
+            };
+            // and its stored blocks q .. q + nb - 1 (columns kx .. of them)
+            auto request_blocks = [&](uint32_t it, int q, int kx, int nb) {
+                const int s = it % STAGES;
+                const uint32_t sb = smem_base + s * Cfg::kStageBytes;
                 if constexpr (H == B) {
                     if (lane == 8) {
-                        tma_load_2d_hint(sb + Cfg::kAOff, few ? &tmA0 : &tmA, full_bar(s), kx, q * B, keep);
+                        tma_load_2d_hint(sb + Cfg::kAOff, few_blocks(nb) ? &tmA0 : &tmA, full_bar(s), kx, q * B, keep);
                     } else if (Cfg::kBB > 128 && lane == 9) {
                         tma_load_2d_hint(sb + Cfg::kAOff + B * 128, &tmA, full_bar(s), 128 / ES, q * B, keep);
                     }
@@ -362,14 +367,19 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const int nvalid = valid_tokens(rec0.y * Cfg::kBnT);
                 for (uint32_t u = pw; u < early; u += NP) {
                     const int jq = static_cast<int>(u) / Cfg::kKS * Cfg::kBps;
-                    request_blocks(u, rec0.z + jq, static_cast<int>(u) % Cfg::kKS * Cfg::kKB, min(Cfg::kBps, nq - jq), nvalid);
+                    expect_stage(u, min(Cfg::kBps, nq - jq), nvalid);
+                    request_blocks(u, rec0.z + jq, static_cast<int>(u) % Cfg::kKS * Cfg::kKB, min(Cfg::kBps, nq - jq));
                 }
             }
             operands_ready();
+            // The order of a stage's requests, see bcsr_tiles_first in api.cu, is chosen outside the loop: a test of it per
+            // stage cost small launches up to 5 % (15,584 x 2008, b = 64, TF32, N = 680, us: 37.4 so, 39.3 with the test).
+            auto walk = [&](auto order) {
+            constexpr bool kTilesFirst = decltype(order)::value;
             for (uint32_t nth = 0; ok && next_tile(nth, &tcd, &tcd_next, &ok); ++nth) {
                 const int nvalid = valid_tokens(tcd.y * Cfg::kBnT);
                 const int n0 = tcd.y * Cfg::kBnT + (Cfg::kHalfTok ? half * Cfg::kTok : 0);         // this CTA's first token
-                const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
+                [[maybe_unused]] const int nbox = (nvalid + Cfg::kTokBox - 1) / Cfg::kTokBox;
                 const bool whole_tile = !Cfg::kHalfTok && p.use_3d && nvalid == Cfg::kBnT;
                 const int pb = tcd.z, pe = tcd.w;
                 const int Jl_first = have_next ? Jl_next : ((pb + lane < pe) ? __ldg(p.block_col_idx + pb + lane) : 0);
@@ -392,9 +402,12 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                         const int s = it % STAGES;
                         const uint32_t ph = (it / STAGES) & 1u;
                         // (an early unit's stage is fresh; it may even have been used already, where it has no tokens)
-                        if (it >= early && !__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, ctl, 1))) { ok = false; break; }
+                        if (it >= early) {
+                            if (!__all_sync(0xffffffffu, mbar_wait(empty_bar(s), ph ^ 1u, ctl, 1))) { ok = false; break; }
+                            expect_stage(it, nb, nvalid);
+                            if (!kTilesFirst) request_blocks(it, q, kx, nb);
+                        }
                         const uint32_t sb = smem_base + s * Cfg::kStageBytes;
-                        if (it >= early) request_blocks(it, q, kx, nb, nvalid);
                         if constexpr (CM) {
                             // X as [N / 128][128][k]: box = GROUPS x 128 tokens x min(b, 64) elements
                             // of block column J (b = 128: lanes nb.. fetch the second K half)
@@ -427,9 +440,13 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                                      n0 + lane * Cfg::kTokBox, J * B + kx, keep);
                             }
                         }
+                        if (kTilesFirst && it >= early) request_blocks(it, q, kx, nb);
                     }
                 }
             }
+            };
+            if (H == B && B >= 64 && p.tiles_first) walk(std::bool_constant<H == B && B >= 64>());
+            else walk(std::false_type());
             if (lane == 0) issued[pw] = it;
         }
     } else if (warp == 1) {

@@ -344,6 +344,40 @@ def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16)
             lib.spmm_destroy(h1)
 
 
+@pytest.mark.parametrize("dtype,b,layout,c16", [("tf32", 64, "row", False), ("tf32", 64, "col", False), ("tf32", 128, "row", False), ("bf16", 64, "row", False),
+                                                ("fp16", 64, "col", True), ("fp8", 64, "col", False), ("bf16", 128, "col", True), ("fp8", 128, "row", False)])
+def test_bcsr_order_of_requests_changes_no_bit(lib, dtype, b, layout, c16):
+    """Few block-rows for the grid (a fifth; TF32 blocks of 64: a third): a stage's token tiles are requested before its stored
+    blocks.  Grids on either side of the line, rows of one block to several rings full, an empty one, a ragged last token
+    tile: the same bits, and the oracle's result."""
+    third = dtype == "tf32" and b == 64
+    nbr, nbc = 3, 40
+    rng = np.random.default_rng(b)
+    mask = np.zeros((nbr, nbc), bool)
+    mask[0] = True
+    mask[2, rng.permutation(nbc)[:1]] = True
+    m, k = nbr * b - 8, nbc * b - 16
+    full = np.kron(mask, np.ones((b, b), bool))[:m, :k]
+    rp = np.concatenate(([0], np.cumsum(full.sum(1)))).astype(np.int64)
+    ci = np.nonzero(full)[1].astype(np.int32)
+    vals = wl.to_storage(rng.uniform(-1, 1, ci.size), dtype)
+    N = 128 * 55 + 16                                     # two token groups to a tile on 10 CTAs
+    Bs = wl.dense(11, k, N, ("uniform", -1.0, 1.0), dtype)
+    got = []
+    for n_ctas in ((9, 10) if third else (15, 16)):
+        h = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, n_ctas=n_ctas, layout=lib.COLMAJOR if layout == "col" else lib.ROWMAJOR,
+                                     c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
+        try:
+            got.append(run_gpu_variant(lib, h, Bs, m, N, dtype, c16=c16, col_major=layout == "col"))
+            assert lib.spmm_get_info(h, N)["plan_token_tile"] > 128 or not third
+        finally:
+            lib.spmm_destroy(h)
+    assert np.array_equal(got[0], got[1])
+    cols = np.arange(0, N, 37)
+    Cr, S = reference({"m": m, "k": k, "row_ptr": rp, "col_idx": ci, "vals": vals}, Bs, dtype, cols=cols)
+    assert_close(got[0][:, cols], Cr, S, dtype, "order of requests b=%d" % b)
+
+
 @pytest.mark.parametrize("dtype", ["tf32", "fp16", "fp8"])
 def test_bcsr_gpu_builder_with_many_block_columns(lib, dtype):
     """More than 196,608 block columns: the builder's bitmap takes more than 48 KB of shared memory."""
