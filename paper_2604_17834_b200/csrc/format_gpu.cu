@@ -343,7 +343,8 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     const int64_t nbr = (m + b - 1) / b, nbc = (k + b - 1) / b;
     const int words = static_cast<int>((nbc + 31) / 32);
     const size_t smem = static_cast<size_t>(2) * (words > 0 ? words : 1) * 4;
-    if (smem > 200 * 1024) return SPMM_ERR_TOO_LARGE;
+    constexpr int kMostSmem = 200 * 1024;
+    if (smem > kMostSmem) return SPMM_ERR_TOO_LARGE;
     *d_block_row_ptr = nullptr;
     *d_block_col_idx = nullptr;
     *d_blocks = nullptr;
@@ -389,11 +390,11 @@ int build_bcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     *nnz_out = nnz;
 
     // 2. stored blocks per block-row, 3. block_row_ptr
-    if (smem > 48 * 1024) {
-        cudaFuncSetAttribute(bcsr_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        cudaFuncSetAttribute(bcsr_fill_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        cudaFuncSetAttribute(bcsr_fill_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        cudaFuncSetAttribute(bcsr_fill_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (smem > 48 * 1024) {                  // (the most there may be: threads that build for other widths set it too)
+        cudaFuncSetAttribute(bcsr_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+        cudaFuncSetAttribute(bcsr_fill_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+        cudaFuncSetAttribute(bcsr_fill_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
+        cudaFuncSetAttribute(bcsr_fill_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostSmem);
     }
     if (nbr > 0) bcsr_count_kernel<<<static_cast<unsigned>(nbr), kThreads, smem, st>>>(m, b, words, d_row_ptr, d_col_idx, d_counts);
     exclusive_scan_kernel<<<1, 1024, 0, st>>>(d_counts, nbr, *d_block_row_ptr, d_flags + 1);
@@ -696,6 +697,7 @@ __device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w
 }
 
 constexpr int kMostBitmap = 216 * 1024;                       // bits and their prefixes, 8 bytes per 32 columns
+static_assert(kLargeWindow * 12 <= kMostBitmap, "the merging kernels' shared memory");
 template <int WH>
 __global__ void __launch_bounds__(kBitmapThreads) wcsr_bitmap_windows_kernel(const CondenseParams p, int max_words) {
     extern __shared__ int32_t dyn[];
@@ -929,7 +931,8 @@ template <int WH>
 bool condense(CondenseParams p, const WindowLists& lists, const int* count, cudaStream_t st) {
     bool first = true;
     auto launch = [&](auto kernel, int64_t grid, int threads, size_t smem, const auto&... args) {
-        if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)) != cudaSuccess) return false;
+        // (the most there may be: threads that build for other widths set it too)
+        if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostBitmap) != cudaSuccess) return false;
         if (!first) return launch_dependent(kernel, dim3(static_cast<unsigned>(grid)), threads, smem, st, p, args...) == cudaSuccess;
         first = false;
         kernel<<<static_cast<unsigned>(grid), threads, smem, st>>>(p, args...);

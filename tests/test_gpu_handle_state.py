@@ -325,3 +325,40 @@ def test_waits_do_not_count_the_launch_before(lib):
         lib.spmm_set_wait_limit_ns(2_000_000_000)
         for h in hs:
             lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["bcsr", "wcsr"])
+def test_handles_built_by_several_threads_for_different_widths(lib, kind):
+    """The GPU builders' shared memory grows with the matrix's width: threads that build for a narrow and for a wide one at the
+    same time do not take each other's allowance away."""
+    import threading
+    import torch
+    m, n = 16, 256                                         # (one entry per 256 columns: WCSR's bitmap kernel)
+    widths = (500_000, 800_000) if kind == "wcsr" else (4_000_000, 12_000_000)
+    mats = []
+    for k in widths:
+        rp = torch.arange(m + 1, dtype=torch.int64, device="cuda") * n
+        ci = (torch.arange(n, device="cuda") * (k // n)).to(torch.int32).repeat(m)
+        mats.append((k, rp, ci, torch.ones(m * n, dtype=torch.float16, device="cuda")))
+    torch.cuda.synchronize()
+    create = lib.spmm_bcsr_create_csr_device if kind == "bcsr" else lib.spmm_wcsr_create_csr_device
+    failed = []
+
+    def build(i):
+        k, rp, ci, va = mats[i % 2]
+        stream = torch.cuda.Stream()
+        try:
+            for _ in range(200):
+                h = create(m, k, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), "fp16", 16, stream.cuda_stream)
+                units = lib.spmm_get_info(h, 64)["n_units"]
+                lib.spmm_destroy(h)
+                assert units == n
+        except Exception as e:                             # for the main thread to raise
+            failed.append(e)
+
+    threads = [threading.Thread(target=build, args=(i,)) for i in range(8)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed, failed[0]
