@@ -16,8 +16,8 @@
 //
 // WCSR (window condensation of Sec. 2.3): a window's entries are one contiguous range of the CSR arrays, wh ascending
 // runs.  A short window is sorted by one warp in registers, a longer one goes through a bitmap of its columns or, where
-// the matrix is too wide for that, is merged run by run in shared memory; each way an entry gets its place among the
-// window's distinct columns.  A prefix sum of the lengths padded to b_col is window_row_ptr; a last pass, entry by entry, writes the
+// the matrix is too wide for that, is merged run by run in shared memory; one too long for that is cut into pieces by
+// column, which go either way, a CTA each.  An entry gets its place among the window's distinct columns.  A prefix sum of the lengths padded to b_col is window_row_ptr; a last pass, entry by entry, writes the
 // columns over a -1 fill and the values straight into the packed tile layout.
 #include <cstring>
 #include <numeric>
@@ -43,13 +43,32 @@ constexpr int kThreads = 256;
 constexpr int kWarpWindow = 256, kMergeWindow = 2048, kLargeWindow = 18432;
 constexpr int kColumnsPerEntry = 256;        // a bitmap from one entry per that many columns on
 enum { kListBitmap, kListMerge, kListLarge, kLists };
+constexpr int kMostBitmap = 216 * 1024;      // bits and their prefixes, 8 bytes per 32 columns
+constexpr int64_t kBitmapColumns = kMostBitmap / 8 * 32;
+static_assert(kLargeWindow * 12 <= kMostBitmap, "the merging kernels' shared memory");
+// Windows of more than kLargeWindow entries are cut into pieces of about kPiece, at columns chosen so that no piece holds more
+// than kPieceCap (wcsr_cut_windows_kernel), unless a bitmap reads no more than kBitmapReads entries for them: the four launches
+// for the pieces cost a small handle about as much as that (R-MAT 2^15, 24 a row, all windows above 18,432 entries cut:
+// 254 -> 267 us).
+constexpr int kBitmapReads = 48 * 1024;
+constexpr int kPiece = 4032, kPieceSlack = 512, kPieceCap = kPiece + kPieceSlack + 64;
+__host__ __device__ constexpr int64_t pieces_of(int64_t n) { return (n + kPiece - 1) / kPiece; }
+constexpr int64_t kMostLong = (int64_t{1} << 31) / kLargeWindow + 1;      // windows there can be, with less than 2^31 entries
+constexpr int kLongShift = 40;               // a count of windows above this bit, of their pieces below it
 struct WindowLists {
     int wh;                                  // 0: no lists are wanted
     int64_t k;
     int32_t* list[kLists];
     int* count;                              // [kLists], zero before
+    int32_t *long_window, *long_first;       // [max_long] the windows that are cut, and their first pieces
+    unsigned long long* long_count;          // both counts in one, zero before: the first pieces ascend with the windows' places
+    int64_t max_long;
+    __device__ __forceinline__ bool is_long(int64_t n) const {
+        if (n <= kLargeWindow) return false;
+        return n > kBitmapReads || n * ((k + kBitmapColumns - 1) / kBitmapColumns) > kBitmapReads;
+    }
     __device__ __forceinline__ int which(int64_t n) const {
-        if (n <= kWarpWindow) return -1;
+        if (n <= kWarpWindow || is_long(n)) return -1;
         if (n > kLargeWindow || n * kColumnsPerEntry >= k) return kListBitmap;
         return n <= kMergeWindow ? kListMerge : kListLarge;
     }
@@ -71,6 +90,14 @@ __global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* er
             const int64_t n = row_ptr[min(i + longer.wh, m)] - row_ptr[i];
             const int which = longer.which(n);
             if (which >= 0) longer.list[which][atomicAdd(longer.count + which, 1)] = static_cast<int32_t>(i / longer.wh);
+            if (longer.is_long(n) && n < (int64_t{1} << 31)) {
+                const unsigned long long one = 1ull << kLongShift, before = atomicAdd(longer.long_count, one + static_cast<unsigned long long>(pieces_of(n)));
+                const int64_t at = static_cast<int64_t>(before >> kLongShift);
+                if (at < longer.max_long) {              // (not so with a row_ptr that is refused)
+                    longer.long_window[at] = static_cast<int32_t>(i / longer.wh);
+                    longer.long_first[at] = static_cast<int32_t>(before & (one - 1));
+                }
+            }
         }
     }
 }
@@ -471,8 +498,21 @@ __device__ __forceinline__ int row_in_window(const int* off, int j) {
     return r;
 }
 
+// Where the entries of a window, or of a piece of one, lie: entry j, of its row r.
+struct WholeWindow {
+    int64_t p0;
+    const int* off;
+    __device__ __forceinline__ int64_t at(int, int j) const { return p0 + j; }
+    __device__ __forceinline__ int64_t row_start(int r) const { return p0 + off[r]; }
+};
+struct WindowPiece {
+    const int64_t *base, *start;             // per row: the place of its first entry here minus that entry's number; its start
+    __device__ __forceinline__ int64_t at(int r, int j) const { return base[r] + j; }
+    __device__ __forceinline__ int64_t row_start(int r) const { return start[r]; }
+};
+
 // One warp: at most 32 * ITEMS entries, sorted in registers by a bitonic network over positions lane * ITEMS + i; the
-// distinct ones then lie ascending in cols (padded to 256 with the largest int), where every entry looks its own up.
+// distinct ones then lie ascending in cols (padded to 32 * ITEMS with the largest int), where every entry looks its own up.
 // For 60,000 power-law rows the network takes about four warp instructions per entry, merging in shared memory 44.
 template <int WH, int ITEMS>
 __device__ __forceinline__ void sort_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, int32_t* own, int32_t* cols) {
@@ -550,16 +590,18 @@ __device__ __forceinline__ void sort_window(const CondenseParams& p, int64_t w, 
     }
 }
 
-// n entries from p0 on: keys[2][cap], rank[cap] in shared memory; off has WH + 1 entries.
-template <int WH, int THREADS>
-__device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, int32_t* keys, int cap, uint32_t* rank) {
+// n entries: keys[2][cap], rank[cap] in shared memory; off has WH + 1 entries.  *found: distinct columns.
+template <int WH, int THREADS, class Entries>
+__device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w, const Entries& e, int n, const int* off, int32_t* keys, int cap, uint32_t* rank,
+                                             int32_t* found) {
     __shared__ int warp_sum[THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j < n; j += THREADS) {
         const int r = row_in_window<WH>(off, j);
-        keys[j] = checked_column(p, p0 + j, p0 + off[r]);
+        const int64_t at = e.at(r, j);
+        keys[j] = checked_column(p, at, e.row_start(r));
         rank[j] = static_cast<uint32_t>(j) | static_cast<uint32_t>(r) << 16;     // the row stays beside the rank
-        p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
+        p.row_of[at] = static_cast<int32_t>(w * WH + r);
     }
     __syncthreads();
     int32_t *src = keys, *dst = keys + cap;
@@ -608,8 +650,8 @@ __device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w,
         carry = all;
         __syncthreads();
     }
-    if (threadIdx.x == 0) p.ucount[w] = carry;
-    for (int j = threadIdx.x; j < n; j += THREADS) p.pos_of[p0 + j] = dst[rank[j] & 0xffffu] - 1;
+    if (threadIdx.x == 0) *found = carry;
+    for (int j = threadIdx.x; j < n; j += THREADS) p.pos_of[e.at(static_cast<int>(rank[j] >> 16), j)] = dst[rank[j] & 0xffffu] - 1;
 }
 
 // One warp per window; the last of the launches that run side by side, it ends after the others.
@@ -650,27 +692,29 @@ __global__ void __launch_bounds__(THREADS) wcsr_merge_windows_kernel(const Conde
     grid_trigger();
     const int64_t w = p.list[blockIdx.x];
     load_offsets<WH, THREADS>(p, w, off);
-    merge_window<WH, THREADS>(p, w, p.row_ptr[w * WH], off[WH], off, dyn, kCap, reinterpret_cast<uint32_t*>(dyn + 2 * kCap));
+    merge_window<WH, THREADS>(p, w, WholeWindow{p.row_ptr[w * WH], off}, off[WH], off, dyn, kCap, reinterpret_cast<uint32_t*>(dyn + 2 * kCap), p.ucount + w);
     grid_wait();
 }
 
-// Bits of the columns [c0, c0 + 32 words) and the set bits before each word, as many at a time as there is room for.
+// Bits of the columns [c0, c0 + 32 words) and the set bits before each word, as many at a time as there is room for, of the
+// columns [begin, end) that the entries lie in.  *found: distinct columns.
 constexpr int kBitmapThreads = 512;
-template <int WH>
-__device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w, int64_t p0, int n, const int* off, uint32_t* bits, int max_words) {
+template <int WH, class Entries>
+__device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w, const Entries& e, int n, const int* off, uint32_t* bits, int max_words,
+                                              int64_t begin, int64_t end, int32_t* found_columns) {
     __shared__ long long scratch[32];
     constexpr int T = kBitmapThreads;
     uint32_t* prefix = bits + max_words;
     int found = 0;                           // condensed columns before c0
-    for (int64_t c0 = 0; c0 < p.k; c0 += int64_t{32} * max_words) {
-        const int words = static_cast<int>(min(static_cast<int64_t>(max_words), (p.k - c0 + 31) / 32));
+    for (int64_t c0 = begin; c0 < end; c0 += int64_t{32} * max_words) {
+        const int words = static_cast<int>(min(static_cast<int64_t>(max_words), (end - c0 + 31) / 32));
         __syncthreads();
         for (int i = threadIdx.x; i < words; i += T) bits[i] = 0u;
         __syncthreads();
         for (int j = threadIdx.x; j < n; j += T) {
             const int r = row_in_window<WH>(off, j);
-            const int64_t c = checked_column(p, p0 + j, p0 + off[r]) - c0;
-            if (c0 == 0) p.row_of[p0 + j] = static_cast<int32_t>(w * WH + r);
+            const int64_t at = e.at(r, j), c = checked_column(p, at, e.row_start(r)) - c0;
+            if (c0 == begin) p.row_of[at] = static_cast<int32_t>(w * WH + r);
             if (c >= 0 && c < int64_t{32} * words) atomicOr(&bits[c >> 5], 1u << (c & 31));
         }
         __syncthreads();
@@ -686,18 +730,19 @@ __device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w
         found = static_cast<int>(carry);
         for (int j = threadIdx.x; j < n; j += T) {
             const int r = row_in_window<WH>(off, j);
-            const int64_t c = checked_column(p, p0 + j, p0 + off[r]) - c0;
+            const int64_t at = e.at(r, j), c = checked_column(p, at, e.row_start(r)) - c0;
             if (c < 0 || c >= int64_t{32} * words) continue;
-            p.pos_of[p0 + j] = static_cast<int32_t>(prefix[c >> 5] + __popc(bits[c >> 5] & ((1u << (c & 31)) - 1u)));
+            p.pos_of[at] = static_cast<int32_t>(prefix[c >> 5] + __popc(bits[c >> 5] & ((1u << (c & 31)) - 1u)));
         }
         for (int i = threadIdx.x; i < words; i += T)
-            for (uint32_t x = bits[i]; x; x &= x - 1) atomicAdd(p.refs + c0 + 32 * int64_t{i} + (__ffs(x) - 1), 1);
+            for (uint32_t x = bits[i]; x; x &= x - 1) {
+                const int64_t c = c0 + 32 * int64_t{i} + (__ffs(x) - 1);
+                atomicAdd(p.refs + c, 1);
+            }
     }
-    if (threadIdx.x == 0) p.ucount[w] = found;
+    if (threadIdx.x == 0) *found_columns = found;
 }
 
-constexpr int kMostBitmap = 216 * 1024;                       // bits and their prefixes, 8 bytes per 32 columns
-static_assert(kLargeWindow * 12 <= kMostBitmap, "the merging kernels' shared memory");
 template <int WH>
 __global__ void __launch_bounds__(kBitmapThreads) wcsr_bitmap_windows_kernel(const CondenseParams p, int max_words) {
     extern __shared__ int32_t dyn[];
@@ -705,8 +750,166 @@ __global__ void __launch_bounds__(kBitmapThreads) wcsr_bitmap_windows_kernel(con
     grid_trigger();
     const int64_t w = p.list[blockIdx.x];
     load_offsets<WH, kBitmapThreads>(p, w, off);
-    bitmap_window<WH>(p, w, p.row_ptr[w * WH], off[WH], off, reinterpret_cast<uint32_t*>(dyn), max_words);
+    bitmap_window<WH>(p, w, WholeWindow{p.row_ptr[w * WH], off}, off[WH], off, reinterpret_cast<uint32_t*>(dyn), max_words, 0, p.k, p.ucount + w);
     grid_wait();
+}
+
+// ---- windows cut into pieces
+// A CTA to a piece; with one to a whole window a dense row was one SM's work.  ms to build a handle (in brackets the builder
+// before that one, which sorted all entries): 16 x 1,000,000, full 72 (4.6) -> 0.52; 16 rows of 1,000,000 entries among
+// 5 x 10^7 columns 1530 (25) -> 8.4; 1,000,000 rows of 8 and a full one 8.4 (9.2) -> 3.9; R-MAT 2^21, 16 a row 16.8 (22.7) -> 15.9.
+struct LongWindows {
+    int windows, pieces;
+    const int32_t *window, *first;           // [windows]: see WindowLists
+    int32_t* cut_at;                         // [pieces + windows][WH]: where the rows are cut, counted from their starts
+    int32_t* cut_col;                        // [pieces + windows]: and the column
+    int32_t* found;                          // [pieces]: distinct columns, then those in the pieces of the window before
+    // the window that piece q belongs to (its place in the lists); its cuts are cut q + its place and the one behind
+    __device__ __forceinline__ int of_piece(int q) const {
+        int lo = 0, hi = windows - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (first[mid] <= q) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    }
+    __device__ __forceinline__ int of_cut(int g) const {
+        int lo = 0, hi = windows - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (first[mid] + mid <= g) lo = mid; else hi = mid - 1;
+        }
+        return lo;
+    }
+};
+
+// A warp per cut: cut i lies at a column before which there are from i * n / pieces to kPieceSlack entries more than that,
+// or, a column holding at most WH of them, at the smallest one with that many.  Found by bisection, which narrows every row's
+// part with the columns'; where the rows are cut is looked up in the whole rows, so that whatever they hold the cuts do
+// not go back as long as the columns do not (checked by the pieces).
+template <int WH>
+__global__ void __launch_bounds__(128) wcsr_cut_windows_kernel(const CondenseParams p, const LongWindows lw) {
+    constexpr int R = (WH + 31) / 32;        // rows of a lane
+    grid_trigger();
+    const int lane = threadIdx.x & 31;
+    const int g = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (g >= lw.pieces + lw.windows) return;
+    const int l = lw.of_cut(g), i = g - lw.first[l] - l;
+    const int64_t r0 = int64_t{lw.window[l]} * WH, n = p.row_ptr[min(r0 + WH, p.m)] - p.row_ptr[r0], pieces = pieces_of(n);
+    const int32_t* row[R];
+    int len[R], a[R], b[R], x[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const int64_t r = r0 + lane + 32 * j;
+        const bool mine = lane + 32 * j < WH && r < p.m;
+        const int64_t start = mine ? p.row_ptr[r] : 0;
+        row[j] = p.col_idx + start;
+        len[j] = mine ? static_cast<int>(p.row_ptr[r + 1] - start) : 0;
+        a[j] = 0;
+        b[j] = len[j];
+    }
+    auto before = [&](int j, int64_t c, int lo, int hi) {        // entries of the row in columns before c, known to be lo .. hi
+        while (lo < hi) {
+            const int mid = lo + ((hi - lo) >> 1);
+            if (row[j][mid] < c) lo = mid + 1; else hi = mid;
+        }
+        return lo;
+    };
+    int64_t col = i == 0 ? 0 : p.k;
+    if (i > 0 && i < pieces) {
+        const unsigned target = static_cast<unsigned>(n * i / pieces);
+        int64_t clo = 0;
+        while (col - clo > 1) {
+            const int64_t mid = (clo + col) >> 1;
+            unsigned sum = 0;
+#pragma unroll
+            for (int j = 0; j < R; ++j) sum += static_cast<unsigned>(x[j] = before(j, mid, a[j], b[j]));
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            if (sum >= target) {
+                col = mid;
+                if (sum < target + kPieceSlack) break;
+            } else {
+                clo = mid;
+            }
+#pragma unroll
+            for (int j = 0; j < R; ++j) (sum >= target ? b[j] : a[j]) = x[j];
+        }
+    }
+    if (lane == 0) lw.cut_col[g] = static_cast<int32_t>(col);
+#pragma unroll
+    for (int j = 0; j < R; ++j)
+        if (lane + 32 * j < WH) lw.cut_at[int64_t{g} * WH + lane + 32 * j] = i == 0 ? 0 : (i == pieces ? len[j] : before(j, col, 0, len[j]));
+}
+
+// One CTA per piece: by bitmap where its columns fit one, merged otherwise.
+constexpr int kPieceSmem = kPieceCap * 12, kPieceWords = kPieceSmem / 8;
+template <int WH>
+__global__ void __launch_bounds__(kBitmapThreads) wcsr_pieces_kernel(const CondenseParams p, const LongWindows lw) {
+    extern __shared__ int32_t dyn[];
+    __shared__ int off[WH + 1];
+    __shared__ int64_t base[WH], start[WH];
+    __shared__ bool bad;
+    grid_trigger();
+    grid_wait();                             // the cuts
+    const int q = blockIdx.x, l = lw.of_piece(q), g = q + l;
+    const int64_t w = lw.window[l];
+    const int32_t *lo = lw.cut_at + int64_t{g} * WH, *hi = lo + WH;
+    for (int r = threadIdx.x; r < WH; r += kBitmapThreads) {
+        start[r] = p.row_ptr[min(w * WH + r, p.m)];
+        base[r] = start[r] + lo[r];
+        off[r + 1] = hi[r] - lo[r];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int64_t n = 0;
+        bad = false;
+        off[0] = 0;
+        for (int r = 0; r < WH; ++r) {
+            base[r] -= n;
+            n += off[r + 1];
+            // (only rows that do not ascend, or hold columns the matrix does not have)
+            if (off[r + 1] < 0 || n > kPieceCap) { bad = true; break; }
+            off[r + 1] = static_cast<int>(n);
+        }
+        if (bad) {
+            *p.bad = 1;
+            lw.found[q] = 0;
+        }
+    }
+    __syncthreads();
+    if (bad) return;
+    const int n = off[WH];
+    const int64_t begin = lw.cut_col[g], end = lw.cut_col[g + 1];
+    const WindowPiece e = {base, start};
+    if (end - begin <= int64_t{32} * kPieceWords) bitmap_window<WH>(p, w, e, n, off, reinterpret_cast<uint32_t*>(dyn), kPieceWords, begin, end, lw.found + q);
+    else merge_window<WH, kBitmapThreads>(p, w, e, n, off, dyn, kPieceCap, reinterpret_cast<uint32_t*>(dyn + 2 * kPieceCap), lw.found + q);
+}
+
+// One CTA per window: its distinct columns, and in found those of the pieces before each.
+__global__ void __launch_bounds__(1024) wcsr_piece_sums_kernel(const CondenseParams p, const LongWindows lw) {
+    __shared__ long long scratch[32];
+    const int q1 = blockIdx.x + 1 < lw.windows ? lw.first[blockIdx.x + 1] : lw.pieces;
+    long long carry = 0, total;
+    for (int q0 = lw.first[blockIdx.x]; q0 < q1; q0 += 1024) {
+        const int q = q0 + threadIdx.x;
+        const long long before = block_exclusive_sum(q < q1 ? lw.found[q] : 0, scratch, &total);
+        if (q < q1) lw.found[q] = static_cast<int32_t>(carry + before);
+        carry += total;
+    }
+    if (threadIdx.x == 0) p.ucount[lw.window[blockIdx.x]] = static_cast<int32_t>(carry);
+}
+
+// One CTA per piece, a warp per row: places in the piece become places in the window.
+template <int WH>
+__global__ void __launch_bounds__(256) wcsr_piece_places_kernel(const CondenseParams p, const LongWindows lw) {
+    const int q = blockIdx.x, l = lw.of_piece(q), lane = threadIdx.x & 31;
+    const int32_t first = lw.found[q];
+    if (first == 0) return;
+    const int32_t *lo = lw.cut_at + int64_t{q + l} * WH, *hi = lo + WH;
+    for (int r = threadIdx.x >> 5; r < WH; r += 8) {
+        const int64_t start = p.row_ptr[min(int64_t{lw.window[l]} * WH + r, p.m)];
+        for (int64_t j = lo[r] + lane; j < hi[r]; j += 32) p.pos_of[start + j] += first;
+    }
 }
 
 // CTA 0: window_row_ptr; the others: how many columns are referenced at all
@@ -926,10 +1129,17 @@ cudaError_t expand_wcsr_fills(int64_t n_items, const void* d_tasks, const int32_
 namespace {
 
 // Every window by its kernel.  The launches touch disjoint data and run side by side, each ending behind the one before
-// it (grid_wait); the first starts when the stream gets there.
+// it (grid_wait); the first starts when the stream gets there.  What follows from the pieces' counts comes behind them all.
 template <int WH>
-bool condense(CondenseParams p, const WindowLists& lists, const int* count, cudaStream_t st) {
-    bool first = true;
+bool condense(CondenseParams p, const WindowLists& lists, const int* count, const LongWindows& lw, cudaStream_t st) {
+    const unsigned pieces = static_cast<unsigned>(lw.pieces);
+    if (lw.windows > 0) {
+        wcsr_cut_windows_kernel<WH><<<(pieces + static_cast<unsigned>(lw.windows) + 3) / 4, 128, 0, st>>>(p, lw);
+        if (cudaGetLastError() != cudaSuccess) return false;
+        if (cudaFuncSetAttribute(wcsr_pieces_kernel<WH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPieceSmem) != cudaSuccess) return false;
+        if (launch_dependent(wcsr_pieces_kernel<WH>, dim3(pieces), kBitmapThreads, kPieceSmem, st, p, lw) != cudaSuccess) return false;
+    }
+    bool first = lw.windows == 0;
     auto launch = [&](auto kernel, int64_t grid, int threads, size_t smem, const auto&... args) {
         // (the most there may be: threads that build for other widths set it too)
         if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostBitmap) != cudaSuccess) return false;
@@ -942,11 +1152,16 @@ bool condense(CondenseParams p, const WindowLists& lists, const int* count, cuda
         p.list = lists.list[which];
         return count[which] == 0 || launch(kernel, count[which], threads, smem, args...);
     };
-    const int words = static_cast<int>(std::min<int64_t>((p.k + 31) / 32, kMostBitmap / 8));
+    const int words = static_cast<int>(std::min<int64_t>((p.k + 31) / 32, kBitmapColumns / 32));
     return list(kListBitmap, wcsr_bitmap_windows_kernel<WH>, kBitmapThreads, static_cast<size_t>(words) * 8, words) &&
            list(kListLarge, wcsr_merge_windows_kernel<WH, 1024>, 1024, size_t{kLargeWindow} * 12) &&
            list(kListMerge, wcsr_merge_windows_kernel<WH, 256>, 256, size_t{kMergeWindow} * 12) &&
-           launch(wcsr_sort_windows_kernel<WH>, (p.nwin + kSortWarps - 1) / kSortWarps, 32 * kSortWarps, 0);
+           launch(wcsr_sort_windows_kernel<WH>, (p.nwin + kSortWarps - 1) / kSortWarps, 32 * kSortWarps, 0) && [&]() {
+               if (lw.windows == 0) return true;
+               wcsr_piece_sums_kernel<<<static_cast<unsigned>(lw.windows), 1024, 0, st>>>(p, lw);
+               wcsr_piece_places_kernel<WH><<<pieces, 256, 0, st>>>(p, lw);
+               return cudaGetLastError() == cudaSuccess;
+           }();
 }
 
 }  // namespace
@@ -976,12 +1191,14 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
         int n_listed[kLists];                 // windows of the condensation kernels that go by lists
         int bad;                              // an entry out of range or not ascending
         int64_t nnz;
+        unsigned long long long_count;        // windows that are cut into pieces, and the pieces
         unsigned long long distinct;          // columns that are referenced
     } flags = {};
     Flags* d_flags = nullptr;
     int32_t* d_lists = nullptr;               // those windows
     uint8_t* d_work = nullptr;                // the entries' rows and places, window lengths, gather counts
-    auto release = [&]() { dev_free(d_flags, st); dev_free(d_lists, st); dev_free(d_work, st); };
+    int32_t* d_cuts = nullptr;                // LongWindows' arrays
+    auto release = [&]() { dev_free(d_flags, st); dev_free(d_lists, st); dev_free(d_work, st); dev_free(d_cuts, st); };
     auto fail = [&](int code) {
         cudaGetLastError();                  // (of a call that failed: not for a later check to find)
         release();
@@ -991,14 +1208,16 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     };
     auto alloc = [&](void** ptr, size_t bytes) { return dev_alloc(ptr, bytes, st) == cudaSuccess; };
 
-    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags)) || !alloc(reinterpret_cast<void**>(&d_lists), static_cast<size_t>(kLists * nwin + 1) * 4))
+    const int64_t max_long = std::min(nwin, kMostLong);
+    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags)) || !alloc(reinterpret_cast<void**>(&d_lists), static_cast<size_t>(kLists * nwin + 2 * max_long + 1) * 4))
         return fail(SPMM_ERR_ALLOC);
     if (cudaMemsetAsync(d_flags, 0, sizeof(Flags), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
     auto read_flags = [&]() {
         return cudaMemcpyAsync(&flags, d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
     };
     const unsigned check_grid = static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048));
-    const WindowLists lists = {wh, k, {d_lists, d_lists + nwin, d_lists + 2 * nwin}, d_flags->n_listed};
+    const WindowLists lists = {wh, k, {d_lists, d_lists + nwin, d_lists + 2 * nwin}, d_flags->n_listed,
+                               d_lists + kLists * nwin, d_lists + kLists * nwin + max_long, &d_flags->long_count, max_long};
     if (m > 0) csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, &d_flags->err, &d_flags->nnz, lists);
     if (!read_flags()) return fail(SPMM_ERR_CUDA);
     if (flags.err != 0) return fail(flags.err);
@@ -1033,7 +1252,19 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     const unsigned entry_grid = static_cast<unsigned>(std::min<int64_t>((nnz + 255) / 256, 16384));
     if (cudaMemsetAsync(cp.ucount, 0, work_bytes - o_ucount, st) != cudaSuccess) return fail(SPMM_ERR_CUDA);     // and the gather counts behind it
     if (nnz > 0 && k == 0) return fail(SPMM_ERR_OUT_OF_RANGE);
-    if (nnz > 0 && !(wh == 16 ? condense<16>(cp, lists, flags.n_listed, st) : condense<64>(cp, lists, flags.n_listed, st))) return fail(SPMM_ERR_CUDA);
+    LongWindows lw = {};
+    lw.windows = static_cast<int>(flags.long_count >> kLongShift);
+    lw.pieces = static_cast<int>(flags.long_count & ((1ull << kLongShift) - 1));
+    if (lw.windows > 0) {
+        const int64_t cuts = int64_t{lw.pieces} + lw.windows;
+        if (!alloc(reinterpret_cast<void**>(&d_cuts), static_cast<size_t>(cuts * (wh + 1) + lw.pieces) * 4)) return fail(SPMM_ERR_ALLOC);
+        lw.window = lists.long_window;
+        lw.first = lists.long_first;
+        lw.cut_at = d_cuts;
+        lw.cut_col = d_cuts + cuts * wh;
+        lw.found = lw.cut_col + cuts;
+    }
+    if (nnz > 0 && !(wh == 16 ? condense<16>(cp, lists, flags.n_listed, lw, st) : condense<64>(cp, lists, flags.n_listed, lw, st))) return fail(SPMM_ERR_CUDA);
     wcsr_row_ptr_kernel<<<1 + static_cast<unsigned>(std::min<int64_t>((k + 1023) / 1024, 128)), 1024, 0, st>>>(
         cp.ucount, nwin, b_col, *d_window_row_ptr, &d_flags->overflow, cp.refs, k, &d_flags->distinct);
     if (cudaMemcpyAsync(out->window_row_ptr.data(), *d_window_row_ptr, static_cast<size_t>(nwin + 1) * 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||

@@ -378,6 +378,114 @@ def test_bcsr_order_of_requests_changes_no_bit(lib, dtype, b, layout, c16):
     assert_close(got[0][:, cols], Cr, S, dtype, "order of requests b=%d" % b)
 
 
+def _long_window_rows(rng, kind, wh, k):
+    """Columns of the rows of four windows of more than 18,432 entries (the last one ragged, one from which on it is cut where a
+    bitmap holds all columns), and a short one between them."""
+    rows = []
+    for w in range(5):
+        n = (18433, 0, 60000, 49153, 49500)[w]
+        if w == 1:
+            rows += [rng.choice(k, 3, replace=False) for _ in range(wh)]
+        elif kind == "spread":
+            rows += [rng.choice(k, n // wh + (i < n % wh), replace=False) for i in range(wh)]
+        elif kind == "one row":
+            rows += [rng.choice(k, n, replace=False)] + [np.zeros(0, np.int64)] * (wh - 1)
+        elif kind == "same columns":
+            rows += [rng.permutation(rng.choice(k, -(-n // wh), replace=False))] * wh
+        elif kind == "two ends":                           # runs of neighbours at the first and the last columns
+            rows += [np.concatenate((np.arange(n // wh - 7), k - 1 - rng.choice(k // 2, 9, replace=False))) for _ in range(wh)]
+        else:                                              # powers: most entries among few columns
+            rows += [np.unique((k * rng.random(2 * n // wh) ** 6).astype(np.int64))[:n // wh + 40] for _ in range(wh)]
+    return [np.sort(np.asarray(r, np.int64)) for r in rows[:len(rows) - wh // 2]]
+
+
+@pytest.mark.parametrize("dtype,wh,k", [("fp16", 16, 70_000), ("tf32", 16, 3_000_000), ("bf16", 64, 70_000), ("fp8", 64, 40_000_000)])
+@pytest.mark.parametrize("kind", ["spread", "one row", "same columns", "two ends", "powers"])
+def test_wcsr_gpu_builder_long_windows(lib, kind, dtype, wh, k):
+    """Windows of more than 18,432 entries that a bitmap does not serve are cut into pieces by column: the same arrays as the host
+    builder's."""
+    import torch
+    rows = _long_window_rows(np.random.default_rng(wh + k), kind, wh, k)
+    m = len(rows)
+    rp = np.concatenate(([0], np.cumsum([r.size for r in rows]))).astype(np.int64)
+    ci = np.concatenate(rows).astype(np.int32)
+    vals = wl.to_storage(np.random.default_rng(1).uniform(-1, 1, ci.size), dtype)
+    d = [torch.from_numpy(rp).cuda(), torch.from_numpy(ci).cuda(), to_device(vals)]
+    h = lib.spmm_wcsr_create_csr_device(m, k, *[x.data_ptr() for x in d], dtype, wh)
+    h0 = lib.spmm_wcsr_create_csr(m, k, rp, ci, vals, dtype, wh)
+    try:
+        bits = {4: np.uint32, 2: np.uint16, 1: np.uint8}[wl.elem_size(dtype)]
+        for which, t in ((lib.X_WCSR_WINDOW_ROW_PTR, np.int32), (lib.X_WCSR_WINDOW_COL_IDX, np.int32), (lib.X_WCSR_VALUES, bits),
+                         (lib.X_WCSR_GROUP_CLASS, np.uint8), (lib.X_WCSR_TASKS, np.int32)):
+            assert np.array_equal(lib.spmm_export(h, which, t), lib.spmm_export(h0, which, t)), which
+        assert lib.spmm_get_info(h, 64) == lib.spmm_get_info(h0, 64)
+    finally:
+        lib.spmm_destroy(h)
+        lib.spmm_destroy(h0)
+
+
+@pytest.mark.parametrize("wh,k", [(16, 100_000), (64, 20_000_000)])
+def test_wcsr_gpu_builder_refuses_bad_entries_of_long_windows(lib, wh, k):
+    """Columns out of range, doubled, or out of order anywhere in a window that is cut into pieces: the status of the host's check
+    (the cuts are looked up in the rows before anything is known of their order)."""
+    import torch
+    rng = np.random.default_rng(5)
+    rows = _long_window_rows(rng, "spread", wh, k)
+    m = len(rows)
+    rp = np.concatenate(([0], np.cumsum([r.size for r in rows]))).astype(np.int64)
+    good = np.concatenate(rows).astype(np.int32)
+    zeros = np.zeros(good.size, np.float16)
+    first, last = int(rp[2 * wh]), int(rp[2 * wh + 1]) - 1           # a row of the window of 60,000 entries
+
+    def put(at, value):
+        c = good.copy()
+        c[at] = value
+        return c
+
+    def shuffled(a, b):
+        c = good.copy()
+        c[a:b] = rng.permutation(c[a:b])
+        return c
+
+    bad = [put(first, -1), put(last, k), put(last, 2**31 - 1), put(first + 9, good[first + 8]), put((first + last) // 2, 0), put(last, good[first]),
+           put(first + 5, k - 1), shuffled(first, last + 1), shuffled(int(rp[2 * wh]), int(rp[3 * wh])), np.zeros_like(good), np.full_like(good, k), good[::-1].copy()]
+    for i, ci in enumerate(bad):
+        d = [torch.from_numpy(rp).cuda(), torch.from_numpy(np.ascontiguousarray(ci)).cuda(), to_device(zeros)]
+        codes = []
+        for create, args in ((lib.spmm_wcsr_create_csr_device, [x.data_ptr() for x in d]), (lib.spmm_wcsr_create_csr, [rp, ci, zeros])):
+            with pytest.raises(lib.SpmmError) as e:
+                create(m, k, *args, "fp16", wh)
+            codes.append(e.value.code)
+        assert codes[0] == codes[1] and codes[0] in (lib.SPMM_ERR_UNSORTED, lib.SPMM_ERR_OUT_OF_RANGE), (i, codes)
+
+
+def test_wcsr_gpu_builder_takes_long_windows_in_its_stride(lib):
+    """16 million entries in one window (16 full rows) cost no multiple of what they cost in 62,500 windows: 72 ms against 7
+    where one CTA condensed a whole window, half a millisecond where it is cut.  Three times as much is allowed; medians of five, in turn."""
+    import time
+    import torch
+    k = 1_000_000
+    mats = []
+    for m, n in ((16, k), (k, 16)):
+        rp = torch.arange(m + 1, dtype=torch.int64, device="cuda") * n
+        ci = (torch.arange(n, device="cuda") * (k // n)).to(torch.int32).repeat(m)
+        if m > 16:                                         # (a window's rows do not share their columns)
+            ci += (torch.arange(m, device="cuda", dtype=torch.int32) % (k // n)).repeat_interleave(n)
+        mats.append((m, rp, ci, torch.ones(m * n, dtype=torch.float16, device="cuda")))
+    took = [[], []]
+    for rep in range(6):
+        for i, (m, rp, ci, va) in enumerate(mats):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            h = lib.spmm_wcsr_create_csr_device(m, k, rp.data_ptr(), ci.data_ptr(), va.data_ptr(), "fp16", 16)
+            took[i].append(time.perf_counter() - t0)
+            if rep == 0 and i == 0:
+                assert lib.spmm_get_info(h, 64)["n_units"] == k
+            lib.spmm_destroy(h)
+    long_windows, short_windows = (sorted(t[1:])[2] for t in took)
+    assert long_windows < 3 * short_windows, (long_windows, short_windows)
+
+
 @pytest.mark.parametrize("dtype", ["tf32", "fp16", "fp8"])
 def test_bcsr_gpu_builder_with_many_block_columns(lib, dtype):
     """More than 196,608 block columns: the builder's bitmap takes more than 48 KB of shared memory."""
