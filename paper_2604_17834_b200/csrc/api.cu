@@ -128,8 +128,8 @@ struct spmm_handle_s {
     int32_t* d_scta_ptr = nullptr;
     CUtensorMap tmAs;                // map of d_svals
     int stack_groups = 0;            // token groups of the stacked launch's tile (2, or 1: see ensure_schedule)
-    // launches by half tiles (see ensure_schedule), and their maps: boxes of 64 rows of stacked blocks, of 64 tokens of X, of
-    // 16 tokens of C or Y
+    // launches by half tiles (see ensure_schedule; a function of the handle and N), and their maps: boxes of 64 rows of stacked
+    // blocks, and, where split, of 64 tokens of X and of 16 tokens of C or Y
     bool split = false, stack_split = false;
     CUtensorMap tmAsh, tmBh, tmCh;
     CUtensorMap tmB3s;               // whole-tile map of B for the stacked launch's token tile
@@ -637,7 +637,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
         const CUtensorMapSwizzle swz = row_bytes == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                                       : (row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
         rc = encode_2d(&h->tmB, h->dtype, B, static_cast<uint64_t>(N), static_cast<uint64_t>(h->k), 128, bw, swz);
-        if (!rc) rc = encode_2d(&h->tmBh, h->dtype, B, static_cast<uint64_t>(N), static_cast<uint64_t>(h->k), 64, bw, swz);
+        if (!rc && h->split) rc = encode_2d(&h->tmBh, h->dtype, B, static_cast<uint64_t>(N), static_cast<uint64_t>(h->k), 64, bw, swz);
         EncodeTiledFn fn = get_encode_fn();
         auto whole_tile_map = [&](int g, CUtensorMap* out, bool* ok) {
             *ok = false;
@@ -719,7 +719,7 @@ int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     };
     CUresult r = encode(&h->tmC, 32);
-    if (r == CUDA_SUCCESS) r = encode(&h->tmCh, 16);
+    if (r == CUDA_SUCCESS && h->split) r = encode(&h->tmCh, 16);
     if (r != CUDA_SUCCESS) return cuda_error();
     h->tmC_ptr = C;
     h->tmC_N = N;
