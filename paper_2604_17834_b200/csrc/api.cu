@@ -694,10 +694,7 @@ int ensure_tmB(spmm_handle_s* h, const void* B, int64_t N, int groups) {
 // Store map of C for the BCSR epilogue (shared-memory staging tile -> TMA store).
 int ensure_tmC(spmm_handle_s* h, void* C, int64_t N) {
     if (h->tmC_ptr == C && h->tmC_N == N) return SPMM_OK;
-    if (h->col_major && h->c16) {            // stored without a map; the kernel is given a valid one all the same
-        h->tmC = h->tmCh = h->tmB;
-        return SPMM_OK;
-    }
+    if (h->col_major && h->c16) return SPMM_OK;          // stored without a map
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return cuda_error();
     const uint32_t w = static_cast<uint32_t>(bcsr_epi_cols(h->bcsr.b, h->c16, h->col_major));
@@ -1042,12 +1039,14 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.k = h->k;
     p.overlap = 0;
     p.tiles_first = bcsr_tiles_first(h, h->sched.groups) ? 1 : 0;
-    CUtensorMap tmA = h->sched.groups <= 1 ? h->tmA1 : h->tmA, tmA0 = h->tmA;
+    BcsrMaps tm;
+    tm.A = h->sched.groups <= 1 ? h->tmA1 : h->tmA;
+    tm.A0 = h->tmA;
     if (!h->tmA_ok) {
         // no stored block at all: the kernel never touches A, any valid map will do
-        rc = encode_2d(&tmA, h->dtype, h->d_vals, 8, 8, 8, 8, CU_TENSOR_MAP_SWIZZLE_NONE);
+        rc = encode_2d(&tm.A, h->dtype, h->d_vals, 8, 8, 8, 8, CU_TENSOR_MAP_SWIZZLE_NONE);
         if (rc) return rc;
-        tmA0 = tmA;
+        tm.A0 = tm.A;
     }
     rc = ensure_tmB(h, B, N, h->sched.groups);
     if (rc) return rc;
@@ -1070,25 +1069,26 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
         ps.overlap = 1;
         p.overlap = 2;
         const int n_tiles = static_cast<int>(h->sched_stack.tiles.size() / 2);
-        cudaError_t es = h->stack_split ? launch_bcsr_stacked(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, h->tmAsh, h->tmAsh, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
-                                                             n_tiles, stream)
-                                       : launch_bcsr_stacked(h->dtype, f.b, h->stack_groups, h->c16, h->col_major, h->tmAs, h->tmAs, h->tmB, h->tmB3s, h->tmC, h->tmC, ps,
-                                                             h->n_ctas, stream);
+        const BcsrMaps ts = {h->stack_split ? h->tmAsh : h->tmAs, {}, h->tmB, h->tmB3s, h->tmC, {}};
+        cudaError_t es = launch_bcsr_stacked(h->dtype, f.b, h->stack_split ? kSplitGroups : h->stack_groups, h->c16, h->col_major, ts, ps,
+                                             h->stack_split ? n_tiles : h->n_ctas, stream);
         if (es != cudaSuccess) return cuda_error();
         if (h->sched.tiles.empty()) return SPMM_OK;
     }
     // dynamic: one CTA per tile, the schedule was built as a single list in the global order
     const int grid = h->dynamic ? static_cast<int>(h->sched.tiles.size() / 2) : h->n_ctas;
     if (grid <= 0) return SPMM_OK;
+    tm.B = h->split ? h->tmBh : h->tmB;
+    tm.B3 = h->tmB3;
+    tm.C = h->split ? h->tmCh : h->tmC;
     if (h->split) {
-        const cudaError_t eh = launch_bcsr(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, 0, tmA, tmA0, h->tmBh, h->tmB3, h->tmCh, h->tmCh, p,
-                                           static_cast<int>(h->sched.tiles.size() / 2), stream);
+        const cudaError_t eh = launch_bcsr(h->dtype, f.b, kSplitGroups, h->c16, h->col_major, 0, tm, p, static_cast<int>(h->sched.tiles.size() / 2), stream);
         return eh == cudaSuccess ? SPMM_OK : cuda_error();
     }
     const bool ksplit = h->sched.n_slots > 0 && h->tmP_ok;
     if (ksplit) p.overlap = 1;          // the merge kernel's CTAs may be placed while this grid runs
-    cudaError_t e = launch_bcsr(h->dtype, f.b, h->sched.groups, h->c16, h->col_major, h->dynamic, tmA, tmA0, h->tmB, h->tmB3,
-                                h->tmC, ksplit ? h->tmP : h->tmC, p, grid, stream);
+    tm.P = ksplit ? h->tmP : h->tmC;
+    cudaError_t e = launch_bcsr(h->dtype, f.b, h->sched.groups, h->c16, h->col_major, h->dynamic, tm, p, grid, stream);
     if (e != cudaSuccess) return cuda_error();
     if (ksplit) {
         BcsrMergeParams mp;

@@ -27,7 +27,7 @@
 // uses the 128-byte swizzle with 32-byte atoms, and blocks wider than 32 columns pass through the
 // ring in 32-column slices), E4M3 (K = 32): a K step is 32 bytes of an operand row in all of them.
 // A tile of one part of a K-split block-row (record x < 0) stores an fp32 partial tile through
-// tmP instead of C; bcsr_merge_kernel adds the parts in order.
+// map P instead of C; bcsr_merge_kernel adds the parts in order.
 // Optional variants, all template parameters:
 //   CT = 1   C is written in the input's 16-bit type instead of fp32.
 //   CM = 1   "column-major" operands (the layout of the paper's BCSR kernel, Sec. 3.2, and of a
@@ -92,7 +92,7 @@ struct BcsrCfg {
     // Halves of stacked rows, whose MMAs are half as long, have twice the blocks as well: 3000 x
     // 16000, b = 16, 10 % full rows, bf16, N = 256 75.3 -> 67.8, 600 x 6000 TF32, N = 200 44.0 ->
     // 41.1 (whole stacked blocks, three stages of 64 KB for six of 32: 49.0 -> 50.5 on 6000 x 5000).
-    // A stage that is at most half full asks for half of the A blocks (tmA0): kFew.
+    // A stage that is at most half full asks for half of the A blocks (map A0): kFew.
     static constexpr int kBps = H == B ? bcsr_blocks_per_stage(B, ES, GROUPS) : bcsr_stacked_per_stage(B, ES) * (SPLIT ? 2 : 1);
     static constexpr int kFew = H == B ? bcsr_blocks_per_stage(B, ES, 2) : kBps;
     static constexpr int kStageBytes = ((kBps * (kDenseBytes + kABytes) + 1023) / 1024) * 1024;
@@ -185,16 +185,37 @@ __device__ __noinline__ float plain_product(const int32_t* block_row_ptr, const 
     return s;
 }
 
+// The maps that a kernel reads: a launch's parameters are copied for every call (three to five maps in
+// place of six, host time of a call, 512 x 512, N = 256: row-major 3.76 -> 3.70 us, column-major 3.73 -> 3.63, 16-bit result 3.58).
+struct BcsrOperandMaps { CUtensorMap A, B, B3; };
+template <bool HAS> struct BcsrMapA0 {};
+template <> struct BcsrMapA0<true> { CUtensorMap A0; };
+template <bool HAS> struct BcsrMapC {};
+template <> struct BcsrMapC<true> { CUtensorMap C; };
+template <bool HAS> struct BcsrMapP {};
+template <> struct BcsrMapP<true> { CUtensorMap P; };
+template <int BS, int H, int GROUPS, int FMT, int CT, int CM, int DYN, int SPLIT, int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2)>
+struct BcsrKernelMaps : BcsrOperandMaps,
+                        BcsrMapA0<H == BS && (bcsr_blocks_per_stage(BS, ES, 2) < bcsr_blocks_per_stage(BS, ES, GROUPS))>,
+                        BcsrMapC<!(CM && CT)>,
+                        BcsrMapP<H == BS && !CT && !CM && !DYN && !SPLIT> {
+    static constexpr bool kParts = H == BS && !CT && !CM && !DYN && !SPLIT;     // K-split: static schedule, fp32, row-major
+    explicit BcsrKernelMaps(const BcsrMaps& m) : BcsrOperandMaps{m.A, m.B, m.B3} {
+        if constexpr (std::is_base_of_v<BcsrMapA0<true>, BcsrKernelMaps>) this->A0 = m.A0;
+        if constexpr (std::is_base_of_v<BcsrMapC<true>, BcsrKernelMaps>) this->C = m.C;
+        if constexpr (kParts) this->P = m.P;
+    }
+};
+
 template <int B, int H, int GROUPS, int STAGES, int FMT, int CT, int CM, int DYN, int SPLIT>
 __global__ void __launch_bounds__((BcsrProducers<B, GROUPS, STAGES, FMT == 3 ? 1 : (FMT == 2 ? 4 : 2), DYN>::kThreads), 1)
-bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB,
-                 const __grid_constant__ CUtensorMap tmB3, const __grid_constant__ CUtensorMap tmC,
-                 const __grid_constant__ CUtensorMap tmP, const BcsrParams p) {
+bcsr_spmm_kernel(const __grid_constant__ BcsrKernelMaps<B, H, GROUPS, FMT, CT, CM, DYN, SPLIT> tm, const BcsrParams p) {
     constexpr int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2);
     static_assert(FMT != 2 || (!CT && !DYN && (H == B || B <= 32)), "TF32: fp32 C, static schedule, row groups of rows up to 128 bytes");
     static_assert(H == B || !DYN, "stacked blocks: static schedule only");
     using CElem = typename CType<FMT, CT>::type;
     using Cfg = BcsrCfg<B, H, GROUPS, STAGES, ES, static_cast<int>(sizeof(CElem)), CM, SPLIT>;
+    using Maps = BcsrKernelMaps<B, H, GROUPS, FMT, CT, CM, DYN, SPLIT>;
     static_assert(!SPLIT || !DYN, "half tiles: static schedule only");
     extern __shared__ uint8_t smem_raw[];
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -228,12 +249,12 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
         }
         *abort_flag = 0;
         fence_mbar_init();
-        prefetch_tmap(&tmA);
-        if (Cfg::kFew < Cfg::kBps) prefetch_tmap(&tmA0);
-        prefetch_tmap(&tmB);
-        prefetch_tmap(&tmB3);
-        prefetch_tmap(&tmC);
-        prefetch_tmap(&tmP);
+        prefetch_tmap(&tm.A);
+        if constexpr (Cfg::kFew < Cfg::kBps) prefetch_tmap(&tm.A0);
+        prefetch_tmap(&tm.B);
+        prefetch_tmap(&tm.B3);
+        if constexpr (!Cfg::kDirect) prefetch_tmap(&tm.C);
+        if constexpr (Maps::kParts) prefetch_tmap(&tm.P);
     }
     if (warp == 1) {
         tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_slot)), Cfg::kTmemCols);
@@ -343,13 +364,15 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                 const uint32_t sb = smem_base + s * Cfg::kStageBytes;
                 if constexpr (H == B) {
                     if (lane == 8) {
-                        tma_load_2d_hint(sb + Cfg::kAOff, few_blocks(nb) ? &tmA0 : &tmA, full_bar(s), kx, q * B, keep);
+                        const CUtensorMap* blocks = &tm.A;
+                        if constexpr (Cfg::kFew < Cfg::kBps) blocks = few_blocks(nb) ? &tm.A0 : &tm.A;
+                        tma_load_2d_hint(sb + Cfg::kAOff, blocks, full_bar(s), kx, q * B, keep);
                     } else if (Cfg::kBB > 128 && lane == 9) {
-                        tma_load_2d_hint(sb + Cfg::kAOff + B * 128, &tmA, full_bar(s), 128 / ES, q * B, keep);
+                        tma_load_2d_hint(sb + Cfg::kAOff + B * 128, &tm.A, full_bar(s), 128 / ES, q * B, keep);
                     }
                 } else {
                     if (lane >= 8 && lane < 8 + nb)
-                        tma_load_2d_hint(sb + Cfg::kAOff + (lane - 8) * Cfg::kABytes, &tmA, full_bar(s), 0, (q + lane - 8) * H + half * (H - Cfg::kRows), keep);
+                        tma_load_2d_hint(sb + Cfg::kAOff + (lane - 8) * Cfg::kABytes, &tm.A, full_bar(s), 0, (q + lane - 8) * H + half * (H - Cfg::kRows), keep);
                 }
             };
             // The first tile's first units: their block columns and stored blocks belong to the handle and are
@@ -416,7 +439,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                             const int J = __shfl_sync(0xffffffffu, Jl, jq + (blk < nb ? blk : 0));
                             if (whole_tile) {
                                 if (blk < nb && hf < kHalves)
-                                    tma_load_3d_hint(sb + blk * Cfg::kDenseBytes + hf * (GROUPS * Cfg::kXGroupBytes), &tmB3,
+                                    tma_load_3d_hint(sb + blk * Cfg::kDenseBytes + hf * (GROUPS * Cfg::kXGroupBytes), &tm.B3,
                                                      full_bar(s), J * B + kx + hf * (128 / ES), 0, n0 >> 7, keep);
                             } else {
                                 // ragged tile, or half of one: one request per token group, rows >= N are zero filled
@@ -424,19 +447,19 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                                 for (int g = 0; g < ngrp; ++g)
                                     if (blk < nb && hf < kHalves)
                                         tma_load_2d_hint(sb + blk * Cfg::kDenseBytes + hf * (GROUPS * Cfg::kXGroupBytes) + g * Cfg::kXGroupBytes,
-                                                         &tmB, full_bar(s), J * B + kx + hf * (128 / ES), n0 + g * 128, keep);
+                                                         &tm.B, full_bar(s), J * B + kx + hf * (128 / ES), n0 + g * 128, keep);
                             }
                         } else
                         if (whole_tile) {
                             // all boxes of a unit with one request: B seen as [token box][k][128 bytes of
                             // tokens], box = kNBox x kKB x 128 bytes; lane i takes block i
                             const int J = __shfl_sync(0xffffffffu, Jl, jq + (lane < nb ? lane : 0));
-                            if (lane < nb) tma_load_3d_hint(sb + lane * Cfg::kDenseBytes, &tmB3, full_bar(s), 0, J * B + kx, n0 / Cfg::kTokBox, keep);
+                            if (lane < nb) tma_load_3d_hint(sb + lane * Cfg::kDenseBytes, &tm.B3, full_bar(s), 0, J * B + kx, n0 / Cfg::kTokBox, keep);
                         } else {
                             for (int i = 0; i < nb; ++i) {
                                 const int J = __shfl_sync(0xffffffffu, Jl, jq + i);
                                 if (lane < nbox)
-                                    tma_load_2d_hint(sb + i * Cfg::kDenseBytes + lane * Cfg::kBoxBytes, &tmB, full_bar(s),
+                                    tma_load_2d_hint(sb + i * Cfg::kDenseBytes + lane * Cfg::kBoxBytes, &tm.B, full_bar(s),
                                                      n0 + lane * Cfg::kTokBox, J * B + kx, keep);
                             }
                         }
@@ -552,9 +575,8 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
             tc_fence_after_sync();
             // K-split: a tile of one part of a long block-row (record x = -1 - slot) writes its fp32
             // partial tile, rows slot * b .. of the partial array, instead of C (fp32 row-major C only)
-            const bool part = tI < 0;
+            const bool part = Maps::kParts && tI < 0;
             const int64_t row0 = static_cast<int64_t>(part ? -1 - tI : tI) * B;
-            const CUtensorMap* tm_out = part ? &tmP : &tmC;
             constexpr int W = Cfg::kDirect ? (B < 64 ? B : 64) : Cfg::kEpiCols;     // accumulator columns at a time
             for (int g = 0; g < ngrp; ++g) {
                 const int nw = n0 + g * 128 + (Cfg::kHalfTok ? half * 64 : 0) + qd * Cfg::kWarpTok;          // first token of this warp
@@ -642,6 +664,8 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
+                        const CUtensorMap* tm_out = &tm.C;
+                        if constexpr (Maps::kParts) tm_out = part ? &tm.P : &tm.C;
                         // row-major: box = 32 tokens x W rows at (token, row); column-major: box =
                         // W columns x 32 tokens at (column, token).  Out-of-range parts are clipped.
                         if constexpr (!CM) tma_store_2d(tm_out, stg, nw, crow);
@@ -717,7 +741,7 @@ bcsr_spmm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // CAP = the deepest ring the shape is given; the ring actually used also leaves room for the
 // epilogue's staging tiles (bcsr_fit_stages).
 template <int B, int H, int GROUPS, int CAP, int FMT, int CT, int CM, int DYN, int SPLIT = 0>
-cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
+cudaError_t launch_one(const BcsrMaps& tm, const BcsrParams& p,
                        int grid, cudaStream_t stream) {
     constexpr int ES = FMT == 3 ? 1 : (FMT == 2 ? 4 : 2);
     constexpr int CS = static_cast<int>(sizeof(typename CType<FMT, CT>::type));
@@ -740,37 +764,37 @@ cudaError_t launch_one(const CUtensorMap& tmA, const CUtensorMap& tmA0, const CU
             attr_done[dev] = true;
         }
     }
+    const BcsrKernelMaps<B, H, GROUPS, FMT, CT, CM, DYN, SPLIT> maps(tm);
     if constexpr (DYN) {        // (its grid is a queue of CTAs that running ones cancel: launched when the stream gets there)
-        kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(tmA, tmA0, tmB, tmB3, tmC, tmP, p);
+        kfn<<<grid, kThreads, Cfg::kSmemBytes, stream>>>(maps, p);
         return cudaGetLastError();
     } else {
-        return launch_dependent(kfn, dim3(static_cast<unsigned>(SPLIT ? 2 * grid : grid)), kThreads, Cfg::kSmemBytes, stream, tmA, tmA0, tmB, tmB3, tmC, tmP, p);
+        return launch_dependent(kfn, dim3(static_cast<unsigned>(SPLIT ? 2 * grid : grid)), kThreads, Cfg::kSmemBytes, stream, maps, p);
     }
 }
 
 template <int FMT, int CT, int CM, int DYN>
-cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
-                         const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
+cudaError_t launch_shape(int b, int groups, const BcsrMaps& tm, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 161: return launch_one<16, 16, 1, 10, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 162: return launch_one<16, 16, 2, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 164: return launch_one<16, 16, 4, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 321: return launch_one<32, 32, 1, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 32, 2, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 324: return launch_one<32, 32, 4, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 641: return launch_one<64, 64, 1, 4, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 642: return launch_one<64, 64, 2, 5, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 644: return launch_one<64, 64, 4, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1281: return launch_one<128, 128, 1, 3, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1282: return launch_one<128, 128, 2, 2, FMT, CT, CM, DYN>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 161: return launch_one<16, 16, 1, 10, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 162: return launch_one<16, 16, 2, 5, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 164: return launch_one<16, 16, 4, 3, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 321: return launch_one<32, 32, 1, 5, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 322: return launch_one<32, 32, 2, 5, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 324: return launch_one<32, 32, 4, 3, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 641: return launch_one<64, 64, 1, 4, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 642: return launch_one<64, 64, 2, 5, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 644: return launch_one<64, 64, 4, 3, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 1281: return launch_one<128, 128, 1, 3, FMT, CT, CM, DYN>(tm, p, grid, stream);
+        case 1282: return launch_one<128, 128, 2, 2, FMT, CT, CM, DYN>(tm, p, grid, stream);
         default: break;
     }
     if constexpr (!DYN) {
         switch (b * 10 + groups) {
-            case 160: return launch_one<16, 16, 1, 16, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 320: return launch_one<32, 32, 1, 8, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 640: return launch_one<64, 64, 1, 5, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 1280: return launch_one<128, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 160: return launch_one<16, 16, 1, 16, FMT, CT, CM, 0, 1>(tm, p, grid, stream);
+            case 320: return launch_one<32, 32, 1, 8, FMT, CT, CM, 0, 1>(tm, p, grid, stream);
+            case 640: return launch_one<64, 64, 1, 5, FMT, CT, CM, 0, 1>(tm, p, grid, stream);
+            case 1280: return launch_one<128, 128, 1, 4, FMT, CT, CM, 0, 1>(tm, p, grid, stream);
             default: break;
         }
     }
@@ -779,57 +803,54 @@ cudaError_t launch_shape(int b, int groups, const CUtensorMap& tmA, const CUtens
 
 // Stacked blocks (row groups): 128 rows x b; token tile 256 and four stages of 48 KB, or 128 and six of 32 KB.
 template <int FMT, int CT, int CM>
-cudaError_t launch_stack_shape(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
-                               const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
+cudaError_t launch_stack_shape(int b, int groups, const BcsrMaps& tm, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 161: return launch_one<16, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 160: return launch_one<16, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 320: return launch_one<32, 128, 1, 4, FMT, CT, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 161: return launch_one<16, 128, 1, 6, FMT, CT, CM, 0>(tm, p, grid, stream);
+        case 162: return launch_one<16, 128, 2, 4, FMT, CT, CM, 0>(tm, p, grid, stream);
+        case 321: return launch_one<32, 128, 1, 6, FMT, CT, CM, 0>(tm, p, grid, stream);
+        case 322: return launch_one<32, 128, 2, 4, FMT, CT, CM, 0>(tm, p, grid, stream);
+        case 160: return launch_one<16, 128, 1, 4, FMT, CT, CM, 0, 1>(tm, p, grid, stream);
+        case 320: return launch_one<32, 128, 1, 4, FMT, CT, CM, 0, 1>(tm, p, grid, stream);
         default: break;
     }
     if constexpr (FMT != 2) {
-        if (b == 64 && groups == 1) return launch_one<64, 128, 1, 6, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        if (b == 64 && groups == 2) return launch_one<64, 128, 2, 4, FMT, CT, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        if (b == 64 && groups == 1) return launch_one<64, 128, 1, 6, FMT, CT, CM, 0>(tm, p, grid, stream);
+        if (b == 64 && groups == 2) return launch_one<64, 128, 2, 4, FMT, CT, CM, 0>(tm, p, grid, stream);
     }
     return cudaErrorInvalidValue;
 }
 
 template <int FMT>
-cudaError_t launch_stack_fmt(int b, int groups, int c16, int cm, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
-                             const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
+cudaError_t launch_stack_fmt(int b, int groups, int c16, int cm, const BcsrMaps& tm, const BcsrParams& p, int grid, cudaStream_t stream) {
     if constexpr (FMT != 2) {
-        if (c16) return cm ? launch_stack_shape<FMT, 1, 1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
-                           : launch_stack_shape<FMT, 1, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        if (c16) return cm ? launch_stack_shape<FMT, 1, 1>(b, groups, tm, p, grid, stream)
+                           : launch_stack_shape<FMT, 1, 0>(b, groups, tm, p, grid, stream);
     }
     if (c16) return cudaErrorInvalidValue;
-    return cm ? launch_stack_shape<FMT, 0, 1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
-              : launch_stack_shape<FMT, 0, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+    return cm ? launch_stack_shape<FMT, 0, 1>(b, groups, tm, p, grid, stream)
+              : launch_stack_shape<FMT, 0, 0>(b, groups, tm, p, grid, stream);
 }
 
 // E4M3 inputs: fp32 C, static schedule; b = 32, 64 or 128 (a block row must hold at least one
 // 32-element K step).  Stages are half the bytes of the 16-bit ones.
 template <int CM>
-cudaError_t launch_fp8(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
-                       const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
+cudaError_t launch_fp8(int b, int groups, const BcsrMaps& tm, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 321: return launch_one<32, 32, 1, 8, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 32, 2, 10, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 324: return launch_one<32, 32, 4, 6, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 641: return launch_one<64, 64, 1, 7, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 642: return launch_one<64, 64, 2, 10, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 644: return launch_one<64, 64, 4, 5, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1281: return launch_one<128, 128, 1, 6, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1282: return launch_one<128, 128, 2, 4, 3, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 321: return launch_one<32, 32, 1, 8, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 322: return launch_one<32, 32, 2, 10, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 324: return launch_one<32, 32, 4, 6, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 641: return launch_one<64, 64, 1, 7, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 642: return launch_one<64, 64, 2, 10, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 644: return launch_one<64, 64, 4, 5, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 1281: return launch_one<128, 128, 1, 6, 3, 0, CM, 0>(tm, p, grid, stream);
+        case 1282: return launch_one<128, 128, 2, 4, 3, 0, CM, 0>(tm, p, grid, stream);
         default: break;
     }
     if constexpr (CM) {
         switch (b * 10 + groups) {
-            case 320: return launch_one<32, 32, 1, 8, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 640: return launch_one<64, 64, 1, 8, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 1280: return launch_one<128, 128, 1, 8, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 320: return launch_one<32, 32, 1, 8, 3, 0, 1, 0, 1>(tm, p, grid, stream);
+            case 640: return launch_one<64, 64, 1, 8, 3, 0, 1, 0, 1>(tm, p, grid, stream);
+            case 1280: return launch_one<128, 128, 1, 8, 3, 0, 1, 0, 1>(tm, p, grid, stream);
             default: break;
         }
     }
@@ -838,35 +859,33 @@ cudaError_t launch_fp8(int b, int groups, const CUtensorMap& tmA, const CUtensor
 
 // TF32 (fp32 storage): fp32 C, static schedule; the deepest rings the stage sizes allow.
 template <int CM>
-cudaError_t launch_tf32(int b, int groups, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB, const CUtensorMap& tmB3,
-                        const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
+cudaError_t launch_tf32(int b, int groups, const BcsrMaps& tm, const BcsrParams& p, int grid, cudaStream_t stream) {
     switch (b * 10 + groups) {
-        case 161: return launch_one<16, 16, 1, 5, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 162: return launch_one<16, 16, 2, 3, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 321: return launch_one<32, 32, 1, 5, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 322: return launch_one<32, 32, 2, 3, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 641: return launch_one<64, 64, 1, 8, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 642: return launch_one<64, 64, 2, 5, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 644: return launch_one<64, 64, 4, 3, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1281: return launch_one<128, 128, 1, 6, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1282: return launch_one<128, 128, 2, 4, 2, 0, CM, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 160: return launch_one<16, 16, 1, 10, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 320: return launch_one<32, 32, 1, 8, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 640: return launch_one<64, 64, 1, 10, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-        case 1280: return launch_one<128, 128, 1, 8, 2, 0, CM, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        case 161: return launch_one<16, 16, 1, 5, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 162: return launch_one<16, 16, 2, 3, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 321: return launch_one<32, 32, 1, 5, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 322: return launch_one<32, 32, 2, 3, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 641: return launch_one<64, 64, 1, 8, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 642: return launch_one<64, 64, 2, 5, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 644: return launch_one<64, 64, 4, 3, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 1281: return launch_one<128, 128, 1, 6, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 1282: return launch_one<128, 128, 2, 4, 2, 0, CM, 0>(tm, p, grid, stream);
+        case 160: return launch_one<16, 16, 1, 10, 2, 0, CM, 0, 1>(tm, p, grid, stream);
+        case 320: return launch_one<32, 32, 1, 8, 2, 0, CM, 0, 1>(tm, p, grid, stream);
+        case 640: return launch_one<64, 64, 1, 10, 2, 0, CM, 0, 1>(tm, p, grid, stream);
+        case 1280: return launch_one<128, 128, 1, 8, 2, 0, CM, 0, 1>(tm, p, grid, stream);
         default: return cudaErrorInvalidValue;
     }
 }
 
 template <int FMT>
-cudaError_t launch_fmt(int b, int groups, int c16, int cm, int dyn, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB,
-                       const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid, cudaStream_t stream) {
+cudaError_t launch_fmt(int b, int groups, int c16, int cm, int dyn, const BcsrMaps& tm, const BcsrParams& p, int grid, cudaStream_t stream) {
     // dynamic scheduling is built for the default output (fp32, row-major) only
-    if (dyn) return (c16 || cm) ? cudaErrorInvalidValue : launch_shape<FMT, 0, 0, 1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-    if (cm) return c16 ? launch_shape<FMT, 1, 1, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
-                       : launch_shape<FMT, 0, 1, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-    return c16 ? launch_shape<FMT, 1, 0, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
-               : launch_shape<FMT, 0, 0, 0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+    if (dyn) return (c16 || cm) ? cudaErrorInvalidValue : launch_shape<FMT, 0, 0, 1>(b, groups, tm, p, grid, stream);
+    if (cm) return c16 ? launch_shape<FMT, 1, 1, 0>(b, groups, tm, p, grid, stream)
+                       : launch_shape<FMT, 0, 1, 0>(b, groups, tm, p, grid, stream);
+    return c16 ? launch_shape<FMT, 1, 0, 0>(b, groups, tm, p, grid, stream)
+               : launch_shape<FMT, 0, 0, 0>(b, groups, tm, p, grid, stream);
 }
 
 }  // namespace
@@ -883,38 +902,36 @@ int bcsr_token_groups_max(int dtype, int b, int c16, int col_major) {
     return (b == 64 && !c16 && !col_major) ? 2 : 4;
 }
 
-cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA, const CUtensorMap& tmA0,
-                        const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
+cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const BcsrMaps& tm, const BcsrParams& p,
                         int grid, cudaStream_t stream) {
-    if (dtype == 1) return launch_fmt<0>(b, groups, c16, col_major, dynamic, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
-    if (dtype == 0) return launch_fmt<1>(b, groups, c16, col_major, dynamic, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
+    if (dtype == 1) return launch_fmt<0>(b, groups, c16, col_major, dynamic, tm, p, grid, stream);   // fp16
+    if (dtype == 0) return launch_fmt<1>(b, groups, c16, col_major, dynamic, tm, p, grid, stream);   // bf16
     if (dtype == 3) {
         if (c16 || dynamic) return cudaErrorInvalidValue;
-        return col_major ? launch_fp8<1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
-                         : launch_fp8<0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        return col_major ? launch_fp8<1>(b, groups, tm, p, grid, stream)
+                         : launch_fp8<0>(b, groups, tm, p, grid, stream);
     }
     if (dtype == 2) {
         if (c16 || dynamic) return cudaErrorInvalidValue;
-        return col_major ? launch_tf32<1>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream)
-                         : launch_tf32<0>(b, groups, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+        return col_major ? launch_tf32<1>(b, groups, tm, p, grid, stream)
+                         : launch_tf32<0>(b, groups, tm, p, grid, stream);
     }
     return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB,
-                                const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p, int grid,
+cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const BcsrMaps& tm, const BcsrParams& p, int grid,
                                 cudaStream_t stream) {
-    if (dtype == 1) return launch_stack_fmt<0>(b, groups, c16, col_major, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // fp16
-    if (dtype == 0) return launch_stack_fmt<1>(b, groups, c16, col_major, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // bf16
-    if (dtype == 2) return launch_stack_fmt<2>(b, groups, c16, col_major, tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);   // TF32: b = 16, 32
+    if (dtype == 1) return launch_stack_fmt<0>(b, groups, c16, col_major, tm, p, grid, stream);   // fp16
+    if (dtype == 0) return launch_stack_fmt<1>(b, groups, c16, col_major, tm, p, grid, stream);   // bf16
+    if (dtype == 2) return launch_stack_fmt<2>(b, groups, c16, col_major, tm, p, grid, stream);   // TF32: b = 16, 32
     if (dtype == 3 && !c16 && col_major) {
         // E4M3: half the bytes per stage, deeper rings
         switch (b * 10 + groups) {
-            case 321: return launch_one<32, 128, 1, 10, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
-            case 320: return launch_one<32, 128, 1, 6, 3, 0, 1, 0, 1>(tmA, tmA0, tmB, tmB3, tmC, tmP, p, grid, stream);
+            case 321: return launch_one<32, 128, 1, 10, 3, 0, 1, 0>(tm, p, grid, stream);
+            case 322: return launch_one<32, 128, 2, 8, 3, 0, 1, 0>(tm, p, grid, stream);
+            case 641: return launch_one<64, 128, 1, 10, 3, 0, 1, 0>(tm, p, grid, stream);
+            case 642: return launch_one<64, 128, 2, 8, 3, 0, 1, 0>(tm, p, grid, stream);
+            case 320: return launch_one<32, 128, 1, 6, 3, 0, 1, 0, 1>(tm, p, grid, stream);
             default: break;
         }
     }

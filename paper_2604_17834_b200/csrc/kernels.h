@@ -58,34 +58,33 @@ struct BcsrParams {
 // operands, fp32 C).  groups: token tile = 128 * groups columns of B (1, 2 or 4).
 // c16: C in the input's 16-bit type.  With es = bytes per element, t = 128 / es tokens per
 // 128-byte box row and kb = b / bcsr_k_split(b, es) rows of B per stage unit --
-// row-major operands: tmB = B as [k][N], box kb x t; tmB3 = B as [N / t][k][t], box
+// row-major operands: map B = B as [k][N], box kb x t; B3 = B as [N / t][k][t], box
 // (es * groups) x kb x t; 128-byte swizzle (with 32-byte atoms for es = 4).  Column-major operands
-// (col_major): tmB = X as [N][k], box 128 tokens x min(kb * es, 128) bytes; tmB3 = X as
+// (col_major): B = X as [N][k], box 128 tokens x min(kb * es, 128) bytes; B3 = X as
 // [N / 128][128][k], box groups x 128 x the same; both with the swizzle of that row length.
-// tmA0: tmA as wider tiles have it, fewer blocks to a box (stacked blocks: not used).
-// tmA: the stored blocks as [blocks * b][b], box (b * bcsr_blocks_per_stage) rows x min(kb * es, 128) bytes.
-// tmC: C as [m][N], box 32 x bcsr_epi_cols, no swizzle; or fp32 Y as [N][m], box 16 x 32, 64-byte swizzle (16-bit Y:
-// any valid map, it is stored without one).
+// A: the stored blocks as [blocks * b][b], box (b * bcsr_blocks_per_stage) rows x min(kb * es, 128) bytes.
+// A0: A as wider tiles have it, fewer blocks to a box (read by 128-token tiles whose stages hold more).
+// C: C as [m][N], box 32 x bcsr_epi_cols, no swizzle; or fp32 Y as [N][m], box 16 x 32, 64-byte swizzle (16-bit Y: not
+// read, it is stored without a map).
+// P: K-split, the partial tiles as [slots * b][N] fp32, box as C's (the tile record of a part holds -1 - slot in place of the
+// block-row); C where the plan has no parts.
 // dynamic: the grid is one CTA per tile (grid = number of tiles, p.tiles in the schedule's global
 // order, p.cta_ptr unused) and CTAs steal tiles through Cluster Launch Control; fp32 row-major only.
-cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const CUtensorMap& tmA, const CUtensorMap& tmA0,
-                        const CUtensorMap& tmB, const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP,
-                        const BcsrParams& p, int grid, cudaStream_t stream);
+struct BcsrMaps { CUtensorMap A, A0, B, B3, C, P; };
+cudaError_t launch_bcsr(int dtype, int b, int groups, int c16, int col_major, int dynamic, const BcsrMaps& tm, const BcsrParams& p,
+                        int grid, cudaStream_t stream);
 // Row groups: the same kernel with 128 x b stacked blocks (MMA N = 128) and a 256-token tile (groups = 2), or a
 // 128-token one (groups = 1; see ensure_schedule).
-// tmA: the stacked values as [blocks * 128][b], box 128 x b; tmB3 built for `groups`; b = 16, 32, 64 (tf32: 16, 32).
+// A: the stacked values as [blocks * 128][b], box 128 x b; B3 built for `groups`; b = 16, 32, 64 (tf32: 16, 32).
 // `groups` of a launch by half tiles (both kinds of launch): the lists of a 128-token schedule, two CTAs to each, with 64 of
-// its tiles' tokens in either (tmC: boxes of 16 tokens instead of 32; column-major tmB: box of 64 tokens; E4M3: column-major
-// operands only) or, for stacked blocks of b = 16 and 32, 64 of their rows (tmA: box of 64 rows).
+// its tiles' tokens in either (C: boxes of 16 tokens instead of 32; column-major B: box of 64 tokens; E4M3: column-major
+// operands only) or, for stacked blocks of b = 16 and 32, 64 of their rows (A: box of 64 rows).
 constexpr int kSplitGroups = 0;
 constexpr int kStackRows = 128;
 constexpr int kStackGroups = 2;
-cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const CUtensorMap& tmA, const CUtensorMap& tmA0, const CUtensorMap& tmB,
-                                const CUtensorMap& tmB3, const CUtensorMap& tmC, const CUtensorMap& tmP, const BcsrParams& p,
+cudaError_t launch_bcsr_stacked(int dtype, int b, int groups, int c16, int col_major, const BcsrMaps& tm, const BcsrParams& p,
                                 int grid, cudaStream_t stream);
-// K-split: tmP = the partial tiles as [slots * b][N] fp32, box as tmC's (the tile record of a
-// part holds -1 - slot in place of the block-row); pass tmC where the plan has no parts.
-// The merge: C rows of every split block-row = sum of its parts' partial tiles in part order.
+// K-split, the merge: C rows of every split block-row = sum of its parts' partial tiles in part order.
 struct BcsrMergeParams {
     const int32_t* row;      // [n] split block-rows
     const int32_t* first;    // first slot
