@@ -865,6 +865,12 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
         return N > 64 && 2 * n_tiles <= h->n_ctas && longest * (128 + rows) * f.b * h->es >= kSplitMinBytes && !h->dynamic &&
                !(h->dtype == SPMM_FP8_E4M3 && !h->col_major);
     };
+    // Such a launch has two CTAs to each of the first lists, as many as there are tiles: they hold all of them (tiles are dealt to
+    // the least loaded CTA, the first of several), or it is none.
+    auto in_first_lists = [](const BcsrSchedule& s) {
+        const size_t n = s.tiles.size() / 2;
+        return n < s.cta_ptr.size() && static_cast<size_t>(s.cta_ptr[n]) == n;
+    };
     try {
         // dynamic scheduling: one list in the global order (slab by slab, longest block-row first)
         // b = 64 gains little per stacked block (its MMAs, not the operand traffic, bound it), so
@@ -890,7 +896,7 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
             } else if (!rc) {
                 rc = build_bcsr_schedule(f, n_tt, static_cast<int>(sw), h->dynamic ? 1 : h->n_ctas, &sc);
                 const int32_t I = f.nbr > 0 ? f.row_order[0] : 0;
-                split = !rc && groups == 1 && f.nbr > 0 && split_fits(f.nbr * n_tt, f.block_row_ptr[I + 1] - f.block_row_ptr[I], f.b);
+                split = !rc && groups == 1 && f.nbr > 0 && split_fits(f.nbr * n_tt, f.block_row_ptr[I + 1] - f.block_row_ptr[I], f.b) && in_first_lists(sc);
             }
         } else {
             // The row groups get a launch and a schedule of their own; the launch of the remaining
@@ -951,7 +957,8 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
                     // dealt for one CTA per tile, so that some of its lists start when the halves are done and count twice)
                     const int64_t n_tiles = static_cast<int64_t>(ks.tiles.size() / 2);
                     const int64_t whole = (most + kStackTileFixedCost) * bcsr_stack_block_cost(1);
-                    stack_split = !rc && split_fits(n_tiles, most, kStackRows) && (whole * 3 / 4 + 2 * rest / (h->n_ctas - n_tiles)) * 10 < whole * 9;
+                    stack_split = !rc && split_fits(n_tiles, most, kStackRows) && (whole * 3 / 4 + 2 * rest / (h->n_ctas - n_tiles)) * 10 < whole * 9 &&
+                                  in_first_lists(ks);
                     if (!rc) {
                         std::sort(loads.begin(), loads.end());
                         rc = build_tile_schedule(units, lens, kTileFixedCost, n_tt, static_cast<int>(sw), h->n_ctas, &kc,

@@ -96,9 +96,31 @@ def assert_close(C_gpu, C_ref, S, dtype, what=""):
     return float(np.max(err / bound))
 
 
-def captured_run(lib, h, B, C, N, relaxed=False, replay=False, static=False):
+def kernel_launch(cu, node):
+    """(CTAs, threads per CTA) of a kernel node of a captured graph."""
+    import ctypes
+
+    class Params(ctypes.Structure):                                          # CUDA_KERNEL_NODE_PARAMS (v2)
+        _fields_ = [("func", ctypes.c_void_p)] + [(x, ctypes.c_uint) for x in ("gx", "gy", "gz", "bx", "by", "bz", "shared")] + \
+                   [(x, ctypes.c_void_p) for x in ("params", "extra", "kern", "ctx")]
+
+    p = Params()
+    assert cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+    return p.gx * p.gy * p.gz, p.bx * p.by * p.bz
+
+
+def captured_launches(lib, h, B, C, N):
+    """(CTAs, threads per CTA) of every kernel that one spmm_run launches, in order; nothing runs."""
+    found = []
+    code, kinds = captured_run(lib, h, B, C, N, launches=found)
+    assert code == lib.SPMM_OK and len(found) == len(kinds), (code, kinds)
+    return found
+
+
+def captured_run(lib, h, B, C, N, relaxed=False, replay=False, static=False, launches=None):
     """One spmm_run (static: spmm_wcsr_run_static) inside a stream capture of its own stream.  -> (status code of the run, kinds of the captured
-    nodes, or None where the capture gave no graph).  replay: launch the graph once, unless the run was refused."""
+    nodes, or None where the capture gave no graph).  replay: launch the graph once, unless the run was refused.  launches: a list
+    that the kernel nodes' sizes are added to (the nodes of a graph of one stream come in its order)."""
     import ctypes
     import torch
     cu = ctypes.CDLL("libcuda.so.1")
@@ -121,6 +143,8 @@ def captured_run(lib, h, B, C, N, relaxed=False, replay=False, static=False):
         t = ctypes.c_int(-1)
         assert cu.cuGraphNodeGetType(ctypes.c_void_p(x), ctypes.byref(t)) == 0
         kinds.append("kernel" if t.value == 0 else "type %d" % t.value)      # CU_GRAPH_NODE_TYPE_KERNEL
+        if launches is not None and t.value == 0:
+            launches.append(kernel_launch(cu, x))
     if replay and code == lib.SPMM_OK:
         ex = ctypes.c_void_p()
         assert cu.cuGraphInstantiateWithFlags(ctypes.byref(ex), graph, ctypes.c_ulonglong(0)) == 0

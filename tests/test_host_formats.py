@@ -485,3 +485,35 @@ def test_bcsr_plan_of_a_few_long_row_groups_is_the_one_that_runs(lib, b, N):
         assert lib.spmm_export(h, lib.X_BCSR_STACK_TILES, np.int32).size // 2 == rows.shape[0] * -(-N // (128 if narrow else 256))
     finally:
         lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("b,N,n_ctas,density,skewed", [(16, 128, 148, 0.05, False), (32, 256, 148, 0.3, True), (64, 200, 20, 0.1, False),
+                                                       (64, 72, 148, 0.02, False), (128, 128, 9, 0.5, True), (16, 256, 148, 1.0, True)])
+def test_bcsr_few_tiles_lie_in_the_first_lists(lib, b, N, n_ctas, density, skewed):
+    """With no more tiles than CTAs, every tile is dealt to a list of its own and the first lists are the ones: a launch by half
+    tiles has two CTAs to each of them and none to the others.  Empty block-rows (tiles without blocks) included."""
+    rng = np.random.default_rng(b + N)
+    n_tt = -(-N // 128)
+    nbr, nbc = max(1, n_ctas // n_tt // 2), 24
+    mask = rng.random((nbr, nbc)) < density
+    mask[0] |= skewed
+    if density < 1 and nbr > 2:
+        mask[nbr // 2] = False
+    full = np.kron(mask, np.ones((b, b), bool))
+    rp = np.concatenate(([0], np.cumsum(full.sum(1)))).astype(np.int64)
+    ci = np.nonzero(full)[1].astype(np.int32)
+    h = lib.spmm_bcsr_create_csr(nbr * b, nbc * b, rp, ci, np.zeros(ci.size, np.float16), "fp16", b, host_only=True, n_ctas=n_ctas)
+    try:
+        lib.spmm_bcsr_plan(h, N)
+        assert lib.spmm_get_info(h, N)["plan_token_tile"] == 128
+        seen = 0
+        for ptr, tiles in ((lib.X_BCSR_TILE_PTR, lib.X_BCSR_TILES), (lib.X_BCSR_STACK_TILE_PTR, lib.X_BCSR_STACK_TILES)):
+            n = lib.spmm_export(h, tiles, np.int32).size // 2
+            if n == 0 or (ptr == lib.X_BCSR_TILE_PTR and seen == 0 and lib.spmm_export(h, lib.X_BCSR_STACK_TILES, np.int32).size):
+                continue                                   # (beside row groups the other block-rows start where those leave room)
+            seen += n
+            cta_ptr = lib.spmm_export(h, ptr, np.int32)
+            assert cta_ptr.size == n_ctas + 1 and np.array_equal(cta_ptr, np.minimum(np.arange(n_ctas + 1), n))
+        assert seen > 0
+    finally:
+        lib.spmm_destroy(h)
