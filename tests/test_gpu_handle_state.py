@@ -313,11 +313,17 @@ def test_waits_do_not_count_the_launch_before(lib):
         B = torch.ones((ks[0], N), dtype=torch.bfloat16, device="cuda")
         C = torch.zeros((2, m, N), dtype=torch.float32, device="cuda")
         st = torch.cuda.current_stream().cuda_stream
-        for limit in (2_000_000_000, 300_000, 300_000):            # (the first pass: kernels loaded, plans made)
-            for i in range(2):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        for limit in (2_000_000_000, 0, 300_000, 300_000):         # (the first pass: kernels loaded, plans made; the second: the long one alone)
+            for i in range(2 if limit else 1):
+                if not limit:
+                    ev[0].record()
                 lib.spmm_set_wait_limit_ns(limit if i else 2_000_000_000)
                 lib.spmm_run(hs[i], B.data_ptr(), C[i].data_ptr(), N, st)
+                if not limit:
+                    ev[1].record()
         torch.cuda.synchronize()
+        assert ev[0].elapsed_time(ev[1]) > 0.6                     # (twice the limit)
         for i in range(2):
             lib.spmm_check(hs[i])
             assert bool(torch.all(C[i] == ks[i]))

@@ -8,7 +8,7 @@ import pytest
 
 from paper_2604_17834_b200 import workloads as wl
 
-from helpers import assert_close, captured_run, reference, run_gpu, run_gpu_variant, to_device
+from helpers import assert_close, captured_launches, captured_run, reference, run_gpu, run_gpu_variant, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -313,8 +313,10 @@ def test_wcsr_gpu_builder_by_window_size(lib, dtype, wh, k):
     ("fp8", 32, 1.0, "col", False)])
 def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16):
     """Launches with at most half as many 128-token tiles as CTAs, each of 768 KB and more: two CTAs to a tile (halves of its
-    tokens for plain blocks, of the stacked blocks' rows for row groups).  The same bits as with one CTA per tile (a grid too
-    small for two), and the oracle's result; token counts around the halves of a tile, an empty block-row, ragged last rows."""
+    tokens for plain blocks, of the stacked blocks' rows for row groups; the launches' sizes show it).  The same bits as with
+    one CTA per tile (a grid too small for two), and the oracle's result; token counts around the halves of a tile, an empty
+    block-row, ragged last rows."""
+    import torch
     m = 328 if dens < 1 else 264
     need = (768 << 10) // ((128 + (b if dens < 1 else 128)) * b * wl.elem_size(dtype)) + 2       # blocks of the longest tile
     k = (need * b + 8) // 16 * 16
@@ -330,6 +332,9 @@ def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16)
     vals = wl.to_storage(rng.uniform(-1, 1, ci.size), dtype)
     a = {"m": m, "k": k, "row_ptr": rp, "col_idx": ci, "vals": vals}
     opt = dict(layout=lib.COLMAJOR if layout == "col" else lib.ROWMAJOR, c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
+    if dens < 1:
+        opt["stack_min_fill"] = -1                          # plain blocks
+    assert need * (128 + (b if dens < 1 else 128)) * b * wl.elem_size(dtype) >= 768 << 10
     for N in ((128, 129, 200, 321) if layout == "col" else (72, 96, 128, 136, 256)):
         h = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, **opt)
         h1 = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, n_ctas=3, **opt)
@@ -339,6 +344,12 @@ def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16)
             Cr, S = reference(a, Bs, dtype)
             assert_close(C, Cr, S, dtype, "half tiles b=%d N=%d" % (b, N))
             assert np.array_equal(C, C1), N
+            Bd, Cd = to_device(np.ascontiguousarray(Bs.T) if layout == "col" else Bs), torch.empty((m, N), dtype=torch.float32, device="cuda")
+            grouped = lib.spmm_export(h, lib.X_BCSR_STACK_TILES, np.int32).size // 2
+            assert (grouped > 0) == (dens == 1)
+            tiles = grouped or lib.spmm_export(h, lib.X_BCSR_TILES, np.int32).size // 2
+            assert captured_launches(lib, h, Bd, Cd, N)[0][0] == 2 * tiles, (N, tiles)
+            assert captured_launches(lib, h1, Bd, Cd, N)[0][0] == 3
         finally:
             lib.spmm_destroy(h)
             lib.spmm_destroy(h1)

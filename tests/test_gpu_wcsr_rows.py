@@ -7,7 +7,7 @@ import pytest
 
 from paper_2604_17834_b200 import workloads as wl
 
-from helpers import CANARY, GUARD, assert_close, captured_run, check_guards, reference, run_gpu_variant, to_device
+from helpers import CANARY, GUARD, assert_close, captured_launches, captured_run, check_guards, reference, run_gpu_variant, to_device
 
 pytestmark = pytest.mark.gpu
 
@@ -217,7 +217,8 @@ def test_static_run_takes_the_kernel_of_spmm_run(lib):
 @pytest.mark.parametrize("dtype,widths", [("tf32", (36, 64, 128, 320)), ("fp16", (72, 128, 320, 520))])
 def test_the_sums_do_not_depend_on_the_cta_size(lib, dtype, widths):
     """A small launch takes CTAs of 128 or 256 threads by the groups that its dense width leaves a warp (8 to 1 of them
-    here); a column's sums are those of the widest run, bit by bit."""
+    here; 256 with up to three, as the launches show); a column's sums are those of the widest run, bit by bit."""
+    import torch
     m, k = 3001, 20000
     a = _matrix(m, k, 16, dtype)
     Bs = wl.dense(64, k, widths[-1], ("uniform", -1.0, 1.0), dtype)
@@ -226,7 +227,11 @@ def test_the_sums_do_not_depend_on_the_cta_size(lib, dtype, widths):
         want = run_gpu_variant(lib, h, Bs, m, widths[-1], dtype)
         Cr, S = reference(a, Bs, dtype)
         assert_close(want, Cr, S, dtype, "rows N=%d" % widths[-1])
-        for N in (16,) + widths[:-1]:
-            assert np.array_equal(run_gpu_variant(lib, h, np.ascontiguousarray(Bs[:, :N]), m, N, dtype), want[:, :N]), N
+        for N in (16,) + widths:
+            B = np.ascontiguousarray(Bs[:, :N])
+            assert np.array_equal(run_gpu_variant(lib, h, B, m, N, dtype), want[:, :N]), N
+            launches = captured_launches(lib, h, to_device(B), torch.empty((m, N), dtype=torch.float32, device="cuda"), N)
+            groups = {16: 8 if dtype == "tf32" else 16, 36: 3, 64: 4, 72: 3, 128: 2 if dtype == "tf32" else 4, 320: 2 if dtype == "tf32" else 1, 520: 1}[N]
+            assert {t for _, t in launches} == {256 if groups < 4 else 128}, (N, launches)
     finally:
         lib.spmm_destroy(h)
