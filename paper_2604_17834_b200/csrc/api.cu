@@ -1005,20 +1005,23 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
 
 // Which request of a stage goes first, its stored blocks or its B tiles: the one that is longer on its way.  Many
 // block-rows share a token tile, which is then close by in L2, and the blocks go first; where few do, the tiles do.  The line, by
-// block-rows (148 CTAs), from the speed with the tiles first over that with the blocks first, geometric mean (and range) of
-// products of random sizes, 0.3 - 5 ms, N = 300 - 50,000, row-major:
-//   block-rows    under 10            10 - 20             20 - 30             30 - 50             60 - 100            100 - 200
-//   b = 128 TF32  1.016 (0.97 - 1.04) 1.011 (0.96 - 1.06) 1.008 (0.96 - 1.23) 1.003 (0.97 - 1.05) 0.983 (0.92 - 1.09) 0.951 (0.92 - 1.00)
-//           bf16  1.015 (0.92 - 1.05) 1.014 (0.95 - 1.07) 1.005 (0.93 - 1.11) 0.997 (0.87 - 1.10) 0.961 (0.89 - 1.02) 0.977 (0.91 - 1.02)
-//   b = 64  TF32  1.014 (1.00 - 1.02) 1.006 (0.98 - 1.04) 1.007 (0.98 - 1.02) 1.007 (0.98 - 1.06) 1.000 (0.96 - 1.07) 0.995 (0.95 - 1.06), under 16 blocks a row
-//           bf16  1.007 (1.00 - 1.03) 1.006 (0.99 - 1.03) 1.002 (0.94 - 1.04) 0.998 (0.98 - 1.04) 0.996 (0.94 - 1.02) 0.99  (0.96 - 1.02)
-// b <= 32 (and stacked blocks) do not gain on either side.  TF32 at b = 64 has the longest B tiles beside its blocks (32 KB to
-// 8): long tiles, 32 blocks a row and more, gain at any number of block-rows, 1.009 (0.96 - 1.08); not in decode steps (0.97
-// - 0.99 with N under 200).
+// block-rows (148 CTAs), from the speed with the tiles first over that with the blocks first, geometric means over products
+// of random sizes, row-major, N = 300 - 50,000 (single ones are within 0.94 and 1.06, and so are two runs of one with
+// other buffers, now and then):
+//   block-rows    under 10   10 - 20   20 - 30   30 - 50   60 - 100   100 - 200
+//   b = 128 TF32  1.016      1.011     1.008     1.003     0.983      0.951
+//           bf16  1.015      1.014     1.005     0.997     0.961      0.977
+//   b = 64  TF32  1.014      1.006     1.007     1.007     1.000      0.995, under 16 blocks a row
+//           bf16  1.007      1.006     1.002     0.998     0.996      0.99
+// b <= 32 and stacked blocks do not gain on either side, nor do short stages (b = 64 in tiles of 128 tokens).  TF32 at b = 64
+// has the longest B tiles beside its blocks (32 KB to 8): long tiles, 32 blocks a row and more, gain at any number of
+// block-rows.  us, blocks first and tiles first: 8192 x 8192, b = 64, density 0.4, TF32, N = 16,384 2225 and 2134; 5000 x 7000,
+// 10 % full rows, N = 16,384 947 and 927; 1819 x 5601, b = 128, 10 % full rows, N = 9288 105.1 and 103.2; 3584 x 18944, b = 128,
+// bf16, N = 2048 87.5 and 82.3.
 bool bcsr_tiles_first(const spmm_handle_s* h, int groups) {
     const BcsrHost& f = h->bcsr;
-    if (f.b < 64) return false;
-    if (h->es == 4 && f.b == 64 && groups > 1) return 3 * f.nbr < h->n_ctas || f.nnzb >= 32 * f.nbr;
+    if (f.b < 64 || (f.b == 64 && groups == 1)) return false;
+    if (h->es == 4 && f.b == 64) return 3 * f.nbr < h->n_ctas || f.nnzb >= 32 * f.nbr;
     return 5 * f.nbr < h->n_ctas;
 }
 

@@ -395,8 +395,10 @@ bcsr_spmm_kernel(const __grid_constant__ BcsrKernelMaps<B, H, GROUPS, FMT, CT, C
                 }
             }
             operands_ready();
-            // The order of a stage's requests, see bcsr_tiles_first in api.cu, is chosen outside the loop: a test of it per
-            // stage cost small launches up to 5 % (15,584 x 2008, b = 64, TF32, N = 680, us: 37.4 so, 39.3 with the test).
+            // The order of a stage's requests, see bcsr_tiles_first in api.cu, is chosen outside the loop, and only in the
+            // shapes that gain from it: a test of it per stage cost small launches up to 5 % (15,584 x 2008, b = 64, TF32,
+            // N = 680, us: 37.4 so, 39.3 with the test), and so did a second loop beside the one in use where a stage is
+            // short (TF32, b = 64, column-major, 512 x 11264, N = 128: 21.1 with it, 19.6 without).
             auto walk = [&](auto order) {
             constexpr bool kTilesFirst = decltype(order)::value;
             for (uint32_t nth = 0; ok && next_tile(nth, &tcd, &tcd_next, &ok); ++nth) {
@@ -468,7 +470,8 @@ bcsr_spmm_kernel(const __grid_constant__ BcsrKernelMaps<B, H, GROUPS, FMT, CT, C
                 }
             }
             };
-            if (H == B && B >= 64 && p.tiles_first) walk(std::bool_constant<H == B && B >= 64>());
+            constexpr bool kEither = H == B && !SPLIT && !DYN && (B == 128 || (B == 64 && GROUPS > 1));
+            if (kEither && p.tiles_first) walk(std::bool_constant<kEither>());
             else walk(std::false_type());
             if (lane == 0) issued[pw] = it;
         }

@@ -359,8 +359,8 @@ def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16)
                                                 ("fp16", 64, "col", True), ("fp8", 64, "col", False), ("bf16", 128, "col", True), ("fp8", 128, "row", False)])
 def test_bcsr_order_of_requests_changes_no_bit(lib, dtype, b, layout, c16):
     """Few block-rows for the grid (a fifth; TF32 blocks of 64: a third): a stage's token tiles are requested before its stored
-    blocks.  Grids on either side of the line, rows of one block to several rings full, an empty one, a ragged last token
-    tile: the same bits, and the oracle's result."""
+    blocks, with blocks of 64 in tiles of more than 128 tokens.  Grids on either side of the line, rows of one block to several
+    rings full, an empty one, a ragged last token tile: the same bits, and the oracle's result."""
     third = dtype == "tf32" and b == 64
     nbr, nbc = 3, 40
     rng = np.random.default_rng(b)
@@ -372,7 +372,7 @@ def test_bcsr_order_of_requests_changes_no_bit(lib, dtype, b, layout, c16):
     rp = np.concatenate(([0], np.cumsum(full.sum(1)))).astype(np.int64)
     ci = np.nonzero(full)[1].astype(np.int32)
     vals = wl.to_storage(rng.uniform(-1, 1, ci.size), dtype)
-    N = 128 * 55 + 16                                     # two token groups to a tile on 10 CTAs
+    N = 128 * 95 + 16                                     # two token groups and more to a tile on 16 CTAs
     Bs = wl.dense(11, k, N, ("uniform", -1.0, 1.0), dtype)
     got = []
     for n_ctas in ((9, 10) if third else (15, 16)):
@@ -380,7 +380,7 @@ def test_bcsr_order_of_requests_changes_no_bit(lib, dtype, b, layout, c16):
                                      c_type=lib.C_SAME_AS_INPUT if c16 else lib.C_FP32)
         try:
             got.append(run_gpu_variant(lib, h, Bs, m, N, dtype, c16=c16, col_major=layout == "col"))
-            assert lib.spmm_get_info(h, N)["plan_token_tile"] > 128 or not third
+            assert lib.spmm_get_info(h, N)["plan_token_tile"] > 128
         finally:
             lib.spmm_destroy(h)
     assert np.array_equal(got[0], got[1])
