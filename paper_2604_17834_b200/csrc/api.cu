@@ -848,22 +848,39 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     int rc;
     // Where the 128-token tiles of a launch are half as many as the CTAs or fewer, each is computed by two CTAs: half of
     // its tokens in either, or, where 128-row stacked blocks are multiplied, half of their rows.  An SM's load rate and its
-    // tensor core bound such a launch; an SM then loads two thirds to three quarters as much.  The sums are the same.  Only
-    // from kSplitMinBytes in the longest tile on (shorter ones are latencies, and two CTAs fetch the blocks, or the tokens,
-    // twice); row groups only where their longest tile, not the work as a whole, decides when the last CTA ends.  us:
+    // tensor core bound such a launch; an SM then loads (64 + b) / (128 + b) as much (0.56 / 0.60 / 0.67 / 0.75; stacked blocks
+    // 0.75).  The sums are the same.  Only from kSplitMinBytes in the longest tile on (shorter ones are latencies, and two CTAs
+    // fetch the blocks, or the tokens, twice); row groups only where their longest tile, not the work as a whole, decides when
+    // the last CTA ends.  us:
     //   1500 x 9000, b = 64, 10 % full rows, fp16, N = 200 (3.4 MB a tile)   35.0 -> 22.5
     //   3000 x 16000, b = 16, 10 % full rows, bf16, N = 256 (8 MB, grouped)  93.2 -> 67.9
     //   600 x 6000, b = 16, 10 % full rows, TF32, N = 200 (6 MB, grouped)    55.2 -> 41.6
     //   3000 x 6000, b = 32, 10 % full rows, fp16, N = 512 (3 MB, grouped)   25.9 -> 26.6: left alone
-    //   3584 x 18944, b = 64, density 0.1, bf16, N = 128 (1 MB)              9.6 -> 9.4
     //   1024 x 4096 and back, b = 64, density 0.2, N = 300 (0.3 MB)          10.7 -> 11.0: left alone
     //   6000 x 5000, b = 32, TF32, N = 1500 (5 MB; 3.7 MB of work per CTA)   48.8 -> 60.7: left alone
+    // Row groups of 150 random skewed products: 1.02 to 1.66 of the speed with whole tiles, none slower.  Plain blocks, speed
+    // over that with whole tiles, at 0.8 - 1 / 2 - 2.5 MB a tile and 8 to 66 tiles; with 74 (148 CTAs):
+    //   bf16  b = 16   row-major 1.00 - 1.01 / 1.01 - 1.02; 1.01    column-major 1.20 - 1.23 / 1.24 - 1.25; 1.20
+    //         b = 32             0.98 - 1.01 / 0.99 - 1.02; 1.02                 1.14 - 1.18 / 1.22 - 1.24; 1.16
+    //         b = 64             1.07 - 1.15 / 1.14 - 1.17; 1.11 - 1.29          1.09 - 1.20 / 1.18 - 1.20; 1.14 - 1.31
+    //         b = 128            0.99 - 1.09 / 1.05 - 1.14; 1.04 - 1.16          1.05 - 1.14 / 1.08 - 1.17; 1.10 - 1.20
+    //   E4M3  b = 32 / 64 / 128                                                  1.27 - 1.32 / 1.05 - 1.12 / 0.98 - 1.05; 1.06 - 1.33
+    //   TF32  b = 16   row-major 0.97 - 0.99 / 0.99 - 1.00; 0.97 - 1.00: left alone    column-major 1.08 - 1.10 / 1.14; 1.08
+    //         b = 32             1.00 - 1.05 / 1.04 - 1.07; 1.07 - 1.17          1.00 - 1.07 / 1.03 - 1.07; 1.09 - 1.17
+    //         b = 64             0.95 - 1.00 / 0.95 - 0.97; 0.99 - 1.07          0.95 - 1.03 / 0.94 - 1.02; 0.99 - 1.06
+    //         b = 128            0.94 - 1.01 / 0.96 - 1.03; 0.97 - 1.19          0.98 - 1.04 / 0.99 - 1.03; 1.01 - 1.20
+    // so that TF32 blocks of 64, and row-major ones of 128 of less than 4 MB a tile, are halved only where that fills the grid.
     // (One MMA of two CTAs, cta_group::2, in their place: 16.3 for the fourth, 70 for the last: with N = 64 or 128 its
     // exchange of the other half's block rows takes longer than the product.)
     bool split = false, stack_split = false;
     auto split_fits = [&](int64_t n_tiles, int64_t longest, int64_t rows) {
-        return N > 64 && 2 * n_tiles <= h->n_ctas && longest * (128 + rows) * f.b * h->es >= kSplitMinBytes && !h->dynamic &&
-               !(h->dtype == SPMM_FP8_E4M3 && !h->col_major);
+        const int64_t bytes = longest * (128 + rows) * f.b * h->es;
+        if (rows == f.b && h->es == 4) {
+            if (f.b == 16 && !h->col_major) return false;
+            const bool fills = 32 * n_tiles > 15 * h->n_ctas;
+            if (!fills && (f.b == 64 || (f.b == 128 && !h->col_major && bytes < (int64_t{4} << 20)))) return false;
+        }
+        return N > 64 && 2 * n_tiles <= h->n_ctas && bytes >= kSplitMinBytes && !h->dynamic && !(h->dtype == SPMM_FP8_E4M3 && !h->col_major);
     };
     // Such a launch has two CTAs to each of the first lists, as many as there are tiles: they hold all of them (tiles are dealt to
     // the least loaded CTA, the first of several), or it is none.

@@ -336,7 +336,9 @@ def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16)
         opt["stack_min_fill"] = -1                          # plain blocks
     assert need * (128 + (b if dens < 1 else 128)) * b * wl.elem_size(dtype) >= 768 << 10
     for N in ((128, 129, 200, 321) if layout == "col" else (72, 96, 128, 136, 256)):
-        h = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, **opt)
+        # (TF32 blocks of 64 and 128: halves that fill the grid)
+        fill = {"n_ctas": 2 * nbr * -(-N // 128)} if dtype == "tf32" and b >= 64 else {}
+        h = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, **opt, **fill)
         h1 = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, n_ctas=3, **opt)
         try:
             Bs = wl.dense(7 + N, k, N, ("uniform", -1.0, 1.0), dtype)
@@ -350,6 +352,13 @@ def test_bcsr_few_long_tiles_run_as_half_tiles(lib, dtype, b, dens, layout, c16)
             tiles = grouped or lib.spmm_export(h, lib.X_BCSR_TILES, np.int32).size // 2
             assert captured_launches(lib, h, Bd, Cd, N)[0][0] == 2 * tiles, (N, tiles)
             assert captured_launches(lib, h1, Bd, Cd, N)[0][0] == 3
+            if fill:                                       # and none on a grid they leave half empty
+                h2 = lib.spmm_bcsr_create_csr(m, k, rp, ci, vals, dtype, b, n_ctas=4 * tiles, **opt)
+                try:
+                    assert np.array_equal(run_gpu_variant(lib, h2, Bs, m, N, dtype, c16=c16, col_major=layout == "col"), C1), N
+                    assert captured_launches(lib, h2, Bd, Cd, N)[0][0] == (2 * tiles if b == 128 and layout == "col" else 4 * tiles)
+                finally:
+                    lib.spmm_destroy(h2)
         finally:
             lib.spmm_destroy(h)
             lib.spmm_destroy(h1)
