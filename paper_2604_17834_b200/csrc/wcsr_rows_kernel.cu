@@ -61,10 +61,16 @@ __device__ __forceinline__ void st_vec(uint8_t* p, const uint32_t* w) {
 
 // acc[e] += a * b[e] over one vector of B.  16-bit types: the product of two 16-bit values is exact in
 // fp32, so the mixed-precision FMA rounds once, like an FMA of the widened values.  (Widening first and
-// a packed fma.rn.f32x2 measured 9 % slower.)  fp32 goes two columns at a time: R-MAT 2^17, 16 a row, N = 200
-// 120.9 -> 118.6 us, 200,000 power-law rows N = 64 47.2 -> 46.2.
+// a packed fma.rn.f32x2 measured 9 % slower.)  fp32 in 32-byte vectors goes two columns at a time: R-MAT 2^17, 16 a row, N = 200
+// 120.9 -> 118.6 us, 200,000 power-law rows N = 64 47.2 -> 46.2.  In 16-byte vectors, whose launches are short chains of
+// gathers, not: 303,000 power-law rows, N = 16, 26.1 us so, 30.0 two at a time; R-MAT 2^20, 16 a row, N = 36, 299 and 306.
 template <int FMT, int VB, int VE>
 __device__ __forceinline__ void fma_vec(float (&acc)[VE], uint32_t a, const Vec<VB>& b) {
+    if constexpr (FMT == 2 && VB == 16) {
+#pragma unroll
+        for (int i = 0; i < VE; ++i) acc[i] = fmaf(__uint_as_float(a), __uint_as_float(b.w[i]), acc[i]);
+        return;
+    }
     if constexpr (FMT == 2) {
 #pragma unroll
         for (int i = 0; i < VE; i += 2)
@@ -161,9 +167,11 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     constexpr int ES = FMT == 2 ? 4 : 2;
     constexpr int VE = VB / ES;                           // dense columns per lane
     using CElem = typename CType<FMT, CT>::type;
-    // long rows: [kStrands][lanes][VE + 1]; with a pitch of VE (or of lanes, transposed) the strands of a warp and the
-    // columns of the adding threads met in a quarter of the banks: 11 of 41 million wavefronts of the L1 data path on
-    // R-MAT 2^19, fp16, N = 128; on 2^21 812 -> 794 us
+    // long rows' strands: wide vectors [kStrands][lanes][VE + 1]; with a pitch of VE (or of lanes, transposed) the strands of a
+    // warp and the columns of the adding threads met in a quarter of the banks: 11 of 41 million wavefronts of the L1 data
+    // path on R-MAT 2^19, fp16, N = 128; on 2^21 812 -> 794 us.  16-byte vectors, whose rows of B are narrow, [kStrands][VE]
+    // [lanes]: they feel the shared memory that the pitch takes from L1 instead (100,000 power-law rows, fp16, N = 32 13.6 us so,
+    // 14.0 with it; R-MAT 2^20, 16 a row, TF32, N = 32 219 and 221)
     extern __shared__ float red[];
     __shared__ unsigned arrived;
 
@@ -227,6 +235,8 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     grid_wait();
     const int n_groups = kWarps * p.groups;
     const int tile_cols = p.lanes * VE;
+    const int strand_pitch = VB == 32 ? p.lanes * (VE + 1) : tile_cols;
+    auto red_at = [&](int strand, int lane_of, int i) { return strand * strand_pitch + (VB == 32 ? lane_of * (VE + 1) + i : i * p.lanes + lane_of); };
     if (g < p.groups) {
         for (int strand = warp * p.groups + g; strand < kStrands; strand += n_groups) {
 #pragma unroll
@@ -246,7 +256,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
                 }
             }
 #pragma unroll
-            for (int i = 0; i < VE; ++i) red[(strand * p.lanes + l) * (VE + 1) + i] = acc[i];
+            for (int i = 0; i < VE; ++i) red[red_at(strand, l, i)] = acc[i];
         }
     }
     __syncthreads();
@@ -257,7 +267,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     for (int t = threadIdx.x; t < tile_cols; t += THREADS) {
         float s = 0.f;
 #pragma unroll
-        for (int i = 0; i < kStrands; ++i) s += red[i * (p.lanes * (VE + 1)) + t + t / VE];
+        for (int i = 0; i < kStrands; ++i) s += red[red_at(i, t / VE, t % VE)];
         if (lr.z == 1) {
             if (n_tile + t < p.N) Crow[t] = from_f32<CElem>(s);
         } else {
@@ -340,7 +350,7 @@ cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsPar
     const int64_t ctas = p.n_parts + (static_cast<int64_t>(p.n_tasks) + per_cta - 1) / per_cta;
     if (ctas <= 0 || tiles <= 0) return cudaSuccess;
     const dim3 grid(static_cast<unsigned>(ctas), static_cast<unsigned>(tiles));
-    const size_t smem = p.n_parts > 0 ? static_cast<size_t>(kStrands) * (s.tile_cols + s.lanes) * 4 : 0;     // at most 34 KB
+    const size_t smem = p.n_parts > 0 ? static_cast<size_t>(kStrands) * (s.tile_cols + (s.vec == 32 ? s.lanes : 0)) * 4 : 0;     // at most 34 KB
     if (threads == 256) return s.vec == 32 ? launch_vb<32, 256>(dtype, c16, p, grid, smem, stream) : launch_vb<16, 256>(dtype, c16, p, grid, smem, stream);
     return s.vec == 32 ? launch_vb<32, kRowsThreads>(dtype, c16, p, grid, smem, stream) : launch_vb<16, kRowsThreads>(dtype, c16, p, grid, smem, stream);
 }
