@@ -629,10 +629,10 @@ bcsr_spmm_kernel(const __grid_constant__ BcsrKernelMaps<B, H, GROUPS, FMT, CT, C
                                             (static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&hi)) << 16);
                                 }
                                 if (wide && crow + c + kPer <= p.m) {
-                                    st_global_v8(dst + c, w8);
+                                    st_global_vec<32>(dst + c, w8);
                                 } else {
-                                    if (crow + c + kPer / 2 <= p.m) st_global_v4(dst + c, w8);
-                                    if (crow + c + kPer <= p.m) st_global_v4(dst + c + kPer / 2, w8 + 4);
+                                    if (crow + c + kPer / 2 <= p.m) st_global_vec<16>(dst + c, w8);
+                                    if (crow + c + kPer <= p.m) st_global_vec<16>(dst + c + kPer / 2, w8 + 4);
                                 }
                             }
                         }

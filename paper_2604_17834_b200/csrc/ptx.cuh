@@ -471,13 +471,15 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-// 32 / 16 bytes to global memory; the address is a multiple of that.
-__device__ __forceinline__ void st_global_v8(void* p, const uint32_t* w) {
-    asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-                 ::"r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "l"(p) : "memory");
-}
-__device__ __forceinline__ void st_global_v4(void* p, const uint32_t* w) {
-    asm volatile("st.global.v4.b32 [%4], {%0, %1, %2, %3};" ::"r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "l"(p) : "memory");
+// 32 or 16 bytes to global memory; the address is a multiple of that.
+template <int BYTES>
+__device__ __forceinline__ void st_global_vec(void* p, const uint32_t* w) {
+    static_assert(BYTES == 32 || BYTES == 16, "one store");
+    if constexpr (BYTES == 32)
+        asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+                     ::"r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "l"(p) : "memory");
+    else
+        asm volatile("st.global.v4.b32 [%4], {%0, %1, %2, %3};" ::"r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "l"(p) : "memory");
 }
 
 // ----------------------------------------------------------------------------- output element

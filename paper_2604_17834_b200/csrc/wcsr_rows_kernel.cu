@@ -50,14 +50,6 @@ __device__ __forceinline__ Vec<VB> ld_row(const uint8_t* p) {
                      : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]) : "l"(p));
     return r;
 }
-template <int BYTES>
-__device__ __forceinline__ void st_vec(uint8_t* p, const uint32_t* w) {
-    if constexpr (BYTES == 32)
-        asm volatile("st.global.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
-                     ::"r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]), "l"(p) : "memory");
-    else
-        asm volatile("st.global.v4.b32 [%4], {%0, %1, %2, %3};" ::"r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "l"(p) : "memory");
-}
 
 // acc[e] += a * b[e] over one vector of B.  16-bit types: the product of two 16-bit values is exact in
 // fp32, so the mixed-precision FMA rounds once, like an FMA of the widened values.  (Widening first and
@@ -142,7 +134,7 @@ __device__ __forceinline__ void store_c(uint8_t* dst, const float (&acc)[VE]) {
             uint32_t w[kPer];
 #pragma unroll
             for (int j = 0; j < kPer; ++j) w[j] = __float_as_uint(acc[i + j]);
-            st_vec<kPer * 4>(dst + i * 4, w);
+            st_global_vec<kPer * 4>(dst + i * 4, w);
         }
     } else {
         uint32_t w[VE / 2];
@@ -152,7 +144,7 @@ __device__ __forceinline__ void store_c(uint8_t* dst, const float (&acc)[VE]) {
             w[j] = static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&lo)) |
                    (static_cast<uint32_t>(*reinterpret_cast<const unsigned short*>(&hi)) << 16);
         }
-        st_vec<VE * 2>(dst, w);
+        st_global_vec<VE * 2>(dst, w);
     }
 }
 
