@@ -1030,15 +1030,16 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
 //           bf16  1.015      1.014     1.005     0.997     0.961      0.977
 //   b = 64  TF32  1.014      1.006     1.007     1.007     1.000      0.995, under 16 blocks a row
 //           bf16  1.007      1.006     1.002     0.998     0.996      0.99
-// b <= 32 and stacked blocks do not gain on either side, nor do short stages (b = 64 in tiles of 128 tokens); column-major E4M3
-// loses (b = 128 under 30 block-rows 0.988, row-major 1.005).  TF32 at b = 64
+// b <= 32 and stacked blocks do not gain on either side, nor do short stages (b = 64 in tiles of 128 tokens), narrow operands
+// (under 1000 columns 0.997: their weights are what comes from afar) or column-major ones (b = 128, under 30 block-rows: 16-bit
+// 1.002, TF32 0.99, E4M3 0.988).  TF32 at b = 64
 // has the longest B tiles beside its blocks (32 KB to 8): long tiles, 32 blocks a row and more, gain at any number of
 // block-rows.  us, blocks first and tiles first: 8192 x 8192, b = 64, density 0.4, TF32, N = 16,384 2225 and 2134; 5000 x 7000,
 // 10 % full rows, N = 16,384 947 and 927; 1819 x 5601, b = 128, 10 % full rows, N = 9288 105.1 and 103.2; 3584 x 18944, b = 128,
 // bf16, N = 2048 87.5 and 82.3.
-bool bcsr_tiles_first(const spmm_handle_s* h, int groups) {
+bool bcsr_tiles_first(const spmm_handle_s* h, int64_t N, int groups) {
     const BcsrHost& f = h->bcsr;
-    if (f.b < 64 || (f.b == 64 && groups == 1) || (h->es == 1 && h->col_major)) return false;
+    if (f.b < 64 || (f.b == 64 && groups == 1) || N < 1024 || h->col_major) return false;
     if (h->es == 4 && f.b == 64) return 3 * f.nbr < h->n_ctas || f.nnzb >= 32 * f.nbr;
     return 5 * f.nbr < h->n_ctas;
 }
@@ -1066,7 +1067,7 @@ int run_bcsr(spmm_handle_s* h, const void* B, void* C, int64_t N, cudaStream_t s
     p.B = nullptr;
     p.k = h->k;
     p.overlap = 0;
-    p.tiles_first = bcsr_tiles_first(h, h->sched.groups) ? 1 : 0;
+    p.tiles_first = bcsr_tiles_first(h, N, h->sched.groups) ? 1 : 0;
     BcsrMaps tm;
     tm.A = h->sched.groups <= 1 ? h->tmA1 : h->tmA;
     tm.A0 = h->tmA;

@@ -470,7 +470,7 @@ bcsr_spmm_kernel(const __grid_constant__ BcsrKernelMaps<B, H, GROUPS, FMT, CT, C
                 }
             }
             };
-            constexpr bool kEither = H == B && !SPLIT && !DYN && (B == 128 || (B == 64 && GROUPS > 1));
+            constexpr bool kEither = H == B && !CM && !SPLIT && !DYN && (B == 128 || (B == 64 && GROUPS > 1));
             if (kEither && p.tiles_first) walk(std::bool_constant<kEither>());
             else walk(std::false_type());
             if (lane == 0) issued[pw] = it;

@@ -38,7 +38,7 @@ struct BcsrParams {
     int* status;
     uint64_t wait_limit_ns;
     int32_t use_3d;     // tmB3 is valid: whole token tiles are fetched with one 3-D request
-    int32_t tiles_first;        // a stage's B tiles are requested before its stored blocks (whole tiles of plain blocks of 128, or of 64 with groups > 1)
+    int32_t tiles_first;        // a stage's B tiles are requested before its stored blocks (row-major whole tiles of plain blocks of 128, or of 64 with groups > 1)
     // stacked launch only: [groups][128 / b] block-rows of every row group (see BcsrStack); the
     // tile records then name {group, token tile, first stacked block, end stacked block} and
     // block_col_idx is the stacked blocks' column index
