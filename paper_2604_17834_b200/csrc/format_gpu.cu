@@ -58,18 +58,15 @@ constexpr int kLongShift = 40;               // a count of windows above this bi
 struct WindowLists {
     int wh;                                  // 0: no lists are wanted
     int64_t k;
-    int32_t* list[kLists];
+    int32_t* list[kLists];                   // kListBitmap: its first place; the others are filled from their last place down
     int* count;                              // [kLists], zero before
     int32_t *long_window, *long_first;       // [max_long] the windows that are cut, and their first pieces
     unsigned long long* long_count;          // both counts in one, zero before: the first pieces ascend with the windows' places
     int64_t max_long;
-    __device__ __forceinline__ bool is_long(int64_t n) const {
-        if (n <= kLargeWindow) return false;
-        return n > kBitmapReads || n * ((k + kBitmapColumns - 1) / kBitmapColumns) > kBitmapReads;
-    }
-    __device__ __forceinline__ int which(int64_t n) const {
-        if (n <= kWarpWindow || is_long(n)) return -1;
-        if (n > kLargeWindow || n * kColumnsPerEntry >= k) return kListBitmap;
+    int64_t long_from;                       // they have that many entries and more
+    __device__ __forceinline__ int which(int64_t n) const {                  // kLists: it is cut
+        if (n >= long_from) return kLists;
+        if (n * kColumnsPerEntry >= k) return kListBitmap;
         return n <= kMergeWindow ? kListMerge : kListLarge;
     }
 };
@@ -88,9 +85,12 @@ __global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* er
         if (row_ptr[i + 1] < row_ptr[i]) atomicMin(err, SPMM_ERR_INVALID_ARG);
         if (longer.wh && i % longer.wh == 0) {
             const int64_t n = row_ptr[min(i + longer.wh, m)] - row_ptr[i];
+            if (n <= kWarpWindow) continue;
             const int which = longer.which(n);
-            if (which >= 0) longer.list[which][atomicAdd(longer.count + which, 1)] = static_cast<int32_t>(i / longer.wh);
-            if (longer.is_long(n) && n < (int64_t{1} << 31)) {
+            if (which < kLists) {
+                const int at = atomicAdd(longer.count + which, 1);
+                longer.list[which][which == kListBitmap ? at : -at] = static_cast<int32_t>(i / longer.wh);
+            } else if (n < (int64_t{1} << 31)) {
                 const unsigned long long one = 1ull << kLongShift, before = atomicAdd(longer.long_count, one + static_cast<unsigned long long>(pieces_of(n)));
                 const int64_t at = static_cast<int64_t>(before >> kLongShift);
                 if (at < longer.max_long) {              // (not so with a row_ptr that is refused)
@@ -590,10 +590,9 @@ __device__ __forceinline__ void sort_window(const CondenseParams& p, int64_t w, 
     }
 }
 
-// n entries: keys[2][cap], rank[cap] in shared memory; off has WH + 1 entries.  *found: distinct columns.
+// n entries: keys[2][cap], rank[cap] in shared memory; off has WH + 1 entries.  Returns the number of distinct columns.
 template <int WH, int THREADS, class Entries>
-__device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w, const Entries& e, int n, const int* off, int32_t* keys, int cap, uint32_t* rank,
-                                             int32_t* found) {
+__device__ __forceinline__ int merge_window(const CondenseParams& p, int64_t w, const Entries& e, int n, const int* off, int32_t* keys, int cap, uint32_t* rank) {
     __shared__ int warp_sum[THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j < n; j += THREADS) {
@@ -650,8 +649,8 @@ __device__ __forceinline__ void merge_window(const CondenseParams& p, int64_t w,
         carry = all;
         __syncthreads();
     }
-    if (threadIdx.x == 0) *found = carry;
     for (int j = threadIdx.x; j < n; j += THREADS) p.pos_of[e.at(static_cast<int>(rank[j] >> 16), j)] = dst[rank[j] & 0xffffu] - 1;
+    return carry;
 }
 
 // One warp per window; the last of the launches that run side by side, it ends after the others.
@@ -692,16 +691,17 @@ __global__ void __launch_bounds__(THREADS) wcsr_merge_windows_kernel(const Conde
     grid_trigger();
     const int64_t w = p.list[blockIdx.x];
     load_offsets<WH, THREADS>(p, w, off);
-    merge_window<WH, THREADS>(p, w, WholeWindow{p.row_ptr[w * WH], off}, off[WH], off, dyn, kCap, reinterpret_cast<uint32_t*>(dyn + 2 * kCap), p.ucount + w);
+    const int found = merge_window<WH, THREADS>(p, w, WholeWindow{p.row_ptr[w * WH], off}, off[WH], off, dyn, kCap, reinterpret_cast<uint32_t*>(dyn + 2 * kCap));
+    if (threadIdx.x == 0) p.ucount[w] = found;
     grid_wait();
 }
 
 // Bits of the columns [c0, c0 + 32 words) and the set bits before each word, as many at a time as there is room for, of the
-// columns [begin, end) that the entries lie in.  *found: distinct columns.
+// columns [begin, end) that the entries lie in.  Returns the number of distinct columns.
 constexpr int kBitmapThreads = 512;
 template <int WH, class Entries>
-__device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w, const Entries& e, int n, const int* off, uint32_t* bits, int max_words,
-                                              int64_t begin, int64_t end, int32_t* found_columns) {
+__device__ __forceinline__ int bitmap_window(const CondenseParams& p, int64_t w, const Entries& e, int n, const int* off, uint32_t* bits, int max_words,
+                                             int64_t begin, int64_t end) {
     __shared__ long long scratch[32];
     constexpr int T = kBitmapThreads;
     uint32_t* prefix = bits + max_words;
@@ -735,12 +735,9 @@ __device__ __forceinline__ void bitmap_window(const CondenseParams& p, int64_t w
             p.pos_of[at] = static_cast<int32_t>(prefix[c >> 5] + __popc(bits[c >> 5] & ((1u << (c & 31)) - 1u)));
         }
         for (int i = threadIdx.x; i < words; i += T)
-            for (uint32_t x = bits[i]; x; x &= x - 1) {
-                const int64_t c = c0 + 32 * int64_t{i} + (__ffs(x) - 1);
-                atomicAdd(p.refs + c, 1);
-            }
+            for (uint32_t x = bits[i]; x; x &= x - 1) atomicAdd(p.refs + c0 + 32 * int64_t{i} + (__ffs(x) - 1), 1);
     }
-    if (threadIdx.x == 0) *found_columns = found;
+    return found;
 }
 
 template <int WH>
@@ -750,7 +747,8 @@ __global__ void __launch_bounds__(kBitmapThreads) wcsr_bitmap_windows_kernel(con
     grid_trigger();
     const int64_t w = p.list[blockIdx.x];
     load_offsets<WH, kBitmapThreads>(p, w, off);
-    bitmap_window<WH>(p, w, WholeWindow{p.row_ptr[w * WH], off}, off[WH], off, reinterpret_cast<uint32_t*>(dyn), max_words, 0, p.k, p.ucount + w);
+    const int found = bitmap_window<WH>(p, w, WholeWindow{p.row_ptr[w * WH], off}, off[WH], off, reinterpret_cast<uint32_t*>(dyn), max_words, 0, p.k);
+    if (threadIdx.x == 0) p.ucount[w] = found;
     grid_wait();
 }
 
@@ -881,8 +879,10 @@ __global__ void __launch_bounds__(kBitmapThreads) wcsr_pieces_kernel(const Conde
     const int n = off[WH];
     const int64_t begin = lw.cut_col[g], end = lw.cut_col[g + 1];
     const WindowPiece e = {base, start};
-    if (end - begin <= int64_t{32} * kPieceWords) bitmap_window<WH>(p, w, e, n, off, reinterpret_cast<uint32_t*>(dyn), kPieceWords, begin, end, lw.found + q);
-    else merge_window<WH, kBitmapThreads>(p, w, e, n, off, dyn, kPieceCap, reinterpret_cast<uint32_t*>(dyn + 2 * kPieceCap), lw.found + q);
+    const int found = end - begin <= int64_t{32} * kPieceWords
+                          ? bitmap_window<WH>(p, w, e, n, off, reinterpret_cast<uint32_t*>(dyn), kPieceWords, begin, end)
+                          : merge_window<WH, kBitmapThreads>(p, w, e, n, off, dyn, kPieceCap, reinterpret_cast<uint32_t*>(dyn + 2 * kPieceCap));
+    if (threadIdx.x == 0) lw.found[q] = found;
 }
 
 // One CTA per window: its distinct columns, and in found those of the pieces before each.
@@ -1149,7 +1149,7 @@ bool condense(CondenseParams p, const WindowLists& lists, const int* count, cons
         return cudaGetLastError() == cudaSuccess;
     };
     auto list = [&](int which, auto kernel, int threads, size_t smem, const auto&... args) {
-        p.list = lists.list[which];
+        p.list = which == kListBitmap ? lists.list[which] : lists.list[which] + 1 - count[which];
         return count[which] == 0 || launch(kernel, count[which], threads, smem, args...);
     };
     const int words = static_cast<int>(std::min<int64_t>((p.k + 31) / 32, kBitmapColumns / 32));
@@ -1209,15 +1209,18 @@ int build_wcsr_device(int64_t m, int64_t k, const int64_t* d_row_ptr, const int3
     auto alloc = [&](void** ptr, size_t bytes) { return dev_alloc(ptr, bytes, st) == cudaSuccess; };
 
     const int64_t max_long = std::min(nwin, kMostLong);
-    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags)) || !alloc(reinterpret_cast<void**>(&d_lists), static_cast<size_t>(kLists * nwin + 2 * max_long + 1) * 4))
+    if (!alloc(reinterpret_cast<void**>(&d_flags), sizeof(Flags)) || !alloc(reinterpret_cast<void**>(&d_lists), static_cast<size_t>(2 * nwin + max_long + 1) * 4))
         return fail(SPMM_ERR_ALLOC);
     if (cudaMemsetAsync(d_flags, 0, sizeof(Flags), st) != cudaSuccess) return fail(SPMM_ERR_CUDA);
     auto read_flags = [&]() {
         return cudaMemcpyAsync(&flags, d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
     };
     const unsigned check_grid = static_cast<unsigned>(std::min<int64_t>((m + 255) / 256, 2048));
-    const WindowLists lists = {wh, k, {d_lists, d_lists + nwin, d_lists + 2 * nwin}, d_flags->n_listed,
-                               d_lists + kLists * nwin, d_lists + kLists * nwin + max_long, &d_flags->long_count, max_long};
+    // a window is cut where a bitmap would read more than kBitmapReads entries, once per kBitmapColumns
+    const int64_t long_from = std::max<int64_t>(kLargeWindow, kBitmapReads / std::max<int64_t>(1, (k + kBitmapColumns - 1) / kBitmapColumns)) + 1;
+    // (no window is in two lists: two of them share nwin places, one from either end)
+    const WindowLists lists = {wh, k, {d_lists, d_lists + nwin - 1, d_lists + 2 * nwin - 1}, d_flags->n_listed,
+                               d_lists + nwin, d_lists + 2 * nwin, &d_flags->long_count, max_long, long_from};
     if (m > 0) csr_check_rows_kernel<<<check_grid, 256, 0, st>>>(m, d_row_ptr, &d_flags->err, &d_flags->nnz, lists);
     if (!read_flags()) return fail(SPMM_ERR_CUDA);
     if (flags.err != 0) return fail(flags.err);
