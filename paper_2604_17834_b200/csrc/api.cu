@@ -1194,6 +1194,27 @@ int wcsr_rows_threads(const spmm_handle_s* h, const RowsShape& s) {
     return h->rows.n_parts > 0 && groups < 4 && wcsr_rows_load(h->m, h->nnz, h->sms) < (groups == 1 ? 8 : 7) ? 256 : kRowsThreads;
 }
 
+// fp32 sums of one column per instruction and strands without padding, for TF32 in 16-byte vectors (rows of B that are no
+// multiple of 32 bytes, or narrow): where the rows are short, the operand is narrow or the launch large, it is chains of
+// gathers, and what two columns per instruction and the padding save in issue slots they cost in latency and L1.  Speed over
+// that with both, by entries a row and entries per SM and 128 groups (load):
+//                              row  load   N = 16   36     52     76     252
+//   power-law rows, 300,000     3    70    1.01     1.07   1.11   1.12   1.08
+//                    50,000     6    20    1.15     1.00   1.00   1.02   1.01
+//   R-MAT 2^20                  4   280    1.04     1.03   1.04   1.03   1.03
+//         2^20                 16   900    1.01     1.02          1.02
+//   power-law rows, 400,000    17   390    1.00     1.03          1.06
+//   R-MAT 2^15                  7    15    1.05     1.00   0.99   0.99   0.93
+//         2^16                 21    80    1.03     0.98   1.00   0.98   0.98
+//   power-law rows, 100,000    14    78    1.06     0.98   1.00   0.96   1.00
+//                    20,000    12    14    1.02     1.00   0.98   0.96   0.96
+//                    6000      12     4    0.98     1.00   1.01   1.00   0.99
+bool wcsr_rows_plain(const spmm_handle_s* h, const RowsShape& s) {
+    if (h->es != 4 || s.vec != 16) return false;
+    const int64_t load = wcsr_rows_load(h->m, h->nnz, h->sms);
+    return load >= 128 || (load >= 8 && (s.tiles * s.lanes <= 8 || h->nnz < 6 * h->m));
+}
+
 // partial: room for cap bytes of partial rows; the column tiles go in as few launches as that and the counters allow,
 // and are made narrower where it does not hold one (sums do not depend on the cut).  A tile of one vector takes
 // kRowsMaxSlots * 32 bytes at most, which the built-in scratch holds.
@@ -1224,10 +1245,11 @@ int launch_wcsr_rows_all(spmm_handle_s* h, const void* B, void* C, float* partia
     p.n_tasks = r.n_tasks;
     p.n_parts = r.n_parts;
     const int threads = wcsr_rows_threads(h, s);
+    const bool plain = wcsr_rows_plain(h, s);
     int step = std::min(s.tiles, kRowsMaxTiles);
     while (step > 1 && rows_partial_bytes(h, s, step) > cap) --step;
     for (int t = 0; t < s.tiles; t += step)
-        if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), threads, stream) != cudaSuccess)
+        if (launch_wcsr_rows(h->dtype, h->c16 ? 1 : 0, s, p, t, std::min(step, s.tiles - t), threads, plain, stream) != cudaSuccess)
             return cuda_error();
     return SPMM_OK;
 }

@@ -205,8 +205,8 @@ constexpr int kRowsMaxTiles = 8;     // column tiles one launch covers at most
 struct RowsShape { int vec, lanes, tiles, tile_cols; };
 // aligned32: every row of B and of C starts on a 32-byte boundary.
 RowsShape wcsr_rows_shape(int64_t N, int es, bool aligned32);
-// bf16, fp16, tf32; threads: kRowsThreads or 256.  Column tiles [tile0, tile0 + tiles), at most kRowsMaxTiles of them.
-cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, int threads, cudaStream_t stream);
+// bf16, fp16, tf32; threads: kRowsThreads or 256; plain: tf32 in 16-byte vectors only, see wcsr_rows_kernel.  Column tiles [tile0, tile0 + tiles), at most kRowsMaxTiles of them.
+cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, int threads, bool plain, cudaStream_t stream);
 
 // In the row kernel's place where the wait limit is zero, which makes the kernels that wait give up at their first wait:
 // the row kernel waits for nothing, and this reports to `status` what they would.

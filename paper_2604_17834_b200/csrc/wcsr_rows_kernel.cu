@@ -53,12 +53,12 @@ __device__ __forceinline__ Vec<VB> ld_row(const uint8_t* p) {
 
 // acc[e] += a * b[e] over one vector of B.  16-bit types: the product of two 16-bit values is exact in
 // fp32, so the mixed-precision FMA rounds once, like an FMA of the widened values.  (Widening first and
-// a packed fma.rn.f32x2 measured 9 % slower.)  fp32 in 32-byte vectors goes two columns at a time: R-MAT 2^17, 16 a row, N = 200
-// 120.9 -> 118.6 us, 200,000 power-law rows N = 64 47.2 -> 46.2.  In 16-byte vectors, whose launches are short chains of
-// gathers, not: 303,000 power-law rows, N = 16, 26.1 us so, 30.0 two at a time; R-MAT 2^20, 16 a row, N = 36, 299 and 306.
-template <int FMT, int VB, int VE>
+// a packed fma.rn.f32x2 measured 9 % slower.)  fp32 goes two columns at a time: R-MAT 2^17, 16 a row, N = 200
+// 120.9 -> 118.6 us, 200,000 power-law rows N = 64 47.2 -> 46.2.  PLAIN: one column at a time
+// (wcsr_rows_plain in api.cu).
+template <int FMT, bool PLAIN, int VB, int VE>
 __device__ __forceinline__ void fma_vec(float (&acc)[VE], uint32_t a, const Vec<VB>& b) {
-    if constexpr (FMT == 2 && VB == 16) {
+    if constexpr (FMT == 2 && PLAIN) {
 #pragma unroll
         for (int i = 0; i < VE; ++i) acc[i] = fmaf(__uint_as_float(a), __uint_as_float(b.w[i]), acc[i]);
         return;
@@ -152,18 +152,16 @@ __device__ __forceinline__ void store_c(uint8_t* dst, const float (&acc)[VE]) {
 // on R-MAT 2^21 fp16 N = 128, 5 CTAs 858, 8 CTAs 893; 16-byte vectors: 8 (with 6: R-MAT 2^20 TF32 N = 76 645 -> 703, 2^17 bf16
 // N = 40 38.4 -> 40.2, of 45,000 rows fp16 N = 48 12.9 -> 11.5; with 10: 30,000 rows fp16 N = 48 8.8 -> 9.3).
 // THREADS: kRowsThreads, or 256 (wcsr_rows_threads in api.cu).
-template <int FMT, int CT, int VB, int THREADS>
+template <int FMT, int CT, int VB, int THREADS, bool PLAIN = false>
 __global__ void __launch_bounds__(THREADS, THREADS > kRowsThreads ? 3 : (VB == 32 ? 7 : 8))
 wcsr_rows_kernel(const WcsrRowsParams p) {
     constexpr int kWarps = THREADS / 32;
     constexpr int ES = FMT == 2 ? 4 : 2;
     constexpr int VE = VB / ES;                           // dense columns per lane
     using CElem = typename CType<FMT, CT>::type;
-    // long rows' strands: wide vectors [kStrands][lanes][VE + 1]; with a pitch of VE (or of lanes, transposed) the strands of a
+    // long rows' strands: [kStrands][lanes][VE + 1]; with a pitch of VE (or of lanes, transposed) the strands of a
     // warp and the columns of the adding threads met in a quarter of the banks: 11 of 41 million wavefronts of the L1 data
-    // path on R-MAT 2^19, fp16, N = 128; on 2^21 812 -> 794 us.  16-byte vectors, whose rows of B are narrow, [kStrands][VE]
-    // [lanes]: they feel the shared memory that the pitch takes from L1 instead (100,000 power-law rows, fp16, N = 32 13.6 us so,
-    // 14.0 with it; R-MAT 2^20, 16 a row, TF32, N = 32 219 and 221)
+    // path on R-MAT 2^19, fp16, N = 128; on 2^21 812 -> 794 us.  PLAIN: [kStrands][VE][lanes], which takes less from L1
     extern __shared__ float red[];
     __shared__ unsigned arrived;
 
@@ -208,7 +206,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
             const Ent4<ES> nxt = ld_ent4<ES>(p.col, p.val, d.x + e + 4, e + 4 < d.y);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                fma_vec<FMT, VB, VE>(acc, cur.val(u), b[u]);
+                fma_vec<FMT, PLAIN, VB, VE>(acc, cur.val(u), b[u]);
                 if (cur.c[u] < 0) {                       // the row's last entry
                     store_c<FMT, CT, VB, VE>(C + row * c_pitch, acc);
 #pragma unroll
@@ -227,8 +225,6 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     grid_wait();
     const int n_groups = kWarps * p.groups;
     const int tile_cols = p.lanes * VE;
-    const int strand_pitch = VB == 32 ? p.lanes * (VE + 1) : tile_cols;
-    auto red_at = [&](int strand, int lane_of, int i) { return strand * strand_pitch + (VB == 32 ? lane_of * (VE + 1) + i : i * p.lanes + lane_of); };
     if (g < p.groups) {
         for (int strand = warp * p.groups + g; strand < kStrands; strand += n_groups) {
 #pragma unroll
@@ -242,13 +238,13 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
                     const int en = (e & 4) ? e + kStrands * 8 - 4 : e + 4;      // the strand's next four entries
                     const Ent4<ES> nxt = ld_ent4<ES>(p.col, p.val, d.x + en, en < d.y);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) fma_vec<FMT, VB, VE>(acc, cur.val(u), b[u]);
+                    for (int u = 0; u < 4; ++u) fma_vec<FMT, PLAIN, VB, VE>(acc, cur.val(u), b[u]);
                     cur = nxt;
                     e = en;
                 }
             }
 #pragma unroll
-            for (int i = 0; i < VE; ++i) red[red_at(strand, l, i)] = acc[i];
+            for (int i = 0; i < VE; ++i) red[PLAIN ? strand * tile_cols + i * p.lanes + l : (strand * p.lanes + l) * (VE + 1) + i] = acc[i];
         }
     }
     __syncthreads();
@@ -259,7 +255,7 @@ wcsr_rows_kernel(const WcsrRowsParams p) {
     for (int t = threadIdx.x; t < tile_cols; t += THREADS) {
         float s = 0.f;
 #pragma unroll
-        for (int i = 0; i < kStrands; ++i) s += red[red_at(i, t / VE, t % VE)];
+        for (int i = 0; i < kStrands; ++i) s += red[PLAIN ? i * tile_cols + (t % VE) * p.lanes + t / VE : i * (p.lanes * (VE + 1)) + t + t / VE];
         if (lr.z == 1) {
             if (n_tile + t < p.N) Crow[t] = from_f32<CElem>(s);
         } else {
@@ -301,9 +297,14 @@ __global__ void wcsr_rows_give_up_kernel(int* status) {
 }
 
 template <int VB, int THREADS>
-cudaError_t launch_vb(int dtype, int c16, const WcsrRowsParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
+cudaError_t launch_vb(int dtype, int c16, bool plain, const WcsrRowsParams& p, dim3 grid, size_t smem, cudaStream_t stream) {
     auto go = [&](auto kfn) { return launch_dependent(kfn, grid, THREADS, smem, stream, p); };
-    if (dtype == 2) return go(wcsr_rows_kernel<2, 0, VB, THREADS>);
+    if (dtype == 2) {
+        if constexpr (VB == 16) {
+            if (plain) return go(wcsr_rows_kernel<2, 0, VB, THREADS, true>);
+        }
+        return go(wcsr_rows_kernel<2, 0, VB, THREADS>);
+    }
     if (dtype == 1) return c16 ? go(wcsr_rows_kernel<0, 1, VB, THREADS>) : go(wcsr_rows_kernel<0, 0, VB, THREADS>);
     if (dtype == 0) return c16 ? go(wcsr_rows_kernel<1, 1, VB, THREADS>) : go(wcsr_rows_kernel<1, 0, VB, THREADS>);
     return cudaErrorInvalidValue;
@@ -334,7 +335,7 @@ cudaError_t launch_wcsr_rows_give_up(int* status, cudaStream_t stream) {
     return launch_dependent(wcsr_rows_give_up_kernel, dim3(1), 1, 0, stream, status);
 }
 
-cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, int threads, cudaStream_t stream) {
+cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsParams p, int tile0, int tiles, int threads, bool plain, cudaStream_t stream) {
     p.lanes = s.lanes;
     p.groups = 32 / s.lanes;
     p.tile0 = tile0;
@@ -342,9 +343,9 @@ cudaError_t launch_wcsr_rows(int dtype, int c16, const RowsShape& s, WcsrRowsPar
     const int64_t ctas = p.n_parts + (static_cast<int64_t>(p.n_tasks) + per_cta - 1) / per_cta;
     if (ctas <= 0 || tiles <= 0) return cudaSuccess;
     const dim3 grid(static_cast<unsigned>(ctas), static_cast<unsigned>(tiles));
-    const size_t smem = p.n_parts > 0 ? static_cast<size_t>(kStrands) * (s.tile_cols + (s.vec == 32 ? s.lanes : 0)) * 4 : 0;     // at most 34 KB
-    if (threads == 256) return s.vec == 32 ? launch_vb<32, 256>(dtype, c16, p, grid, smem, stream) : launch_vb<16, 256>(dtype, c16, p, grid, smem, stream);
-    return s.vec == 32 ? launch_vb<32, kRowsThreads>(dtype, c16, p, grid, smem, stream) : launch_vb<16, kRowsThreads>(dtype, c16, p, grid, smem, stream);
+    const size_t smem = p.n_parts > 0 ? static_cast<size_t>(kStrands) * (s.tile_cols + (plain ? 0 : s.lanes)) * 4 : 0;     // at most 34 KB
+    if (threads == 256) return s.vec == 32 ? launch_vb<32, 256>(dtype, c16, plain, p, grid, smem, stream) : launch_vb<16, 256>(dtype, c16, plain, p, grid, smem, stream);
+    return s.vec == 32 ? launch_vb<32, kRowsThreads>(dtype, c16, plain, p, grid, smem, stream) : launch_vb<16, kRowsThreads>(dtype, c16, plain, p, grid, smem, stream);
 }
 
 }  // namespace spmm

@@ -235,3 +235,29 @@ def test_the_sums_do_not_depend_on_the_cta_size(lib, dtype, widths):
             assert {t for _, t in launches} == {256 if groups < 4 else 128}, (N, launches)
     finally:
         lib.spmm_destroy(h)
+
+
+@pytest.mark.parametrize("m,per_row", [(3001, 5), (30001, 5), (30001, 9), (160000, 16)])
+def test_plain_sums_of_16_byte_vectors_are_the_same_bits(lib, m, per_row):
+    """TF32 with rows of B that are no multiple of 32 bytes: one or two columns per instruction, and the strands of long rows
+    with or without padding, by the width, the entries a row (6) and the size of the launch.  A column's sums are those of an
+    aligned, wider run, which has two columns and the padding, bit by bit."""
+    rng = np.random.default_rng(m + per_row)
+    k = 5000
+    lens = np.full(m, per_row, np.int64)
+    lens[[3, 700]] = (2500, 4001)                          # long rows, one cut into parts
+    rp = np.concatenate(([0], np.cumsum(lens))).astype(np.int64)
+    starts = rng.integers(0, k - 20, m)
+    ci = np.concatenate([starts[i] + np.arange(n) if n < 20 else np.sort(rng.choice(k, n, replace=False)) for i, n in enumerate(lens)]).astype(np.int32)
+    vals = wl.to_storage(rng.uniform(-1, 1, ci.size), "tf32")
+    Bs = wl.dense(12, k, 136, ("uniform", -1.0, 1.0), "tf32")
+    h = lib.spmm_wcsr_create_csr(m, k, rp, ci, vals, "tf32", 16)
+    try:
+        want = run_gpu_variant(lib, h, Bs, m, 136, "tf32")
+        Cr, S = reference({"m": m, "k": k, "row_ptr": rp, "col_idx": ci, "vals": vals}, Bs, "tf32", rows=(0, 800))
+        assert_close(want[:800], Cr[:800], S[:800], "tf32", "rows N=136")
+        for N in (4, 20, 32, 36, 52, 132):
+            got = run_gpu_variant(lib, h, np.ascontiguousarray(Bs[:, :N]), m, N, "tf32")
+            assert np.array_equal(got, want[:, :N]), N
+    finally:
+        lib.spmm_destroy(h)
