@@ -1180,18 +1180,24 @@ RowsShape rows_shape(const spmm_handle_s* h, const void* B, const void* C, int64
 }
 
 // Threads of a CTA of the row kernel.  A long row's part is 16 strands, which the CTA's groups sum one after the other
-// where there are fewer groups than that.  A launch that is over when its slowest part is gains from twice the warps; in
-// larger ones a CTA then holds its slot for its slowest warp.  The line, by entries per SM and 128 groups (load) and groups
-// per warp, from us with 128 / 256 threads (512: 0.6 - 1.07 of the speed of 256):
-//   power-law rows, 4000 (load 3)    TF32 N = 36 6.6 / 5.6   N = 128 8.9 / 6.4    bf16 N = 320 13.6 / 9.8
-//                   12,000 (6)       7.3 / 6.4               9.4 / 7.8            16.2 / 11.6
-//                   9000 (8)         7.6 / 8.1               9.8 / 9.8            17.4 / 14.3
-//   R-MAT 2^13, 4 a row (2)          6.1 / 5.4               8.5 / 6.5            13.0 / 8.3
-//         2^13, 16 a row (7)         7.0 / 8.8               9.0 / 10.5           15.8 / 14.2
-//         2^15, 4 a row (8)          7.2 / 7.5               9.9 / 10.6           21.2 / 21.9
+// where there are fewer groups than that.  A launch that is over when its slowest part is gains from twice the warps (512
+// threads: 0.6 - 1.07 of the speed of 256); in larger ones, and where the parts themselves take turns, a CTA then holds its slot
+// for its slowest warp.  Speed with 256 over 128 threads, TF32, by entries per SM and 128 groups (load) and parts (N = 320 is
+// three tiles, a CTA for every part in each):
+//                          load  parts  N = 36 (3 groups)  128 (2)  256 (1)  320 (2)
+//   power-law rows, 2000    2    189                       1.37     1.58     1.06
+//                   4000    3    240    1.22               1.40     1.73     0.95
+//                   9000    6    536    1.08               1.13     1.47     0.91
+//                   12,000  5    455    1.14               1.18     1.51     0.96
+//                   16,000  3     95    1.20               1.34     1.77     1.17
+//   R-MAT 2^11, 16 a row    1    241    1.27               1.29     1.81     1.03
+//         2^12, 24 a row    4    640    1.04               1.10     1.51     0.87
+//         2^13, 16 a row    6    960    0.83               0.90     1.28     0.81
+//         2^14, 8 a row     7    662    0.98                        1.27
 int wcsr_rows_threads(const spmm_handle_s* h, const RowsShape& s) {
     const int groups = 32 / s.lanes;
-    return h->rows.n_parts > 0 && groups < 4 && wcsr_rows_load(h->m, h->nnz, h->sms) < (groups == 1 ? 8 : 7) ? 256 : kRowsThreads;
+    if (h->rows.n_parts == 0 || groups > 3 || wcsr_rows_load(h->m, h->nnz, h->sms) >= (groups == 1 ? 8 : 7)) return kRowsThreads;
+    return int64_t{3} * h->rows.n_parts * s.tiles <= (groups == 1 ? 21 : 13) * h->sms ? 256 : kRowsThreads;
 }
 
 // fp32 sums of one column per instruction and strands without padding, for TF32 in 16-byte vectors (rows of B that are no

@@ -261,3 +261,28 @@ def test_plain_sums_of_16_byte_vectors_are_the_same_bits(lib, m, per_row):
             assert np.array_equal(got, want[:, :N]), N
     finally:
         lib.spmm_destroy(h)
+
+
+def test_many_parts_of_long_rows_keep_small_ctas(lib):
+    """900 rows of 100 entries, each a part of its own in a launch this small: CTAs of 128 threads where a warp holds two groups,
+    of 256 where it holds one (by the parts that an SM takes in turn); the same bits and the oracle's result."""
+    import torch
+    m, k, n = 900, 6000, 100
+    rng = np.random.default_rng(9)
+    rp = np.arange(m + 1, dtype=np.int64) * n
+    ci = np.concatenate([np.sort(rng.choice(k, n, replace=False)) for _ in range(m)]).astype(np.int32)
+    vals = wl.to_storage(rng.uniform(-1, 1, ci.size), "tf32")
+    Bs = wl.dense(13, k, 128, ("uniform", -1.0, 1.0), "tf32")
+    h = lib.spmm_wcsr_create_csr(m, k, rp, ci, vals, "tf32", 16)
+    try:
+        got = {}
+        for N, threads in ((128, 128), (76, 256)):
+            B = np.ascontiguousarray(Bs[:, :N])
+            got[N] = run_gpu_variant(lib, h, B, m, N, "tf32")
+            launches = captured_launches(lib, h, to_device(B), torch.empty((m, N), dtype=torch.float32, device="cuda"), N)
+            assert {t for _, t in launches} == {threads}, (N, launches)
+        assert np.array_equal(got[76], got[128][:, :76])
+        Cr, S = reference({"m": m, "k": k, "row_ptr": rp, "col_idx": ci, "vals": vals}, Bs, "tf32")
+        assert_close(got[128], Cr, S, "tf32", "many parts")
+    finally:
+        lib.spmm_destroy(h)
