@@ -865,20 +865,26 @@ int ensure_schedule(spmm_handle_s* h, int64_t N) {
     //         b = 64             1.07 - 1.15 / 1.14 - 1.17; 1.11 - 1.29          1.09 - 1.20 / 1.18 - 1.20; 1.14 - 1.31
     //         b = 128            0.99 - 1.09 / 1.05 - 1.14; 1.04 - 1.16          1.05 - 1.14 / 1.08 - 1.17; 1.10 - 1.20
     //   E4M3  b = 32 / 64 / 128                                                  1.27 - 1.32 / 1.05 - 1.12 / 0.98 - 1.05; 1.06 - 1.33
-    //   TF32  b = 16   row-major 0.97 - 0.99 / 0.99 - 1.00; 0.97 - 1.00: left alone    column-major 1.08 - 1.10 / 1.14; 1.08
+    //   TF32  b = 16   row-major 0.97 - 0.99 / 0.99 - 1.00; 0.97 - 1.00                column-major 1.08 - 1.10 / 1.14; 1.08
     //         b = 32             1.00 - 1.05 / 1.04 - 1.07; 1.07 - 1.17          1.00 - 1.07 / 1.03 - 1.07; 1.09 - 1.17
     //         b = 64             0.95 - 1.00 / 0.95 - 0.97; 0.99 - 1.07          0.95 - 1.03 / 0.94 - 1.02; 0.99 - 1.06
     //         b = 128            0.94 - 1.01 / 0.96 - 1.03; 0.97 - 1.19          0.98 - 1.04 / 0.99 - 1.03; 1.01 - 1.20
-    // so that TF32 blocks of 64, and row-major ones of 128 of less than 4 MB a tile, are halved only where that fills the grid.
+    // so that TF32 blocks of 64, and row-major ones of 128 of less than 4 MB a tile, are halved only where that fills the grid
+    // (66 tiles of 5 MB, b = 64: 1.04).
+    // Those are widths of whole tiles of whole 128-byte lines.  A ragged or misaligned row-major tile takes a request per 32
+    // tokens, fewer in a half: TF32, N = 72 / 120 / 200 / 248 / 500, b = 64 1.04 - 1.07 / 1.09 - 1.12 / 1.04 - 1.07 / 1.10 - 1.13 / 1.48,
+    // b = 128 1.00 - 1.04 / 1.15 - 1.25 / 1.10 - 1.18 / 1.15 - 1.24 / 1.31 - 1.39, b = 16 1.03 / 1.13 / 1.03 / 1.12 / 1.51; whole
+    // lines, N = 160 / 320: b = 64 0.98 / 1.03, others 0.97; N = 96, b = 64 1.03 - 1.07.
     // (One MMA of two CTAs, cta_group::2, in their place: 16.3 for the fourth, 70 for the last: with N = 64 or 128 its
     // exchange of the other half's block rows takes longer than the product.)
     bool split = false, stack_split = false;
     auto split_fits = [&](int64_t n_tiles, int64_t longest, int64_t rows) {
         const int64_t bytes = longest * (128 + rows) * f.b * h->es;
         if (rows == f.b && h->es == 4) {
-            if (f.b == 16 && !h->col_major) return false;
-            const bool fills = 32 * n_tiles > 15 * h->n_ctas;
-            if (!fills && (f.b == 64 || (f.b == 128 && !h->col_major && bytes < (int64_t{4} << 20)))) return false;
+            const bool very_long = bytes >= int64_t{4} << 20, fills = 32 * n_tiles > (very_long ? 14 : 15) * h->n_ctas;
+            const bool even = N % 32 == 0 && !(f.b == 64 && N % 128 >= 64);
+            if (h->col_major ? f.b == 64 && !fills
+                             : even && (f.b == 16 || (!fills && (f.b == 64 || (f.b == 128 && !very_long))))) return false;
         }
         return N > 64 && 2 * n_tiles <= h->n_ctas && bytes >= kSplitMinBytes && !h->dynamic && !(h->dtype == SPMM_FP8_E4M3 && !h->col_major);
     };

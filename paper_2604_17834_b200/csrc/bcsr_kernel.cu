@@ -876,12 +876,9 @@ cudaError_t launch_tf32(int b, int groups, const BcsrMaps& tm, const BcsrParams&
         case 320: return launch_one<32, 32, 1, 8, 2, 0, CM, 0, 1>(tm, p, grid, stream);
         case 640: return launch_one<64, 64, 1, 10, 2, 0, CM, 0, 1>(tm, p, grid, stream);
         case 1280: return launch_one<128, 128, 1, 8, 2, 0, CM, 0, 1>(tm, p, grid, stream);
-        default: break;
+        case 160: return launch_one<16, 16, 1, 10, 2, 0, CM, 0, 1>(tm, p, grid, stream);
+        default: return cudaErrorInvalidValue;
     }
-    if constexpr (CM) {
-        if (b * 10 + groups == 160) return launch_one<16, 16, 1, 10, 2, 0, 1, 0, 1>(tm, p, grid, stream);
-    }
-    return cudaErrorInvalidValue;
 }
 
 template <int FMT>
