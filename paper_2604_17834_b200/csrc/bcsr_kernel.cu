@@ -378,9 +378,9 @@ bcsr_spmm_kernel(const __grid_constant__ BcsrKernelMaps<B, H, GROUPS, FMT, CT, C
             // The first tile's first units: their block columns and stored blocks belong to the handle and are
             // fetched while the launch before this one may still be running (a short launch is a chain of index,
             // request, MMA and store latencies, and the weights of a decode step come from HBM); the units' B tiles
-            // follow in the loop below.  Back to back, us: 512 x
-            // 512, N = 256 4.13 -> 3.82; both projections 18944 x 3584, bf16, N = 128 19.4 -> 17.7; 8192 x 8192,
-            // b = 16, N = 4096 222 -> 216; prefill shapes unchanged.
+            // follow in the loop below.  Back to back, us:
+            // both projections 18944 x 3584, bf16, N = 128 19.4 -> 17.7; 512 x 512, N = 256 4.12 -> 3.79 (4.21 -> 4.03
+            // on another box).
             uint32_t early = 0;
             if (!DYN && tile_begin < tile_end && rec0.w > rec0.z) {
                 Jl_next = (rec0.z + lane < rec0.w) ? __ldg(p.block_col_idx + rec0.z + lane) : 0;
