@@ -88,8 +88,10 @@ __global__ void csr_check_rows_kernel(int64_t m, const int64_t* row_ptr, int* er
             if (n <= kWarpWindow) continue;
             const int which = longer.which(n);
             if (which < kLists) {
+                // (chosen, not indexed: an index puts the parameters on the stack.  400,000 power-law rows: 8.9 -> 5.5 us)
+                int32_t* const list = which == kListBitmap ? longer.list[kListBitmap] : which == kListMerge ? longer.list[kListMerge] : longer.list[kListLarge];
                 const int at = atomicAdd(longer.count + which, 1);
-                longer.list[which][which == kListBitmap ? at : -at] = static_cast<int32_t>(i / longer.wh);
+                list[which == kListBitmap ? at : -at] = static_cast<int32_t>(i / longer.wh);
             } else if (n < (int64_t{1} << 31)) {
                 const unsigned long long one = 1ull << kLongShift, before = atomicAdd(longer.long_count, one + static_cast<unsigned long long>(pieces_of(n)));
                 const int64_t at = static_cast<int64_t>(before >> kLongShift);
